@@ -66,7 +66,7 @@ struct Profiler {
 struct UpdateWs {
     DevBuf a, b, c, d, e, f, g, h;   // flags, delete keys/ids/positions, insert keys/ids/xy/ranks
     DevBuf keys, ids, xy;            // the next sorted arrays (swapped with the index's)
-    DevBuf mark, v, t;               // deleted marks, shift counts, their exclusive scan
+    DevBuf marks, dstart, istart;    // deleted bits and counts per tile; deletes, inserts before each tile
 };
 
 }  // namespace sfc

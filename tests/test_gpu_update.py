@@ -85,3 +85,37 @@ def test_insert_into_empty_index(cuda):
     pts, qs, d = W.tiny_dense(23, 900, 100, 10, 40)
     assert sfc.sfc_update(idx, to_dev(pts, cuda), None) == 0 == dyn.apply(pts, np.zeros(0, np.int64))
     check_same(idx, dyn, qs, d, cuda)
+
+
+@pytest.mark.parametrize("n", [1, 2047, 2048, 2049, 6144, 10007])
+def test_tiles_of_the_merge(cuda, n):
+    """The merge counts deletes and inserts per tile of 2,048 entries: array sizes at a tile's
+    edges, stacked equal points over tile borders whose ids are deleted in shuffled order, inserts
+    ranked inside the stack, before every entry and after every entry, and tiles deleted whole."""
+    rng = np.random.default_rng(n)
+    pts = rng.integers(0, 1 << 12, size=(n, 2)).astype(np.int32)
+    pts[rng.permutation(n)[: n // 2]] = (2000, 2000)   # half of the points are one stack
+    qs = rng.integers(0, 1 << 12, size=(50, 2)).astype(np.int32)
+    d = rng.integers(0, 600, size=50).astype(np.int32)
+    idx = sfc.sfc_build(to_dev(pts, cuda), "z")
+    dyn = DynamicOracle(pts)
+    ends = np.array([[0, 0], [(1 << 30) - 1, (1 << 30) - 1]], np.int32)
+    for share in (0.3, 0.9):
+        live = np.nonzero(dyn.alive)[0]
+        dels = rng.permutation(live)[: int(len(live) * share)].astype(np.uint32)
+        ins = np.concatenate([ends, np.full((5, 2), 2000, np.int32),
+                              rng.integers(0, 1 << 12, size=(n // 3, 2)).astype(np.int32)])
+        first = sfc.sfc_update(idx, to_dev(ins, cuda), to_dev(dels.view(np.int32), cuda) if len(dels) else None)
+        assert first == dyn.apply(ins, dels)
+        check_same(idx, dyn, qs, d, cuda)
+    assert sfc.sfc_device_status(idx) == (0, 0)
+
+
+def test_repeated_delete_among_equal_points(cuda):
+    """A repeated id is rejected also when another id of the same coordinates lies between."""
+    pts = np.full((10, 2), 77, np.int32)
+    idx = sfc.sfc_build(to_dev(pts, cuda), "z")
+    with pytest.raises(sfc.SfcError) as e:
+        sfc.sfc_update(idx, None, to_dev(np.array([7, 3, 7], np.int32), cuda))
+    assert e.value.status == sfc.SFC_ERR_NOT_FOUND
+    assert sfc.sfc_get_sorted(idx)[0].numel() == 10
