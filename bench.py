@@ -240,10 +240,10 @@ def committed_traffic(kernel: str, workload: str):
 
 def query_rooflines(agg, scanned: int, hits: int, dim: int, hbm_peak: float, peak_kind: str,
                     workload: str = WORKLOAD, sm_count: int = 152, sm_mhz: float = 2070.0):
-    """Roofline objects of the two query passes (the small queries run inside them), the one
-    with the longer time first.  The count pass is one count_kernel launch; the write pass is
-    write_kernel, preceded by write_big_kernel for the chunks of queries split over warps
-    (its time and DRAM bytes are the two launches together).
+    """Roofline objects of the two query passes, the one with the longer time first.  The count
+    pass is one count_kernel launch; the write pass is write_kernel, followed by refilter_kernel
+    for queries whose hits found no room in the record buffer (its time and DRAM bytes are the
+    two launches together).
 
     write_kernel, bound by HBM: the method must read every reported id and write it, 8 B per
     hit (the hit mask is the two-pass implementation's own traffic and is not counted).
@@ -262,7 +262,7 @@ def query_rooflines(agg, scanned: int, hits: int, dim: int, hbm_peak: float, pea
         o = {"kernel": name, "avg_launch_ms": avg, "traffic": traffic,
              "traffic_source": rec.get("command") if traffic is not None else None}
         if name == "write_kernel":
-            o["launches"] = "write_big_kernel + write_kernel"
+            o["launches"] = "write_kernel + refilter_kernel"
         if traffic is not None:
             gbs = traffic / (avg / 1e3) / 1e9
             o.update({"dram_gbs": gbs, "dram_frac": gbs / hbm_peak, "dram_frac_nominal": gbs / NOMINAL_HBM_GBS})

@@ -98,8 +98,9 @@ typedef struct {
     int train_samples;      /* learned model: keys sampled for root training (default 16384) */
     float learning_rate;    /* learned model: Adam step size (default 0.02) */
     int chunk;              /* scan chunk in points (0 = autotuned/default 1024) */
-    int mask_budget_mb;     /* cap on the hit-mask buffer of the two-pass scan, which is sized
-                               1 KB per query (default cap 4096 MB) */
+    int mask_budget_mb;     /* cap on the buffer that carries the hits from the count pass to the
+                               write pass, sized 1 KB per query and 4 bytes per point; queries
+                               whose hits do not fit are filtered again (default cap 4096 MB) */
     int reorder_queries;    /* order in which queries are processed (outputs are unaffected):
                                0 input order, 1 curve order of the centres (queries that scan
                                overlapping ranges run together and share L2), 2 curve order once
@@ -256,10 +257,9 @@ sfc_status sfc_reserve_queries(sfc_index* idx, uint64_t m, void* stream);
 
 /* Autotuner: when the index was built with cover_refine = -1, first times whole batches
  * (count + write) under the covers 0, 1 and 2; then times the count pass (plan + scan + count)
- * of this query batch for chunk sizes {256, 512, 1024, 2048, 4096} points (threads-per-query
- * granularity of the scan), then the number of chunks taken per work-queue grab
- * {1, 2, 4, 8, 16}, then the queries per write-pass grab {1, 2, 4, 8, 16}, and keeps the
- * fastest in the index (results do not depend on them).  The choice is cached per (device,
+ * of this query batch for chunks of {256, 512, 1024, 2048, 4096} points, then for {1, 2, 4, 8,
+ * 16} work items per work-queue grab, then the write pass for {1, 2, 4, 8, 16} work items per
+ * grab, and keeps the fastest in the index (results do not depend on them).  The choice is cached per (device,
  * curve, log2 n, log2 m, bound search, cover option) for later indexes; force != 0
  * re-measures.  Writes the choice to *h_chunk, *h_batch, *h_qbatch (any may be NULL); the
  * cover is read back with sfc_cover_refine.  Synchronises `stream`; allocates temporary
@@ -268,10 +268,11 @@ sfc_status sfc_autotune(sfc_index* idx, const int32_t* d_q, const int32_t* d_del
                         int* h_chunk, int* h_batch, int* h_qbatch, void* stream);
 
 /* Sets the three scan settings that sfc_autotune chooses, without timing anything: the chunk
- * in points (32 ... 4096, a multiple of 32), the chunks per work-queue grab of the count pass
- * (batch) and the queries per grab of the write pass (qbatch), each 1 ... 1024; otherwise
+ * in points (32 ... 4096, a multiple of 32; past 1024 the count pass takes proportionally more
+ * per grab), the work items (up to 4,096 neighbouring points each) per work-queue grab of the count
+ * pass (batch) and of the write pass (qbatch), each 1 ... 1024; otherwise
  * SFC_ERR_INVALID and nothing changes.  Results do not depend on them, and a count already
- * made keeps its own chunk for its write.  For replaying a measured choice where timing it
+ * made is not changed.  For replaying a measured choice where timing it
  * again would give another (under a profiler, whose overhead changes the timings). */
 sfc_status sfc_set_tuning(sfc_index* idx, int chunk, int batch, int qbatch);
 
@@ -364,8 +365,8 @@ sfc_status sfc_model_fence(const sfc_index* idx, uint64_t* h_fence, int* h_leave
 sfc_status sfc_model_fence_fine(const sfc_index* idx, uint64_t* h_fence, int* h_leaves, void* stream);
 
 /* Work of the last query batch: points scanned (sum over queries of the interval lengths,
- * the S_q of Alg. 1's scan loop), scan chunks (queries that scan at most 64 points have none:
- * one thread scans each of them), and points reported.  Synchronises. */
+ * the S_q of Alg. 1's scan loop), scan chunks (of opt->chunk points; queries that scan at most
+ * 64 points count none), and points reported.  Synchronises. */
 sfc_status sfc_query_stats(const sfc_index* idx, uint64_t* h_scanned, uint64_t* h_chunks,
                            uint64_t* h_hits, void* stream);
 

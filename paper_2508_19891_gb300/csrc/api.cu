@@ -101,7 +101,7 @@ sfc_status ensure_status_buf(sfc_index* idx, cudaStream_t st)
 uint32_t* status_word(sfc_index* idx) { return idx->status.as<uint32_t>(); }
 // status buffer: u32 status word, padding, then u64 counters [0..2] learned-bounds
 // statistics, [3] points scanned by the last batch, [4] cover cells, [5] of them found empty
-// by the early-termination bitmap
+// by the early-termination bitmap, [6] scan chunks
 unsigned long long* model_stats(sfc_index* idx)
 {
     return reinterpret_cast<unsigned long long*>(idx->status.as<unsigned char>() + 16);
@@ -113,7 +113,7 @@ sfc_status build_from_device(sfc_index* idx, const int32_t* d_points, cudaStream
     const uint64_t n = idx->n;
     SFC_TRY(idx->keys.ensure(n * sizeof(uint64_t), st));
     SFC_TRY(idx->ids.ensure(n * sizeof(uint32_t), st));
-    SFC_TRY(idx->xy.ensure(n * sizeof(int2), st));
+    SFC_TRY(idx->xy.ensure(pad_groups(n) * sizeof(int2), st));
     SortSource src;
     src.points = reinterpret_cast<const int2*>(d_points);
     src.curve = idx->curve;
@@ -125,6 +125,10 @@ sfc_status build_from_device(sfc_index* idx, const int32_t* d_points, cudaStream
     {
         ProfScope ps(idx, "sort", st);
         SFC_TRY(radix_sort(src, n, dst, idx->sort_ws, status_word(idx), st));
+    }
+    {
+        ProfScope ps(idx, "boxes", st);
+        SFC_TRY(build_boxes(idx, st));
     }
     if (idx->opt.occupancy_depth > 0) {
         ProfScope ps(idx, "occupancy", st);
@@ -146,7 +150,7 @@ sfc_status build3_from_device(sfc_index* idx, const int32_t* d_points, cudaStrea
     const uint64_t n = idx->n;
     SFC_TRY(idx->keys.ensure(n * sizeof(uint64_t), st));
     SFC_TRY(idx->ids.ensure(n * sizeof(uint32_t), st));
-    SFC_TRY(idx->xyz.ensure(n * sizeof(int4), st));
+    SFC_TRY(idx->xyz.ensure(pad_groups(n) * sizeof(int4), st));
     SFC_TRY(idx->keys_in.ensure(n * sizeof(uint64_t), st));
     ProfScope ps(idx, "sort", st);
     SFC_TRY(launch_keys3(d_points, n, idx->keys_in.as<uint64_t>(), status_word(idx), st));
@@ -157,6 +161,7 @@ sfc_status build3_from_device(sfc_index* idx, const int32_t* d_points, cudaStrea
     dst.vals = idx->ids.as<uint32_t>();
     SFC_TRY(radix_sort(src, n, dst, idx->sort_ws, status_word(idx), st));
     SFC_TRY(launch_decode3(idx->keys.as<uint64_t>(), n, idx->xyz.as<int4>(), st));
+    SFC_TRY(build_boxes(idx, st));
     idx->next_id = (uint32_t)n;
     return SFC_OK;
 }
@@ -178,6 +183,7 @@ QueryArgs base_args(sfc_index* idx, const int32_t* q, const int32_t* delta, uint
     a.norm = idx->norm;
     a.dim = idx->dim;
     a.xyz = idx->xyz.as<int4>();
+    a.box = idx->box.as<int4>();
     if (idx->opt.occupancy_depth > 0 && idx->occ.ptr) {
         a.occ = idx->occ.as<uint32_t>();
         a.occ_depth = idx->opt.occupancy_depth;
@@ -186,33 +192,40 @@ QueryArgs base_args(sfc_index* idx, const int32_t* q, const int32_t* delta, uint
     return a;
 }
 
-sfc_status ensure_query_ws(sfc_index* idx, uint64_t m, cudaStream_t st)
+// Bytes for the hits of a batch of m queries over n points: 1 KB per query (about 100 records and
+// 9 batches of 32 items), and 4 bytes per point so that a few queries over large parts of the
+// array fit too; capped by mask_budget_mb.  A quarter goes to the batches, the rest to the
+// records.  Items past either are filtered again by the write pass.
+constexpr uint64_t kBatchBytes = sizeof(uint4) + sizeof(uint32_t) + sizeof(uint64_t);
+
+sfc_status ensure_query_ws(sfc_index* idx, uint64_t m, uint64_t n, cudaStream_t st)
 {
     QueryWs& w = idx->qws;
-    SFC_TRY(w.ranges.ensure(m * 2 * query_intervals(idx->dim, idx->drop) * sizeof(uint32_t), st));
-    SFC_TRY(w.nchunks.ensure(m * sizeof(uint32_t), st));
-    SFC_TRY(w.chunk_base.ensure((m + 1) * sizeof(uint64_t), st));
+    const uint64_t kint = (uint64_t)query_intervals(idx->dim, idx->drop);
+    SFC_TRY(w.ranges.ensure(m * kint * sizeof(uint2), st));
+    SFC_TRY(w.qrec.ensure(m * sizeof(int4), st));
+    SFC_TRY(w.nitems.ensure(m * sizeof(uint32_t), st));
+    SFC_TRY(w.gbase.ensure((m + 1) * sizeof(uint64_t), st));
+    SFC_TRY(w.ovf.ensure(m, st));
     SFC_TRY(w.counts.ensure(m * sizeof(uint32_t), st));
     SFC_TRY(w.ctr.ensure(kCtrWords * sizeof(unsigned long long), st));
-    SFC_TRY(w.small_list.ensure(m * sizeof(uint32_t), st));
-    SFC_TRY(w.small_mask.ensure(m * kSmallWords * sizeof(unsigned long long), st));
-    SFC_TRY(w.chunk_hits.ensure((kChunkHitsPerQuery * m + 1024) * sizeof(uint32_t), st));
-    SFC_TRY(w.big_items.ensure((kChunkHitsPerQuery * m + 1024) * sizeof(uint32_t), st));
-    SFC_TRY(w.big_list.ensure(m * sizeof(uint32_t), st));
     if (idx->opt.reorder_queries != 0 && idx->dim == 2) {
         SFC_TRY(w.qkeys.ensure(m * sizeof(uint64_t), st));
         SFC_TRY(w.qkeys_sorted.ensure(m * sizeof(uint64_t), st));
         SFC_TRY(w.perm.ensure(m * sizeof(uint32_t), st));
-        SFC_TRY(w.nch_sorted.ensure(m * sizeof(uint32_t), st));
-        SFC_TRY(w.wbase.ensure((m + 1) * sizeof(uint64_t), st));
+        SFC_TRY(w.pstart.ensure(m * sizeof(uint32_t), st));
+        SFC_TRY(w.dbase.ensure(m * sizeof(uint64_t), st));
         SFC_TRY(reserve_sort(idx->sort_ws, std::max<uint64_t>(m, 1), st));
     }
     const uint64_t budget = (uint64_t)idx->opt.mask_budget_mb << 20;
-    // one bit per scanned point: 1 KB per query covers batches whose mean scan is up to 8,192
-    // points; chunks past the buffer are re-filtered by the write pass
-    uint64_t want = m * 1024ull + (1ull << 20);
-    if (want > budget) want = budget;
-    if (w.masks.bytes < want) SFC_TRY(w.masks.ensure(want, st));
+    const uint64_t bytes = std::min<uint64_t>(budget, m * 1024ull + (1ull << 20) + 4 * n);
+    const uint64_t batches = std::min<uint64_t>(bytes / 4 / kBatchBytes, max_batches(idx->dim, m, n, kint));
+    const uint64_t recs = std::min<uint64_t>(bytes / 4 * 3 / sizeof(uint2), 64 * item_groups(idx->dim) * max_batches(idx->dim, m, n, kint) + (1ull << 23));
+    SFC_TRY(w.heads.ensure(batches * sizeof(uint4), st));
+    SFC_TRY(w.bhits.ensure(batches * sizeof(uint32_t), st));
+    SFC_TRY(w.bbase.ensure((batches + 1) * sizeof(uint64_t), st));
+    SFC_TRY(w.recs.ensure(recs * sizeof(uint2), st));
+    SFC_TRY(reserve_scan(idx->scan_ws, std::max<uint64_t>(m, batches + batches / 8 + 64), st));
     return SFC_OK;
 }
 
@@ -236,46 +249,52 @@ bool use_curve_order(const sfc_index* idx, uint64_t m)
     return idx->n >= (1ull << 24);
 }
 
-// The chunk hit counts of big queries (count pass) and their in-query offsets (write pass).
-void set_big_queries(QueryWs& w, QueryArgs& a)
+// The query workspace's buffers and settings of a batch of m queries (count and write pass).
+void set_workspace(sfc_index* idx, QueryArgs& a)
 {
-    a.chunk_hits = w.chunk_hits.as<uint32_t>();
-    a.big_items = w.big_items.as<uint32_t>();
-    a.big_list = w.big_list.as<uint32_t>();
-    a.big_cap = std::min<uint64_t>(std::min(w.chunk_hits.bytes, w.big_items.bytes) / sizeof(uint32_t), a.mask_chunks);
-    a.big_warps = (uint32_t)num_sms() * 64u * kBigShare;
+    QueryWs& w = idx->qws;
+    a.ranges = w.ranges.as<uint2>();
+    a.qrec = w.qrec.as<int4>();
+    a.nitems = w.nitems.as<uint32_t>();
+    a.gbase = w.gbase.as<uint64_t>();
+    a.ovf = w.ovf.as<uint8_t>();
+    a.counts = w.counts.as<uint32_t>();
+    a.heads = w.heads.as<uint4>();
+    a.bhits = w.bhits.as<uint32_t>();
+    a.bbase = w.bbase.as<uint64_t>();
+    a.cap_batches = std::min<uint64_t>({w.heads.bytes / sizeof(uint4), w.bhits.bytes / sizeof(uint32_t),
+                              w.bbase.bytes / sizeof(uint64_t) - 1});
+    a.recs = w.recs.as<uint2>();
+    a.cap_recs = std::min<uint64_t>(w.recs.bytes / sizeof(uint2), 0xffffffffull);
+    // records a warp reserves at a time (a batch has up to 32 item_groups): large while an eighth
+    // of the buffer covers every warp's
+    const uint64_t warps = (uint64_t)num_sms() * 64;
+    a.slab = a.cap_recs >= warps * 512 * 8 ? 512 : (uint32_t)(32 * item_groups(idx->dim));
+    a.cgrab = idx->batch * std::max(1u, idx->chunk / 1024);
+    a.wgrab = idx->qbatch;
+    a.work_ctr = w.ctr.as<unsigned long long>();
 }
 
+// slices > 1: a curve-ordered batch is processed slice by slice of the input (see
+// sfc_query_batch_host), in curve order inside each.
 sfc_status do_count(sfc_index* idx, const int32_t* d_q, const int32_t* d_delta, uint64_t m,
-                    uint64_t* d_out_offsets, cudaStream_t st)
+                    uint64_t* d_out_offsets, cudaStream_t st, int slices = 1)
 {
     SFC_TRY(ensure_status_buf(idx, st));
     if (m == 0) {
         SFC_CUDA_TRY(cudaMemsetAsync(d_out_offsets, 0, sizeof(uint64_t), st));
-        idx->qws.pending = {true, d_q, d_delta, 0, d_out_offsets, 0, false, idx->drop, idx->norm};
+        idx->qws.pending = {true, d_q, d_delta, 0, d_out_offsets, false, idx->drop, idx->norm};
         return SFC_OK;
     }
-    SFC_TRY(ensure_query_ws(idx, m, st));
+    SFC_TRY(ensure_query_ws(idx, m, idx->n, st));
     QueryWs& w = idx->qws;
     QueryArgs a = base_args(idx, d_q, d_delta, m);
-    a.ranges = w.ranges.as<uint32_t>();
-    a.nchunks = w.nchunks.as<uint32_t>();
-    a.chunk_base = w.chunk_base.as<uint64_t>();
-    a.counts = w.counts.as<uint32_t>();
-    a.masks = w.masks.as<uint32_t>();
+    set_workspace(idx, a);
     a.chunk = idx->chunk;
-    a.mask_chunks = w.masks.bytes / (a.chunk / 8);
-    set_big_queries(w, a);
-    a.batch = idx->batch;
-    a.qbatch = idx->qbatch;
-    a.work_ctr = w.ctr.as<unsigned long long>();
-    a.small_list = w.small_list.as<uint32_t>();
-    a.small_mask = w.small_mask.as<unsigned long long>();
     a.out_offsets = d_out_offsets;
     a.scanned = scan_stats(idx);
-    // per-batch statistics: learned-bounds counters and the scanned total
-    SFC_CUDA_TRY(cudaMemsetAsync(model_stats(idx), 0, 6 * sizeof(unsigned long long), st));
-    SFC_CUDA_TRY(cudaMemsetAsync(a.counts, 0, m * sizeof(uint32_t), st));
+    // per-batch statistics: learned-bounds counters, the scanned total, cells and chunks
+    SFC_CUDA_TRY(cudaMemsetAsync(model_stats(idx), 0, 7 * sizeof(unsigned long long), st));
     SFC_CUDA_TRY(cudaMemsetAsync(a.work_ctr, 0, kCtrWords * sizeof(unsigned long long), st));
     LearnedModelView lv;
     const bool ordered = use_curve_order(idx, m);
@@ -283,7 +302,7 @@ sfc_status do_count(sfc_index* idx, const int32_t* d_q, const int32_t* d_delta, 
         // processing order: queries sorted by the curve key of their centre, so that queries
         // scanning overlapping ranges run close together and share the cache
         ProfScope ps(idx, "order", st);
-        SFC_TRY(launch_query_keys(d_q, m, idx->curve, w.qkeys.as<uint64_t>(), st));
+        SFC_TRY(launch_query_keys(d_q, m, idx->curve, slices, w.qkeys.as<uint64_t>(), st));
         SortSource src;
         src.keys = w.qkeys.as<uint64_t>();
         SortDest dst;
@@ -291,7 +310,9 @@ sfc_status do_count(sfc_index* idx, const int32_t* d_q, const int32_t* d_delta, 
         dst.vals = w.perm.as<uint32_t>();
         dst.curve = idx->curve;
         SFC_TRY(radix_sort(src, m, dst, idx->sort_ws, a.status, st));
-        a.perm = w.perm.as<uint32_t>();   // the plan already runs in processing order
+        a.perm = w.perm.as<uint32_t>();
+        a.pstart = w.pstart.as<uint32_t>();
+        a.dbase = w.dbase.as<uint64_t>();
     }
     {
         ProfScope ps(idx, "plan", st);
@@ -299,13 +320,7 @@ sfc_status do_count(sfc_index* idx, const int32_t* d_q, const int32_t* d_delta, 
     }
     {
         ProfScope ps(idx, "scan", st);
-        SFC_TRY(exclusive_scan_u32(a.nchunks, m, a.chunk_base, idx->scan_ws, a.status, st));
-        if (ordered) {
-            SFC_TRY(launch_gather_u32(a.nchunks, w.perm.as<uint32_t>(), m, w.nch_sorted.as<uint32_t>(), st));
-            SFC_TRY(exclusive_scan_u32(w.nch_sorted.as<uint32_t>(), m, w.wbase.as<uint64_t>(), idx->scan_ws,
-                                       a.status, st));
-            a.wbase = w.wbase.as<uint64_t>();
-        }
+        SFC_TRY(exclusive_scan_u32(a.nitems, m, a.gbase, idx->scan_ws, a.status, st));
     }
     {
         ProfScope ps(idx, "count", st);
@@ -313,48 +328,37 @@ sfc_status do_count(sfc_index* idx, const int32_t* d_q, const int32_t* d_delta, 
     }
     {
         ProfScope ps(idx, "scan", st);
+        SFC_TRY(exclusive_scan_u32(a.bhits, std::min<uint64_t>(a.cap_batches, max_batches(idx->dim, m, idx->n, a.kint)), a.bbase,
+                                   idx->scan_ws, a.status, st, a.gbase + m));
         SFC_TRY(exclusive_scan_u32(a.counts, m, d_out_offsets, idx->scan_ws, a.status, st));
-        SFC_TRY(launch_chunk_prefix(a, st));
+        SFC_TRY(launch_dbase(a, st));
     }
-    w.pending = {true, d_q, d_delta, m, d_out_offsets, a.chunk, ordered, a.drop, a.norm};
+    w.pending = {true, d_q, d_delta, m, d_out_offsets, ordered, a.drop, a.norm};
     return SFC_OK;
 }
 
-// The write pass for the queries [q_begin, q_end) of the pending count (no state checks).
+// The write pass for the processing ranks [q_begin, q_end) of the pending count (no state checks).
 sfc_status do_write_range(sfc_index* idx, const int32_t* d_q, const int32_t* d_delta, uint64_t m,
                           const uint64_t* d_out_offsets, uint32_t* d_out_ids, uint64_t cap, cudaStream_t st,
-                          uint64_t q_begin, uint64_t q_end, const uint32_t* perm = nullptr)
+                          uint64_t q_begin, uint64_t q_end)
 {
     QueryWs& w = idx->qws;
     QueryArgs a = base_args(idx, d_q, d_delta, m);
     a.drop = w.pending.drop;
     a.kint = (uint32_t)query_intervals(idx->dim, a.drop);
     a.norm = w.pending.norm;
-    a.ranges = w.ranges.as<uint32_t>();
-    a.nchunks = w.nchunks.as<uint32_t>();
-    a.chunk_base = w.chunk_base.as<uint64_t>();
-    a.counts = w.counts.as<uint32_t>();
-    a.masks = w.masks.as<uint32_t>();
-    a.chunk = w.pending.chunk;
-    a.mask_chunks = w.masks.bytes / (a.chunk / 8);
-    set_big_queries(w, a);
-    a.batch = idx->batch;
-    a.qbatch = idx->qbatch;
-    a.work_ctr = w.ctr.as<unsigned long long>();
-    a.small_list = w.small_list.as<uint32_t>();
-    a.small_mask = w.small_mask.as<unsigned long long>();
+    set_workspace(idx, a);
     a.out_offsets = const_cast<uint64_t*>(d_out_offsets);
     a.out_ids = d_out_ids;
     if (w.pending.ordered) {
-        a.perm = perm ? perm : w.perm.as<uint32_t>();
-        a.wbase = w.wbase.as<uint64_t>();
+        a.perm = w.perm.as<uint32_t>();
+        a.dbase = w.dbase.as<uint64_t>();
     }
     a.ids_capacity = d_out_ids ? cap : 0;
     a.q_begin = q_begin;
     a.q_end = q_end;
-    // the write pass's own work counters start at zero (a repeated write stays correct)
-    SFC_CUDA_TRY(cudaMemsetAsync(a.work_ctr + kCtrWrite, 0, 2 * sizeof(unsigned long long), st));
-    SFC_CUDA_TRY(cudaMemsetAsync(a.work_ctr + kCtrWriteBig, 0, sizeof(unsigned long long), st));
+    // the write pass's own work counter starts at zero (a repeated write stays correct)
+    SFC_CUDA_TRY(cudaMemsetAsync(a.work_ctr + kCtrWrite, 0, sizeof(unsigned long long), st));
     ProfScope ps(idx, "write", st);
     return launch_write(a, st);
 }
@@ -518,17 +522,18 @@ sfc_status sfc_reserve(sfc_index* idx, uint64_t n_max, uint64_t m_max, void* str
     SFC_TRY(idx->keys.ensure(n1 * sizeof(uint64_t), st));
     SFC_TRY(idx->ids.ensure(n1 * sizeof(uint32_t), st));
     if (idx->dim == 3) {
-        SFC_TRY(idx->xyz.ensure(n1 * sizeof(int4), st));
+        SFC_TRY(idx->xyz.ensure(pad_groups(n1) * sizeof(int4), st));
         SFC_TRY(idx->keys_in.ensure(n1 * sizeof(uint64_t), st));
     } else {
-        SFC_TRY(idx->xy.ensure(n1 * sizeof(int2), st));
+        SFC_TRY(idx->xy.ensure(pad_groups(n1) * sizeof(int2), st));
         SFC_TRY(idx->xy_by_id.ensure(n1 * sizeof(int2), st));
         SFC_TRY(ensure_alive_bits(idx, n1, st));
     }
     if (idx->opt.occupancy_depth > 0)
         SFC_TRY(idx->occ.ensure(occupancy_words(idx->opt.occupancy_depth) * sizeof(uint32_t), st));
     SFC_TRY(reserve_sort(idx->sort_ws, n1, st));
-    SFC_TRY(ensure_query_ws(idx, m_max, st));
+    SFC_TRY(idx->box.ensure(box_bytes(idx->dim, n1), st));
+    SFC_TRY(ensure_query_ws(idx, m_max, n1, st));
     SFC_TRY(reserve_scan(idx->scan_ws, std::max<uint64_t>(m_max, n1) + 1, st));
     if (idx->opt.bounds == SFC_BOUNDS_LEARNED) SFC_TRY(reserve_model(idx, n1, st));
     return SFC_OK;
@@ -858,7 +863,8 @@ sfc_status sfc_query_batch_host(sfc_index* idx, const int32_t* h_q, const int32_
         SFC_CUDA_TRY(cudaMemcpyAsync(dq, h_q, qbytes, cudaMemcpyHostToDevice, st));
         SFC_CUDA_TRY(cudaMemcpyAsync(dd, h_delta, m * sizeof(int32_t), cudaMemcpyHostToDevice, st));
     }
-    SFC_TRY(do_count(idx, dq, dd, m, doff, st));
+    const int S = HostStage::kSlices;
+    SFC_TRY(do_count(idx, dq, dd, m, doff, st, m >= (uint64_t)S ? S : 1));
     SFC_CUDA_TRY(cudaMemcpyAsync(h_out_offsets, doff, (m + 1) * sizeof(uint64_t), cudaMemcpyDeviceToHost, st));
     SFC_CUDA_TRY(cudaStreamSynchronize(st));
     const uint64_t total = h_out_offsets[m];
@@ -868,29 +874,10 @@ sfc_status sfc_query_batch_host(sfc_index* idx, const int32_t* h_q, const int32_
     }
     SFC_TRY(hs.ids.ensure(total * sizeof(uint32_t), st));
     uint32_t* d_ids = hs.ids.as<uint32_t>();
-    const int S = HostStage::kSlices;
     if (m >= (uint64_t)S && total * sizeof(uint32_t) >= (32ull << 20)) {
         // the write pass in query slices; the ids of each finished slice go out on a second
-        // stream while the next slices are written (output offsets are in query order)
-        const uint32_t* sperm = nullptr;
-        if (idx->qws.pending.ordered) {
-            // curve order: regroup the processing order by input slice (a stable one-digit sort
-            // of the slice numbers), so slice s is positions [floor(m s / S), floor(m (s + 1) / S))
-            // and keeps curve order inside
-            SFC_TRY(hs.slice_keys.ensure(m * sizeof(uint64_t), st));
-            SFC_TRY(hs.slice_keys_sorted.ensure(m * sizeof(uint64_t), st));
-            SFC_TRY(hs.slice_perm.ensure(m * sizeof(uint32_t), st));
-            const uint32_t* perm = idx->qws.perm.as<uint32_t>();
-            SFC_TRY(launch_slice_keys(perm, m, S, hs.slice_keys.as<uint64_t>(), st));
-            SortSource src;
-            src.keys = hs.slice_keys.as<uint64_t>();
-            src.vals = perm;
-            SortDest dst;
-            dst.keys = hs.slice_keys_sorted.as<uint64_t>();
-            dst.vals = hs.slice_perm.as<uint32_t>();
-            SFC_TRY(radix_sort(src, m, dst, idx->sort_ws, status_word(idx), st));
-            sperm = hs.slice_perm.as<uint32_t>();
-        }
+        // stream while the next slices are written (output offsets are in query order; a curve
+        // order runs inside the slices, so slice s is ranks [floor(m s / S), floor(m (s + 1) / S)))
         if (!hs.copy) {
             SFC_CUDA_TRY(cudaStreamCreateWithFlags(&hs.copy, cudaStreamNonBlocking));
             for (auto& e : hs.done) SFC_CUDA_TRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
@@ -898,7 +885,7 @@ sfc_status sfc_query_batch_host(sfc_index* idx, const int32_t* h_q, const int32_
         idx->qws.pending.valid = false;
         for (int sl = 0; sl < S; ++sl) {
             const uint64_t qa = m * (uint64_t)sl / S, qb = m * (uint64_t)(sl + 1) / S;
-            SFC_TRY(do_write_range(idx, dq, dd, m, doff, d_ids, total, st, qa, qb, sperm));
+            SFC_TRY(do_write_range(idx, dq, dd, m, doff, d_ids, total, st, qa, qb));
             SFC_CUDA_TRY(cudaEventRecord(hs.done[sl], st));
             SFC_CUDA_TRY(cudaStreamWaitEvent(hs.copy, hs.done[sl], 0));
             const uint64_t a = h_out_offsets[qa], b = h_out_offsets[qb];
@@ -922,7 +909,7 @@ sfc_status sfc_reserve_queries(sfc_index* idx, uint64_t m, void* stream)
     if (!idx) return SFC_ERR_INVALID;
     AllocScope alloc_scope(idx->allocator());
     SFC_TRY(ensure_status_buf(idx, as_stream(stream)));
-    return ensure_query_ws(idx, m, as_stream(stream));
+    return ensure_query_ws(idx, m, idx->n, as_stream(stream));
 }
 
 sfc_status sfc_set_bounds_mode(sfc_index* idx, sfc_bounds mode)
@@ -1006,18 +993,15 @@ sfc_status sfc_query_stats(const sfc_index* cidx, uint64_t* h_scanned, uint64_t*
     sfc_index* idx = const_cast<sfc_index*>(cidx);
     if (!idx || !idx->status.ptr) return SFC_ERR_INVALID;
     cudaStream_t st = as_stream(stream);
-    unsigned long long s = 0;
-    uint64_t g = 0, h = 0;
-    SFC_CUDA_TRY(cudaMemcpyAsync(&s, scan_stats(idx), sizeof(s), cudaMemcpyDeviceToHost, st));
+    unsigned long long s[4] = {0, 0, 0, 0};
+    uint64_t h = 0;
+    SFC_CUDA_TRY(cudaMemcpyAsync(s, scan_stats(idx), sizeof(s), cudaMemcpyDeviceToHost, st));
     const PendingCount& p = idx->qws.pending;
-    if (p.m && idx->qws.chunk_base.ptr)
-        SFC_CUDA_TRY(cudaMemcpyAsync(&g, idx->qws.chunk_base.as<uint64_t>() + p.m, sizeof(g),
-                                     cudaMemcpyDeviceToHost, st));
     if (p.m && p.offsets)
         SFC_CUDA_TRY(cudaMemcpyAsync(&h, p.offsets + p.m, sizeof(h), cudaMemcpyDeviceToHost, st));
     SFC_CUDA_TRY(cudaStreamSynchronize(st));
-    if (h_scanned) *h_scanned = s;
-    if (h_chunks) *h_chunks = g;
+    if (h_scanned) *h_scanned = s[0];
+    if (h_chunks) *h_chunks = p.m ? s[3] : 0;
     if (h_hits) *h_hits = h;
     return SFC_OK;
 }

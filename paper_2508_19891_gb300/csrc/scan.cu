@@ -36,9 +36,9 @@ __device__ __forceinline__ uint64_t warp_incl_scan(uint64_t v)
 }
 
 __global__ void __launch_bounds__(kThreads)
-scan_kernel(const uint32_t* __restrict__ in, uint64_t n, uint64_t* __restrict__ out,
-            uint64_t* flags /* [0] = tile counter, [1 + t] = tile words */, uint32_t* status,
-            int vec)
+scan_kernel(const uint32_t* __restrict__ in, uint64_t n, const uint64_t* __restrict__ per32,
+            uint64_t* __restrict__ out, uint64_t* flags /* [0] = tile counter, [1 + t] = tile words */,
+            uint32_t* status, int vec)
 {
     __shared__ uint32_t s_tile;
     __shared__ uint64_t s_warp[kThreads / 32];
@@ -47,6 +47,8 @@ scan_kernel(const uint32_t* __restrict__ in, uint64_t n, uint64_t* __restrict__ 
     if (tid == 0) s_tile = atomicAdd(reinterpret_cast<unsigned long long*>(flags), 1ull);
     __syncthreads();
     const uint64_t tile = s_tile;
+    if (per32) n = min(n, (*per32 + 31) >> 5);   // the length lives on the device
+    if (tile * kTile >= n) return;
     const uint64_t base = tile * kTile + (uint64_t)tid * kItems;
 
     uint32_t v[kItems];
@@ -138,7 +140,7 @@ sfc_status reserve_scan(ScanWorkspace& ws, uint64_t n, cudaStream_t st)
 }
 
 sfc_status exclusive_scan_u32(const uint32_t* in, uint64_t n, uint64_t* out, ScanWorkspace& ws,
-                              uint32_t* status, cudaStream_t st)
+                              uint32_t* status, cudaStream_t st, const uint64_t* per32)
 {
     if (n == 0) {
         SFC_CUDA_TRY(cudaMemsetAsync(out, 0, sizeof(uint64_t), st));
@@ -149,7 +151,7 @@ sfc_status exclusive_scan_u32(const uint32_t* in, uint64_t n, uint64_t* out, Sca
     SFC_TRY(ws.flags.ensure((tiles + 1) * sizeof(uint64_t), st));
     SFC_CUDA_TRY(cudaMemsetAsync(ws.flags.ptr, 0, (tiles + 1) * sizeof(uint64_t), st));
     int vec = ((((uintptr_t)in) & 15) == 0) && ((((uintptr_t)out) & 15) == 0);
-    scan_kernel<<<(unsigned)tiles, kThreads, 0, st>>>(in, n, out, ws.flags.as<uint64_t>(), status, vec);
+    scan_kernel<<<(unsigned)tiles, kThreads, 0, st>>>(in, n, per32, out, ws.flags.as<uint64_t>(), status, vec);
     count_launch();
     return launch_status();
 }
@@ -173,7 +175,7 @@ sfc_status exclusive_scan_standalone(const uint32_t* in, uint64_t n, uint64_t* o
     if (cudaMemsetAsync(words, 0, (tiles + 2) * sizeof(uint64_t), st) != cudaSuccess) s = SFC_ERR_CUDA;
     if (s == SFC_OK) {
         const int vec = ((((uintptr_t)in) & 15) == 0) && ((((uintptr_t)out) & 15) == 0);
-        scan_kernel<<<(unsigned)tiles, kThreads, 0, st>>>(in, n, out, words + 1, reinterpret_cast<uint32_t*>(words),
+        scan_kernel<<<(unsigned)tiles, kThreads, 0, st>>>(in, n, nullptr, out, words + 1, reinterpret_cast<uint32_t*>(words),
                                                           vec);
         count_launch();
         s = launch_status();
@@ -283,7 +285,7 @@ extern "C" sfc_status sfc_exclusive_scan_noalloc(const uint32_t* d_in, uint64_t 
         return SFC_OK;
     }
     const int vec = ((((uintptr_t)d_in) & 15) == 0) && ((((uintptr_t)d_out) & 15) == 0);
-    scan_kernel<<<(unsigned)tiles, kThreads, 0, st>>>(d_in, n, d_out, words + 1, reinterpret_cast<uint32_t*>(words),
+    scan_kernel<<<(unsigned)tiles, kThreads, 0, st>>>(d_in, n, nullptr, d_out, words + 1, reinterpret_cast<uint32_t*>(words),
                                                       vec);
     count_launch();
     return launch_status();

@@ -44,6 +44,10 @@ inline sfc_status launch_status()
 
 int num_sms();   // SM count of the current device (cached per device)
 
+// Points that a coordinate array has room for: whole groups of 32, so that a group can be loaded
+// without a bounds check (what lies past the last point is never used).
+inline uint64_t pad_groups(uint64_t n) { return (n + 31) / 32 * 32; }
+
 // First bit of depth t in the early-termination bitmap (depths stored one after another).
 __host__ __device__ __forceinline__ uint64_t occupancy_level_start(int t)
 {
@@ -404,12 +408,13 @@ sfc_status launch_decode(const uint64_t* keys, uint64_t n, int curve, int2* pts,
 sfc_status launch_keys3(const int32_t* pts, uint64_t n, uint64_t* keys, uint32_t* status, cudaStream_t st);
 sfc_status launch_decode3(const uint64_t* keys, uint64_t n, int4* xyz, cudaStream_t st);
 
-// scan.cu: exclusive scan of uint32 (or a uint32 view) into uint64[n+1].
+// scan.cu: exclusive scan of uint32 (or a uint32 view) into uint64[n+1]; with per32 (device), of
+// the first min(n, ceil(*per32 / 32)) elements only.
 struct ScanWorkspace {
     DevBuf flags;
 };
 sfc_status exclusive_scan_u32(const uint32_t* in, uint64_t n, uint64_t* out, ScanWorkspace& ws,
-                              uint32_t* status, cudaStream_t st);
+                              uint32_t* status, cudaStream_t st, const uint64_t* per32 = nullptr);
 sfc_status reserve_scan(ScanWorkspace& ws, uint64_t n, cudaStream_t st);
 // the same with its own workspace and status word; synchronises st and returns
 // SFC_ERR_TIMEOUT if a look-back wait gave up

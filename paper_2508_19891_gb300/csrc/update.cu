@@ -245,19 +245,18 @@ void release_index(sfc_index* idx, cudaStream_t st)
     idx->alive.release(st);
     idx->status.release(st);
     idx->occ.release(st);
+    idx->box.release(st);
     idx->xyz.release(st);
     idx->keys_in.release(st);
     release_sort_ws(idx->sort_ws, st);
     idx->scan_ws.flags.release(st);
     QueryWs& q = idx->qws;
-    q.ranges.release(st); q.nchunks.release(st); q.chunk_base.release(st);
-    q.counts.release(st); q.masks.release(st); q.ctr.release(st);
-    q.qkeys.release(st); q.qkeys_sorted.release(st); q.perm.release(st);
-    q.nch_sorted.release(st); q.wbase.release(st); q.small_list.release(st); q.small_mask.release(st);
-    q.chunk_hits.release(st); q.big_items.release(st); q.big_list.release(st);
+    for (DevBuf* d : {&q.ranges, &q.qrec, &q.nitems, &q.gbase, &q.ovf, &q.counts, &q.ctr, &q.heads, &q.bhits, &q.bbase,
+                      &q.recs, &q.qkeys, &q.qkeys_sorted, &q.perm, &q.pstart, &q.dbase})
+        d->release(st);
     HostStage& h = idx->stage;
     h.q.release(st); h.delta.release(st); h.offsets.release(st); h.ids.release(st);
-    h.points.release(st); h.slice_keys.release(st); h.slice_keys_sorted.release(st); h.slice_perm.release(st);
+    h.points.release(st);
     if (h.copy) {
         cudaStreamSynchronize(h.copy);
         cudaStreamDestroy(h.copy);
@@ -360,7 +359,7 @@ sfc_status apply_update(sfc_index* idx, const int32_t* d_inserts, uint64_t k_ins
     const uint64_t new_n = (uint64_t)n - k_del + k_ins;
     SFC_TRY(U.keys.ensure(std::max<uint64_t>(new_n, 1) * 8, st));
     SFC_TRY(U.ids.ensure(std::max<uint64_t>(new_n, 1) * 4, st));
-    SFC_TRY(U.xy.ensure(std::max<uint64_t>(new_n, 1) * 8, st));
+    SFC_TRY(U.xy.ensure(pad_groups(std::max<uint64_t>(new_n, 1)) * 8, st));
     SFC_TRY(U.istart.ensure(((size_t)tiles + 1) * sizeof(uint32_t), st));
     uint32_t* istart = U.istart.as<uint32_t>();
     const uint64_t* keys = idx->keys.as<uint64_t>();
@@ -413,6 +412,7 @@ sfc_status apply_update(sfc_index* idx, const int32_t* d_inserts, uint64_t k_ins
     if (h_first) *h_first = next_id;
     idx->qws.pending.valid = false;
     SFC_TRY(build_occupancy(idx, st));
+    SFC_TRY(build_boxes(idx, st));
     if (idx->model.trained) {
         const int steps = std::max(20, idx->opt.train_steps / 5);
         SFC_TRY(refit_model(idx, steps, st));
