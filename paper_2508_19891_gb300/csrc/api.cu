@@ -117,6 +117,7 @@ sfc_status build_from_device(sfc_index* idx, const int32_t* d_points, cudaStream
     SortSource src;
     src.points = reinterpret_cast<const int2*>(d_points);
     src.curve = idx->curve;
+    src.bits = 2 * kOmega;
     SortDest dst;
     dst.keys = idx->keys.as<uint64_t>();
     dst.vals = idx->ids.as<uint32_t>();
@@ -156,6 +157,7 @@ sfc_status build3_from_device(sfc_index* idx, const int32_t* d_points, cudaStrea
     SFC_TRY(launch_keys3(d_points, n, idx->keys_in.as<uint64_t>(), status_word(idx), st));
     SortSource src;
     src.keys = idx->keys_in.as<uint64_t>();
+    src.bits = 3 * kOmega3;
     SortDest dst;
     dst.keys = idx->keys.as<uint64_t>();
     dst.vals = idx->ids.as<uint32_t>();
@@ -305,6 +307,8 @@ sfc_status do_count(sfc_index* idx, const int32_t* d_q, const int32_t* d_delta, 
         SFC_TRY(launch_query_keys(d_q, m, idx->curve, slices, w.qkeys.as<uint64_t>(), st));
         SortSource src;
         src.keys = w.qkeys.as<uint64_t>();
+        src.bits = slices > 1 ? 32 : 24;   // launch_query_keys: 24 bits, and the slice above
+        src.partial = false;
         SortDest dst;
         dst.keys = w.qkeys_sorted.as<uint64_t>();
         dst.vals = w.perm.as<uint32_t>();

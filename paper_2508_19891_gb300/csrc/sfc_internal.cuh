@@ -105,38 +105,49 @@ struct DevBuf {
 
 // Z-curve (Alg. 2): x's bit i goes to key bit 2i, y's bit i to key bit 2i + 1.  Done with
 // the magic-mask spread instead of a per-bit loop: each step doubles the gap between
-// groups of bits.
+// groups of bits.  The two 16-bit halves are spread apart in 32-bit words: a step is one shift and
+// one three-input logic instruction, where a 64-bit step takes two of each.
+__device__ __forceinline__ uint32_t spread16(uint32_t x)
+{
+    x = (x | (x << 8)) & 0x00FF00FFu;
+    x = (x | (x << 4)) & 0x0F0F0F0Fu;
+    x = (x | (x << 2)) & 0x33333333u;
+    x = (x | (x << 1)) & 0x55555555u;
+    return x;
+}
+
 __device__ __forceinline__ uint64_t spread_bits(uint32_t v)
 {
-    uint64_t x = v;
-    x = (x | (x << 16)) & 0x0000FFFF0000FFFFull;
-    x = (x | (x << 8)) & 0x00FF00FF00FF00FFull;
-    x = (x | (x << 4)) & 0x0F0F0F0F0F0F0F0Full;
-    x = (x | (x << 2)) & 0x3333333333333333ull;
-    x = (x | (x << 1)) & 0x5555555555555555ull;
+    return (uint64_t)spread16(v >> 16) << 32 | spread16(v & 0xFFFFu);
+}
+
+__device__ __forceinline__ uint32_t gather16(uint32_t x)
+{
+    x &= 0x55555555u;
+    x = (x | (x >> 1)) & 0x33333333u;
+    x = (x | (x >> 2)) & 0x0F0F0F0Fu;
+    x = (x | (x >> 4)) & 0x00FF00FFu;
+    x = (x | (x >> 8)) & 0x0000FFFFu;
     return x;
 }
 
 __device__ __forceinline__ uint32_t gather_bits(uint64_t x)
 {
-    x &= 0x5555555555555555ull;
-    x = (x | (x >> 1)) & 0x3333333333333333ull;
-    x = (x | (x >> 2)) & 0x0F0F0F0F0F0F0F0Full;
-    x = (x | (x >> 4)) & 0x00FF00FF00FF00FFull;
-    x = (x | (x >> 8)) & 0x0000FFFF0000FFFFull;
-    x = (x | (x >> 16)) & 0x00000000FFFFFFFFull;
-    return (uint32_t)x;
+    return gather16((uint32_t)(x >> 32)) << 16 | gather16((uint32_t)x);
 }
 
 __device__ __forceinline__ uint64_t morton_key(uint32_t x, uint32_t y)
 {
-    return spread_bits(x) | (spread_bits(y) << 1);
+    const uint32_t lo = spread16(x & 0xFFFFu) | spread16(y & 0xFFFFu) << 1;
+    const uint32_t hi = spread16(x >> 16) | spread16(y >> 16) << 1;
+    return (uint64_t)hi << 32 | lo;
 }
 
 __device__ __forceinline__ void morton_decode(uint64_t k, uint32_t& x, uint32_t& y)
 {
-    x = gather_bits(k);
-    y = gather_bits(k >> 1);
+    const uint32_t lo = (uint32_t)k, hi = (uint32_t)(k >> 32);
+    x = gather16(hi) << 16 | gather16(lo);
+    y = gather16(hi >> 1) << 16 | gather16(lo >> 1);
 }
 
 // Z curve in 3-D (Alg. 2 with a third coordinate): bit i of x, y, z goes to key bit 3i, 3i + 1,
@@ -426,6 +437,7 @@ struct SortWorkspace {
     DevBuf tmp_vals[2];
     DevBuf lookback;      // per (tile, digit) look-back words, epoch-tagged
     DevBuf small;         // histograms, digit offsets, pass plan, tile counters
+    DevBuf runs;          // runs that the sorted digits leave long
     DevBuf epoch_dev;     // device epoch counter (advanced on the device per sort)
 };
 // Source of the keys to sort: either points (keys computed on the fly for `curve`) or
@@ -436,6 +448,8 @@ struct SortSource {
     const uint32_t* vals = nullptr;
     uint32_t val_base = 0;
     int curve = SFC_CURVE_Z;
+    int bits = 64;         // the keys are below 2^bits
+    bool partial = true;   // may sort the leading digits and then order the runs left over
 };
 struct SortDest {
     uint64_t* keys = nullptr;

@@ -308,6 +308,7 @@ sfc_status apply_update(sfc_index* idx, const int32_t* d_inserts, uint64_t k_ins
         count_launch();
         SortSource src;
         src.keys = dkeys_in;
+        src.bits = 2 * kOmega;
         src.vals = d_del;
         SortDest dst;
         dst.keys = dkeys;
@@ -346,6 +347,7 @@ sfc_status apply_update(sfc_index* idx, const int32_t* d_inserts, uint64_t k_ins
         irank = U.h.as<uint32_t>();
         SortSource src;
         src.points = reinterpret_cast<const int2*>(d_inserts);
+        src.bits = 2 * kOmega;
         src.curve = curve;
         src.val_base = next_id;
         SortDest dst;
