@@ -186,6 +186,8 @@ QueryArgs base_args(sfc_index* idx, const int32_t* q, const int32_t* delta, uint
     a.dim = idx->dim;
     a.xyz = idx->xyz.as<int4>();
     a.box = idx->box.as<int4>();
+    a.dir = idx->dir.as<uint32_t>();
+    a.dir_bits = dir_bits(idx->n);
     if (idx->opt.occupancy_depth > 0 && idx->occ.ptr) {
         a.occ = idx->occ.as<uint32_t>();
         a.occ_depth = idx->opt.occupancy_depth;
@@ -537,6 +539,7 @@ sfc_status sfc_reserve(sfc_index* idx, uint64_t n_max, uint64_t m_max, void* str
         SFC_TRY(idx->occ.ensure(occupancy_words(idx->opt.occupancy_depth) * sizeof(uint32_t), st));
     SFC_TRY(reserve_sort(idx->sort_ws, n1, st));
     SFC_TRY(idx->box.ensure(box_bytes(idx->dim, n1), st));
+    SFC_TRY(idx->dir.ensure(dir_bytes(n1), st));
     SFC_TRY(ensure_query_ws(idx, m_max, n1, st));
     SFC_TRY(reserve_scan(idx->scan_ws, std::max<uint64_t>(m_max, n1) + 1, st));
     if (idx->opt.bounds == SFC_BOUNDS_LEARNED) SFC_TRY(reserve_model(idx, n1, st));

@@ -8,6 +8,10 @@
 // One pass over the coordinates, bound by HBM: a warp takes four groups at a time, one coalesced
 // load each, and reduces them with the warp's min / max instructions (10^8 points: 0.15 ms, 5.7
 // TB/s, against 3.4 ms that the boxes save in each batch of 10^7 queries).
+//
+// The same launch fills the key directory that the bound searches of the plan start from: a thread
+// finds each entry by binary search (neighbouring threads walk nearly the same path, so 2^18
+// entries take a few microseconds beside the boxes).
 #include <algorithm>
 
 #include "sfc_internal.cuh"
@@ -20,11 +24,40 @@ namespace {
 constexpr int kT = 256;
 constexpr int kU = 4;   // groups per warp and iteration
 
-__global__ void __launch_bounds__(kT) boxes_kernel(const int2* __restrict__ xy, uint32_t n, uint32_t groups, int4* box)
+// Entries [0, 2^bits] of the directory, by the blocks [0, blocks) of a launch.
+__device__ __forceinline__ void fill_directory(const uint64_t* __restrict__ keys, uint32_t n, int bits, uint32_t blocks,
+                                               uint32_t* dir)
 {
+    const uint64_t kmin = __ldg(keys), kmax = __ldg(keys + n - 1);
+    const int shift = dir_shift(kmin, kmax, bits);
+    for (uint32_t v = blockIdx.x * kT + threadIdx.x; v <= 1u << bits; v += blocks * kT) {
+        const uint64_t t = kmin + ((uint64_t)v << shift);   // at most 2 kmax: 64 bits hold it
+        // three probes a step: the latency of the steps, not the loads, sets the time of short arrays
+        uint32_t lo = 0, len = n;   // the answer lies in [lo, lo + len]
+        while (len > 0) {
+            const uint32_t q = len >> 2, h = len >> 1;
+            const uint64_t ka = __ldg(keys + lo + q), kb = __ldg(keys + lo + h), kc = __ldg(keys + lo + h + q);
+            const uint32_t from = kc < t ? h + q + 1 : (kb < t ? h + 1 : (ka < t ? q + 1 : 0));
+            const uint32_t to = kc < t ? len : (kb < t ? h + q : (ka < t ? h : q));
+            lo += from;
+            len = to - from;
+        }
+        dir[v] = lo;
+    }
+}
+
+// Blocks [0, dblocks) fill the directory, the others the boxes.
+__global__ void __launch_bounds__(kT) boxes_kernel(const int2* __restrict__ xy, const uint64_t* __restrict__ keys,
+                                                   uint32_t n, uint32_t groups, int bits, uint32_t dblocks, uint32_t* dir,
+                                                   int4* box)
+{
+    if (blockIdx.x < dblocks) {
+        fill_directory(keys, n, bits, dblocks, dir);
+        return;
+    }
     const unsigned lane = lane_id();
-    const uint32_t warps = gridDim.x * (kT / 32);
-    for (uint32_t g0 = (blockIdx.x * (kT / 32) + (threadIdx.x >> 5)) * kU; g0 < groups; g0 += warps * kU) {
+    const uint32_t warps = (gridDim.x - dblocks) * (kT / 32);
+    for (uint32_t g0 = ((blockIdx.x - dblocks) * (kT / 32) + (threadIdx.x >> 5)) * kU; g0 < groups; g0 += warps * kU) {
         int2 p[kU];
 #pragma unroll
         for (int u = 0; u < kU; ++u)   // past the end the last point stands in: it changes no box
@@ -38,11 +71,17 @@ __global__ void __launch_bounds__(kT) boxes_kernel(const int2* __restrict__ xy, 
     }
 }
 
-__global__ void __launch_bounds__(kT) boxes3_kernel(const int4* __restrict__ xyz, uint32_t n, uint32_t groups, int4* box)
+__global__ void __launch_bounds__(kT) boxes3_kernel(const int4* __restrict__ xyz, const uint64_t* __restrict__ keys,
+                                                    uint32_t n, uint32_t groups, int bits, uint32_t dblocks, uint32_t* dir,
+                                                    int4* box)
 {
+    if (blockIdx.x < dblocks) {
+        fill_directory(keys, n, bits, dblocks, dir);
+        return;
+    }
     const unsigned lane = lane_id();
-    const uint32_t warps = gridDim.x * (kT / 32);
-    for (uint32_t g = blockIdx.x * (kT / 32) + (threadIdx.x >> 5); g < groups; g += warps) {
+    const uint32_t warps = (gridDim.x - dblocks) * (kT / 32);
+    for (uint32_t g = (blockIdx.x - dblocks) * (kT / 32) + (threadIdx.x >> 5); g < groups; g += warps) {
         const int4 p = __ldg(xyz + (uint32_t)min((uint64_t)g * 32 + lane, (uint64_t)n - 1));
         const int4 lo = make_int4(__reduce_min_sync(0xffffffffu, p.x), __reduce_min_sync(0xffffffffu, p.y),
                                   __reduce_min_sync(0xffffffffu, p.z), 0);
@@ -58,16 +97,28 @@ __global__ void __launch_bounds__(kT) boxes3_kernel(const int4* __restrict__ xyz
 // Padded to whole items (four groups): a lane loads its item's boxes together.
 size_t box_bytes(int dim, uint64_t n) { return (n + 127) / 128 * 4 * (dim == 3 ? 2 : 1) * sizeof(int4); }
 
+size_t dir_bytes(uint64_t n) { return ((size_t)(1u << dir_bits(n)) + 1) * sizeof(uint32_t); }
+
 sfc_status build_boxes(sfc_index* idx, cudaStream_t st)
 {
     const uint64_t n = idx->n;
     if (n == 0) return SFC_OK;
     SFC_TRY(idx->box.ensure(box_bytes(idx->dim, n), st));
+    SFC_TRY(idx->dir.ensure(dir_bytes(n), st));
     const uint32_t groups = (uint32_t)((n + 31) / 32);
     const uint32_t per_block = (kT / 32) * (idx->dim == 3 ? 1 : kU);
-    const uint32_t grid = std::min((groups + per_block - 1) / per_block, (uint32_t)num_sms() * 8);
-    if (idx->dim == 3) boxes3_kernel<<<grid, kT, 0, st>>>(idx->xyz.as<int4>(), (uint32_t)n, groups, idx->box.as<int4>());
-    else boxes_kernel<<<grid, kT, 0, st>>>(idx->xy.as<int2>(), (uint32_t)n, groups, idx->box.as<int4>());
+    const int bits = dir_bits(n);
+    // of the eight blocks that an SM holds, two fill the directory beside six that stream a large
+    // array (the directory's latency then hides behind the boxes); short arrays take what it needs
+    const bool large = n >= 1ull << 24;
+    const uint32_t dblocks = std::min((1u << bits) / kT + 1, (uint32_t)num_sms() * (large ? 2 : 4));
+    const uint32_t grid = dblocks + std::min((groups + per_block - 1) / per_block, (uint32_t)num_sms() * (large ? 6 : 8));
+    if (idx->dim == 3)
+        boxes3_kernel<<<grid, kT, 0, st>>>(idx->xyz.as<int4>(), idx->keys.as<uint64_t>(), (uint32_t)n, groups, bits, dblocks,
+                                           idx->dir.as<uint32_t>(), idx->box.as<int4>());
+    else
+        boxes_kernel<<<grid, kT, 0, st>>>(idx->xy.as<int2>(), idx->keys.as<uint64_t>(), (uint32_t)n, groups, bits, dblocks,
+                                          idx->dir.as<uint32_t>(), idx->box.as<int4>());
     count_launch();
     return launch_status();
 }

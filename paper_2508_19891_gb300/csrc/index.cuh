@@ -89,6 +89,7 @@ struct sfc_index {
     sfc::DevBuf status;                 // device status word + model statistics
     sfc::DevBuf occ;                    // early-termination bitmap (occupancy_depth > 0)
     sfc::DevBuf box;                    // bounding boxes of the groups of 32 sorted points
+    sfc::DevBuf dir;                    // key directory: positions of equal parts of the key range
     sfc::DevBuf xyz;                    // 3-D: coordinates in sorted order (int4 x, y, z, 0)
     sfc::DevBuf keys_in;                // 3-D: keys in input order (the sort's source)
 
@@ -115,7 +116,8 @@ const RootParams* model_root_device(sfc_index* idx);
 // early-termination bitmap of the sorted keys (no-op when opt.occupancy_depth == 0)
 sfc_status build_occupancy(sfc_index* idx, cudaStream_t st);
 uint64_t occupancy_words(int depth);
-// bounding boxes of the groups of 32 consecutive sorted points
+// bounding boxes of the groups of 32 consecutive sorted points, and the key directory
+size_t dir_bytes(uint64_t n);
 sfc_status build_boxes(sfc_index* idx, cudaStream_t st);
 size_t box_bytes(int dim, uint64_t n);
 

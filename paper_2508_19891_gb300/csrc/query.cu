@@ -11,7 +11,6 @@
 //                  error window, verified, with fallback).  It keeps the non-empty array ranges
 //                  and how many items they make: group g is the 32 array positions
 //                  32 g .. 32 g + 31, an item is four (3-D: two) neighbouring groups.
-//                  plan3_kernel does the same for 3-D points.
 //   scan           exclusive scan of the item counts: the batch's scan is now one list of items,
 //                  in processing order.
 //   count_kernel   a warp takes a batch of 32 items, one per lane.  A lane looks its groups'
@@ -45,7 +44,10 @@ constexpr int kThreads = 256;
 // Binary searches in lock step per thread, and the plan kernel's resident blocks per SM (its
 // register budget) for each bound search.
 #ifndef SFC_BINARY_BATCH
-#define SFC_BINARY_BATCH 8
+#define SFC_BINARY_BATCH 4
+#endif
+#ifndef SFC_BINARY_BATCH3
+#define SFC_BINARY_BATCH3 8
 #endif
 #ifndef SFC_PLAN_BLOCKS_BINARY
 #define SFC_PLAN_BLOCKS_BINARY 4
@@ -71,34 +73,33 @@ constexpr uint32_t kPlanCap = SFC_PLAN_CAP;
 #define SFC_WRITE_BLOCKS 8
 #endif
 
-__device__ __forceinline__ bool query_valid(int32_t qx, int32_t qy, int32_t delta)
-{
-    return point_in_domain(qx, qy) && delta >= 0;
-}
-
 // ------------------------------------------------------------------------------------
-// Bound search: K lower_bounds in lock step (independent loads in flight together)
+// Bound search: lower_bounds in lock step (independent loads in flight together)
 // ------------------------------------------------------------------------------------
-template <int K>
-__device__ __forceinline__ void lower_bounds_window(const uint64_t* __restrict__ keys,
-                                                    const uint64_t* t, uint32_t* lo,
-                                                    uint32_t* len)
+// E lower_bounds in lock step, the answer of search x in [base[x], base[x] + len[x]]; a search that
+// has ended loads nothing more (padding all to the longest made the short ones probe cold lines
+// beyond their part: the plan of 10^6 mixed queries 502 us; the learned search, whose queries run in
+// curve order over lines that their neighbours hold, is the faster padded, 2.35 against 2.58 ms).
+template <int E>
+__device__ __forceinline__ void lower_bounds_each(const uint64_t* __restrict__ keys, const uint64_t* t, uint32_t* base,
+                                                  uint32_t* len)
 {
-    // answer of search e lies in [lo[e], lo[e] + len[e]]
     while (true) {
-        bool any = false;
+        uint32_t any = 0;
 #pragma unroll
-        for (int e = 0; e < K; ++e) any |= len[e] > 0;
+        for (int x = 0; x < E; ++x) any |= len[x];
         if (!any) break;
+        uint64_t k[E];
 #pragma unroll
-        for (int e = 0; e < K; ++e) {
-            if (len[e] > 0) {
-                uint32_t half = len[e] >> 1;
-                uint64_t k = __ldg(keys + lo[e] + half);
-                bool right = k < t[e];
-                lo[e] = right ? lo[e] + half + 1 : lo[e];
-                len[e] = right ? len[e] - half - 1 : half;
-            }
+        for (int x = 0; x < E; ++x)
+            if (len[x]) k[x] = __ldg(keys + base[x] + (len[x] >> 1));
+#pragma unroll
+        for (int x = 0; x < E; ++x) {
+            if (!len[x]) continue;
+            const uint32_t half = len[x] >> 1;
+            const bool below = k[x] < t[x];
+            base[x] = below ? base[x] + half + 1 : base[x];
+            len[x] = below ? len[x] - half - 1 : half;
         }
     }
 }
@@ -130,41 +131,53 @@ struct BoundStats {
     unsigned long long endpoints = 0, misses = 0, window = 0;
 };
 
-// Bound search functors: lower_bound of t[0..ne) (ne <= E) into r[].
+// Bound search functors: search_flat gives lower_bound over the whole array of the warp's flat
+// list of T targets (each lane takes targets lane, lane + 32, ...; kBatch of them in lock step).
+//
+// Binary search behind the key directory (boxes.cu): one lookup leaves the keys of one of 2^bits
+// equal parts of the key range, so a search takes that load and about log2(n / 2^bits) steps where
+// the array is evenly filled (more in a cluster) instead of log2(n).
+// Measured, plan of 10^6 queries over 10^7 points: mixed, cover 1, 421 -> 261 us; Normal points,
+// square windows 209 -> 112 us; 3-D balls 1371 -> 712 us (whose cells also moved from local memory to
+// columns in shared memory).
+template <int DIM>
 struct BinaryBounds {
     static constexpr bool kStats = false;
-    static constexpr int kBatch = SFC_BINARY_BATCH;
-    static constexpr bool kFenceSmem = false;
-    static constexpr int kMinBlocks = SFC_PLAN_BLOCKS_BINARY;   // endpoints searched in lock step per thread
-    __device__ __forceinline__ void prepare(RootParams*) {}
-    template <int E>
-    __device__ __forceinline__ void search(const uint64_t* keys, uint32_t n, const uint64_t* t, uint32_t* r,
-                                           int ne, BoundStats&) const
+    // (3-D: the columns of cell keys leave few warps, which need more loads in flight)
+    static constexpr int kBatch = DIM == 3 ? SFC_BINARY_BATCH3 : SFC_BINARY_BATCH;
+    static constexpr int kMinBlocks = SFC_PLAN_BLOCKS_BINARY;
+    const uint32_t* dir;
+    int bits;
+    uint64_t kmin, kmax;
+    int shift;
+    __device__ __forceinline__ void prepare(RootParams*, const uint64_t* keys, uint32_t n)
     {
-        uint32_t lo[E], len[E];
-#pragma unroll
-        for (int e = 0; e < E; ++e) { lo[e] = 0; len[e] = e < ne ? n : 0; }
-        lower_bounds_window<E>(keys, t, lo, len);
-#pragma unroll
-        for (int e = 0; e < E; ++e) r[e] = lo[e];
+        kmin = n ? __ldg(keys) : 0;
+        kmax = n ? __ldg(keys + n - 1) : 0;
+        shift = dir_shift(kmin, kmax, bits);
     }
-    // lower_bound over the whole array of the warp's flat list of T targets (each lane takes
-    // targets lane, lane + 32, ...; kBatch of them in lock step); results in res
     __device__ __forceinline__ void search_flat(const uint64_t* keys, uint32_t n, const uint64_t* tg, uint32_t* res,
-                                                uint32_t T, BoundStats&, uint64_t*) const
+                                                uint32_t T, BoundStats&) const
     {
         constexpr int E = kBatch;
 #pragma unroll 1
         for (uint32_t e0 = lane_id(); e0 < T; e0 += 32 * E) {
             uint64_t t[E];
-            uint32_t base[E];
+            uint32_t base[E], len[E];
 #pragma unroll
             for (int x = 0; x < E; ++x) {
                 const uint32_t e = e0 + 32 * x;
                 t[x] = e < T ? tg[e] : 0;
-                base[x] = 0;
+                base[x] = len[x] = 0;
+                if (t[x] > kmax) {
+                    base[x] = n;
+                } else if (t[x] > kmin) {
+                    const uint32_t v = (uint32_t)((t[x] - kmin) >> shift);
+                    base[x] = __ldg(dir + v);
+                    len[x] = __ldg(dir + v + 1) - base[x];
+                }
             }
-            lower_bounds_uniform<E>(keys, t, base, n);
+            lower_bounds_each<E>(keys, t, base, len);
 #pragma unroll
             for (int x = 0; x < E; ++x) {
                 const uint32_t e = e0 + 32 * x;
@@ -176,7 +189,6 @@ struct BinaryBounds {
 
 struct LearnedBounds {
     static constexpr bool kStats = true;
-    static constexpr bool kFenceSmem = false;
     static constexpr int kBatch = SFC_LEARNED_BATCH;
     static constexpr int kMinBlocks = SFC_PLAN_BLOCKS_LEARNED;
     const RootParams* root;      // device; after prepare() the block's shared-memory copy
@@ -185,7 +197,7 @@ struct LearnedBounds {
     const uint64_t* fence_fine;  // [leaves][kFenceFine] fine fence keys
     unsigned long long* stats;   // [0] endpoints, [1] misses, [2] window sum
     // every thread of the block calls this, then the block synchronises
-    __device__ __forceinline__ void prepare(RootParams* s)
+    __device__ __forceinline__ void prepare(RootParams* s, const uint64_t*, uint32_t)
     {
         const uint32_t* src = reinterpret_cast<const uint32_t*>(root);
         uint32_t* dst = reinterpret_cast<uint32_t*>(s);
@@ -206,7 +218,7 @@ struct LearnedBounds {
     //      the key beyond the edge, and a target whose window missed is searched over the whole
     //      array.
     __device__ __forceinline__ void search_flat(const uint64_t* keys, uint32_t n, const uint64_t* tg, uint32_t* res,
-                                                uint32_t T, BoundStats& bs, uint64_t*) const
+                                                uint32_t T, BoundStats& bs) const
     {
         constexpr int E = kBatch;
 #pragma unroll 1
@@ -352,11 +364,13 @@ __device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v)
 // ------------------------------------------------------------------------------------
 // plan_kernel: range derivation and bound search, one thread per query
 // ------------------------------------------------------------------------------------
-template <int DROP>
+template <int DIM, int DROP>
 struct Cover {
     // cells per axis at most: 2 for cells(Q) (2 delta <= 2^l), 2^DROP + 1 one or two levels finer
     static constexpr int NX = DROP == 0 ? 2 : (1 << DROP) + 1;
-    static constexpr int K = NX * NX;   // 4, 9, 25 interval slots per query
+    static constexpr int K = DIM == 3 ? NX * NX * NX : NX * NX;   // 2-D: 4, 9, 25 slots per query; 3-D: 8, 27
+    // threads per block: the columns of cell keys are K words a thread
+    static constexpr int kThreads = DIM == 3 ? 128 : 256;
 };
 
 // Early termination (Sec. 2.2): whether the cell of level l whose key interval starts at c may
@@ -367,6 +381,17 @@ __device__ __forceinline__ bool cell_occupied(const uint32_t* __restrict__ occ, 
     const int t = min(kOmega - l, D);
     const uint64_t b = occupancy_level_start(t) + (c >> (2 * (kOmega - t)));
     return (__ldg(occ + (b >> 5)) >> (b & 31)) & 1u;
+}
+
+// Puts key c into its place among the cnt ascending keys of the column.
+__device__ __forceinline__ void insert_cell(uint64_t* col, int stride, int cnt, uint64_t c)
+{
+    int j = cnt;
+    while (j > 0 && col[(j - 1) * stride] > c) {
+        col[j * stride] = col[(j - 1) * stride];
+        --j;
+    }
+    col[j * stride] = c;
 }
 
 // The cells of the cover, each as the key of its first point (its key interval is [c, c | span],
@@ -383,7 +408,6 @@ __device__ __forceinline__ int derive_cells(int curve, int norm, const HilbertTa
                                             int32_t delta, const uint32_t* occ, int D, uint64_t* col, int stride,
                                             uint64_t* span_out, uint32_t& ncell, uint32_t& nempty)
 {
-    constexpr int K = Cover<DROP>::K;
     const int64_t d = delta;
     const int64_t x0 = max((int64_t)0, (int64_t)qx - d), x1 = min((int64_t)kSide - 1, (int64_t)qx + d);
     const int64_t y0 = max((int64_t)0, (int64_t)qy - d), y1 = min((int64_t)kSide - 1, (int64_t)qy + d);
@@ -395,7 +419,7 @@ __device__ __forceinline__ int derive_cells(int curve, int norm, const HilbertTa
     l = max(0, l - DROP);
     const uint64_t span = (l >= kOmega) ? kKeyMax : ((1ull << (2 * l)) - 1);
     *span_out = span;
-    constexpr int NX = Cover<DROP>::NX;   // cells per axis at most
+    constexpr int NX = Cover<2, DROP>::NX;   // cells per axis at most
     const int64_t cx0 = x0 >> l, cy0 = y0 >> l;
     const int nx = (int)min((int64_t)NX, (x1 >> l) - cx0 + 1), ny = (int)min((int64_t)NX, (y1 >> l) - cy0 + 1);
     // per column: the squared distance from q to the column's nearest x and, for the Z curve,
@@ -434,13 +458,59 @@ __device__ __forceinline__ int derive_cells(int curve, int norm, const HilbertTa
                 ++nempty;
                 continue;
             }
-            int j = cnt;
-            while (j > 0 && col[(j - 1) * stride] > c) {
-                col[j * stride] = col[(j - 1) * stride];
-                --j;
+            insert_cell(col, stride, cnt++, c);
+        }
+    }
+    return cnt;
+}
+
+// The same in 3-D.  DROP 0: cells(Q), the cells of level l (2 delta <= 2^l < 4 delta, capped at 21)
+// meeting the clipped cube Q.  DROP 1: the cells of level max(0, l - 1) holding an integer point of
+// the closed ball.
+template <int DROP>
+__device__ __forceinline__ int derive_cells3(int4 w, uint64_t* col, int stride, uint64_t* span_out)
+{
+    constexpr int NX = Cover<3, DROP>::NX;
+    const int64_t d = w.z, d2 = d * d;
+    int l = 0;
+    if (d > 0) {
+        l = 64 - __clzll((unsigned long long)(2 * d - 1));
+        if (l > kOmega3) l = kOmega3;
+    }
+    l = max(0, l - DROP);
+    const uint64_t span = (1ull << (3 * l)) - 1;   // 3 l <= 63
+    *span_out = span;
+    // per axis: the first cell and the squared distance from q to each cell's nearest coordinate
+    // (-1: no such cell)
+    const int c[3] = {w.x, w.y, w.w};
+    int first[3];
+    int64_t dist2[3][NX];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const int a0 = (int)max((int64_t)0, c[k] - d), a1 = (int)min((int64_t)kSide3 - 1, c[k] + d);
+        first[k] = a0 >> l;
+#pragma unroll
+        for (int j = 0; j < NX; ++j) {
+            const int64_t b0 = (int64_t)(first[k] + j) << l, b1 = b0 + ((int64_t)1 << l) - 1;
+            const int64_t e = c[k] < b0 ? b0 - c[k] : (c[k] > b1 ? c[k] - b1 : 0);
+            dist2[k][j] = first[k] + j <= (a1 >> l) ? e * e : -1;
+        }
+    }
+    int cnt = 0;
+#pragma unroll
+    for (int iz = 0; iz < NX; ++iz) {
+        if (dist2[2][iz] < 0) break;
+        const uint64_t sz = spread3_bits((uint32_t)(first[2] + iz) << l) << 2;
+#pragma unroll
+        for (int iy = 0; iy < NX; ++iy) {
+            if (dist2[1][iy] < 0) break;
+            const uint64_t sy = sz | spread3_bits((uint32_t)(first[1] + iy) << l) << 1;
+#pragma unroll
+            for (int ix = 0; ix < NX; ++ix) {
+                if (dist2[0][ix] < 0) break;
+                if (DROP > 0 && dist2[0][ix] + dist2[1][iy] + dist2[2][iz] > d2) continue;
+                insert_cell(col, stride, cnt++, sy | spread3_bits((uint32_t)(first[0] + ix) << l));
             }
-            col[j * stride] = c;
-            ++cnt;
         }
     }
     return cnt;
@@ -505,16 +575,15 @@ struct PlanExport {
 };
 
 
-// Dynamic shared memory of plan_kernel<Bounds, DROP, ..>: each thread's column of K cell keys
+// Dynamic shared memory of plan_kernel<.., DIM, DROP, ..>: each thread's column of K cell keys
 // (column-major, so that the lanes of a warp touch consecutive words), then per warp the flat
-// target list (kPlanCap keys) and its results (kPlanCap positions), and for the learned search
-// per warp one leaf's fine fence (kFenceFine keys).
-template <class Bounds, int DROP>
+// target list (kPlanCap keys) and its results (kPlanCap positions).
+template <int DIM, int DROP>
 constexpr size_t plan_smem_bytes()
 {
-    return (size_t)Cover<DROP>::K * kThreads * sizeof(uint64_t) +
-           (size_t)(kThreads / 32) * kPlanCap * (sizeof(uint64_t) + sizeof(uint32_t)) +
-           (Bounds::kFenceSmem ? (size_t)(kThreads / 32) * kFenceFine * sizeof(uint64_t) : 0);
+    constexpr int T = Cover<DIM, DROP>::kThreads;
+    return (size_t)Cover<DIM, DROP>::K * T * sizeof(uint64_t) +
+           (size_t)(T / 32) * kPlanCap * (sizeof(uint64_t) + sizeof(uint32_t));
 }
 
 // One thread per query for the range derivation: the cells of its cover, sorted, in shared
@@ -524,10 +593,11 @@ constexpr size_t plan_smem_bytes()
 // of interval counts over the warp's queries.  Then each thread writes its query's intervals'
 // (begin, end) to slots 0.. of its K slots (unused slots (0, 0)), the number of chunks of its
 // scan, and adds to the scanned total.  Nothing per query lives in local memory.
-template <class Bounds, int DROP, bool EXPORT>
-__global__ void __launch_bounds__(kThreads, Bounds::kMinBlocks) plan_kernel(QueryArgs a, Bounds bounds_in, PlanExport ex)
+template <class Bounds, int DIM, int DROP, bool EXPORT>
+__global__ void __launch_bounds__((Cover<DIM, DROP>::kThreads), Bounds::kMinBlocks)
+plan_kernel(QueryArgs a, Bounds bounds_in, PlanExport ex)
 {
-    constexpr int K = Cover<DROP>::K;
+    constexpr int K = Cover<DIM, DROP>::K, kThreads = Cover<DIM, DROP>::kThreads;
     __shared__ HilbertTables tb;
     __shared__ RootParams s_root;
     extern __shared__ __align__(16) unsigned char s_dyn[];
@@ -536,34 +606,42 @@ __global__ void __launch_bounds__(kThreads, Bounds::kMinBlocks) plan_kernel(Quer
     uint64_t* tg = reinterpret_cast<uint64_t*>(s_dyn) + (size_t)K * kThreads + (size_t)warp * kPlanCap;
     uint32_t* res = reinterpret_cast<uint32_t*>(reinterpret_cast<uint64_t*>(s_dyn) + (size_t)K * kThreads +
                                                 (size_t)(kThreads / 32) * kPlanCap) + (size_t)warp * kPlanCap;
-    uint64_t* sf = reinterpret_cast<uint64_t*>(s_dyn + (size_t)K * kThreads * sizeof(uint64_t) +
-                                               (size_t)(kThreads / 32) * kPlanCap * (sizeof(uint64_t) + sizeof(uint32_t))) +
-                   (size_t)warp * kFenceFine;
     Bounds bounds = bounds_in;
-    bounds.prepare(&s_root);
-    __syncthreads();
-    if (a.curve == SFC_CURVE_HILBERT) hilbert_tables_init(&tb);   // ends with a block barrier
+    bounds.prepare(&s_root, a.keys, a.n);
+    if constexpr (Bounds::kStats) __syncthreads();   // the root's shared-memory copy
+    if (DIM == 2 && a.curve == SFC_CURVE_HILBERT) hilbert_tables_init(&tb);   // ends with a block barrier
     // thread r takes the query of processing rank r (curve order of the centres when a
     // processing order is given: neighbouring threads then search neighbouring keys)
     const uint64_t r = (uint64_t)blockIdx.x * kThreads + threadIdx.x;
     const bool active = r < a.m;
     const uint64_t i = active && a.perm ? (uint64_t)__ldg(a.perm + r) : r;
-    int2 q = make_int2(0, 0);
-    int32_t delta = -1;
+    int4 q = make_int4(0, 0, -1, 0);   // x, y, delta, z
     if (active) {
-        q = __ldg(reinterpret_cast<const int2*>(a.q) + i);
-        delta = __ldg(a.delta + i);
+        if (DIM == 3) {
+            q.x = __ldg(a.q + 3 * i);
+            q.y = __ldg(a.q + 3 * i + 1);
+            q.w = __ldg(a.q + 3 * i + 2);
+        } else {
+            const int2 c = __ldg(reinterpret_cast<const int2*>(a.q) + i);
+            q.x = c.x;
+            q.y = c.y;
+        }
+        q.z = __ldg(a.delta + i);
     }
-    const bool ok = active && query_valid(q.x, q.y, delta);
+    const bool ok = active && q.z >= 0 && (DIM == 3 ? point3_in_domain(q.x, q.y, q.w) : point_in_domain(q.x, q.y));
     if (active && !ok) set_status(a.status, SFC_DEV_BAD_QUERY);
     BoundStats bs;
     uint32_t ncell = 0, nempty = 0;
     uint64_t span = 0;
-    const int nc = ok ? derive_cells<DROP>(a.curve, a.norm, &tb, q.x, q.y, delta, a.occ, a.occ_depth, col, kThreads,
-                                           &span, ncell, nempty)
-                      : 0;
+    int nc = 0;
+    if (ok) {
+        if constexpr (DIM == 3) nc = derive_cells3<DROP>(q, col, kThreads, &span);
+        else nc = derive_cells<DROP>(a.curve, a.norm, &tb, q.x, q.y, q.z, a.occ, a.occ_depth, col, kThreads, &span, ncell,
+                                     nempty);
+    }
     uint32_t cnt = 0;   // merged intervals
     for_each_endpoint(col, kThreads, nc, span, [&](uint32_t ep, uint64_t) { cnt += ep & 1u; });
+    if (DIM == 3) ncell = cnt;
     const uint32_t ne = 2u * cnt;
     const uint32_t incl = warp_incl_scan_u32(ne);
     const uint32_t off = incl - ne;
@@ -579,7 +657,7 @@ __global__ void __launch_bounds__(kThreads, Bounds::kMinBlocks) plan_kernel(Quer
             if (f >= r0 && f < r1) tg[f - r0] = key;
         });
         __syncwarp();
-        bounds.search_flat(a.keys, a.n, tg, res, r1 - r0, bs, sf);
+        bounds.search_flat(a.keys, a.n, tg, res, r1 - r0, bs);
         __syncwarp();
         const uint32_t f0 = max(off, r0), f1 = min(off + ne, r1);
         for (uint32_t f = f0; f < f1; ++f) {
@@ -591,7 +669,7 @@ __global__ void __launch_bounds__(kThreads, Bounds::kMinBlocks) plan_kernel(Quer
                     open = pos;
                 } else if (pos > open) {   // a non-empty range
                     *rp++ = make_uint2(open, pos);
-                    items += range_items<kItemGroups2>(open, pos);
+                    items += range_items<DIM == 3 ? kItemGroups3 : kItemGroups2>(open, pos);
                 }
             } else {
                 const uint64_t o = (uint64_t)K * i + (ep >> 1);
@@ -631,7 +709,7 @@ __global__ void __launch_bounds__(kThreads, Bounds::kMinBlocks) plan_kernel(Quer
     }
     if (!active) return;
     if (!EXPORT) {
-        plan_store(a, r, i, make_int4(q.x, q.y, delta, 0), items);
+        plan_store(a, r, i, q, items);
     } else {
         for (uint32_t k = cnt; k < (uint32_t)K; ++k) {
             const uint64_t o = (uint64_t)K * i + k;
@@ -641,145 +719,6 @@ __global__ void __launch_bounds__(kThreads, Bounds::kMinBlocks) plan_kernel(Quer
             if (ex.e) ex.e[o] = 0;
         }
         if (ex.cnt) ex.cnt[i] = cnt;
-    }
-}
-
-// ------------------------------------------------------------------------------------
-// plan3_kernel: the same for 3-D points (Z curve in Z^3, binary bound search)
-// ------------------------------------------------------------------------------------
-// cells(Q) in 3-D: at most two cells per axis, 8 in all; one level finer, at most 3 per axis
-template <int DROP>
-struct Cover3 {
-    static constexpr int NX = DROP == 0 ? 2 : 3;
-    static constexpr int K = NX * NX * NX;
-};
-
-// DROP 0: cells(Q) in 3-D, the cells of level l (2 delta <= 2^l < 4 delta, capped at 21)
-// meeting the clipped cube Q.  DROP 1: the cells of level max(0, l - 1) holding an integer
-// point of the closed ball.  Key intervals of length 8^l, sorted, abutting ones merged.
-template <int DROP>
-__device__ __forceinline__ int derive_ranges3(int32_t qx, int32_t qy, int32_t qz, int32_t delta, uint64_t* lo,
-                                              uint64_t* hi)
-{
-    constexpr int K = Cover3<DROP>::K;
-    const int64_t d = delta;
-    const int64_t c[3] = {qx, qy, qz};
-    int64_t a0[3], a1[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        a0[k] = max((int64_t)0, c[k] - d);
-        a1[k] = min((int64_t)kSide3 - 1, c[k] + d);
-    }
-    int l = 0;
-    if (d > 0) {
-        l = 64 - __clzll((unsigned long long)(2 * d - 1));
-        if (l > kOmega3) l = kOmega3;
-    }
-    l = max(0, l - DROP);
-    const uint64_t span = (1ull << (3 * l)) - 1;   // 3 l <= 63
-    int cnt = 0;
-    for (int64_t cz = a0[2] >> l; cz <= (a1[2] >> l); ++cz)
-        for (int64_t cy = a0[1] >> l; cy <= (a1[1] >> l); ++cy)
-            for (int64_t cx = a0[0] >> l; cx <= (a1[0] >> l); ++cx) {
-                if (DROP > 0) {
-                    const int64_t cc[3] = {cx, cy, cz};
-                    int64_t dist2 = 0;
-#pragma unroll
-                    for (int k = 0; k < 3; ++k) {
-                        const int64_t b0 = cc[k] << l, b1 = ((cc[k] + 1) << l) - 1;
-                        const int64_t e = c[k] < b0 ? b0 - c[k] : (c[k] > b1 ? c[k] - b1 : 0);
-                        dist2 += e * e;
-                    }
-                    if (dist2 > d * d) continue;
-                }
-                if (cnt == K) break;   // unreachable: at most Cover3<DROP>::NX cells per axis
-                const uint64_t k0 = morton3_key((uint32_t)(cx << l), (uint32_t)(cy << l), (uint32_t)(cz << l)) & ~span;
-                int j = cnt;
-                while (j > 0 && lo[j - 1] > k0) { lo[j] = lo[j - 1]; hi[j] = hi[j - 1]; --j; }
-                lo[j] = k0;
-                hi[j] = k0 | span;
-                ++cnt;
-            }
-    int m = 0;
-    for (int i = 0; i < cnt; ++i) {
-        if (m > 0 && hi[m - 1] + 1 == lo[i]) {
-            hi[m - 1] = hi[i];
-        } else {
-            lo[m] = lo[i];
-            hi[m] = hi[i];
-            ++m;
-        }
-    }
-    return m;
-}
-
-template <int DROP, bool EXPORT>
-__global__ void __launch_bounds__(kThreads, 4) plan3_kernel(QueryArgs a, PlanExport ex)
-{
-    constexpr int kCells3 = Cover3<DROP>::K;
-    constexpr int NB = (2 * kCells3 + 7) / 8;
-    const uint64_t i = (uint64_t)blockIdx.x * kThreads + threadIdx.x;
-    const bool active = i < a.m;
-    int32_t qx = 0, qy = 0, qz = 0, delta = -1;
-    if (active) {
-        qx = __ldg(a.q + 3 * i);
-        qy = __ldg(a.q + 3 * i + 1);
-        qz = __ldg(a.q + 3 * i + 2);
-        delta = __ldg(a.delta + i);
-    }
-    const bool ok = active && point3_in_domain(qx, qy, qz) && delta >= 0;
-    if (active && !ok) set_status(a.status, SFC_DEV_BAD_QUERY);
-    uint64_t lo[kCells3], hi[kCells3];
-    uint32_t b[kCells3], e[kCells3];
-    const int cnt = ok ? derive_ranges3<DROP>(qx, qy, qz, delta, lo, hi) : 0;
-    BoundStats bs;
-    const BinaryBounds bounds{};
-#pragma unroll 1
-    for (int bi = 0; bi < NB && 8 * bi < 2 * cnt; ++bi) {
-        uint64_t t[8];
-        uint32_t r[8];
-#pragma unroll
-        for (int x = 0; x < 8; ++x) {
-            const int ep = 8 * bi + x;
-            t[x] = ep < 2 * cnt ? ((ep & 1) ? hi[ep >> 1] + 1 : lo[ep >> 1]) : 0;
-        }
-        bounds.search<8>(a.keys, a.n, t, r, min(2 * cnt - 8 * bi, 8), bs);
-#pragma unroll
-        for (int x = 0; x < 8; ++x) {
-            const int ep = 8 * bi + x;
-            if (ep < 2 * cnt) {
-                if (ep & 1) e[ep >> 1] = r[x];
-                else b[ep >> 1] = r[x];
-            }
-        }
-    }
-    uint64_t S = 0;
-    for (int k = 0; k < cnt; ++k) S += e[k] - b[k];
-    if (!EXPORT) {   // statistics: one atomic per warp and counter
-        plan_stats(a, S);
-        const unsigned long long tc = warp_sum_u64((unsigned long long)cnt);
-        if (lane_id() == 0 && tc) atomicAdd(a.cells, tc);
-    }
-    if (!active) return;
-    if (!EXPORT) {
-        uint2* rp = a.ranges + (uint64_t)kCells3 * i;
-        uint32_t items = 0;
-        for (int k = 0; k < cnt; ++k) {
-            if (e[k] <= b[k]) continue;
-            *rp++ = make_uint2(b[k], e[k]);
-            items += range_items<kItemGroups3>(b[k], e[k]);
-        }
-        plan_store(a, i, i, make_int4(qx, qy, delta, qz), items);
-    } else {
-        for (int k = 0; k < kCells3; ++k) {
-            const bool u = k < cnt;
-            const uint64_t o = (uint64_t)kCells3 * i + k;
-            if (ex.lo) ex.lo[o] = u ? lo[k] : 1;
-            if (ex.hi) ex.hi[o] = u ? hi[k] : 0;
-            if (ex.b) ex.b[o] = u ? b[k] : 0;
-            if (ex.e) ex.e[o] = u ? e[k] : 0;
-        }
-        if (ex.cnt) ex.cnt[i] = (uint32_t)cnt;
     }
 }
 
@@ -1375,32 +1314,29 @@ void launch_write_geom(const QueryArgs& a, cudaStream_t st)
 
 }  // namespace
 
-// Opts plan_kernel<Bounds, DROP, EXPORT> into its dynamic shared memory (more than 48 KB for
-// the finest cover), once per instantiation and device.
-template <class Bounds, int DROP, bool EXPORT>
-static void allow_plan_smem()
+// Launches plan_kernel<Bounds, DIM, DROP, EXPORT>, opted into its dynamic shared memory (more
+// than 48 KB for the finest covers) once per instantiation and device.
+template <class Bounds, int DIM, int DROP, bool EXPORT>
+static void plan_dispatch(const QueryArgs& a, const Bounds& bounds, const PlanExport& ex, cudaStream_t st)
 {
     static bool done[64] = {false};
+    constexpr size_t smem = plan_smem_bytes<DIM, DROP>();
+    constexpr int T = Cover<DIM, DROP>::kThreads;
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 || done[dev]) return;
-    cudaFuncSetAttribute(plan_kernel<Bounds, DROP, EXPORT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)plan_smem_bytes<Bounds, DROP>());
-    done[dev] = true;
+    if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 && !done[dev]) {
+        cudaFuncSetAttribute(plan_kernel<Bounds, DIM, DROP, EXPORT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        done[dev] = true;
+    }
+    plan_kernel<Bounds, DIM, DROP, EXPORT><<<(unsigned)((a.m + T - 1) / T), T, smem, st>>>(a, bounds, ex);
+    count_launch();
 }
 
-template <int DROP, bool EXPORT>
-static void plan_dispatch(const QueryArgs& a, const LearnedModelView* lm, const PlanExport& ex, cudaStream_t st)
+template <class Bounds, bool EXPORT>
+static void plan_launch2(const QueryArgs& a, const Bounds& bounds, const PlanExport& ex, cudaStream_t st)
 {
-    const unsigned g = (unsigned)((a.m + kThreads - 1) / kThreads);
-    if (lm) {
-        allow_plan_smem<LearnedBounds, DROP, EXPORT>();
-        plan_kernel<LearnedBounds, DROP, EXPORT><<<g, kThreads, plan_smem_bytes<LearnedBounds, DROP>(), st>>>(
-            a, LearnedBounds{lm->root, lm->leaf, lm->fence, lm->fence_fine, lm->stats}, ex);
-    } else {
-        allow_plan_smem<BinaryBounds, DROP, EXPORT>();
-        plan_kernel<BinaryBounds, DROP, EXPORT><<<g, kThreads, plan_smem_bytes<BinaryBounds, DROP>(), st>>>(
-            a, BinaryBounds{}, ex);
-    }
+    if (a.drop == 0) plan_dispatch<Bounds, 2, 0, EXPORT>(a, bounds, ex, st);
+    else if (a.drop == 1) plan_dispatch<Bounds, 2, 1, EXPORT>(a, bounds, ex, st);
+    else plan_dispatch<Bounds, 2, 2, EXPORT>(a, bounds, ex, st);
 }
 
 template <bool EXPORT>
@@ -1408,16 +1344,15 @@ static sfc_status plan_launch(const QueryArgs& a, const LearnedModelView* lm, co
 {
     if (a.m == 0) return SFC_OK;
     if (a.dim == 3) {
-        const unsigned g = (unsigned)((a.m + kThreads - 1) / kThreads);
-        if (a.drop == 0) plan3_kernel<0, EXPORT><<<g, kThreads, 0, st>>>(a, ex);
-        else plan3_kernel<1, EXPORT><<<g, kThreads, 0, st>>>(a, ex);
-        count_launch();
-        return launch_status();
+        const BinaryBounds<3> binary{a.dir, a.dir_bits, 0, 0, 0};
+        if (a.drop == 0) plan_dispatch<BinaryBounds<3>, 3, 0, EXPORT>(a, binary, ex, st);
+        else plan_dispatch<BinaryBounds<3>, 3, 1, EXPORT>(a, binary, ex, st);
+    } else if (lm) {
+        plan_launch2<LearnedBounds, EXPORT>(a, LearnedBounds{lm->root, lm->leaf, lm->fence, lm->fence_fine, lm->stats}, ex,
+                                            st);
+    } else {
+        plan_launch2<BinaryBounds<2>, EXPORT>(a, BinaryBounds<2>{a.dir, a.dir_bits, 0, 0, 0}, ex, st);
     }
-    if (a.drop == 0) plan_dispatch<0, EXPORT>(a, lm, ex, st);
-    else if (a.drop == 1) plan_dispatch<1, EXPORT>(a, lm, ex, st);
-    else plan_dispatch<2, EXPORT>(a, lm, ex, st);
-    count_launch();
     return launch_status();
 }
 
@@ -1426,12 +1361,10 @@ sfc_status launch_plan(const QueryArgs& a, const LearnedModelView* lm, cudaStrea
     return plan_launch<false>(a, lm, PlanExport{}, st);
 }
 
-int cover_intervals(int drop) { return drop == 0 ? Cover<0>::K : (drop == 1 ? Cover<1>::K : Cover<2>::K); }
-
 int query_intervals(int dim, int drop)
 {
-    if (dim == 3) return drop == 0 ? Cover3<0>::K : Cover3<1>::K;
-    return cover_intervals(drop);
+    if (dim == 3) return drop == 0 ? Cover<3, 0>::K : Cover<3, 1>::K;
+    return drop == 0 ? Cover<2, 0>::K : (drop == 1 ? Cover<2, 1>::K : Cover<2, 2>::K);
 }
 
 static unsigned flat_grid(uint64_t m)

@@ -28,6 +28,8 @@ struct QueryArgs {
     const int32_t* q;            // [m][dim]
     const int32_t* delta;        // [m]
     uint64_t m;
+    const uint32_t* dir;         // key directory (boxes.cu), 2^dir_bits + 1 positions
+    int dir_bits;
     const int4* box;             // bounding boxes of the groups of 32 sorted points (boxes.cu)
     // plan results, by processing rank (the order in which queries are handed out)
     uint2* ranges;               // [m][kint]: the non-empty (begin, end) array ranges, in order
@@ -77,8 +79,7 @@ struct LearnedModelView {
 };
 
 sfc_status launch_plan(const QueryArgs& a, const LearnedModelView* lm, cudaStream_t st);
-int cover_intervals(int drop);   // intervals stored per query for a cover refinement
-int query_intervals(int dim, int drop);   // ... for an index of dimension dim
+int query_intervals(int dim, int drop);   // range slots per query for a cover refinement
 sfc_status launch_count(const QueryArgs& a, cudaStream_t st);
 // queries that scan at most this many points have no chunks in the statistics
 constexpr uint32_t kSmallScan = 64;

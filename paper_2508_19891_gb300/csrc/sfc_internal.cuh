@@ -48,6 +48,21 @@ int num_sms();   // SM count of the current device (cached per device)
 // without a bounds check (what lies past the last point is never used).
 inline uint64_t pad_groups(uint64_t n) { return (n + 31) / 32 * 32; }
 
+// Key directory (boxes.cu): the range of the sorted keys, kmin .. kmax, is cut into 2^bits parts of
+// 2^shift keys; entry v is the position of the first key of part v (lower_bound of kmin + v 2^shift).
+// Up to 2^18 parts (1 MB, kept in L2) of eight keys or more on average.
+inline int dir_bits(uint64_t n)
+{
+    int b = 1;
+    while (b < 18 && (n >> (b + 4)) != 0) ++b;
+    return b;
+}
+
+__device__ __forceinline__ int dir_shift(uint64_t kmin, uint64_t kmax, int bits)
+{
+    return max(64 - __clzll((long long)(kmax - kmin)) - bits, 0);
+}
+
 // First bit of depth t in the early-termination bitmap (depths stored one after another).
 __host__ __device__ __forceinline__ uint64_t occupancy_level_start(int t)
 {

@@ -85,3 +85,28 @@ def test_items_past_the_budget(cuda, reorder):
     got = u32(out)
     assert np.array_equal(got[:cap], rids[:cap]) and (got[cap:] == 0xFFFFFFFF).all()
     assert sfc.sfc_device_status(idx)[1] == sfc.SFC_DEV_CAPACITY
+
+
+@pytest.mark.parametrize("n", [1, 2, 15, 16, 17, 4096, 70_001])
+@pytest.mark.parametrize("spread", ["stack", "two", "corner", "domain"])
+def test_bounds_behind_the_directory(cuda, n, spread):
+    """Array positions of interval ends for key ranges of every kind: one key only, two far apart,
+    a small corner (directory parts narrower than a cell), the whole domain."""
+    rng = np.random.default_rng(n)
+    top = (1 << 30) - 1
+    pts = {"stack": np.full((n, 2), 12345), "two": rng.integers(0, 2, size=(n, 1)) * np.array([[top, top]]),
+           "corner": rng.integers(0, 50, size=(n, 2)), "domain": rng.integers(0, top + 1, size=(n, 2))}[spread].astype(np.int32)
+    m = 64
+    qs = np.concatenate([rng.integers(0, top + 1, size=(m // 2, 2)), pts[rng.integers(0, n, m // 2)]]).astype(np.int32)
+    d = np.exp(rng.uniform(0, np.log(2.0 ** 31 - 1), m)).astype(np.int32)
+    for curve in ("z", "h"):
+        ref = oracle.build(pts, 30, curve)
+        for cover in (0, 1, 2):
+            idx = sfc.sfc_build(to_dev(pts, cuda), curve, cover_refine=cover)
+            K = sfc.sfc_query_max_intervals(idx)
+            lo, hi, b, e, c = sfc.sfc_query_ranges(idx, to_dev(qs, cuda), to_dev(d, cuda))
+            lo, hi, b, e, c = u64(lo), u64(hi), u32(b), u32(e), u32(c)
+            for i in range(m):
+                for r in range(int(c[i])):
+                    assert b[K * i + r] == oracle.lower_bound(ref.keys, int(lo[K * i + r]))
+                    assert e[K * i + r] == oracle.lower_bound(ref.keys, int(hi[K * i + r]) + 1)
