@@ -229,7 +229,8 @@ sfc_status ensure_query_ws(sfc_index* idx, uint64_t m, uint64_t n, cudaStream_t 
     SFC_TRY(w.bhits.ensure(batches * sizeof(uint32_t), st));
     SFC_TRY(w.bbase.ensure((batches + 1) * sizeof(uint64_t), st));
     SFC_TRY(w.recs.ensure(recs * sizeof(uint2), st));
-    SFC_TRY(reserve_scan(idx->scan_ws, std::max<uint64_t>(m, batches + batches / 8 + 64), st));
+    // look-back words of the batch's three scans
+    SFC_TRY(w.flags.ensure((2 * scan_flag_words(m) + scan_flag_words(batches + batches / 8 + 64)) * sizeof(uint64_t), st));
     return SFC_OK;
 }
 
@@ -297,9 +298,16 @@ sfc_status do_count(sfc_index* idx, const int32_t* d_q, const int32_t* d_delta, 
     a.chunk = idx->chunk;
     a.out_offsets = d_out_offsets;
     a.scanned = scan_stats(idx);
-    // per-batch statistics: learned-bounds counters, the scanned total, cells and chunks
-    SFC_CUDA_TRY(cudaMemsetAsync(model_stats(idx), 0, 7 * sizeof(unsigned long long), st));
-    SFC_CUDA_TRY(cudaMemsetAsync(a.work_ctr, 0, kCtrWords * sizeof(unsigned long long), st));
+    // look-back words of the scans of the item counts, the batches' hits and the queries' hits
+    const uint64_t nb = std::min<uint64_t>(a.cap_batches, max_batches(idx->dim, m, idx->n, a.kint));
+    SFC_TRY(w.flags.ensure((2 * scan_flag_words(m) + scan_flag_words(nb)) * sizeof(uint64_t), st));
+    uint64_t* flags_items = w.flags.as<uint64_t>();
+    uint64_t* flags_counts = flags_items + scan_flag_words(m);
+    uint64_t* flags_hits = flags_counts + scan_flag_words(m);
+    // per-batch statistics (learned-bounds counters, the scanned total, cells and chunks) start at
+    // zero with the rest
+    SFC_TRY(launch_reset(model_stats(idx), 7, a.work_ctr, flags_items, 2 * scan_flag_words(m) + scan_flag_words(nb), st));
+    w.write_ctr_zero = true;
     LearnedModelView lv;
     const bool ordered = use_curve_order(idx, m);
     if (ordered) {
@@ -326,7 +334,7 @@ sfc_status do_count(sfc_index* idx, const int32_t* d_q, const int32_t* d_delta, 
     }
     {
         ProfScope ps(idx, "scan", st);
-        SFC_TRY(exclusive_scan_u32(a.nitems, m, a.gbase, idx->scan_ws, a.status, st));
+        SFC_TRY(launch_scan(a.nitems, m, a.gbase, flags_items, a.status, st));
     }
     {
         ProfScope ps(idx, "count", st);
@@ -334,9 +342,8 @@ sfc_status do_count(sfc_index* idx, const int32_t* d_q, const int32_t* d_delta, 
     }
     {
         ProfScope ps(idx, "scan", st);
-        SFC_TRY(exclusive_scan_u32(a.bhits, std::min<uint64_t>(a.cap_batches, max_batches(idx->dim, m, idx->n, a.kint)), a.bbase,
-                                   idx->scan_ws, a.status, st, a.gbase + m));
-        SFC_TRY(exclusive_scan_u32(a.counts, m, d_out_offsets, idx->scan_ws, a.status, st));
+        SFC_TRY(launch_scan_pair(a.bhits, nb, a.gbase + m, a.bbase, flags_hits, a.counts, m, d_out_offsets, flags_counts,
+                                 a.status, st));
         SFC_TRY(launch_dbase(a, st));
     }
     w.pending = {true, d_q, d_delta, m, d_out_offsets, ordered, a.drop, a.norm};
@@ -363,8 +370,10 @@ sfc_status do_write_range(sfc_index* idx, const int32_t* d_q, const int32_t* d_d
     a.ids_capacity = d_out_ids ? cap : 0;
     a.q_begin = q_begin;
     a.q_end = q_end;
-    // the write pass's own work counter starts at zero (a repeated write stays correct)
-    SFC_CUDA_TRY(cudaMemsetAsync(a.work_ctr + kCtrWrite, 0, sizeof(unsigned long long), st));
+    // the write pass's own work counter starts at zero: the count's reset serves the first write
+    // after it, a repeated one or the next slice clears it
+    if (!w.write_ctr_zero) SFC_CUDA_TRY(cudaMemsetAsync(a.work_ctr + kCtrWrite, 0, sizeof(unsigned long long), st));
+    w.write_ctr_zero = false;
     ProfScope ps(idx, "write", st);
     return launch_write(a, st);
 }
@@ -549,6 +558,7 @@ sfc_status sfc_reserve(sfc_index* idx, uint64_t n_max, uint64_t m_max, void* str
 }  // extern "C"
 
 struct sfc_graph {
+    sfc_index* idx = nullptr;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
 };
@@ -581,6 +591,7 @@ sfc_status sfc_graph_capture(sfc_index* idx, unsigned flags, const int32_t* d_po
     if (s == SFC_OK && ce != cudaSuccess) s = SFC_ERR_CUDA;
     if (s == SFC_OK && cudaGraphInstantiate(&g->exec, graph, 0) != cudaSuccess) s = SFC_ERR_CUDA;
     g->graph = graph;
+    g->idx = idx;
     cudaStreamDestroy(cs);
     idx->last_stream = st;
     if (s != SFC_OK) {
@@ -595,6 +606,7 @@ sfc_status sfc_graph_capture(sfc_index* idx, unsigned flags, const int32_t* d_po
 sfc_status sfc_graph_launch(sfc_graph* g, void* stream)
 {
     if (!g || !g->exec) return SFC_ERR_INVALID;
+    g->idx->qws.write_ctr_zero = false;   // a replayed batch uses the write pass's counter
     SFC_CUDA_TRY(cudaGraphLaunch(g->exec, as_stream(stream)));
     count_launch();
     return SFC_OK;

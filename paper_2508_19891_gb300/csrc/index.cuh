@@ -22,7 +22,9 @@ struct QueryWs {
     DevBuf ranges, qrec, nitems, gbase, ovf, counts, ctr;   // per query
     DevBuf heads, bhits, bbase;      // per batch of 32 items
     DevBuf recs;                     // the records of the items with hits
+    DevBuf flags;                    // look-back words of a batch's scans
     DevBuf qkeys, qkeys_sorted, perm, pstart, dbase;         // curve-order processing
+    bool write_ctr_zero = false;     // the write pass's work counter has not been used since the count
     PendingCount pending{false, nullptr, nullptr, 0, nullptr, false, 0, 0};
 };
 

@@ -1267,6 +1267,15 @@ __global__ void query_keys_kernel(const int32_t* __restrict__ q, uint64_t m, int
     }
 }
 
+__global__ void reset_kernel(unsigned long long* stats, int nstats, unsigned long long* ctr, uint64_t* flags,
+                             uint64_t nflags)
+{
+    const uint64_t i = blockIdx.x * (uint64_t)kThreads + threadIdx.x;
+    if (i < (uint64_t)nstats) stats[i] = 0;
+    if (i < (uint64_t)kCtrWords) ctr[i] = 0;
+    for (uint64_t w = i; w < nflags; w += (uint64_t)gridDim.x * kThreads) flags[w] = 0;
+}
+
 int persistent_grid(const void* fn)
 {
     int per_sm = 0;
@@ -1378,6 +1387,14 @@ sfc_status launch_query_keys(const int32_t* q, uint64_t m, int curve, int slices
 {
     if (m == 0) return SFC_OK;
     query_keys_kernel<<<flat_grid(m), kThreads, 0, st>>>(q, m, curve, slices, keys);
+    count_launch();
+    return launch_status();
+}
+
+sfc_status launch_reset(unsigned long long* stats, int nstats, unsigned long long* ctr, uint64_t* flags, uint64_t nflags,
+                        cudaStream_t st)
+{
+    reset_kernel<<<flat_grid(nflags), kThreads, 0, st>>>(stats, nstats, ctr, flags, nflags);
     count_launch();
     return launch_status();
 }

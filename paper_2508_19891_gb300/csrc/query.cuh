@@ -93,6 +93,10 @@ inline uint64_t max_batches(int dim, uint64_t m, uint64_t n, uint64_t kint)
 {
     return m * (n / 32 / item_groups(dim) + 2 * kint + 1) / 32 + 1;
 }
+// Zeroes what a query batch counts in: the statistics, the work counters and the look-back words
+// of its scans.
+sfc_status launch_reset(unsigned long long* stats, int nstats, unsigned long long* ctr, uint64_t* flags, uint64_t nflags,
+                        cudaStream_t st);
 // sort keys of the processing order: (input slice, top 24 bits of the centre's curve key)
 sfc_status launch_query_keys(const int32_t* q, uint64_t m, int curve, int slices, uint64_t* keys, cudaStream_t st);
 // dbase from the scans (with perm)

@@ -35,14 +35,37 @@ __device__ __forceinline__ uint64_t warp_incl_scan(uint64_t v)
     return v;
 }
 
-__global__ void __launch_bounds__(kThreads)
-scan_kernel(const uint32_t* __restrict__ in, uint64_t n, const uint64_t* __restrict__ per32,
-            uint64_t* __restrict__ out, uint64_t* flags /* [0] = tile counter, [1 + t] = tile words */,
-            uint32_t* status, int vec)
+// One scan: in[0 .. n) -> out[0 .. n]; flags[0] = tile counter, flags[1 + t] = tile words, all zero
+// before the launch; per32 (device): only the first min(n, ceil(*per32 / 32)) elements.
+struct ScanJob {
+    const uint32_t* in;
+    uint64_t n;
+    const uint64_t* per32;
+    uint64_t* out;
+    uint64_t* flags;
+    int vec;   // in and out 16-byte aligned
+};
+
+ScanJob scan_job(const uint32_t* in, uint64_t n, const uint64_t* per32, uint64_t* out, uint64_t* flags)
+{
+    return {in, n, per32, out, flags, ((((uintptr_t)in) & 15) == 0) && ((((uintptr_t)out) & 15) == 0)};
+}
+
+uint64_t scan_tiles(uint64_t n) { return (n + kTile - 1) / kTile; }
+
+// Blocks [0, blocks0) take the tiles of the first scan, the others those of the second.
+__global__ void __launch_bounds__(kThreads) scan_kernel(ScanJob j0, ScanJob j1, uint32_t blocks0, uint32_t* status)
 {
     __shared__ uint32_t s_tile;
     __shared__ uint64_t s_warp[kThreads / 32];
     __shared__ uint64_t s_excl;
+    const bool second = blockIdx.x >= blocks0;
+    const uint32_t* __restrict__ in = second ? j1.in : j0.in;
+    uint64_t* __restrict__ out = second ? j1.out : j0.out;
+    uint64_t* flags = second ? j1.flags : j0.flags;
+    const uint64_t* per32 = second ? j1.per32 : j0.per32;
+    uint64_t n = second ? j1.n : j0.n;
+    const int vec = second ? j1.vec : j0.vec;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) s_tile = atomicAdd(reinterpret_cast<unsigned long long*>(flags), 1ull);
     __syncthreads();
@@ -133,25 +156,42 @@ scan_kernel(const uint32_t* __restrict__ in, uint64_t n, const uint64_t* __restr
 
 }  // namespace
 
+uint64_t scan_flag_words(uint64_t n) { return scan_tiles(n) + 1; }
+
 sfc_status reserve_scan(ScanWorkspace& ws, uint64_t n, cudaStream_t st)
 {
-    const uint64_t tiles = (n + kTile - 1) / kTile;
-    return ws.flags.ensure((tiles + 1) * sizeof(uint64_t), st);
+    return ws.flags.ensure(scan_flag_words(n) * sizeof(uint64_t), st);
 }
 
 sfc_status exclusive_scan_u32(const uint32_t* in, uint64_t n, uint64_t* out, ScanWorkspace& ws,
-                              uint32_t* status, cudaStream_t st, const uint64_t* per32)
+                              uint32_t* status, cudaStream_t st)
 {
     if (n == 0) {
         SFC_CUDA_TRY(cudaMemsetAsync(out, 0, sizeof(uint64_t), st));
         return SFC_OK;
     }
-    uint64_t tiles = (n + kTile - 1) / kTile;
-    if (tiles > 0x7fffffffull) return SFC_ERR_INVALID;
-    SFC_TRY(ws.flags.ensure((tiles + 1) * sizeof(uint64_t), st));
-    SFC_CUDA_TRY(cudaMemsetAsync(ws.flags.ptr, 0, (tiles + 1) * sizeof(uint64_t), st));
-    int vec = ((((uintptr_t)in) & 15) == 0) && ((((uintptr_t)out) & 15) == 0);
-    scan_kernel<<<(unsigned)tiles, kThreads, 0, st>>>(in, n, per32, out, ws.flags.as<uint64_t>(), status, vec);
+    if (scan_tiles(n) > 0x7fffffffull) return SFC_ERR_INVALID;
+    SFC_TRY(reserve_scan(ws, n, st));
+    SFC_CUDA_TRY(cudaMemsetAsync(ws.flags.ptr, 0, scan_flag_words(n) * sizeof(uint64_t), st));
+    return launch_scan(in, n, out, ws.flags.as<uint64_t>(), status, st);
+}
+
+sfc_status launch_scan(const uint32_t* in, uint64_t n, uint64_t* out, uint64_t* flags, uint32_t* status, cudaStream_t st)
+{
+    const ScanJob j = scan_job(in, n, nullptr, out, flags);
+    const uint32_t blocks = (uint32_t)scan_tiles(n);
+    scan_kernel<<<blocks, kThreads, 0, st>>>(j, j, blocks, status);
+    count_launch();
+    return launch_status();
+}
+
+sfc_status launch_scan_pair(const uint32_t* in0, uint64_t n0, const uint64_t* per32, uint64_t* out0, uint64_t* flags0,
+                            const uint32_t* in1, uint64_t n1, uint64_t* out1, uint64_t* flags1, uint32_t* status,
+                            cudaStream_t st)
+{
+    const uint32_t b0 = (uint32_t)scan_tiles(n0), b1 = (uint32_t)scan_tiles(n1);
+    scan_kernel<<<b0 + b1, kThreads, 0, st>>>(scan_job(in0, n0, per32, out0, flags0),
+                                              scan_job(in1, n1, nullptr, out1, flags1), b0, status);
     count_launch();
     return launch_status();
 }
@@ -174,9 +214,8 @@ sfc_status exclusive_scan_standalone(const uint32_t* in, uint64_t n, uint64_t* o
     uint32_t bits = 0;
     if (cudaMemsetAsync(words, 0, (tiles + 2) * sizeof(uint64_t), st) != cudaSuccess) s = SFC_ERR_CUDA;
     if (s == SFC_OK) {
-        const int vec = ((((uintptr_t)in) & 15) == 0) && ((((uintptr_t)out) & 15) == 0);
-        scan_kernel<<<(unsigned)tiles, kThreads, 0, st>>>(in, n, nullptr, out, words + 1, reinterpret_cast<uint32_t*>(words),
-                                                          vec);
+        const ScanJob j = scan_job(in, n, nullptr, out, words + 1);
+        scan_kernel<<<(unsigned)tiles, kThreads, 0, st>>>(j, j, (uint32_t)tiles, reinterpret_cast<uint32_t*>(words));
         count_launch();
         s = launch_status();
     }
@@ -284,9 +323,8 @@ extern "C" sfc_status sfc_exclusive_scan_noalloc(const uint32_t* d_in, uint64_t 
         SFC_CUDA_TRY(cudaMemsetAsync(d_out, 0, sizeof(uint64_t), st));
         return SFC_OK;
     }
-    const int vec = ((((uintptr_t)d_in) & 15) == 0) && ((((uintptr_t)d_out) & 15) == 0);
-    scan_kernel<<<(unsigned)tiles, kThreads, 0, st>>>(d_in, n, nullptr, d_out, words + 1, reinterpret_cast<uint32_t*>(words),
-                                                      vec);
+    const ScanJob j = scan_job(d_in, n, nullptr, d_out, words + 1);
+    scan_kernel<<<(unsigned)tiles, kThreads, 0, st>>>(j, j, (uint32_t)tiles, reinterpret_cast<uint32_t*>(words));
     count_launch();
     return launch_status();
 }

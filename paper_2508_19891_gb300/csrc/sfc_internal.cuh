@@ -434,14 +434,20 @@ sfc_status launch_decode(const uint64_t* keys, uint64_t n, int curve, int2* pts,
 sfc_status launch_keys3(const int32_t* pts, uint64_t n, uint64_t* keys, uint32_t* status, cudaStream_t st);
 sfc_status launch_decode3(const uint64_t* keys, uint64_t n, int4* xyz, cudaStream_t st);
 
-// scan.cu: exclusive scan of uint32 (or a uint32 view) into uint64[n+1]; with per32 (device), of
-// the first min(n, ceil(*per32 / 32)) elements only.
+// scan.cu: exclusive scan of uint32 (or a uint32 view) into uint64[n+1].
 struct ScanWorkspace {
     DevBuf flags;
 };
 sfc_status exclusive_scan_u32(const uint32_t* in, uint64_t n, uint64_t* out, ScanWorkspace& ws,
-                              uint32_t* status, cudaStream_t st, const uint64_t* per32 = nullptr);
+                              uint32_t* status, cudaStream_t st);
 sfc_status reserve_scan(ScanWorkspace& ws, uint64_t n, cudaStream_t st);
+// the launch alone, with scan_flag_words(n) words of flags that the caller has zeroed (n > 0)
+uint64_t scan_flag_words(uint64_t n);
+sfc_status launch_scan(const uint32_t* in, uint64_t n, uint64_t* out, uint64_t* flags, uint32_t* status, cudaStream_t st);
+// two scans in one launch; per32 (device): the first takes its first min(n0, ceil(*per32 / 32)) elements
+sfc_status launch_scan_pair(const uint32_t* in0, uint64_t n0, const uint64_t* per32, uint64_t* out0, uint64_t* flags0,
+                            const uint32_t* in1, uint64_t n1, uint64_t* out1, uint64_t* flags1, uint32_t* status,
+                            cudaStream_t st);
 // the same with its own workspace and status word; synchronises st and returns
 // SFC_ERR_TIMEOUT if a look-back wait gave up
 sfc_status exclusive_scan_standalone(const uint32_t* in, uint64_t n, uint64_t* out, cudaStream_t st);

@@ -253,7 +253,7 @@ void release_index(sfc_index* idx, cudaStream_t st)
     idx->scan_ws.flags.release(st);
     QueryWs& q = idx->qws;
     for (DevBuf* d : {&q.ranges, &q.qrec, &q.nitems, &q.gbase, &q.ovf, &q.counts, &q.ctr, &q.heads, &q.bhits, &q.bbase,
-                      &q.recs, &q.qkeys, &q.qkeys_sorted, &q.perm, &q.pstart, &q.dbase})
+                      &q.recs, &q.flags, &q.qkeys, &q.qkeys_sorted, &q.perm, &q.pstart, &q.dbase})
         d->release(st);
     HostStage& h = idx->stage;
     h.q.release(st); h.delta.release(st); h.offsets.release(st); h.ids.release(st);
