@@ -234,9 +234,12 @@ def _pts(t, dim: int = 2):
 
 
 class _CudaView:
-    """Zero-copy view of library-owned device memory for torch.as_tensor."""
+    """Zero-copy view of library-owned device memory for torch.as_tensor.  The tensor holds this
+    object, and this object the index that owns the memory: a view outlives the caller's last
+    reference to the index."""
 
-    def __init__(self, ptr, shape, typestr):
+    def __init__(self, ptr, shape, typestr, owner):
+        self.owner = owner
         self.__cuda_array_interface__ = {"shape": shape, "typestr": typestr,
                                          "data": (int(ptr or 0), False), "version": 3,
                                          "strides": None, "stream": None}
@@ -671,9 +674,9 @@ def sfc_get_sorted(index: Index, copy: bool = True):
         return (torch.empty(0, dtype=torch.int64, device=dev), torch.empty(0, dtype=torch.int32, device=dev),
                 torch.empty((0, c), dtype=torch.int32, device=dev))
     with torch.cuda.device(dev):
-        kt = torch.as_tensor(_CudaView(k.value, (n,), "<i8"), device=dev)
-        it = torch.as_tensor(_CudaView(i.value, (n,), "<i4"), device=dev)
-        xt = torch.as_tensor(_CudaView(x.value, (n, c), "<i4"), device=dev)
+        kt = torch.as_tensor(_CudaView(k.value, (n,), "<i8", index), device=dev)
+        it = torch.as_tensor(_CudaView(i.value, (n,), "<i4", index), device=dev)
+        xt = torch.as_tensor(_CudaView(x.value, (n, c), "<i4", index), device=dev)
     if copy:
         return kt.clone(), it.clone(), xt.clone()
     return kt, it, xt

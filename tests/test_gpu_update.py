@@ -119,3 +119,21 @@ def test_repeated_delete_among_equal_points(cuda):
         sfc.sfc_update(idx, None, to_dev(np.array([7, 3, 7], np.int32), cuda))
     assert e.value.status == sfc.SFC_ERR_NOT_FOUND
     assert sfc.sfc_get_sorted(idx)[0].numel() == 10
+
+
+def test_sorted_views_outlive_the_callers_index(cuda):
+    """Zero-copy views of the sorted array keep the index that owns their memory alive."""
+    import gc
+    import weakref
+
+    pts, _, _ = W.tiny_dense(31, 5000, 1, 20, 10)
+    idx = sfc.sfc_build(to_dev(pts, cuda), "z")
+    want = u64(sfc.sfc_get_sorted(idx)[0])
+    keys, _, _ = sfc.sfc_get_sorted(idx, copy=False)
+    ref = weakref.ref(idx)
+    del idx, _
+    gc.collect()
+    assert ref() is not None and np.array_equal(u64(keys), want)
+    del keys
+    gc.collect()
+    assert ref() is None
