@@ -51,6 +51,7 @@ __global__ void __launch_bounds__(kT) boxes_kernel(const int2* __restrict__ xy, 
                                                    uint32_t n, uint32_t groups, int bits, uint32_t dblocks, uint32_t* dir,
                                                    int4* box)
 {
+    chain_start();
     if (blockIdx.x < dblocks) {
         fill_directory(keys, n, bits, dblocks, dir);
         return;
@@ -75,6 +76,7 @@ __global__ void __launch_bounds__(kT) boxes3_kernel(const int4* __restrict__ xyz
                                                     uint32_t n, uint32_t groups, int bits, uint32_t dblocks, uint32_t* dir,
                                                     int4* box)
 {
+    chain_start();
     if (blockIdx.x < dblocks) {
         fill_directory(keys, n, bits, dblocks, dir);
         return;
@@ -114,10 +116,10 @@ sfc_status build_boxes(sfc_index* idx, cudaStream_t st)
     const uint32_t dblocks = std::min((1u << bits) / kT + 1, (uint32_t)num_sms() * (large ? 2 : 4));
     const uint32_t grid = dblocks + std::min((groups + per_block - 1) / per_block, (uint32_t)num_sms() * (large ? 6 : 8));
     if (idx->dim == 3)
-        boxes3_kernel<<<grid, kT, 0, st>>>(idx->xyz.as<int4>(), idx->keys.as<uint64_t>(), (uint32_t)n, groups, bits, dblocks,
+        launch_chain(boxes3_kernel, grid, kT, 0, st, idx->xyz.as<int4>(), idx->keys.as<uint64_t>(), (uint32_t)n, groups, bits, dblocks,
                                            idx->dir.as<uint32_t>(), idx->box.as<int4>());
     else
-        boxes_kernel<<<grid, kT, 0, st>>>(idx->xy.as<int2>(), idx->keys.as<uint64_t>(), (uint32_t)n, groups, bits, dblocks,
+        launch_chain(boxes_kernel, grid, kT, 0, st, idx->xy.as<int2>(), idx->keys.as<uint64_t>(), (uint32_t)n, groups, bits, dblocks,
                                           idx->dir.as<uint32_t>(), idx->box.as<int4>());
     count_launch();
     return launch_status();

@@ -17,6 +17,7 @@ __global__ void __launch_bounds__(kThreads) keys_kernel(const int2* __restrict__
                                                         uint64_t* __restrict__ keys,
                                                         uint32_t* status, int vec)
 {
+    chain_start();
     __shared__ HilbertTables tb;
     if (CURVE == SFC_CURVE_HILBERT) hilbert_tables_init(&tb);
     if (!vec) {   // operands not 16-byte aligned: one point per thread
@@ -55,6 +56,7 @@ template <int CURVE>
 __global__ void __launch_bounds__(kThreads) decode_kernel(const uint64_t* __restrict__ keys,
                                                           uint64_t n, int2* __restrict__ pts)
 {
+    chain_start();
     __shared__ HilbertTables tb;
     if (CURVE == SFC_CURVE_HILBERT) hilbert_tables_init(&tb);
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
@@ -72,6 +74,7 @@ __global__ void __launch_bounds__(kThreads) decode_kernel(const uint64_t* __rest
 __global__ void __launch_bounds__(kThreads) keys3_kernel(const int32_t* __restrict__ pts, uint64_t n,
                                                          uint64_t* __restrict__ keys, uint32_t* status)
 {
+    chain_start();
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     bool bad = false;
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
@@ -85,6 +88,7 @@ __global__ void __launch_bounds__(kThreads) keys3_kernel(const int32_t* __restri
 __global__ void __launch_bounds__(kThreads) decode3_kernel(const uint64_t* __restrict__ keys, uint64_t n,
                                                            int4* __restrict__ xyz)
 {
+    chain_start();
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
         const uint64_t k = keys[i];
@@ -110,9 +114,9 @@ sfc_status launch_keys(const int2* pts, uint64_t n, int curve, uint64_t* keys, u
     int vec = (((uintptr_t)pts | (uintptr_t)keys) & 15) == 0;
     int g = grid_for(vec ? (n + 1) / 2 : n, kThreads);
     if (curve == SFC_CURVE_HILBERT)
-        keys_kernel<SFC_CURVE_HILBERT><<<g, kThreads, 0, st>>>(pts, n, keys, status, vec);
+        launch_chain(keys_kernel<SFC_CURVE_HILBERT>, g, kThreads, 0, st, pts, n, keys, status, vec);
     else
-        keys_kernel<SFC_CURVE_Z><<<g, kThreads, 0, st>>>(pts, n, keys, status, vec);
+        launch_chain(keys_kernel<SFC_CURVE_Z>, g, kThreads, 0, st, pts, n, keys, status, vec);
     count_launch();
     return launch_status();
 }
@@ -122,9 +126,9 @@ sfc_status launch_decode(const uint64_t* keys, uint64_t n, int curve, int2* pts,
     if (n == 0) return SFC_OK;
     int g = grid_for(n, kThreads);
     if (curve == SFC_CURVE_HILBERT)
-        decode_kernel<SFC_CURVE_HILBERT><<<g, kThreads, 0, st>>>(keys, n, pts);
+        launch_chain(decode_kernel<SFC_CURVE_HILBERT>, g, kThreads, 0, st, keys, n, pts);
     else
-        decode_kernel<SFC_CURVE_Z><<<g, kThreads, 0, st>>>(keys, n, pts);
+        launch_chain(decode_kernel<SFC_CURVE_Z>, g, kThreads, 0, st, keys, n, pts);
     count_launch();
     return launch_status();
 }
@@ -132,7 +136,7 @@ sfc_status launch_decode(const uint64_t* keys, uint64_t n, int curve, int2* pts,
 sfc_status launch_keys3(const int32_t* pts, uint64_t n, uint64_t* keys, uint32_t* status, cudaStream_t st)
 {
     if (n == 0) return SFC_OK;
-    keys3_kernel<<<grid_for(n, kThreads), kThreads, 0, st>>>(pts, n, keys, status);
+    launch_chain(keys3_kernel, grid_for(n, kThreads), kThreads, 0, st, pts, n, keys, status);
     count_launch();
     return launch_status();
 }
@@ -140,7 +144,7 @@ sfc_status launch_keys3(const int32_t* pts, uint64_t n, uint64_t* keys, uint32_t
 sfc_status launch_decode3(const uint64_t* keys, uint64_t n, int4* xyz, cudaStream_t st)
 {
     if (n == 0) return SFC_OK;
-    decode3_kernel<<<grid_for(n, kThreads), kThreads, 0, st>>>(keys, n, xyz);
+    launch_chain(decode3_kernel, grid_for(n, kThreads), kThreads, 0, st, keys, n, xyz);
     count_launch();
     return launch_status();
 }

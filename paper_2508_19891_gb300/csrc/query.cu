@@ -597,6 +597,7 @@ template <class Bounds, int DIM, int DROP, bool EXPORT>
 __global__ void __launch_bounds__((Cover<DIM, DROP>::kThreads), Bounds::kMinBlocks)
 plan_kernel(QueryArgs a, Bounds bounds_in, PlanExport ex)
 {
+    chain_start();
     constexpr int K = Cover<DIM, DROP>::K, kThreads = Cover<DIM, DROP>::kThreads;
     __shared__ HilbertTables tb;
     __shared__ RootParams s_root;
@@ -1009,6 +1010,7 @@ __device__ __forceinline__ uint32_t lanemask_le() { return lanemask_lt() | (1u <
 template <int GEOM>
 __global__ void __launch_bounds__(kThreads, SFC_COUNT_BLOCKS) count_kernel(QueryArgs a)
 {
+    chain_start();
     constexpr int kGroups = Geom<GEOM>::kGroups;
     __shared__ FilterSmem<GEOM> s_filter[kThreads / 32];
     FilterSmem<GEOM>* sm = &s_filter[threadIdx.x >> 5];
@@ -1151,6 +1153,7 @@ __device__ __forceinline__ void copy_records(const QueryArgs& a, bool fits, uint
 // 48.8 ms -> 0.08 ms, as no warp owns a query.
 __global__ void __launch_bounds__(kThreads, SFC_WRITE_BLOCKS) write_kernel(QueryArgs a)
 {
+    chain_start();
     __shared__ CopySmem s_copy[kThreads / 32];
     CopySmem* sm = &s_copy[threadIdx.x >> 5];
     const unsigned lane = lane_id();
@@ -1200,6 +1203,7 @@ __global__ void __launch_bounds__(kThreads, SFC_WRITE_BLOCKS) write_kernel(Query
 template <int GEOM>
 __global__ void __launch_bounds__(kThreads) refilter_kernel(QueryArgs a)
 {
+    chain_start();
     constexpr int kGroups = Geom<GEOM>::kGroups;
     __shared__ FilterSmem<GEOM> s_filter[kThreads / 32];
     __shared__ CopySmem s_copy[kThreads / 32];
@@ -1242,6 +1246,7 @@ __global__ void __launch_bounds__(kThreads) refilter_kernel(QueryArgs a)
 // minus the hits before its first item.
 __global__ void dbase_kernel(QueryArgs a)
 {
+    chain_start();
     for (uint64_t r = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; r < a.m; r += (uint64_t)gridDim.x * blockDim.x) {
         const uint64_t b = a.gbase[r] >> 5;
         if (b < a.cap_batches)
@@ -1253,6 +1258,7 @@ __global__ void dbase_kernel(QueryArgs a)
 // cut into [floor(m s / slices), floor(m (s + 1) / slices))), then the curve key of its centre.
 __global__ void query_keys_kernel(const int32_t* __restrict__ q, uint64_t m, int curve, int slices, uint64_t* keys)
 {
+    chain_start();
     __shared__ HilbertTables tb;
     if (curve == SFC_CURVE_HILBERT) hilbert_tables_init(&tb);
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < m; i += (uint64_t)gridDim.x * blockDim.x) {
@@ -1270,6 +1276,7 @@ __global__ void query_keys_kernel(const int32_t* __restrict__ q, uint64_t m, int
 __global__ void reset_kernel(unsigned long long* stats, int nstats, unsigned long long* ctr, uint64_t* flags,
                              uint64_t nflags)
 {
+    chain_start();
     const uint64_t i = blockIdx.x * (uint64_t)kThreads + threadIdx.x;
     if (i < (uint64_t)nstats) stats[i] = 0;
     if (i < (uint64_t)kCtrWords) ctr[i] = 0;
@@ -1305,7 +1312,7 @@ template <int GEOM>
 void launch_count_geom(const QueryArgs& a, cudaStream_t st)
 {
     static const int g = persistent_grid((const void*)count_kernel<GEOM>);
-    count_kernel<GEOM><<<batch_grid(a, g), kThreads, 0, st>>>(a);
+    launch_chain(count_kernel<GEOM>, batch_grid(a, g), kThreads, 0, st, a);
     count_launch();
 }
 
@@ -1313,10 +1320,10 @@ template <int GEOM>
 void launch_write_geom(const QueryArgs& a, cudaStream_t st)
 {
     static const int g = persistent_grid((const void*)write_kernel);
-    write_kernel<<<batch_grid(a, g), kThreads, 0, st>>>(a);
+    launch_chain(write_kernel, batch_grid(a, g), kThreads, 0, st, a);
     count_launch();
     if (may_overflow(a)) {
-        refilter_kernel<GEOM><<<num_sms() * 4, kThreads, 0, st>>>(a);
+        launch_chain(refilter_kernel<GEOM>, num_sms() * 4, kThreads, 0, st, a);
         count_launch();
     }
 }
@@ -1336,7 +1343,7 @@ static void plan_dispatch(const QueryArgs& a, const Bounds& bounds, const PlanEx
         cudaFuncSetAttribute(plan_kernel<Bounds, DIM, DROP, EXPORT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         done[dev] = true;
     }
-    plan_kernel<Bounds, DIM, DROP, EXPORT><<<(unsigned)((a.m + T - 1) / T), T, smem, st>>>(a, bounds, ex);
+    launch_chain(plan_kernel<Bounds, DIM, DROP, EXPORT>, (unsigned)((a.m + T - 1) / T), T, smem, st, a, bounds, ex);
     count_launch();
 }
 
@@ -1386,7 +1393,7 @@ static unsigned flat_grid(uint64_t m)
 sfc_status launch_query_keys(const int32_t* q, uint64_t m, int curve, int slices, uint64_t* keys, cudaStream_t st)
 {
     if (m == 0) return SFC_OK;
-    query_keys_kernel<<<flat_grid(m), kThreads, 0, st>>>(q, m, curve, slices, keys);
+    launch_chain(query_keys_kernel, flat_grid(m), kThreads, 0, st, q, m, curve, slices, keys);
     count_launch();
     return launch_status();
 }
@@ -1394,7 +1401,7 @@ sfc_status launch_query_keys(const int32_t* q, uint64_t m, int curve, int slices
 sfc_status launch_reset(unsigned long long* stats, int nstats, unsigned long long* ctr, uint64_t* flags, uint64_t nflags,
                         cudaStream_t st)
 {
-    reset_kernel<<<flat_grid(nflags), kThreads, 0, st>>>(stats, nstats, ctr, flags, nflags);
+    launch_chain(reset_kernel, flat_grid(nflags), kThreads, 0, st, stats, nstats, ctr, flags, nflags);
     count_launch();
     return launch_status();
 }
@@ -1402,7 +1409,7 @@ sfc_status launch_reset(unsigned long long* stats, int nstats, unsigned long lon
 sfc_status launch_dbase(const QueryArgs& a, cudaStream_t st)
 {
     if (a.m == 0 || !a.dbase) return SFC_OK;
-    dbase_kernel<<<flat_grid(a.m), kThreads, 0, st>>>(a);
+    launch_chain(dbase_kernel, flat_grid(a.m), kThreads, 0, st, a);
     count_launch();
     return launch_status();
 }

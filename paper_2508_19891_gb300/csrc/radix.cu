@@ -121,6 +121,7 @@ __device__ __forceinline__ uint64_t source_key(const SortSource& s, const Hilber
 template <int CURVE, int SAMPLE>
 __global__ void __launch_bounds__(1024) sample_kernel(SortSource src, uint64_t n, Small* sm)
 {
+    chain_start();
     __shared__ HilbertTables tb;
     __shared__ unsigned long long s_pairs, s_live;
     constexpr uint32_t kSlots = 2 * SAMPLE;
@@ -189,6 +190,7 @@ template <int CURVE>
 __global__ void __launch_bounds__(kHistThreads) hist_kernel(SortSource src, uint64_t n, uint64_t* keys_out, Small* sm,
                                                             uint32_t* status)
 {
+    chain_start();
     __shared__ HilbertTables tb;
     extern __shared__ uint32_t s_rows[];   // [passes][kRadix][kHistRow]
     if (CURVE == SFC_CURVE_HILBERT && src.points) hilbert_tables_init(&tb);
@@ -252,6 +254,7 @@ __global__ void __launch_bounds__(kHistThreads) hist_kernel(SortSource src, uint
 // One block of 256 threads (thread = digit).
 __global__ void __launch_bounds__(kRadix) plan_kernel(Small* sm, uint64_t n, int bits, uint32_t* epoch_ctr)
 {
+    chain_start();
     if (threadIdx.x == 0) {
         // 30-bit epochs, never 0 (the value of a cleared word); wraps after 2^27 sorts
         uint32_t e = *epoch_ctr;
@@ -382,6 +385,7 @@ __device__ __forceinline__ void rank_keys(const uint64_t (&key)[ITEMS], int shif
 template <int CURVE, int ITEMS>
 __global__ void __launch_bounds__(kThreads, SFC_SORT_BLOCKS) onesweep_kernel(PassArgs a)
 {
+    chain_start();
     const PassPlan pl = a.sm->plan[a.pass];
     if (!pl.active) return;
     const uint32_t epoch = a.sm->epoch_base + (uint32_t)a.pass;
@@ -561,6 +565,7 @@ static_assert(kFixSpan <= 1 << kFixAt && kFixHalo * 2 <= kFixThreads, "");
 template <int CURVE>
 __global__ void __launch_bounds__(kFixThreads, SFC_FIX_BLOCKS) fix_kernel(PassArgs a)
 {
+    chain_start();
     const uint32_t low = a.sm->low;
     if (low == 0) return;   // sorted by all digits
     __shared__ HilbertTables tb;
@@ -670,6 +675,7 @@ __global__ void __launch_bounds__(kFixThreads, SFC_FIX_BLOCKS) fix_kernel(PassAr
 template <int CURVE>
 __global__ void __launch_bounds__(kThreads) long_kernel(PassArgs a)
 {
+    chain_start();
     const uint32_t runs = a.sm->runs;
     if (runs == 0) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -771,7 +777,7 @@ void launch_sample(const PassArgs& a, cudaStream_t st)
     static bool ok[64] = {false};
     constexpr size_t smem = 3 * SAMPLE * sizeof(uint32_t);
     allow_smem((const void*)sample_kernel<CURVE, SAMPLE>, smem, ok);
-    sample_kernel<CURVE, SAMPLE><<<1, 1024, smem, st>>>(a.src, a.n, a.sm);
+    launch_chain(sample_kernel<CURVE, SAMPLE>, 1, 1024, smem, st, a.src, a.n, a.sm);
     count_launch();
 }
 
@@ -782,7 +788,7 @@ void launch_pass(const PassArgs& a, cudaStream_t st)
     allow_smem((const void*)onesweep_kernel<CURVE, ITEMS>, sizeof(PassSmem<ITEMS>), ok);
     const uint64_t tiles = (a.n + kThreads * ITEMS - 1) / (kThreads * ITEMS);
     const unsigned grid = (unsigned)std::min<uint64_t>(tiles, (uint64_t)num_sms() * SFC_SORT_BLOCKS);
-    onesweep_kernel<CURVE, ITEMS><<<grid, kThreads, sizeof(PassSmem<ITEMS>), st>>>(a);
+    launch_chain(onesweep_kernel<CURVE, ITEMS>, grid, kThreads, sizeof(PassSmem<ITEMS>), st, a);
     count_launch();
 }
 
@@ -805,12 +811,12 @@ sfc_status run_sort(const PassArgs& args, uint32_t* epoch, cudaStream_t st)
     allow_smem((const void*)hist_kernel<CURVE>, (size_t)kPasses * kRadix * kHistRow * sizeof(uint32_t), hist_ok);
     const uint64_t hgrid = std::min<uint64_t>((a.n + kHistThreads * 4 - 1) / (kHistThreads * 4),
                                               std::max<uint64_t>(num_sms(), a.n / kHistMost + 1));
-    hist_kernel<CURVE><<<(unsigned)hgrid, kHistThreads, hsmem, st>>>(a.src, a.n, a.tmp_keys[1], a.sm, a.status);
+    launch_chain(hist_kernel<CURVE>, (unsigned)hgrid, kHistThreads, hsmem, st, a.src, a.n, a.tmp_keys[1], a.sm, a.status);
     if (a.src.points) {   // the passes read the keys
         a.src.points = nullptr;
         a.src.keys = a.tmp_keys[1];
     }
-    plan_kernel<<<1, kRadix, 0, st>>>(a.sm, a.n, a.src.bits, epoch);
+    launch_chain(plan_kernel, 1, kRadix, 0, st, a.sm, a.n, a.src.bits, epoch);
     count_launch(2);
     for (int p = 0; p < all; ++p) {
         a.pass = p;
@@ -820,10 +826,10 @@ sfc_status run_sort(const PassArgs& args, uint32_t* epoch, cudaStream_t st)
     if (sample) {
         static bool ok[64] = {false};
         const uint64_t ftiles = (a.n + kFixTile - 1) / kFixTile;
-        fix_kernel<CURVE><<<(unsigned)std::min<uint64_t>(ftiles, (uint64_t)num_sms() * 8), kFixThreads, 0, st>>>(a);
+        launch_chain(fix_kernel<CURVE>, (unsigned)std::min<uint64_t>(ftiles, (uint64_t)num_sms() * 8), kFixThreads, 0, st, a);
         allow_smem((const void*)long_kernel<CURVE>, sizeof(PassSmem<kItems>), ok);
         const unsigned lgrid = (unsigned)std::min<uint64_t>(a.n / kMaxRun + 1, (uint64_t)num_sms());
-        long_kernel<CURVE><<<lgrid, kThreads, sizeof(PassSmem<kItems>), st>>>(a);
+        launch_chain(long_kernel<CURVE>, lgrid, kThreads, sizeof(PassSmem<kItems>), st, a);
         count_launch(2);
     }
     return launch_status();

@@ -56,6 +56,7 @@ uint64_t scan_tiles(uint64_t n) { return (n + kTile - 1) / kTile; }
 // Blocks [0, blocks0) take the tiles of the first scan, the others those of the second.
 __global__ void __launch_bounds__(kThreads) scan_kernel(ScanJob j0, ScanJob j1, uint32_t blocks0, uint32_t* status)
 {
+    chain_start();
     __shared__ uint32_t s_tile;
     __shared__ uint64_t s_warp[kThreads / 32];
     __shared__ uint64_t s_excl;
@@ -180,7 +181,7 @@ sfc_status launch_scan(const uint32_t* in, uint64_t n, uint64_t* out, uint64_t* 
 {
     const ScanJob j = scan_job(in, n, nullptr, out, flags);
     const uint32_t blocks = (uint32_t)scan_tiles(n);
-    scan_kernel<<<blocks, kThreads, 0, st>>>(j, j, blocks, status);
+    launch_chain(scan_kernel, blocks, kThreads, 0, st, j, j, blocks, status);
     count_launch();
     return launch_status();
 }
@@ -190,7 +191,7 @@ sfc_status launch_scan_pair(const uint32_t* in0, uint64_t n0, const uint64_t* pe
                             cudaStream_t st)
 {
     const uint32_t b0 = (uint32_t)scan_tiles(n0), b1 = (uint32_t)scan_tiles(n1);
-    scan_kernel<<<b0 + b1, kThreads, 0, st>>>(scan_job(in0, n0, per32, out0, flags0),
+    launch_chain(scan_kernel, b0 + b1, kThreads, 0, st, scan_job(in0, n0, per32, out0, flags0),
                                               scan_job(in1, n1, nullptr, out1, flags1), b0, status);
     count_launch();
     return launch_status();
@@ -215,7 +216,7 @@ sfc_status exclusive_scan_standalone(const uint32_t* in, uint64_t n, uint64_t* o
     if (cudaMemsetAsync(words, 0, (tiles + 2) * sizeof(uint64_t), st) != cudaSuccess) s = SFC_ERR_CUDA;
     if (s == SFC_OK) {
         const ScanJob j = scan_job(in, n, nullptr, out, words + 1);
-        scan_kernel<<<(unsigned)tiles, kThreads, 0, st>>>(j, j, (uint32_t)tiles, reinterpret_cast<uint32_t*>(words));
+        launch_chain(scan_kernel, (unsigned)tiles, kThreads, 0, st, j, j, (uint32_t)tiles, reinterpret_cast<uint32_t*>(words));
         count_launch();
         s = launch_status();
     }
@@ -324,7 +325,7 @@ extern "C" sfc_status sfc_exclusive_scan_noalloc(const uint32_t* d_in, uint64_t 
         return SFC_OK;
     }
     const ScanJob j = scan_job(d_in, n, nullptr, d_out, words + 1);
-    scan_kernel<<<(unsigned)tiles, kThreads, 0, st>>>(j, j, (uint32_t)tiles, reinterpret_cast<uint32_t*>(words));
+    launch_chain(scan_kernel, (unsigned)tiles, kThreads, 0, st, j, j, (uint32_t)tiles, reinterpret_cast<uint32_t*>(words));
     count_launch();
     return launch_status();
 }

@@ -42,6 +42,33 @@ inline sfc_status launch_status()
     return e == cudaErrorMemoryAllocation ? SFC_ERR_OOM : SFC_ERR_CUDA;
 }
 
+// Launches of a chain: the next kernel is set up while the blocks of the one before it in the stream
+// are ending (programmatic dependent launch).  Every kernel launched this way begins with
+// chain_start(), which waits until the one before has completed with its writes visible, so
+// nothing it touches is still in use.  After any other stream operation the launch is an ordinary
+// one.  Takes part of the gaps between launches, which set the time of small calls (one lookup 68 ->
+// 54 us, 3*10^5 points built and queried 185 -> 129 us, an update of 5*10^7 points 810 -> 725 us).
+// No kernel lets the next one go before its own blocks end: waiting blocks would take room beside
+// working ones (let go at its start by every kernel, 10^7 3-D points with 10^6 balls took 5.35 ms
+// instead of 3.96, by grids of up to 456 blocks 10^8 points with 10^7 queries 20.7 instead of 19.6).
+template <class... P, class... A>
+inline void launch_chain(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, A&&... args)
+{
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3(grid);
+    c.blockDim = dim3(block);
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+
+__device__ __forceinline__ void chain_start() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 int num_sms();   // SM count of the current device (cached per device)
 
 // Points that a coordinate array has room for: whole groups of 32, so that a group can be loaded

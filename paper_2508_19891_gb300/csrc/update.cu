@@ -40,6 +40,7 @@ int grid_of(uint64_t n)
 __global__ void del_keys_kernel(const uint32_t* __restrict__ del, uint64_t k, const int2* __restrict__ xy_by_id,
                                 uint32_t next_id, int curve, uint64_t* keys_out)
 {
+    chain_start();
     __shared__ HilbertTables tb;
     if (curve == SFC_CURVE_HILBERT) hilbert_tables_init(&tb);
     for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < k; t += (uint64_t)gridDim.x * blockDim.x) {
@@ -66,6 +67,7 @@ __global__ void del_locate_kernel(const uint64_t* __restrict__ keys, const uint3
                                   const uint32_t* __restrict__ alive, uint32_t next_id, uint32_t* dpos,
                                   uint32_t* dbits, uint32_t* dcount, uint32_t* bad)
 {
+    chain_start();
     for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < k; t += (uint64_t)gridDim.x * blockDim.x) {
         const uint64_t kk = dkeys[t];
         const uint32_t id = dids[t];
@@ -92,6 +94,7 @@ __global__ void del_locate_kernel(const uint64_t* __restrict__ keys, const uint3
 __global__ void ins_rank_kernel(const uint64_t* __restrict__ keys, uint32_t n, const uint64_t* __restrict__ ikeys,
                                 uint64_t k, uint32_t* rank)
 {
+    chain_start();
     for (uint64_t j = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; j < k; j += (uint64_t)gridDim.x * blockDim.x) {
         const uint64_t kk = ikeys[j];
         uint32_t lo = 0, len = n;
@@ -110,6 +113,7 @@ __global__ void ins_rank_kernel(const uint64_t* __restrict__ keys, uint32_t n, c
 // rest).  A position may be n (an insert after every entry).
 __global__ void tile_starts_kernel(const uint32_t* __restrict__ pos, uint64_t k, uint32_t tiles, uint32_t* starts)
 {
+    chain_start();
     for (uint64_t j = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; j <= k; j += (uint64_t)gridDim.x * blockDim.x) {
         const uint32_t t0 = j ? pos[j - 1] / kMoveTile + 1 : 0;
         const uint32_t t1 = j < k ? min(pos[j] / kMoveTile, tiles) : tiles;
@@ -128,6 +132,7 @@ __global__ void __launch_bounds__(kT) move_kernel(const uint64_t* __restrict__ k
                                                   const uint32_t* __restrict__ rank, const uint32_t* __restrict__ istart,
                                                   uint64_t* nkeys, uint32_t* nids, int2* nxy)
 {
+    chain_start();
     __shared__ uint32_t s_ins[kMoveTile];   // inserts ranked at each entry, then its slot in the tile's output
     __shared__ uint32_t s_warp[kT / 32];
     const int tid = threadIdx.x;
@@ -193,6 +198,7 @@ __global__ void ins_place_kernel(const uint64_t* __restrict__ ikeys, const uint3
                                  const uint32_t* __restrict__ dpos, uint64_t kdel, uint64_t* nkeys, uint32_t* nids,
                                  int2* nxy)
 {
+    chain_start();
     for (uint64_t j = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; j < k; j += (uint64_t)gridDim.x * blockDim.x) {
         const uint32_t r = rank[j];
         // deletes at positions < r (dpos is ascending)
@@ -212,6 +218,7 @@ __global__ void ins_place_kernel(const uint64_t* __restrict__ ikeys, const uint3
 
 __global__ void alive_clear_kernel(const uint32_t* __restrict__ del, uint64_t k, uint32_t* alive)
 {
+    chain_start();
     for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < k; t += (uint64_t)gridDim.x * blockDim.x) {
         const uint32_t id = del[t];
         atomicAnd(alive + (id >> 5), ~(1u << (id & 31)));
@@ -305,7 +312,7 @@ sfc_status apply_update(sfc_index* idx, const int32_t* d_inserts, uint64_t k_ins
         dkeys = dkeys_in + k_del;
         dids = U.c.as<uint32_t>();
         dpos = U.d.as<uint32_t>();
-        del_keys_kernel<<<grid_of(k_del), kT, 0, st>>>(d_del, k_del, idx->xy_by_id.as<int2>(), next_id, curve, dkeys_in);
+        launch_chain(del_keys_kernel, grid_of(k_del), kT, 0, st, d_del, k_del, idx->xy_by_id.as<int2>(), next_id, curve, dkeys_in);
         count_launch();
         SortSource src;
         src.keys = dkeys_in;
@@ -321,7 +328,7 @@ sfc_status apply_update(sfc_index* idx, const int32_t* d_inserts, uint64_t k_ins
         dbits = U.marks.as<uint32_t>();
         uint32_t* dcount = dbits + (n / 32 + 1);
         SFC_CUDA_TRY(cudaMemsetAsync(dbits, 0, ((size_t)(n / 32 + 1) + tiles) * sizeof(uint32_t), st));
-        del_locate_kernel<<<grid_of(k_del), kT, 0, st>>>(idx->keys.as<uint64_t>(), idx->ids.as<uint32_t>(), n, dkeys, dids,
+        launch_chain(del_locate_kernel, grid_of(k_del), kT, 0, st, idx->keys.as<uint64_t>(), idx->ids.as<uint32_t>(), n, dkeys, dids,
                                                          k_del, idx->alive.as<uint32_t>(), next_id, dpos, dbits, dcount,
                                                          bad);
         count_launch();
@@ -368,8 +375,8 @@ sfc_status apply_update(sfc_index* idx, const int32_t* d_inserts, uint64_t k_ins
     const uint64_t* keys = idx->keys.as<uint64_t>();
     const uint32_t* ids = idx->ids.as<uint32_t>();
     if (k_ins) {
-        ins_rank_kernel<<<grid_of(k_ins), kT, 0, st>>>(keys, n, ikeys, k_ins, irank);
-        tile_starts_kernel<<<grid_of(k_ins + 1), kT, 0, st>>>(irank, k_ins, tiles, istart);
+        launch_chain(ins_rank_kernel, grid_of(k_ins), kT, 0, st, keys, n, ikeys, k_ins, irank);
+        launch_chain(tile_starts_kernel, grid_of(k_ins + 1), kT, 0, st, irank, k_ins, tiles, istart);
         count_launch(2);
     }
     SFC_TRY(launch_status());
@@ -377,17 +384,17 @@ sfc_status apply_update(sfc_index* idx, const int32_t* d_inserts, uint64_t k_ins
     uint32_t* nids = U.ids.as<uint32_t>();
     int2* nxy = U.xy.as<int2>();
     if (n) {
-        move_kernel<<<tiles, kT, 0, st>>>(keys, ids, idx->xy.as<int2>(), n, dbits, U.dstart.as<uint64_t>(), irank, istart,
+        launch_chain(move_kernel, tiles, kT, 0, st, keys, ids, idx->xy.as<int2>(), n, dbits, U.dstart.as<uint64_t>(), irank, istart,
                                           nkeys, nids, nxy);
         count_launch();
     }
     if (k_ins) {
-        ins_place_kernel<<<grid_of(k_ins), kT, 0, st>>>(ikeys, iids, ixy, k_ins, irank, dpos, k_del, nkeys, nids, nxy);
+        launch_chain(ins_place_kernel, grid_of(k_ins), kT, 0, st, ikeys, iids, ixy, k_ins, irank, dpos, k_del, nkeys, nids, nxy);
         count_launch();
     }
     // ---- liveness and the id -> coordinates table ----
     if (k_del) {
-        alive_clear_kernel<<<grid_of(k_del), kT, 0, st>>>(d_del, k_del, idx->alive.as<uint32_t>());
+        launch_chain(alive_clear_kernel, grid_of(k_del), kT, 0, st, d_del, k_del, idx->alive.as<uint32_t>());
         count_launch();
     }
     SFC_TRY(launch_status());
