@@ -144,14 +144,15 @@ sfc_status build_from_device(sfc_index* idx, const int32_t* d_points, cudaStream
     return SFC_OK;
 }
 
-// 3-D: keys of the input points, the (key, id) sort, and the coordinates decoded from the sorted
-// keys into 16-byte records.
+// 3-D: keys of the input points, the (key, id) sort, and (with the boxes) the coordinates decoded
+// from the sorted keys.
 sfc_status build3_from_device(sfc_index* idx, const int32_t* d_points, cudaStream_t st)
 {
     const uint64_t n = idx->n;
     SFC_TRY(idx->keys.ensure(n * sizeof(uint64_t), st));
     SFC_TRY(idx->ids.ensure(n * sizeof(uint32_t), st));
-    SFC_TRY(idx->xyz.ensure(pad_groups(n) * sizeof(int4), st));
+    SFC_TRY(idx->xyz.ensure(n * sizeof(int4), st));
+    SFC_TRY(idx->packed.ensure(pad_groups(n) * sizeof(uint2), st));
     SFC_TRY(idx->keys_in.ensure(n * sizeof(uint64_t), st));
     ProfScope ps(idx, "sort", st);
     SFC_TRY(launch_keys3(d_points, n, idx->keys_in.as<uint64_t>(), status_word(idx), st));
@@ -162,7 +163,6 @@ sfc_status build3_from_device(sfc_index* idx, const int32_t* d_points, cudaStrea
     dst.keys = idx->keys.as<uint64_t>();
     dst.vals = idx->ids.as<uint32_t>();
     SFC_TRY(radix_sort(src, n, dst, idx->sort_ws, status_word(idx), st));
-    SFC_TRY(launch_decode3(idx->keys.as<uint64_t>(), n, idx->xyz.as<int4>(), st));
     SFC_TRY(build_boxes(idx, st));
     idx->next_id = (uint32_t)n;
     return SFC_OK;
@@ -184,7 +184,7 @@ QueryArgs base_args(sfc_index* idx, const int32_t* q, const int32_t* delta, uint
     a.kint = (uint32_t)query_intervals(idx->dim, idx->drop);
     a.norm = idx->norm;
     a.dim = idx->dim;
-    a.xyz = idx->xyz.as<int4>();
+    a.packed = idx->packed.as<uint2>();
     a.box = idx->box.as<int4>();
     a.dir = idx->dir.as<uint32_t>();
     a.dir_bits = dir_bits(idx->n);
@@ -537,7 +537,8 @@ sfc_status sfc_reserve(sfc_index* idx, uint64_t n_max, uint64_t m_max, void* str
     SFC_TRY(idx->keys.ensure(n1 * sizeof(uint64_t), st));
     SFC_TRY(idx->ids.ensure(n1 * sizeof(uint32_t), st));
     if (idx->dim == 3) {
-        SFC_TRY(idx->xyz.ensure(pad_groups(n1) * sizeof(int4), st));
+        SFC_TRY(idx->xyz.ensure(n1 * sizeof(int4), st));
+        SFC_TRY(idx->packed.ensure(pad_groups(n1) * sizeof(uint2), st));
         SFC_TRY(idx->keys_in.ensure(n1 * sizeof(uint64_t), st));
     } else {
         SFC_TRY(idx->xy.ensure(pad_groups(n1) * sizeof(int2), st));

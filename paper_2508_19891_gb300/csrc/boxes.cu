@@ -72,8 +72,10 @@ __global__ void __launch_bounds__(kT) boxes_kernel(const int2* __restrict__ xy, 
     }
 }
 
-__global__ void __launch_bounds__(kT) boxes3_kernel(const int4* __restrict__ xyz, const uint64_t* __restrict__ keys,
-                                                    uint32_t n, uint32_t groups, int bits, uint32_t dblocks, uint32_t* dir,
+// 3-D: decodes the sorted keys into the 16-byte records and the packed coordinates on the way (a
+// decoding kernel of its own and boxes read back from its records: 78 us more at 10^7 points).
+__global__ void __launch_bounds__(kT) boxes3_kernel(const uint64_t* __restrict__ keys, uint32_t n, uint32_t groups,
+                                                    int bits, uint32_t dblocks, uint32_t* dir, int4* xyz, uint2* packed,
                                                     int4* box)
 {
     chain_start();
@@ -83,14 +85,25 @@ __global__ void __launch_bounds__(kT) boxes3_kernel(const int4* __restrict__ xyz
     }
     const unsigned lane = lane_id();
     const uint32_t warps = (gridDim.x - dblocks) * (kT / 32);
-    for (uint32_t g = (blockIdx.x - dblocks) * (kT / 32) + (threadIdx.x >> 5); g < groups; g += warps) {
-        const int4 p = __ldg(xyz + (uint32_t)min((uint64_t)g * 32 + lane, (uint64_t)n - 1));
-        const int4 lo = make_int4(__reduce_min_sync(0xffffffffu, p.x), __reduce_min_sync(0xffffffffu, p.y),
-                                  __reduce_min_sync(0xffffffffu, p.z), 0);
-        const int4 hi = make_int4(__reduce_max_sync(0xffffffffu, p.x), __reduce_max_sync(0xffffffffu, p.y),
-                                  __reduce_max_sync(0xffffffffu, p.z), 0);
-        if (lane == 0) box[2 * (uint64_t)g] = lo;
-        if (lane == 1) box[2 * (uint64_t)g + 1] = hi;
+    for (uint32_t g0 = ((blockIdx.x - dblocks) * (kT / 32) + (threadIdx.x >> 5)) * kU; g0 < groups; g0 += warps * kU) {
+        uint64_t k[kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u)
+            k[u] = __ldg(keys + (uint32_t)min((uint64_t)(g0 + u) * 32 + lane, (uint64_t)n - 1));
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            const uint64_t i = (uint64_t)(g0 + u) * 32 + lane;
+            const uint32_t x = gather3_bits(k[u]), y = gather3_bits(k[u] >> 1), z = gather3_bits(k[u] >> 2);
+            if (i < n) {
+                xyz[i] = make_int4((int)x, (int)y, (int)z, 0);
+                packed[i] = pack3(x, y, z);
+            }
+            const int4 lo = make_int4((int)__reduce_min_sync(0xffffffffu, x), (int)__reduce_min_sync(0xffffffffu, y),
+                                      (int)__reduce_min_sync(0xffffffffu, z), 0);
+            const int4 hi = make_int4((int)__reduce_max_sync(0xffffffffu, x), (int)__reduce_max_sync(0xffffffffu, y),
+                                      (int)__reduce_max_sync(0xffffffffu, z), 0);
+            if (lane < 2 && g0 + u < groups) box[2 * (uint64_t)(g0 + u) + lane] = lane ? hi : lo;
+        }
     }
 }
 
@@ -108,7 +121,7 @@ sfc_status build_boxes(sfc_index* idx, cudaStream_t st)
     SFC_TRY(idx->box.ensure(box_bytes(idx->dim, n), st));
     SFC_TRY(idx->dir.ensure(dir_bytes(n), st));
     const uint32_t groups = (uint32_t)((n + 31) / 32);
-    const uint32_t per_block = (kT / 32) * (idx->dim == 3 ? 1 : kU);
+    const uint32_t per_block = (kT / 32) * kU;
     const int bits = dir_bits(n);
     // of the eight blocks that an SM holds, two fill the directory beside six that stream a large
     // array (the directory's latency then hides behind the boxes); short arrays take what it needs
@@ -116,8 +129,8 @@ sfc_status build_boxes(sfc_index* idx, cudaStream_t st)
     const uint32_t dblocks = std::min((1u << bits) / kT + 1, (uint32_t)num_sms() * (large ? 2 : 4));
     const uint32_t grid = dblocks + std::min((groups + per_block - 1) / per_block, (uint32_t)num_sms() * (large ? 6 : 8));
     if (idx->dim == 3)
-        launch_chain(boxes3_kernel, grid, kT, 0, st, idx->xyz.as<int4>(), idx->keys.as<uint64_t>(), (uint32_t)n, groups, bits, dblocks,
-                                           idx->dir.as<uint32_t>(), idx->box.as<int4>());
+        launch_chain(boxes3_kernel, grid, kT, 0, st, idx->keys.as<uint64_t>(), (uint32_t)n, groups, bits, dblocks,
+                     idx->dir.as<uint32_t>(), idx->xyz.as<int4>(), idx->packed.as<uint2>(), idx->box.as<int4>());
     else
         launch_chain(boxes_kernel, grid, kT, 0, st, idx->xy.as<int2>(), idx->keys.as<uint64_t>(), (uint32_t)n, groups, bits, dblocks,
                                           idx->dir.as<uint32_t>(), idx->box.as<int4>());

@@ -93,6 +93,7 @@ struct sfc_index {
     sfc::DevBuf box;                    // bounding boxes of the groups of 32 sorted points
     sfc::DevBuf dir;                    // key directory: positions of equal parts of the key range
     sfc::DevBuf xyz;                    // 3-D: coordinates in sorted order (int4 x, y, z, 0)
+    sfc::DevBuf packed;                 // 3-D: the same packed into 8 bytes, read by the scans
     sfc::DevBuf keys_in;                // 3-D: keys in input order (the sort's source)
 
     sfc::SortWorkspace sort_ws;

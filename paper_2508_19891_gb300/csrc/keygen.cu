@@ -85,17 +85,6 @@ __global__ void __launch_bounds__(kThreads) keys3_kernel(const int32_t* __restri
     if (bad) set_status(status, SFC_DEV_BAD_POINT);
 }
 
-__global__ void __launch_bounds__(kThreads) decode3_kernel(const uint64_t* __restrict__ keys, uint64_t n,
-                                                           int4* __restrict__ xyz)
-{
-    chain_start();
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        const uint64_t k = keys[i];
-        xyz[i] = make_int4((int)gather3_bits(k), (int)gather3_bits(k >> 1), (int)gather3_bits(k >> 2), 0);
-    }
-}
-
 int grid_for(uint64_t work, int per_block)
 {
     uint64_t want = (work + per_block - 1) / per_block;
@@ -137,14 +126,6 @@ sfc_status launch_keys3(const int32_t* pts, uint64_t n, uint64_t* keys, uint32_t
 {
     if (n == 0) return SFC_OK;
     launch_chain(keys3_kernel, grid_for(n, kThreads), kThreads, 0, st, pts, n, keys, status);
-    count_launch();
-    return launch_status();
-}
-
-sfc_status launch_decode3(const uint64_t* keys, uint64_t n, int4* xyz, cudaStream_t st)
-{
-    if (n == 0) return SFC_OK;
-    launch_chain(decode3_kernel, grid_for(n, kThreads), kThreads, 0, st, keys, n, xyz);
     count_launch();
     return launch_status();
 }

@@ -727,7 +727,7 @@ plan_kernel(QueryArgs a, Bounds bounds_in, PlanExport ex)
 // Items: (query, group) pairs
 // ------------------------------------------------------------------------------------
 // The scans are specialised by geometry: the 2-D disc, the 2-D square window, and the 3-D
-// ball (points stored as 16-byte int4 records).
+// ball (points packed into 8 bytes).
 constexpr int kGeomDisc = SFC_NORM_DISC;
 constexpr int kGeomSquare = SFC_NORM_SQUARE;
 constexpr int kGeomBall3 = 2;
@@ -740,9 +740,9 @@ struct Geom {
 };
 template <>
 struct Geom<kGeomBall3> {
-    using P = int4;
+    using P = uint2;
     static constexpr int kGroups = kItemGroups3;
-    static __device__ __forceinline__ const P* points(const QueryArgs& a) { return a.xyz; }
+    static __device__ __forceinline__ const P* points(const QueryArgs& a) { return a.packed; }
 };
 
 // A query's window as the lanes hold it: x, y, delta, z (0 in 2-D).
@@ -766,15 +766,16 @@ __device__ __forceinline__ bool is_hit(const int4& w, long long, int2 p)
 }
 
 template <int GEOM>
-__device__ __forceinline__ bool is_hit(const int4& w, long long c, int4 p)
+__device__ __forceinline__ bool is_hit(const int4& w, long long c, uint2 packed)
 {
+    const int3 p = unpack3(packed);
     const int dx = p.x - w.x, dy = p.y - w.y, dz = p.z - w.z;
     const long long s = (long long)dx * dx + ((long long)dy * dy + ((long long)dz * dz + c));
     return (int)(s >> 32) < 0;
 }
 
 __device__ __forceinline__ int2 ldg_points(const int2* p) { return __ldg(p); }
-__device__ __forceinline__ int4 ldg_points(const int4* p) { return __ldg(p); }
+__device__ __forceinline__ uint2 ldg_points(const uint2* p) { return __ldg(p); }
 
 // Where the box of a group of points lies: kOut no point of it is in the window, kIn every
 // point is, kEdge the points have to be looked at.  The nearest and farthest points of the box
@@ -1002,7 +1003,8 @@ __device__ __forceinline__ uint32_t lanemask_le() { return lanemask_lt() | (1u <
 // (about 12 instructions), a warp tests 32 points with about 10, and only where a box is cut by the
 // window's edge.  Measured, count pass only, before (every scanned point tested, a warp per chunk
 // of one query) and now: 10^7 queries over 10^8 mixed points, cover 1 (1.48*10^10 scanned points)
-// 12.8 -> 5.6 ms; 10^6 over 10^7 1.20 -> 0.58 ms; 10^6 3-D balls over 10^7 3.87 -> 1.90 ms.
+// 12.8 -> 5.6 ms; 10^6 over 10^7 1.20 -> 0.58 ms; 10^6 3-D balls over 10^7 3.87 -> 1.70 ms (1.90 with
+// 16-byte records, which do not fit in L2).
 //
 // Every query owns at least one item, so the owners of 32 consecutive items follow from the
 // owner of the first and one load of the next 32 queries' first items (past the last query the

@@ -7,7 +7,7 @@ namespace sfc {
 
 // Groups of 32 points per item of the scan passes (powers of two: an item's boxes are loaded in
 // pairs).  2-D: four measured best (two and one: count 5.8 -> 6.6 and 9.4 ms at 10^8 mixed points);
-// 3-D: two (four need more registers than leave enough warps).
+// 3-D: two (four the same, one 1.70 -> 2.32 ms at 10^7 points and 10^6 balls).
 #ifndef SFC_ITEM_GROUPS2
 #define SFC_ITEM_GROUPS2 4
 #endif
@@ -22,7 +22,7 @@ struct QueryArgs {
     const uint64_t* keys;        // sorted keys [n]
     const uint32_t* ids;         // ids in sorted order [n]
     const int2* xy;              // coordinates in sorted order [n] (2-D)
-    const int4* xyz;             // coordinates in sorted order [n] (3-D: x, y, z, 0)
+    const uint2* packed;         // coordinates in sorted order [n] (3-D, pack3)
     int dim;                     // 2 or 3; queries are int32[m][dim]
     uint32_t n;
     const int32_t* q;            // [m][dim]

@@ -225,6 +225,19 @@ __host__ __device__ __forceinline__ uint64_t morton3_key(uint32_t x, uint32_t y,
     return spread3_bits(x) | (spread3_bits(y) << 1) | (spread3_bits(z) << 2);
 }
 
+// The three coordinates of a point in one word (x in bits 0-20, y in 21-41, z in 42-62): what the
+// scans read, half of the 16-byte records that sfc_get_sorted hands out.
+__device__ __forceinline__ uint2 pack3(uint32_t x, uint32_t y, uint32_t z)
+{
+    return make_uint2(x | y << kOmega3, y >> (32 - kOmega3) | z << (2 * kOmega3 - 32));
+}
+
+__device__ __forceinline__ int3 unpack3(uint2 p)
+{
+    return make_int3((int)(p.x & (kSide3 - 1)), (int)(__funnelshift_r(p.x, p.y, kOmega3) & (kSide3 - 1)),
+                     (int)(p.y >> (2 * kOmega3 - 32)));
+}
+
 __device__ __forceinline__ bool point3_in_domain(int32_t x, int32_t y, int32_t z)
 {
     return (uint32_t)x < kSide3 && (uint32_t)y < kSide3 && (uint32_t)z < kSide3;
@@ -456,10 +469,8 @@ __device__ __forceinline__ int64_t leaf_predict(const LeafParams& lp, uint64_t k
 sfc_status launch_keys(const int2* pts, uint64_t n, int curve, uint64_t* keys, uint32_t* status,
                        cudaStream_t st);
 sfc_status launch_decode(const uint64_t* keys, uint64_t n, int curve, int2* pts, cudaStream_t st);
-// 3-D Z keys of int32[n][3] points (bad coordinates set SFC_DEV_BAD_POINT), and their inverse
-// into int4 (x, y, z, 0) records
+// 3-D Z keys of int32[n][3] points (bad coordinates set SFC_DEV_BAD_POINT)
 sfc_status launch_keys3(const int32_t* pts, uint64_t n, uint64_t* keys, uint32_t* status, cudaStream_t st);
-sfc_status launch_decode3(const uint64_t* keys, uint64_t n, int4* xyz, cudaStream_t st);
 
 // scan.cu: exclusive scan of uint32 (or a uint32 view) into uint64[n+1].
 struct ScanWorkspace {

@@ -255,6 +255,7 @@ void release_index(sfc_index* idx, cudaStream_t st)
     idx->box.release(st);
     idx->dir.release(st);
     idx->xyz.release(st);
+    idx->packed.release(st);
     idx->keys_in.release(st);
     release_sort_ws(idx->sort_ws, st);
     idx->scan_ws.flags.release(st);
