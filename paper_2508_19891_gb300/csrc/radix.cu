@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(1024) sample_kernel(SortSource src, uint64_t n
 {
     chain_start();
     __shared__ HilbertTables tb;
-    __shared__ unsigned long long s_pairs, s_live;
+    __shared__ uint32_t s_pairs, s_live[2];   // 32-bit words: 64-bit shared atomics retry under contention
     constexpr uint32_t kSlots = 2 * SAMPLE;
     extern __shared__ uint32_t s_slots[];            // kSlots fingerprints, then their 16-bit counts
     uint32_t* s_count = s_slots + kSlots;
@@ -136,14 +136,19 @@ __global__ void __launch_bounds__(1024) sample_kernel(SortSource src, uint64_t n
     const uint64_t first = source_key<CURVE>(src, &tb, 0);
 #pragma unroll
     for (int i = 0; i < K; ++i) live |= key[i] ^ first;
-    if (threadIdx.x == 0) s_live = 0;
+    if (threadIdx.x < 2) s_live[threadIdx.x] = 0;
     __syncthreads();
-    atomicOr(&s_live, (unsigned long long)live);
+    const uint32_t l0 = __reduce_or_sync(0xffffffffu, (uint32_t)live), l1 = __reduce_or_sync(0xffffffffu, (uint32_t)(live >> 32));
+    if (lane_id() == 0) {
+        atomicOr(&s_live[0], l0);
+        atomicOr(&s_live[1], l1);
+    }
     __syncthreads();
-    live = s_live;
+    live = (uint64_t)s_live[1] << 32 | s_live[0];
     const int all = (src.bits + kBits - 1) / kBits;
     const int top = live ? 63 - __clzll((long long)live) : 0;
-    const uint64_t most = (uint64_t)SFC_SORT_MEAN_RUN * SAMPLE * SAMPLE / (2 * n);   // pairs of short runs
+    // pairs of short runs (all pairs there are: SAMPLE^2 / 2 < 2^27)
+    const uint32_t most = (uint32_t)min((uint64_t)SFC_SORT_MEAN_RUN * SAMPLE * SAMPLE / (2 * n), (uint64_t)SAMPLE * SAMPLE);
     int passes = 2;
     for (; passes < all; ++passes) {
         const int low = low_bits(src.bits, passes);
@@ -154,7 +159,7 @@ __global__ void __launch_bounds__(1024) sample_kernel(SortSource src, uint64_t n
         __syncthreads();
 #pragma unroll
         for (int i = 0; i < K; ++i) {
-            if (*(volatile unsigned long long*)&s_pairs > most) break;   // long runs, however many more
+            if (*(volatile uint32_t*)&s_pairs > most) break;   // long runs, however many more
             // 32-bit fingerprint of the top bits (multiplicative hashing), never 0
             const uint64_t h = (key[i] >> low) * 0x9e3779b97f4a7c15ull;
             const uint32_t f = (uint32_t)(h >> 32) | 1u;
@@ -167,7 +172,7 @@ __global__ void __launch_bounds__(1024) sample_kernel(SortSource src, uint64_t n
             }
             const uint32_t sh = 16 * (at & 1);
             const uint32_t earlier = (atomicAdd(&s_count[at >> 1], 1u << sh) >> sh) & 0xffffu;
-            if (earlier) atomicAdd(&s_pairs, (unsigned long long)earlier);
+            if (earlier) atomicAdd(&s_pairs, earlier);
         }
         __syncthreads();
         if (s_pairs <= most) break;
