@@ -114,10 +114,12 @@ sfc_status build_from_device(sfc_index* idx, const int32_t* d_points, cudaStream
     SFC_TRY(idx->keys.ensure(n * sizeof(uint64_t), st));
     SFC_TRY(idx->ids.ensure(n * sizeof(uint32_t), st));
     SFC_TRY(idx->xy.ensure(pad_groups(n) * sizeof(int2), st));
+    SFC_TRY(idx->key_by_id.ensure(n * sizeof(uint64_t), st));
     SortSource src;
     src.points = reinterpret_cast<const int2*>(d_points);
     src.curve = idx->curve;
     src.bits = 2 * kOmega;
+    src.keys_out = idx->key_by_id.as<uint64_t>();   // the sort leaves the id -> key table behind
     SortDest dst;
     dst.keys = idx->keys.as<uint64_t>();
     dst.vals = idx->ids.as<uint32_t>();
@@ -135,10 +137,6 @@ sfc_status build_from_device(sfc_index* idx, const int32_t* d_points, cudaStream
         ProfScope ps(idx, "occupancy", st);
         SFC_TRY(build_occupancy(idx, st));
     }
-    // the id -> coordinates table of the dynamic setting starts as a copy of the input
-    SFC_TRY(idx->xy_by_id.ensure(n * sizeof(int2), st));
-    if (n) SFC_CUDA_TRY(cudaMemcpyAsync(idx->xy_by_id.ptr, d_points, n * sizeof(int2),
-                                        cudaMemcpyDeviceToDevice, st));
     idx->next_id = (uint32_t)n;
     SFC_TRY(ensure_alive_bits(idx, n, st));
     return SFC_OK;
@@ -542,7 +540,7 @@ sfc_status sfc_reserve(sfc_index* idx, uint64_t n_max, uint64_t m_max, void* str
         SFC_TRY(idx->keys_in.ensure(n1 * sizeof(uint64_t), st));
     } else {
         SFC_TRY(idx->xy.ensure(pad_groups(n1) * sizeof(int2), st));
-        SFC_TRY(idx->xy_by_id.ensure(n1 * sizeof(int2), st));
+        SFC_TRY(idx->key_by_id.ensure(n1 * sizeof(uint64_t), st));
         SFC_TRY(ensure_alive_bits(idx, n1, st));
     }
     if (idx->opt.occupancy_depth > 0)

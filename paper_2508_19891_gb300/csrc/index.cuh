@@ -86,7 +86,7 @@ struct sfc_index {
     const sfc_allocator* allocator() const { return has_alloc ? &alloc : nullptr; }
 
     sfc::DevBuf keys, ids, xy;          // the sorted array A_P and its keys
-    sfc::DevBuf xy_by_id;               // coordinates by id (dynamic setting)
+    sfc::DevBuf key_by_id;              // keys by id (dynamic setting), written by the sorts
     sfc::DevBuf alive;                  // liveness bitmap by id
     sfc::DevBuf status;                 // device status word + model statistics
     sfc::DevBuf occ;                    // early-termination bitmap (occupancy_depth > 0)

@@ -816,10 +816,11 @@ sfc_status run_sort(const PassArgs& args, uint32_t* epoch, cudaStream_t st)
     allow_smem((const void*)hist_kernel<CURVE>, (size_t)kPasses * kRadix * kHistRow * sizeof(uint32_t), hist_ok);
     const uint64_t hgrid = std::min<uint64_t>((a.n + kHistThreads * 4 - 1) / (kHistThreads * 4),
                                               std::max<uint64_t>(num_sms(), a.n / kHistMost + 1));
-    launch_chain(hist_kernel<CURVE>, (unsigned)hgrid, kHistThreads, hsmem, st, a.src, a.n, a.tmp_keys[1], a.sm, a.status);
+    uint64_t* keys_out = a.src.keys_out ? a.src.keys_out : a.tmp_keys[1];
+    launch_chain(hist_kernel<CURVE>, (unsigned)hgrid, kHistThreads, hsmem, st, a.src, a.n, keys_out, a.sm, a.status);
     if (a.src.points) {   // the passes read the keys
         a.src.points = nullptr;
-        a.src.keys = a.tmp_keys[1];
+        a.src.keys = keys_out;
     }
     launch_chain(plan_kernel, 1, kRadix, 0, st, a.sm, a.n, a.src.bits, epoch);
     count_launch(2);

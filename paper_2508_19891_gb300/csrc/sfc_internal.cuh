@@ -507,6 +507,7 @@ struct SortSource {
     const uint32_t* vals = nullptr;
     uint32_t val_base = 0;
     int curve = SFC_CURVE_Z;
+    uint64_t* keys_out = nullptr;   // receives the keys of the points, in input order (NULL: scratch)
     int bits = 64;         // the keys are below 2^bits
     bool partial = true;   // may sort the leading digits and then order the runs left over
 };

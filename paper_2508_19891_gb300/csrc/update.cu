@@ -5,7 +5,7 @@
 // rebuild from scratch over the live points would produce, because the order is (key, id)
 // and every inserted id is larger than every existing one:
 //
-//   del_keys_kernel    key of each deleted id from the id -> coordinates table
+//   del_keys_kernel    key of each deleted id from the id -> key table
 //   radix sort         deletes by (key, id)
 //   del_locate_kernel  each delete must be an issued, live id; its array position (lexicographic
 //                      lower_bound of (key, id)) goes into a bitmap, where a repeated id meets its
@@ -18,7 +18,7 @@
 //   move_kernel        surviving entry p to slot p - (deletes before p) + (inserts ranked <= p),
 //                      counted tile by tile in shared memory
 //   ins_place_kernel   insert j to slot r_j - (deletes before r_j) + j
-//   then: liveness bits, the id -> coordinates table, and a refit of a trained model.
+//   then: liveness bits, boxes and directory, and a refit of a trained model.
 #include <algorithm>
 
 #include "sfc_internal.cuh"
@@ -37,21 +37,30 @@ int grid_of(uint64_t n)
     return (int)std::max<uint64_t>(1, std::min(g, cap));
 }
 
-__global__ void del_keys_kernel(const uint32_t* __restrict__ del, uint64_t k, const int2* __restrict__ xy_by_id,
-                                uint32_t next_id, int curve, uint64_t* keys_out)
+__global__ void del_keys_kernel(const uint32_t* __restrict__ del, uint64_t k, const uint64_t* __restrict__ key_by_id,
+                                uint32_t next_id, uint64_t* keys_out)
 {
     chain_start();
-    __shared__ HilbertTables tb;
-    if (curve == SFC_CURVE_HILBERT) hilbert_tables_init(&tb);
     for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < k; t += (uint64_t)gridDim.x * blockDim.x) {
         const uint32_t id = del[t];
-        uint64_t key = 0;
-        if (id < next_id) {
-            const int2 p = xy_by_id[id];
-            key = curve_key(curve, &tb, (uint32_t)p.x & (kSide - 1), (uint32_t)p.y & (kSide - 1));
-        }
-        keys_out[t] = key;
+        keys_out[t] = id < next_id ? key_by_id[id] : 0;
     }
+}
+
+// Part of the sorted array that holds the keys equal to kk, from the key directory (boxes.cu): those
+// before [lo, hi) are smaller, those from hi on larger.
+__device__ __forceinline__ void key_part(const uint64_t* __restrict__ keys, uint32_t n, const uint32_t* __restrict__ dir,
+                                         int bits, uint64_t kk, uint32_t& lo, uint32_t& hi)
+{
+    lo = hi = 0;
+    if (n == 0) return;
+    const uint64_t kmin = __ldg(keys), kmax = __ldg(keys + n - 1);
+    if (kk < kmin) return;
+    lo = hi = n;
+    if (kk > kmax) return;
+    const uint32_t v = (uint32_t)((kk - kmin) >> dir_shift(kmin, kmax, bits));
+    lo = __ldg(dir + v);
+    hi = __ldg(dir + v + 1);
 }
 
 // Old entries per tile of move_kernel: eight per thread.
@@ -63,8 +72,8 @@ constexpr uint32_t kGone = 0xffffffffu;   // no slot is this large (n < 2^32 - 1
 // id), a bit per position and a count per tile.  Ids of equal keys come in input order, so the
 // positions ascend key by key only.
 __global__ void del_locate_kernel(const uint64_t* __restrict__ keys, const uint32_t* __restrict__ ids, uint32_t n,
-                                  const uint64_t* __restrict__ dkeys, const uint32_t* __restrict__ dids, uint64_t k,
-                                  const uint32_t* __restrict__ alive, uint32_t next_id, uint32_t* dpos,
+                                  const uint32_t* __restrict__ dir, int bits, const uint64_t* __restrict__ dkeys,
+                                  const uint32_t* __restrict__ dids, uint64_t k, const uint32_t* __restrict__ alive, uint32_t next_id, uint32_t* dpos,
                                   uint32_t* dbits, uint32_t* dcount, uint32_t* bad)
 {
     chain_start();
@@ -72,7 +81,9 @@ __global__ void del_locate_kernel(const uint64_t* __restrict__ keys, const uint3
         const uint64_t kk = dkeys[t];
         const uint32_t id = dids[t];
         bool ok = id < next_id && ((alive[id >> 5] >> (id & 31)) & 1u);
-        uint32_t lo = 0, len = n;
+        uint32_t lo, hi;
+        key_part(keys, n, dir, bits, kk, lo, hi);
+        uint32_t len = hi - lo;
         while (len > 0) {
             const uint32_t half = len >> 1;
             const uint32_t mid = lo + half;
@@ -91,13 +102,15 @@ __global__ void del_locate_kernel(const uint64_t* __restrict__ keys, const uint3
 
 // Rank of each (sorted) insert among the old entries: all old ids are smaller, so it is the
 // number of old keys <= the insert's key.
-__global__ void ins_rank_kernel(const uint64_t* __restrict__ keys, uint32_t n, const uint64_t* __restrict__ ikeys,
-                                uint64_t k, uint32_t* rank)
+__global__ void ins_rank_kernel(const uint64_t* __restrict__ keys, uint32_t n, const uint32_t* __restrict__ dir, int bits,
+                                const uint64_t* __restrict__ ikeys, uint64_t k, uint32_t* rank)
 {
     chain_start();
     for (uint64_t j = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; j < k; j += (uint64_t)gridDim.x * blockDim.x) {
         const uint64_t kk = ikeys[j];
-        uint32_t lo = 0, len = n;
+        uint32_t lo, hi;
+        key_part(keys, n, dir, bits, kk, lo, hi);
+        uint32_t len = hi - lo;
         while (len > 0) {
             const uint32_t half = len >> 1;
             const bool le = keys[lo + half] <= kk;
@@ -248,7 +261,7 @@ void release_index(sfc_index* idx, cudaStream_t st)
     idx->keys.release(st);
     idx->ids.release(st);
     idx->xy.release(st);
-    idx->xy_by_id.release(st);
+    idx->key_by_id.release(st);
     idx->alive.release(st);
     idx->status.release(st);
     idx->occ.release(st);
@@ -313,7 +326,8 @@ sfc_status apply_update(sfc_index* idx, const int32_t* d_inserts, uint64_t k_ins
         dkeys = dkeys_in + k_del;
         dids = U.c.as<uint32_t>();
         dpos = U.d.as<uint32_t>();
-        launch_chain(del_keys_kernel, grid_of(k_del), kT, 0, st, d_del, k_del, idx->xy_by_id.as<int2>(), next_id, curve, dkeys_in);
+        launch_chain(del_keys_kernel, grid_of(k_del), kT, 0, st, d_del, k_del, idx->key_by_id.as<uint64_t>(), next_id,
+                     dkeys_in);
         count_launch();
         SortSource src;
         src.keys = dkeys_in;
@@ -329,9 +343,9 @@ sfc_status apply_update(sfc_index* idx, const int32_t* d_inserts, uint64_t k_ins
         dbits = U.marks.as<uint32_t>();
         uint32_t* dcount = dbits + (n / 32 + 1);
         SFC_CUDA_TRY(cudaMemsetAsync(dbits, 0, ((size_t)(n / 32 + 1) + tiles) * sizeof(uint32_t), st));
-        launch_chain(del_locate_kernel, grid_of(k_del), kT, 0, st, idx->keys.as<uint64_t>(), idx->ids.as<uint32_t>(), n, dkeys, dids,
-                                                         k_del, idx->alive.as<uint32_t>(), next_id, dpos, dbits, dcount,
-                                                         bad);
+        launch_chain(del_locate_kernel, grid_of(k_del), kT, 0, st, idx->keys.as<uint64_t>(), idx->ids.as<uint32_t>(), n,
+                     idx->dir.as<uint32_t>(), dir_bits(n), dkeys, dids, k_del, idx->alive.as<uint32_t>(), next_id, dpos,
+                     dbits, dcount, bad);
         count_launch();
         SFC_TRY(exclusive_scan_u32(dcount, tiles, U.dstart.as<uint64_t>(), idx->scan_ws, status, st));
         SFC_TRY(launch_status());
@@ -355,6 +369,19 @@ sfc_status apply_update(sfc_index* idx, const int32_t* d_inserts, uint64_t k_ins
         ixy = U.g.as<int2>();
         irank = U.h.as<uint32_t>();
         SortSource src;
+        // the id -> key table takes the inserts' keys from their sort (entries past next_id until the
+        // batch is done mean nothing)
+        const uint64_t ids_after = (uint64_t)next_id + k_ins;
+        if (ids_after * sizeof(uint64_t) > idx->key_by_id.bytes) {
+            DevBuf nb;
+            SFC_TRY(nb.ensure(ids_after * sizeof(uint64_t) + ids_after * sizeof(uint64_t) / 2, st));
+            if (next_id)
+                SFC_CUDA_TRY(cudaMemcpyAsync(nb.ptr, idx->key_by_id.ptr, (size_t)next_id * sizeof(uint64_t),
+                                             cudaMemcpyDeviceToDevice, st));
+            idx->key_by_id.release(st);
+            idx->key_by_id = nb;
+        }
+        src.keys_out = idx->key_by_id.as<uint64_t>() + next_id;
         src.points = reinterpret_cast<const int2*>(d_inserts);
         src.bits = 2 * kOmega;
         src.curve = curve;
@@ -376,7 +403,8 @@ sfc_status apply_update(sfc_index* idx, const int32_t* d_inserts, uint64_t k_ins
     const uint64_t* keys = idx->keys.as<uint64_t>();
     const uint32_t* ids = idx->ids.as<uint32_t>();
     if (k_ins) {
-        launch_chain(ins_rank_kernel, grid_of(k_ins), kT, 0, st, keys, n, ikeys, k_ins, irank);
+        launch_chain(ins_rank_kernel, grid_of(k_ins), kT, 0, st, keys, n, idx->dir.as<uint32_t>(), dir_bits(n), ikeys, k_ins,
+                     irank);
         launch_chain(tile_starts_kernel, grid_of(k_ins + 1), kT, 0, st, irank, k_ins, tiles, istart);
         count_launch(2);
     }
@@ -393,27 +421,13 @@ sfc_status apply_update(sfc_index* idx, const int32_t* d_inserts, uint64_t k_ins
         launch_chain(ins_place_kernel, grid_of(k_ins), kT, 0, st, ikeys, iids, ixy, k_ins, irank, dpos, k_del, nkeys, nids, nxy);
         count_launch();
     }
-    // ---- liveness and the id -> coordinates table ----
+    // ---- liveness ----
     if (k_del) {
         launch_chain(alive_clear_kernel, grid_of(k_del), kT, 0, st, d_del, k_del, idx->alive.as<uint32_t>());
         count_launch();
     }
     SFC_TRY(launch_status());
-    if (k_ins) {
-        const uint64_t ids_after = (uint64_t)next_id + k_ins;
-        if (ids_after * sizeof(int2) > idx->xy_by_id.bytes) {
-            DevBuf nb;
-            SFC_TRY(nb.ensure(ids_after * sizeof(int2) + ids_after * sizeof(int2) / 2, st));
-            if (next_id)
-                SFC_CUDA_TRY(cudaMemcpyAsync(nb.ptr, idx->xy_by_id.ptr, (size_t)next_id * sizeof(int2),
-                                             cudaMemcpyDeviceToDevice, st));
-            idx->xy_by_id.release(st);
-            idx->xy_by_id = nb;
-        }
-        SFC_CUDA_TRY(cudaMemcpyAsync(idx->xy_by_id.as<int2>() + next_id, d_inserts, k_ins * sizeof(int2),
-                                     cudaMemcpyDeviceToDevice, st));
-        SFC_TRY(ensure_alive_bits(idx, ids_after, st));
-    }
+    if (k_ins) SFC_TRY(ensure_alive_bits(idx, (uint64_t)next_id + k_ins, st));
     // ---- swap in the new arrays ----
     std::swap(idx->keys, U.keys);
     std::swap(idx->ids, U.ids);
