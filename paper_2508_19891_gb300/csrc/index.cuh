@@ -60,7 +60,7 @@ struct Profiler {
 };
 
 struct UpdateWs {
-    DevBuf a, b, c, d, e, f, g, h;   // flags, delete keys/ids/positions, insert keys/ids/xy/ranks
+    DevBuf a, e, f, g, h;            // flags, insert keys/ids/xy/ranks
     DevBuf keys, ids, xy;            // the next sorted arrays (swapped with the index's)
     DevBuf marks, dstart, istart;    // deleted bits and counts per tile; deletes, inserts before each tile
 };

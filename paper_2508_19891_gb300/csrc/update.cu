@@ -5,11 +5,10 @@
 // rebuild from scratch over the live points would produce, because the order is (key, id)
 // and every inserted id is larger than every existing one:
 //
-//   del_keys_kernel    key of each deleted id from the id -> key table
-//   radix sort         deletes by (key, id)
 //   del_locate_kernel  each delete must be an issued, live id; its array position (lexicographic
-//                      lower_bound of (key, id)) goes into a bitmap, where a repeated id meets its
-//                      own bit, and into the deletes' count per tile
+//                      lower_bound of (key, id), the key from the id -> key table) goes into a
+//                      bitmap, where a repeated id meets its own bit, and into the deletes' count
+//                      per tile
 //   (host)             one synchronisation: a bad batch is rejected before anything changes
 //   scan               deletes before each tile
 //   radix sort         inserts by key with ids next_id + i (keys computed from the points)
@@ -17,7 +16,7 @@
 //   tile_starts_kernel inserts ranked before each tile
 //   move_kernel        surviving entry p to slot p - (deletes before p) + (inserts ranked <= p),
 //                      counted tile by tile in shared memory
-//   ins_place_kernel   insert j to slot r_j - (deletes before r_j) + j
+//   ins_place_kernel   insert j to slot r_j - (deletes before r_j, from the bitmap) + j
 //   then: liveness bits, boxes and directory, and a refit of a trained model.
 #include <algorithm>
 
@@ -35,16 +34,6 @@ int grid_of(uint64_t n)
     uint64_t g = (n + kT - 1) / kT;
     const uint64_t cap = (uint64_t)num_sms() * 16;
     return (int)std::max<uint64_t>(1, std::min(g, cap));
-}
-
-__global__ void del_keys_kernel(const uint32_t* __restrict__ del, uint64_t k, const uint64_t* __restrict__ key_by_id,
-                                uint32_t next_id, uint64_t* keys_out)
-{
-    chain_start();
-    for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < k; t += (uint64_t)gridDim.x * blockDim.x) {
-        const uint32_t id = del[t];
-        keys_out[t] = id < next_id ? key_by_id[id] : 0;
-    }
 }
 
 // Part of the sorted array that holds the keys equal to kk, from the key directory (boxes.cu): those
@@ -68,19 +57,23 @@ constexpr int kMoveItems = 8;
 constexpr int kMoveTile = kT * kMoveItems;
 constexpr uint32_t kGone = 0xffffffffu;   // no slot is this large (n < 2^32 - 1)
 
-// Checks and locates the (sorted) deletes: position of (key, id) in the array sorted by (key,
-// id), a bit per position and a count per tile.  Ids of equal keys come in input order, so the
-// positions ascend key by key only.
+// Checks and locates the deletes: position of (key, id) in the array sorted by (key, id), a bit per
+// position and a count per tile.  In the order they are given: sorting them first, for searches over
+// neighbouring lines and ascending positions, took longer than it saved (5*10^5 deletes at 5*10^7
+// points: the update 636 us sorted, 592 not).
 __global__ void del_locate_kernel(const uint64_t* __restrict__ keys, const uint32_t* __restrict__ ids, uint32_t n,
-                                  const uint32_t* __restrict__ dir, int bits, const uint64_t* __restrict__ dkeys,
-                                  const uint32_t* __restrict__ dids, uint64_t k, const uint32_t* __restrict__ alive, uint32_t next_id, uint32_t* dpos,
-                                  uint32_t* dbits, uint32_t* dcount, uint32_t* bad)
+                                  const uint32_t* __restrict__ dir, int bits, const uint32_t* __restrict__ del, uint64_t k,
+                                  const uint64_t* __restrict__ key_by_id, const uint32_t* __restrict__ alive,
+                                  uint32_t next_id, uint32_t* dbits, uint32_t* dcount, uint32_t* bad)
 {
     chain_start();
     for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < k; t += (uint64_t)gridDim.x * blockDim.x) {
-        const uint64_t kk = dkeys[t];
-        const uint32_t id = dids[t];
-        bool ok = id < next_id && ((alive[id >> 5] >> (id & 31)) & 1u);
+        const uint32_t id = del[t];
+        if (id >= next_id || !((alive[id >> 5] >> (id & 31)) & 1u)) {
+            atomicOr(bad, 1u);
+            continue;
+        }
+        const uint64_t kk = __ldg(key_by_id + id);
         uint32_t lo, hi;
         key_part(keys, n, dir, bits, kk, lo, hi);
         uint32_t len = hi - lo;
@@ -92,8 +85,7 @@ __global__ void del_locate_kernel(const uint64_t* __restrict__ keys, const uint3
             lo = less ? mid + 1 : lo;
             len = less ? len - half - 1 : half;
         }
-        dpos[t] = lo;
-        ok = ok && lo < n && keys[lo] == kk && ids[lo] == id;
+        bool ok = lo < n && keys[lo] == kk && ids[lo] == id;
         if (ok) ok = !((atomicOr(dbits + (lo >> 5), 1u << (lo & 31)) >> (lo & 31)) & 1u);   // a repeated id
         if (ok) atomicAdd(dcount + lo / kMoveTile, 1u);
         else atomicOr(bad, 1u);
@@ -137,7 +129,7 @@ __global__ void tile_starts_kernel(const uint32_t* __restrict__ pos, uint64_t k,
 // Moves a tile of old entries to their new slots.  Bound by HBM: it reads and writes each entry's
 // 20 bytes once and nothing else per entry (a full-length deletion mask, shift counts and their
 // scan took another 26 bytes per entry: 5*10^5 inserts and deletes at 5*10^7 points 1086 us
-// before, 719 us now).  The entries are loaded before the tile's counts are scanned, so the loads
+// before, 719 us after).  The entries are loaded before the tile's counts are scanned, so the loads
 // overlap the shared-memory work.
 __global__ void __launch_bounds__(kT) move_kernel(const uint64_t* __restrict__ keys, const uint32_t* __restrict__ ids,
                                                   const int2* __restrict__ xy, uint32_t n,
@@ -167,7 +159,7 @@ __global__ void __launch_bounds__(kT) move_kernel(const uint64_t* __restrict__ k
     const uint32_t i0 = rank ? istart[blockIdx.x] : 0, i1 = rank ? istart[blockIdx.x + 1] : 0;
     __syncthreads();
     for (uint32_t j = i0 + tid; j < i1; j += kT)
-        if (rank[j] < n) atomicAdd(&s_ins[rank[j] - p0], 1u);
+        atomicAdd(&s_ins[rank[j] - p0], 1u);
     __syncthreads();
     // this thread's stretch of eight entries, the eight bits of its deletions
     const uint32_t at = p0 + tid * kMoveItems;
@@ -208,21 +200,26 @@ __global__ void __launch_bounds__(kT) move_kernel(const uint64_t* __restrict__ k
 
 __global__ void ins_place_kernel(const uint64_t* __restrict__ ikeys, const uint32_t* __restrict__ iids,
                                  const int2* __restrict__ ixy, uint64_t k, const uint32_t* __restrict__ rank,
-                                 const uint32_t* __restrict__ dpos, uint64_t kdel, uint64_t* nkeys, uint32_t* nids,
-                                 int2* nxy)
+                                 const uint32_t* __restrict__ dbits, const uint64_t* __restrict__ dstart, uint64_t* nkeys,
+                                 uint32_t* nids, int2* nxy)
 {
     chain_start();
     for (uint64_t j = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; j < k; j += (uint64_t)gridDim.x * blockDim.x) {
         const uint32_t r = rank[j];
-        // deletes at positions < r (dpos is ascending)
-        uint64_t lo = 0, len = kdel;
-        while (len > 0) {
-            const uint64_t half = len >> 1;
-            const bool lt = dpos[lo + half] < r;
-            lo = lt ? lo + half + 1 : lo;
-            len = lt ? len - half - 1 : half;
+        // deletes at positions < r: those before r's tile, then the tile's bits up to r
+        uint32_t before = 0;
+        if (dbits) {
+            const uint32_t tile = r / kMoveTile;
+            before = (uint32_t)dstart[tile];
+            uint32_t w = tile * (kMoveTile / 32);
+            for (; w + 4 <= r >> 5; w += 4) {
+                const uint4 x = __ldg(reinterpret_cast<const uint4*>(dbits + w));
+                before += __popc(x.x) + __popc(x.y) + __popc(x.z) + __popc(x.w);
+            }
+            for (; w < r >> 5; ++w) before += __popc(dbits[w]);
+            before += __popc(dbits[w] & ((1u << (r & 31)) - 1u));
         }
-        const uint64_t dst = (uint64_t)r - lo + j;
+        const uint64_t dst = (uint64_t)r - before + j;
         nkeys[dst] = ikeys[j];
         nids[dst] = iids[j];
         nxy[dst] = ixy[j];
@@ -293,7 +290,7 @@ void release_index(sfc_index* idx, cudaStream_t st)
     M.tmp.release(st); M.leaves.release(st); M.fence.release(st);
     M.fence_fine.release(st);
     UpdateWs& u = idx->uws;
-    u.a.release(st); u.b.release(st); u.c.release(st); u.d.release(st);
+    u.a.release(st);
     u.e.release(st); u.f.release(st); u.g.release(st); u.h.release(st);
     u.keys.release(st); u.ids.release(st); u.xy.release(st);
     u.marks.release(st); u.dstart.release(st); u.istart.release(st);
@@ -308,44 +305,23 @@ sfc_status apply_update(sfc_index* idx, const int32_t* d_inserts, uint64_t k_ins
     const int curve = idx->curve;
     if ((uint64_t)next_id + k_ins >= 0xffffffffull || (uint64_t)n + k_ins >= 0xffffffffull) return SFC_ERR_INVALID;
     uint32_t* status = idx->status.as<uint32_t>();
-    // scratch: a = flags, b = delete keys in / sorted, c = delete ids sorted, d = delete positions
+    // scratch: a = flags, e .. h = the sorted inserts and their ranks
     SFC_TRY(U.a.ensure(16, st));
     uint32_t* bad = U.a.as<uint32_t>();
     SFC_CUDA_TRY(cudaMemsetAsync(bad, 0, 16, st));
-    uint64_t* dkeys_in = nullptr;
-    uint64_t* dkeys = nullptr;
-    uint32_t* dids = nullptr;
-    uint32_t* dpos = nullptr;
     uint32_t* dbits = nullptr;
-    const uint32_t tiles = (uint32_t)(((uint64_t)n + kMoveTile - 1) / kMoveTile);
+    // tiles of old entries; the last one may be empty, it takes the inserts ranked after all of them
+    const uint32_t tiles = n / kMoveTile + 1;
     if (k_del) {
-        SFC_TRY(U.b.ensure(k_del * 16, st));
-        SFC_TRY(U.c.ensure(k_del * 4, st));
-        SFC_TRY(U.d.ensure(k_del * 4, st));
-        dkeys_in = U.b.as<uint64_t>();
-        dkeys = dkeys_in + k_del;
-        dids = U.c.as<uint32_t>();
-        dpos = U.d.as<uint32_t>();
-        launch_chain(del_keys_kernel, grid_of(k_del), kT, 0, st, d_del, k_del, idx->key_by_id.as<uint64_t>(), next_id,
-                     dkeys_in);
-        count_launch();
-        SortSource src;
-        src.keys = dkeys_in;
-        src.bits = 2 * kOmega;
-        src.vals = d_del;
-        SortDest dst;
-        dst.keys = dkeys;
-        dst.vals = dids;
-        dst.curve = curve;
-        SFC_TRY(radix_sort(src, k_del, dst, idx->sort_ws, status, st));
-        SFC_TRY(U.marks.ensure(((size_t)(n / 32 + 1) + tiles) * sizeof(uint32_t), st));
+        const size_t words = (size_t)tiles * (kMoveTile / 32);
+        SFC_TRY(U.marks.ensure((words + tiles) * sizeof(uint32_t), st));
         SFC_TRY(U.dstart.ensure(((size_t)tiles + 1) * sizeof(uint64_t), st));
         dbits = U.marks.as<uint32_t>();
-        uint32_t* dcount = dbits + (n / 32 + 1);
-        SFC_CUDA_TRY(cudaMemsetAsync(dbits, 0, ((size_t)(n / 32 + 1) + tiles) * sizeof(uint32_t), st));
+        uint32_t* dcount = dbits + words;
+        SFC_CUDA_TRY(cudaMemsetAsync(dbits, 0, (words + tiles) * sizeof(uint32_t), st));
         launch_chain(del_locate_kernel, grid_of(k_del), kT, 0, st, idx->keys.as<uint64_t>(), idx->ids.as<uint32_t>(), n,
-                     idx->dir.as<uint32_t>(), dir_bits(n), dkeys, dids, k_del, idx->alive.as<uint32_t>(), next_id, dpos,
-                     dbits, dcount, bad);
+                     idx->dir.as<uint32_t>(), dir_bits(n), d_del, k_del, idx->key_by_id.as<uint64_t>(),
+                     idx->alive.as<uint32_t>(), next_id, dbits, dcount, bad);
         count_launch();
         SFC_TRY(exclusive_scan_u32(dcount, tiles, U.dstart.as<uint64_t>(), idx->scan_ws, status, st));
         SFC_TRY(launch_status());
@@ -418,7 +394,8 @@ sfc_status apply_update(sfc_index* idx, const int32_t* d_inserts, uint64_t k_ins
         count_launch();
     }
     if (k_ins) {
-        launch_chain(ins_place_kernel, grid_of(k_ins), kT, 0, st, ikeys, iids, ixy, k_ins, irank, dpos, k_del, nkeys, nids, nxy);
+        launch_chain(ins_place_kernel, grid_of(k_ins), kT, 0, st, ikeys, iids, ixy, k_ins, irank, dbits,
+                     U.dstart.as<uint64_t>(), nkeys, nids, nxy);
         count_launch();
     }
     // ---- liveness ----
