@@ -70,8 +70,12 @@ constexpr uint32_t kPlanCap = SFC_PLAN_CAP;
 #define SFC_COUNT_BLOCKS 6
 #endif
 #ifndef SFC_WRITE_BLOCKS
-#define SFC_WRITE_BLOCKS 8
+#define SFC_WRITE_BLOCKS 7
 #endif
+// Records whose ids a warp of the write pass has in flight.  Measured with the blocks that the
+// registers leave, 10^6 queries over 10^7 mixed points (10^7 over 10^8): two on 8 blocks 597 us (5.77 ms),
+// four on 8 588 (5.81), six on 7 553 (5.62), eight on 7 576 (5.77), on 6 632 (5.97).
+constexpr uint32_t kCopyUnroll = 6;
 
 // ------------------------------------------------------------------------------------
 // Bound search: lower_bounds in lock step (independent loads in flight together)
@@ -1102,11 +1106,11 @@ __global__ void __launch_bounds__(kThreads, SFC_COUNT_BLOCKS) count_kernel(Query
 // Per-warp shared memory of a copy: up to 32 records (hit word, first position, output
 // pointer).  A slot past the last has an empty word.
 struct CopySmem {
-    ulonglong2 it[32 + 4];
+    ulonglong2 it[32 + kCopyUnroll];
 };
 
 // Writes the ids of every lane's record (hit word, first position p0) to out_ids[dst ...), the
-// hits in order; with !fits, ids whose slot is past the capacity are dropped.  Four records at a
+// hits in order; with !fits, ids whose slot is past the capacity are dropped.  Six records at a
 // time: the id loads of their 32 positions are in flight together.  Lanes [0, cnt) have records.
 // Every lane calls.
 __device__ __forceinline__ void copy_records(const QueryArgs& a, bool fits, uint32_t cnt, uint32_t word, uint32_t p0,
@@ -1114,7 +1118,7 @@ __device__ __forceinline__ void copy_records(const QueryArgs& a, bool fits, uint
 {
     const unsigned lane = lane_id();
     const uint32_t lt = lanemask_lt(), bit = 1u << lane;
-    constexpr uint32_t U = 4;
+    constexpr uint32_t U = kCopyUnroll;
     __syncwarp();   // the previous records have been read
     if (lane < cnt)
         sm->it[lane] = make_ulonglong2((unsigned long long)p0 << 32 | word,
@@ -1150,9 +1154,9 @@ __device__ __forceinline__ void copy_records(const QueryArgs& a, bool fits, uint
 
 // The records of the items of the queries of processing ranks [q_begin, q_end).  Bound by HBM and
 // the L2 (ids are read where the sorted array lies and written once): 4.23*10^9 ids of 10^7 queries
-// over 10^8 mixed points in 5.8 ms, 5.8 TB/s of id reads and writes (11.4 ms with one warp per query,
+// over 10^8 mixed points in 5.6 ms, 6.0 TB/s of id reads and writes (11.4 ms with one warp per query,
 // whose dependent loads and per-hit shared-memory store set the time); 129 windows of 2*10^5 ids
-// 48.8 ms -> 0.08 ms, as no warp owns a query.
+// 48.8 ms -> 0.07 ms, as no warp owns a query.
 __global__ void __launch_bounds__(kThreads, SFC_WRITE_BLOCKS) write_kernel(QueryArgs a)
 {
     chain_start();
