@@ -781,34 +781,31 @@ __device__ __forceinline__ bool is_hit(const int4& w, long long c, uint2 packed)
 __device__ __forceinline__ int2 ldg_points(const int2* p) { return __ldg(p); }
 __device__ __forceinline__ uint2 ldg_points(const uint2* p) { return __ldg(p); }
 
-// Where the box of a group of points lies: kOut no point of it is in the window, kIn every
-// point is, kEdge the points have to be looked at.  The nearest and farthest points of the box
-// are tested with the window's own arithmetic (the same bounds on every term).
-constexpr int kOut = 0, kEdge = 1, kIn = 2;
+// Where the box of a group of points lies: out, no point of it is in the window; in, every point is;
+// neither, the points have to be looked at.  The nearest and farthest points of the box are
+// tested with the window's own arithmetic (the same bounds on every term).
+struct BoxSide {
+    bool out, in;
+};
 
-__device__ __forceinline__ int class_of(long long near2, long long far2, long long d2)
-{
-    return near2 > d2 ? kOut : (far2 <= d2 ? kIn : kEdge);
-}
-
-// 2-D box (x0, y0, x1, y1).
+// 2-D box (x0, y0, x1, y1); d2 = delta^2.
 template <int GEOM>
-__device__ __forceinline__ int box_class(const Window& w, const int4& b)
+__device__ __forceinline__ BoxSide box_side(const Window& w, long long d2, const int4& b)
 {
     const int nx = max(max(b.x - w.x, w.x - b.z), 0), fx = max(w.x - b.x, b.z - w.x);
     const int ny = max(max(b.y - w.y, w.y - b.w), 0), fy = max(w.y - b.y, b.w - w.y);
-    if (GEOM == kGeomSquare) return max(nx, ny) > w.z ? kOut : (max(fx, fy) <= w.z ? kIn : kEdge);
-    return class_of((long long)nx * nx + (long long)ny * ny, (long long)fx * fx + (long long)fy * fy, (long long)w.z * w.z);
+    if (GEOM == kGeomSquare) return {max(nx, ny) > w.z, max(fx, fy) <= w.z};
+    return {(long long)nx * nx + (long long)ny * ny > d2, (long long)fx * fx + (long long)fy * fy <= d2};
 }
 
 // 3-D box.
-__device__ __forceinline__ int box3_class(const Window& w, const int4& lo, const int4& hi)
+__device__ __forceinline__ BoxSide box3_side(const Window& w, long long d2, const int4& lo, const int4& hi)
 {
     const int nx = max(max(lo.x - w.x, w.x - hi.x), 0), fx = max(w.x - lo.x, hi.x - w.x);
     const int ny = max(max(lo.y - w.y, w.y - hi.y), 0), fy = max(w.y - lo.y, hi.y - w.y);
     const int nz = max(max(lo.z - w.w, w.w - hi.z), 0), fz = max(w.w - lo.z, hi.z - w.w);
-    return class_of((long long)nx * nx + (long long)ny * ny + (long long)nz * nz,
-                    (long long)fx * fx + (long long)fy * fy + (long long)fz * fz, (long long)w.z * w.z);
+    return {(long long)nx * nx + (long long)ny * ny + (long long)nz * nz > d2,
+            (long long)fx * fx + (long long)fy * fy + (long long)fz * fz <= d2};
 }
 
 // Two neighbouring 16-byte records, 32-byte aligned, in one load: a lane's boxes lie side by side,
@@ -818,30 +815,6 @@ __device__ __forceinline__ void ldg_pair(const int4* p, int4& a, int4& b)
     asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
         : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
         : "l"(p));
-}
-
-// The classes of an item's groups (first group g, a multiple of the groups per item), two bits
-// each.
-template <int GEOM>
-__device__ __forceinline__ uint32_t item_classes(const QueryArgs& a, const Window& w, uint32_t g)
-{
-    uint32_t c = 0;
-    if (GEOM == kGeomBall3) {
-#pragma unroll
-        for (int u = 0; u < Geom<GEOM>::kGroups; ++u) {
-            int4 lo, hi;
-            ldg_pair(a.box + 2 * (uint64_t)(g + u), lo, hi);
-            c |= (uint32_t)box3_class(w, lo, hi) << (2 * u);
-        }
-    } else {
-#pragma unroll
-        for (int u = 0; u < Geom<GEOM>::kGroups; u += 2) {
-            int4 b0, b1;
-            ldg_pair(a.box + (g + u), b0, b1);
-            c |= (uint32_t)box_class<GEOM>(w, b0) << (2 * u) | (uint32_t)box_class<GEOM>(w, b1) << (2 * u + 2);
-        }
-    }
-    return c;
 }
 
 // The t-th item of a query whose ranges start at rp: the range [b, e) it belongs to (0, 0 for the
@@ -864,12 +837,11 @@ __device__ __forceinline__ uint2 locate_item(const uint2* __restrict__ rp, uint3
     return make_uint2(0u, 0u);
 }
 
-// Which of the 32 positions from p on lie in [r.x, r.y).
-__device__ __forceinline__ uint32_t group_mask(uint2 r, uint32_t p)
+// Which of an item's positions 32 u .. 32 u + 31 lie in [lo, hi) (0 <= lo, hi <= the item's length).
+__device__ __forceinline__ uint32_t group_mask(int lo, int hi, int u)
 {
-    const uint32_t lo = r.x > p ? r.x - p : 0u;
-    if (p >= r.y || lo >= 32) return 0u;
-    return (0xffffffffu >> (32u - min(r.y - p, 32u))) & (0xffffffffu << lo);
+    // ones from bit max(lo - 32 u, 0) on, none past 31 (the shift clamps at 32)
+    return __funnelshift_lc(0u, 0xffffffffu, max(lo - 32 * u, 0)) & ~__funnelshift_lc(0u, 0xffffffffu, max(hi - 32 * u, 0));
 }
 
 // Per-warp shared memory of the filter: the groups whose points have to be looked at, side by
@@ -903,6 +875,9 @@ __device__ __forceinline__ void filter_init(FilterSmem<GEOM>* sm)
 // Groups that need their points looked at are gathered in shared memory and taken four at a
 // time, so that four coalesced loads are in flight.  The points' array is padded to whole
 // groups.  Every lane of the warp calls.
+// Bound by instruction issue: a group's side, mask and shared-memory slot are made in one step (all
+// classes first, then masks, then slots: count pass of 10^6 queries over 10^7 mixed points 586 us
+// against 564, square windows over Normal points 120 against 110), with masks of two clamped shifts.
 template <int GEOM>
 __device__ __forceinline__ void filter_items(const QueryArgs& a, const Window& w, uint2 r, uint32_t p0,
                                              uint32_t (&word)[Geom<GEOM>::kGroups], FilterSmem<GEOM>* sm)
@@ -912,35 +887,39 @@ __device__ __forceinline__ void filter_items(const QueryArgs& a, const Window& w
     const unsigned lane = lane_id();
     const P* __restrict__ pts = Geom<GEOM>::points(a) + lane;
     uint32_t cnt = 0, slots = 0;   // byte u: 0x80 | slot of group u when its points are looked at
-    const uint32_t classes = r.y > r.x ? item_classes<GEOM>(a, w, p0 >> 5) : 0u;
-#pragma unroll
-    for (int u = 0; u < kGroups; ++u) {
-        word[u] = group_mask(r, p0 + 32 * u);
-        const uint32_t cls = word[u] ? (classes >> (2 * u)) & 3u : kOut;
-        const uint32_t edge = __ballot_sync(0xffffffffu, cls == kEdge);
-        if (cls == kEdge) slots |= (0x80u | (cnt + __popc(edge & lanemask_lt()))) << (8 * u);
-        cnt += __popc(edge);
-        if (cls == kOut) word[u] = 0;
-    }
-    if (cnt == 0) return;
+    const bool item = r.y > r.x;
+    const int lo = r.x > p0 ? (int)(r.x - p0) : 0, hi = item ? (int)min(r.y - p0, 32u * kGroups) : 0;
+    const long long d2 = (long long)w.z * w.z, c = ~d2;   // -(delta^2 + 1)
     __syncwarp();   // the previous groups have been read
-    if (slots) {
-        const long long c = -((long long)w.z * w.z + 1);
 #pragma unroll
-        for (int u = 0; u < kGroups; ++u) {
-            if (!((slots >> (8 * u)) & 0x80u)) continue;
-            const uint32_t s = (slots >> (8 * u)) & 0x7fu, p = p0 + 32 * u;
-            if (GEOM == kGeomDisc) {
-                sm->w[s] = make_int4(w.x, w.y, (int)c, (int)(c >> 32));
-                sm->p[s] = p;
-            } else if (GEOM == kGeomSquare) {
-                sm->w[s] = make_int4(w.x, w.y, w.z, (int)p);
-            } else {
-                sm->w[s] = make_int4(w.x, w.y, w.w, (int)p);
-                sm->c[s] = (unsigned long long)c;
+    for (int v = 0; v < kGroups; v += GEOM == kGeomBall3 ? 1 : 2) {
+        int4 b[2] = {make_int4(0, 0, 0, 0), make_int4(0, 0, 0, 0)};   // two boxes, or the two corners of one
+        if (item) ldg_pair(a.box + (GEOM == kGeomBall3 ? 2 : 1) * (uint64_t)((p0 >> 5) + v), b[0], b[1]);
+#pragma unroll
+        for (int u = v; u < v + (GEOM == kGeomBall3 ? 1 : 2); ++u) {
+            BoxSide side;
+            if constexpr (GEOM == kGeomBall3) side = box3_side(w, d2, b[0], b[1]);
+            else side = box_side<GEOM>(w, d2, b[u - v]);
+            word[u] = side.out ? 0u : group_mask(lo, hi, u);
+            const bool look = word[u] != 0 && !side.in;
+            const uint32_t edge = __ballot_sync(0xffffffffu, look);
+            if (look) {
+                const uint32_t s = cnt + __popc(edge & lanemask_lt()), p = p0 + 32 * u;
+                slots |= (0x80u | s) << (8 * u);
+                if (GEOM == kGeomDisc) {
+                    sm->w[s] = make_int4(w.x, w.y, (int)c, (int)(c >> 32));
+                    sm->p[s] = p;
+                } else if (GEOM == kGeomSquare) {
+                    sm->w[s] = make_int4(w.x, w.y, w.z, (int)p);
+                } else {
+                    sm->w[s] = make_int4(w.x, w.y, w.w, (int)p);
+                    sm->c[s] = (unsigned long long)c;
+                }
             }
+            cnt += __popc(edge);
         }
     }
+    if (cnt == 0) return;
     __syncwarp();
     constexpr uint32_t U = 4;
 #pragma unroll 1
@@ -1007,8 +986,9 @@ __device__ __forceinline__ uint32_t lanemask_le() { return lanemask_lt() | (1u <
 // (about 12 instructions), a warp tests 32 points with about 10, and only where a box is cut by the
 // window's edge.  Measured, count pass only, before (every scanned point tested, a warp per chunk
 // of one query) and now: 10^7 queries over 10^8 mixed points, cover 1 (1.48*10^10 scanned points)
-// 12.8 -> 5.6 ms; 10^6 over 10^7 1.20 -> 0.58 ms; 10^6 3-D balls over 10^7 3.87 -> 1.70 ms (1.90 with
-// 16-byte records, which do not fit in L2).
+// 12.8 -> 5.4 ms; 10^6 over 10^7 1.20 -> 0.56 ms; 10^6 3-D balls over 10^7 3.87 -> 1.66 ms.  Blocks per
+// SM, 10^6 over 10^7 mixed points / Normal points and square windows / 3-D: five 592 / 114 / 1637 us,
+// six 564 / 110 / 1657, seven 637 / 146 / 1601 (spills).
 //
 // Every query owns at least one item, so the owners of 32 consecutive items follow from the
 // owner of the first and one load of the next 32 queries' first items (past the last query the
