@@ -7,7 +7,7 @@
 //
 // One pass over the coordinates, bound by HBM: a warp takes four groups at a time, one coalesced
 // load each, and reduces them with the warp's min / max instructions (10^8 points: 0.15 ms, 5.7
-// TB/s, against 3.4 ms that the boxes save in each batch of 10^7 queries).
+// TB/s, 0.18 ms with the directory below, against the 7 ms that the count pass of 10^7 queries saves).
 //
 // The same launch fills the key directory that the bound searches of the plan start from: a thread
 // finds each entry by binary search (neighbouring threads walk nearly the same path, so 2^18
