@@ -1132,9 +1132,10 @@ __device__ __forceinline__ void copy_records(const QueryArgs& a, bool fits, uint
     }
 }
 
-// The records of the items of the queries of processing ranks [q_begin, q_end).  Bound by HBM and
-// the L2 (ids are read where the sorted array lies and written once): 4.23*10^9 ids of 10^7 queries
-// over 10^8 mixed points in 5.6 ms, 6.0 TB/s of id reads and writes (11.4 ms with one warp per query,
+// The records of the items of the queries of processing ranks [q_begin, q_end).  Bound by the
+// latency of record, id and store and by the L2 (most ids are read from it, all are written once to HBM,
+// 3.6 TB/s): 4.25*10^9 ids of 10^7 queries over 10^8 mixed points in 5.6 ms, 6.1 TB/s of id reads and
+// writes, 1.0 warp instructions per id (11.4 ms and 2.2 with one warp per query,
 // whose dependent loads and per-hit shared-memory store set the time); 129 windows of 2*10^5 ids
 // 48.8 ms -> 0.07 ms, as no warp owns a query.
 __global__ void __launch_bounds__(kThreads, SFC_WRITE_BLOCKS) write_kernel(QueryArgs a)
