@@ -36,6 +36,7 @@
 #include <algorithm>
 
 #include "sfc_internal.cuh"
+#include "sizes.cuh"
 
 namespace sfc {
 
@@ -399,7 +400,7 @@ __global__ void __launch_bounds__(kThreads, SFC_SORT_BLOCKS) onesweep_kernel(Pas
     constexpr int kTile = kThreads * ITEMS, kWarpSpan = 32 * ITEMS;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t n = (uint32_t)a.n;
-    const uint32_t tiles = (uint32_t)((a.n + kTile - 1) / kTile);
+    const uint32_t tiles = tiles_of(a.n, kTile);
     const int shift = (int)pl.shift;
     if (CURVE == SFC_CURVE_HILBERT && pl.dst == 3 && a.dst.xy) hilbert_tables_init(&S.tb);
     uint32_t *wh = S.hist[warp], *wm = S.match[warp];
@@ -580,7 +581,7 @@ __global__ void __launch_bounds__(kFixThreads, SFC_FIX_BLOCKS) fix_kernel(PassAr
     const uint32_t n = (uint32_t)a.n;
     const uint64_t* keys = a.tmp_keys[a.sm->from - 1];
     const uint32_t* vals = a.tmp_vals[a.sm->from - 1];
-    const uint32_t tiles = (n + kFixTile - 1) / kFixTile;
+    const uint32_t tiles = tiles_of(a.n, kFixTile);
     const uint64_t mask = (1ull << low) - 1;   // low <= 48: at least two digits are sorted
     const int tid = threadIdx.x;
     // place in the span of this thread's halo key
@@ -697,17 +698,17 @@ __global__ void __launch_bounds__(kThreads) long_kernel(PassArgs a)
         __syncthreads();
         if (S.tile >= runs) return;
         const uint2 run = a.runs[S.tile];
-        const uint32_t first = run.x, len = run.y;
+        const uint64_t first = run.x, len = run.y;
         int cur = (int)a.sm->from - 1;
         bool ordered = true;
-        for (uint32_t j = tid; j + 1 < len; j += kThreads)
+        for (uint64_t j = tid; j + 1 < len; j += kThreads)
             ordered &= a.tmp_keys[cur][first + j] <= a.tmp_keys[cur][first + j + 1];
         if (!__syncthreads_and(ordered)) {
             for (int shift = 0; shift < low; shift += kBits) {
                 // digit counts of the run, then each digit's next position in it
                 if (tid < kRadix) S.gbase[tid] = 0;
                 __syncthreads();
-                for (uint32_t j = tid; j < len; j += kThreads)
+                for (uint64_t j = tid; j < len; j += kThreads)
                     atomicAdd(&S.gbase[(uint32_t)(a.tmp_keys[cur][first + j] >> shift) & (kRadix - 1)], 1u);
                 __syncthreads();
                 uint32_t v = 0, c = 0;
@@ -725,18 +726,20 @@ __global__ void __launch_bounds__(kThreads) long_kernel(PassArgs a)
                     for (int w = 0; w < warp; ++w) v += S.w[w];
                     S.gbase[tid] = v - c;
                 }
-                for (uint32_t t0 = 0; t0 < len; t0 += kTile) {
-                    const uint32_t wbase = t0 + (uint32_t)(warp * kWarpSpan);
+                for (uint64_t t0 = 0; t0 < len; t0 += kTile) {
+                    // places in the tile, which holds `left` keys
+                    const uint32_t wbase = (uint32_t)(warp * kWarpSpan);
+                    const uint32_t left = (uint32_t)min(len - t0, (uint64_t)kTile);
                     uint64_t key[kItems];
                     uint32_t rank[kItems / 2];
 #pragma unroll
                     for (int i = 0; i < kItems; ++i) {
                         const uint32_t j = wbase + (uint32_t)(i * 32) + lane;
-                        key[i] = j < len ? a.tmp_keys[cur][first + j] : ~0ull;
+                        key[i] = j < left ? a.tmp_keys[cur][first + t0 + j] : ~0ull;
                     }
                     for (int d = lane; d < kRadix; d += 32) wh[d] = 0;
                     __syncwarp();
-                    rank_keys<false>(key, shift, wbase, len, wh, wm, rank);
+                    rank_keys<false>(key, shift, wbase, left, wh, wm, rank);
                     __syncthreads();
                     if (tid < kRadix) {
                         uint32_t next = S.gbase[tid];
@@ -751,19 +754,19 @@ __global__ void __launch_bounds__(kThreads) long_kernel(PassArgs a)
 #pragma unroll
                     for (int i = 0; i < kItems; ++i) {
                         const uint32_t j = wbase + (uint32_t)(i * 32) + lane;
-                        if (j >= len) continue;
-                        const uint32_t at = first + wh[(uint32_t)(key[i] >> shift) & (kRadix - 1)] +
+                        if (j >= left) continue;
+                        const uint64_t at = first + wh[(uint32_t)(key[i] >> shift) & (kRadix - 1)] +
                                             ((rank[i / 2] >> (16 * (i & 1))) & 0xffffu);
                         a.tmp_keys[cur ^ 1][at] = key[i];
-                        a.tmp_vals[cur ^ 1][at] = a.tmp_vals[cur][first + j];
+                        a.tmp_vals[cur ^ 1][at] = a.tmp_vals[cur][first + t0 + j];
                     }
                     __syncthreads();
                 }
                 cur ^= 1;
             }
         }
-        for (uint32_t j = tid; j < len; j += kThreads)
-            store_final<CURVE>(a.dst, &S.tb, first + j, a.tmp_keys[cur][first + j], a.tmp_vals[cur][first + j]);
+        for (uint64_t j = tid; j < len; j += kThreads)
+            store_final<CURVE>(a.dst, &S.tb, (uint32_t)(first + j), a.tmp_keys[cur][first + j], a.tmp_vals[cur][first + j]);
     }
 }
 
@@ -791,7 +794,7 @@ void launch_pass(const PassArgs& a, cudaStream_t st)
 {
     static bool ok[64] = {false};
     allow_smem((const void*)onesweep_kernel<CURVE, ITEMS>, sizeof(PassSmem<ITEMS>), ok);
-    const uint64_t tiles = (a.n + kThreads * ITEMS - 1) / (kThreads * ITEMS);
+    const uint32_t tiles = tiles_of(a.n, kThreads * ITEMS);
     const unsigned grid = (unsigned)std::min<uint64_t>(tiles, (uint64_t)num_sms() * SFC_SORT_BLOCKS);
     launch_chain(onesweep_kernel<CURVE, ITEMS>, grid, kThreads, sizeof(PassSmem<ITEMS>), st, a);
     count_launch();
@@ -831,7 +834,7 @@ sfc_status run_sort(const PassArgs& args, uint32_t* epoch, cudaStream_t st)
     }
     if (sample) {
         static bool ok[64] = {false};
-        const uint64_t ftiles = (a.n + kFixTile - 1) / kFixTile;
+        const uint32_t ftiles = tiles_of(a.n, kFixTile);
         launch_chain(fix_kernel<CURVE>, (unsigned)std::min<uint64_t>(ftiles, (uint64_t)num_sms() * 8), kFixThreads, 0, st, a);
         allow_smem((const void*)long_kernel<CURVE>, sizeof(PassSmem<kItems>), ok);
         const unsigned lgrid = (unsigned)std::min<uint64_t>(a.n / kMaxRun + 1, (uint64_t)num_sms());
