@@ -5,8 +5,9 @@
 // passes over the top bits of the keys, as many as leave only short runs of equal top bits, and
 // a last local step puts each run in order.
 //
-//   1. sample_kernel   4096 keys; for each number of passes, how many sampled pairs agree in the
-//                      bits those passes sort estimates the mean length of the runs left over.
+//   1. sample_kernel   2,048 keys (16,384 of 2^22 or more) at hashed positions; for each number of
+//                      passes, how many sampled pairs agree in the bits those passes sort
+//                      estimates the mean length of the runs left over.
 //                      The fewest passes with short runs are chosen (all of them if none is).
 //   2. hist_kernel     one read of the input: the keys of the points are computed and written
 //                      out, and the 256-bin histograms of all digits are accumulated at once.
@@ -117,8 +118,8 @@ __device__ __forceinline__ uint64_t source_key(const SortSource& s, const Hilber
     return __ldg(s.keys + i);
 }
 
-// Chooses the number of passes (one block).  Of S sampled keys, C pairs agree in their top bits: a
-// key shares its run with about n * 2 C / S^2 others.
+// Chooses the number of passes (one block).  Of S sampled keys, C pairs agree in their top bits: the
+// run of a key is about n * 2 C / S^2 keys long, itself counted (a position may be drawn twice).
 template <int CURVE, int SAMPLE>
 __global__ void __launch_bounds__(1024) sample_kernel(SortSource src, uint64_t n, Small* sm)
 {
@@ -132,7 +133,7 @@ __global__ void __launch_bounds__(1024) sample_kernel(SortSource src, uint64_t n
     constexpr int K = SAMPLE / 1024;
     uint64_t key[K], live = 0;
 #pragma unroll
-    for (int i = 0; i < K; ++i) key[i] = source_key<CURVE>(src, &tb, n * (uint64_t)(i * 1024 + threadIdx.x) / SAMPLE);
+    for (int i = 0; i < K; ++i) key[i] = source_key<CURVE>(src, &tb, sample_position(i * 1024 + threadIdx.x, n));
     // bits in which the sampled keys differ: passes above them leave one run
     const uint64_t first = source_key<CURVE>(src, &tb, 0);
 #pragma unroll

@@ -81,3 +81,21 @@ def test_build_with_stacks_and_a_tight_cluster(cuda, curve):
     assert np.array_equal(u64(k), ref.keys) and np.array_equal(u32(i), ref.ids)
     assert np.array_equal(xy.cpu().numpy(), ref.xy)
     assert sfc.sfc_device_status(idx) == (0, 0)
+
+
+@pytest.mark.parametrize("order", ["sorted", "reversed", "every second", "every 256th"])
+@pytest.mark.parametrize("n", [1 << 20, 1 << 23])
+def test_order_of_the_input(cuda, order, n):
+    """Keys of which half lie in dense clusters, in orders that follow the curve or interleave the
+    two kinds with a period that divides the array."""
+    rng = np.random.default_rng(n)
+    keys = rng.integers(0, 1 << 60, n, dtype=np.uint64)
+    top = rng.integers(0, 1 << 60, 40, dtype=np.uint64) >> np.uint64(34) << np.uint64(34)
+    dense = np.ones(n, bool) if "every" in order else rng.random(n) < 0.5
+    if "every" in order:
+        dense[:: 2 if order == "every second" else 256] = False
+    keys[dense] = top[rng.integers(0, 40, int(dense.sum()))] | rng.integers(0, 1 << 34, int(dense.sum()), dtype=np.uint64)
+    if order in ("sorted", "reversed"):
+        keys.sort()
+        keys = keys[::-1].copy() if order == "reversed" else keys
+    _check(keys, cuda)

@@ -15,6 +15,10 @@ SOURCE = """
 using namespace sfc;
 extern "C" {
 uint32_t c_tiles_of(uint64_t n, uint32_t per) { return tiles_of(n, per); }
+void c_sample_positions(uint32_t samples, uint64_t n, uint64_t* out)
+{
+    for (uint32_t i = 0; i < samples; ++i) out[i] = sample_position(i, n);
+}
 }
 """
 
@@ -45,3 +49,49 @@ def test_no_tile_count_of_the_sort_is_in_32_bits():
     src = open(os.path.join(CSRC, "radix.cu")).read()
     counts = [line for line in src.splitlines() if "tiles =" in line and "small_tiles" not in line]
     assert counts and all("tiles_of(" in line or "uint64_t tiles" in line for line in counts), counts
+
+
+MEAN_RUN = 16   # the mean run that fewer passes may leave
+
+
+def _sample(rules, samples, n):
+    out = np.empty(samples, np.uint64)
+    rules.c_sample_positions(ctypes.c_uint32(samples), ctypes.c_uint64(n), out.ctypes.data_as(ctypes.c_void_p))
+    return out
+
+
+def _pairs(keys):
+    c = np.unique(keys, return_counts=True)[1].astype(np.int64)
+    return int((c * (c - 1) // 2).sum())
+
+
+@pytest.mark.parametrize("order", ["shuffled", "sorted", "reversed", "every second"])
+@pytest.mark.parametrize("n,samples", [(1 << 20, 2048), (1 << 23, 16384)])
+def test_sample_sees_the_runs_whatever_the_order(rules, order, n, samples):
+    """Half of the keys spread out, half in dense clusters: the passes that the sample chooses leave
+    runs of at most twice the intended mean length (the estimate's spread) for every input order."""
+    rng = np.random.default_rng(n)
+    keys = rng.integers(0, 1 << 60, n, dtype=np.uint64)
+    dense = rng.integers(0, 1 << 60, 40, dtype=np.uint64)[rng.integers(0, 40, n // 2)] >> np.uint64(34) << np.uint64(34)
+    keys[n // 2:] = dense | rng.integers(0, 1 << 34, n // 2, dtype=np.uint64)
+    if order == "shuffled":
+        keys = keys[rng.permutation(n)]
+    elif order == "every second":
+        keys = np.stack([keys[: n // 2], keys[n // 2:]], 1).reshape(-1)
+    else:
+        keys.sort()
+        keys = keys[::-1] if order == "reversed" else keys
+    at = _sample(rules, samples, n)
+    assert int(at.max()) < n
+    most = MEAN_RUN * samples * samples // (2 * n)
+    for passes in range(2, 8):
+        low = np.uint64(60 - 8 * passes)
+        if _pairs(keys[at] >> low) <= most:
+            break
+    run = np.unique(keys >> low, return_counts=True)[1].astype(np.float64)
+    assert (run * run).sum() / n <= 2 * MEAN_RUN, (passes, (run * run).sum() / n, run.max())
+
+
+def test_sample_positions_stay_inside(rules):
+    for n in (1, 2, 8192, 10 ** 8, (1 << 32) - 2):
+        assert int(_sample(rules, 16384, n).max()) < n
