@@ -200,6 +200,13 @@ QueryArgs base_args(sfc_index* idx, const int32_t* q, const int32_t* delta, uint
 // records.  Items past either are filtered again by the write pass.
 constexpr uint64_t kBatchBytes = sizeof(uint4) + sizeof(uint32_t) + sizeof(uint64_t);
 
+// Batches that every per-batch buffer has room for.
+uint64_t batch_capacity(const QueryWs& w)
+{
+    return std::min<uint64_t>({w.heads.bytes / sizeof(uint4), w.bhits.bytes / sizeof(uint32_t),
+                              std::max<uint64_t>(w.bbase.bytes / sizeof(uint64_t), 1) - 1});
+}
+
 sfc_status ensure_query_ws(sfc_index* idx, uint64_t m, uint64_t n, cudaStream_t st)
 {
     QueryWs& w = idx->qws;
@@ -227,9 +234,9 @@ sfc_status ensure_query_ws(sfc_index* idx, uint64_t m, uint64_t n, cudaStream_t 
     SFC_TRY(w.bhits.ensure(batches * sizeof(uint32_t), st));
     SFC_TRY(w.bbase.ensure((batches + 1) * sizeof(uint64_t), st));
     SFC_TRY(w.recs.ensure(recs * sizeof(uint2), st));
-    // look-back words of the batch's three scans
-    SFC_TRY(w.flags.ensure((2 * scan_flag_words(m) + scan_flag_words(batches + batches / 8 + 64)) * sizeof(uint64_t), st));
-    return SFC_OK;
+    // look-back words of the batch's three scans: of the batches that there is room for, which an
+    // earlier call over more points may have left larger than this one asks for
+    return w.flags.ensure((2 * scan_flag_words(m) + scan_flag_words(batch_capacity(w))) * sizeof(uint64_t), st);
 }
 
 const LearnedModelView* model_view(sfc_index* idx, LearnedModelView& v)
@@ -265,8 +272,7 @@ void set_workspace(sfc_index* idx, QueryArgs& a)
     a.heads = w.heads.as<uint4>();
     a.bhits = w.bhits.as<uint32_t>();
     a.bbase = w.bbase.as<uint64_t>();
-    a.cap_batches = std::min<uint64_t>({w.heads.bytes / sizeof(uint4), w.bhits.bytes / sizeof(uint32_t),
-                              w.bbase.bytes / sizeof(uint64_t) - 1});
+    a.cap_batches = batch_capacity(w);
     a.recs = w.recs.as<uint2>();
     a.cap_recs = std::min<uint64_t>(w.recs.bytes / sizeof(uint2), 0xffffffffull);
     // records a warp reserves at a time (a batch has up to 32 item_groups): large while an eighth
@@ -298,7 +304,6 @@ sfc_status do_count(sfc_index* idx, const int32_t* d_q, const int32_t* d_delta, 
     a.scanned = scan_stats(idx);
     // look-back words of the scans of the item counts, the batches' hits and the queries' hits
     const uint64_t nb = std::min<uint64_t>(a.cap_batches, max_batches(idx->dim, m, idx->n, a.kint));
-    SFC_TRY(w.flags.ensure((2 * scan_flag_words(m) + scan_flag_words(nb)) * sizeof(uint64_t), st));
     uint64_t* flags_items = w.flags.as<uint64_t>();
     uint64_t* flags_counts = flags_items + scan_flag_words(m);
     uint64_t* flags_hits = flags_counts + scan_flag_words(m);

@@ -120,3 +120,34 @@ def test_allocator_out_of_memory_is_reported(cuda):
     assert e.value.status == sfc.SFC_ERR_OOM
     torch.cuda.synchronize()
     assert not A.live and A.frees == A.allocs
+
+
+def test_capture_after_a_batch_over_more_points_allocates_nothing(cuda):
+    """An earlier batch over many points leaves room for more item batches than a smaller rebuild
+    with more queries asks for: sfc_reserve sizes the rest of the workspace for that room, so the
+    captured calls run no allocator callback, and replays are right."""
+    gen = torch.Generator(device=cuda)
+    gen.manual_seed(4)
+    big = torch.randint(0, 1 << 30, (80_000_000, 2), generator=gen, device=cuda, dtype=torch.int32)
+    n, m = 1_000_000, 290_000
+    pts, q = big[:n].clone(), big[-m:].clone()
+    d = torch.full((m,), 1 << 20, dtype=torch.int32, device=cuda)
+    A = sfc.TorchAllocator(cuda)
+    idx = sfc.sfc_build(big, "z", allocator=A)
+    sfc.query(idx, q[:1000].contiguous(), d[:1000].contiguous())
+    ref = sfc.sfc_build(pts, "z")
+    want_off, want_ids = sfc.query(ref, q, d)
+    off, ids = torch.zeros_like(want_off), torch.zeros_like(want_ids)
+    sfc.sfc_reserve(idx, n, m)
+    allocs, frees = A.allocs, A.frees
+    g = sfc.sfc_graph_capture(idx, pts, q, d, off, ids)
+    assert (A.allocs, A.frees) == (allocs, frees)
+    for _ in range(2):
+        off.zero_()
+        ids.zero_()
+        g.launch()
+        torch.cuda.synchronize()
+        assert torch.equal(off, want_off) and torch.equal(ids, want_ids)
+    assert (A.allocs, A.frees) == (allocs, frees) and sfc.sfc_device_status(idx) == (0, 0)
+    g.close()
+    idx.close()
