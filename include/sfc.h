@@ -252,7 +252,8 @@ sfc_status sfc_query_batch_host(sfc_index* idx, const int32_t* h_q, const int32_
                                 uint64_t ids_capacity, void* stream);
 
 /* Pre-sizes the query workspace for batches of up to m queries, so that later query calls
- * allocate nothing (needed before capturing them in a CUDA graph). */
+ * allocate nothing (needed before capturing them in a CUDA graph).  Where a later sfc_rebuild or
+ * sfc_update grows the index's arrays, that call grows the workspace for the same m as well. */
 sfc_status sfc_reserve_queries(sfc_index* idx, uint64_t m, void* stream);
 
 /* Autotuner: when the index was built with cover_refine = -1, first times whole batches

@@ -139,6 +139,7 @@ sfc_status build_from_device(sfc_index* idx, const int32_t* d_points, cudaStream
     }
     idx->next_id = (uint32_t)n;
     SFC_TRY(ensure_alive_bits(idx, n, st));
+    follow_arrays(idx, st);
     return SFC_OK;
 }
 
@@ -163,6 +164,7 @@ sfc_status build3_from_device(sfc_index* idx, const int32_t* d_points, cudaStrea
     SFC_TRY(radix_sort(src, n, dst, idx->sort_ws, status_word(idx), st));
     SFC_TRY(build_boxes(idx, st));
     idx->next_id = (uint32_t)n;
+    follow_arrays(idx, st);
     return SFC_OK;
 }
 
@@ -207,7 +209,35 @@ uint64_t batch_capacity(const QueryWs& w)
                               std::max<uint64_t>(w.bbase.bytes / sizeof(uint64_t), 1) - 1});
 }
 
-sfc_status ensure_query_ws(sfc_index* idx, uint64_t m, uint64_t n, cudaStream_t st)
+bool capturing(cudaStream_t st)
+{
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) == cudaSuccess) return cs != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return true;
+}
+
+// Sizes the buffers of hits for batches of m queries over as many points as the index's arrays
+// hold (not as it has: a batch over more points within the same arrays, or a replayed graph of one,
+// finds the buffers that it found before).  A capture that was sized for its m uses what is there
+// (any size is right, what does not fit is filtered again) and allocates nothing.
+sfc_status ensure_hits(sfc_index* idx, uint64_t m, cudaStream_t st)
+{
+    QueryWs& w = idx->qws;
+    const uint64_t n = idx->keys.bytes / sizeof(uint64_t), kint = (uint64_t)query_intervals(idx->dim, idx->drop);
+    const uint64_t budget = (uint64_t)idx->opt.mask_budget_mb << 20;
+    const uint64_t bytes = std::min<uint64_t>(budget, m * 1024ull + (1ull << 20) + 4 * n);
+    const uint64_t batches = std::min<uint64_t>(bytes / 4 / kBatchBytes, max_batches(idx->dim, m, n, kint));
+    const uint64_t recs = std::min<uint64_t>(bytes / 4 * 3 / sizeof(uint2), 64 * item_groups(idx->dim) * max_batches(idx->dim, m, n, kint) + (1ull << 23));
+    if (batch_capacity(w) >= batches && w.recs.bytes >= recs * sizeof(uint2)) return SFC_OK;
+    if (m <= w.sized_m && w.recs.bytes && capturing(st)) return SFC_OK;
+    SFC_TRY(w.heads.ensure(batches * sizeof(uint4), st));
+    SFC_TRY(w.bhits.ensure(batches * sizeof(uint32_t), st));
+    SFC_TRY(w.bbase.ensure((batches + 1) * sizeof(uint64_t), st));
+    return w.recs.ensure(recs * sizeof(uint2), st);
+}
+
+sfc_status ensure_query_ws(sfc_index* idx, uint64_t m, cudaStream_t st)
 {
     QueryWs& w = idx->qws;
     const uint64_t kint = (uint64_t)query_intervals(idx->dim, idx->drop);
@@ -226,14 +256,8 @@ sfc_status ensure_query_ws(sfc_index* idx, uint64_t m, uint64_t n, cudaStream_t 
         SFC_TRY(w.dbase.ensure(m * sizeof(uint64_t), st));
         SFC_TRY(reserve_sort(idx->sort_ws, std::max<uint64_t>(m, 1), st));
     }
-    const uint64_t budget = (uint64_t)idx->opt.mask_budget_mb << 20;
-    const uint64_t bytes = std::min<uint64_t>(budget, m * 1024ull + (1ull << 20) + 4 * n);
-    const uint64_t batches = std::min<uint64_t>(bytes / 4 / kBatchBytes, max_batches(idx->dim, m, n, kint));
-    const uint64_t recs = std::min<uint64_t>(bytes / 4 * 3 / sizeof(uint2), 64 * item_groups(idx->dim) * max_batches(idx->dim, m, n, kint) + (1ull << 23));
-    SFC_TRY(w.heads.ensure(batches * sizeof(uint4), st));
-    SFC_TRY(w.bhits.ensure(batches * sizeof(uint32_t), st));
-    SFC_TRY(w.bbase.ensure((batches + 1) * sizeof(uint64_t), st));
-    SFC_TRY(w.recs.ensure(recs * sizeof(uint2), st));
+    SFC_TRY(ensure_hits(idx, m, st));
+    w.sized_m = std::max(w.sized_m, m);
     // look-back words of the batch's three scans: of the batches that there is room for, which an
     // earlier call over more points may have left larger than this one asks for
     return w.flags.ensure((2 * scan_flag_words(m) + scan_flag_words(batch_capacity(w))) * sizeof(uint64_t), st);
@@ -249,6 +273,15 @@ const LearnedModelView* model_view(sfc_index* idx, LearnedModelView& v)
     v.stats = model_stats(idx);
     return &v;
 }
+
+}  // namespace
+
+void sfc::follow_arrays(sfc_index* idx, cudaStream_t st)
+{
+    if (idx->qws.sized_m) ensure_hits(idx, idx->qws.sized_m, st);   // a later batch asks again if this fails
+}
+
+namespace {
 
 // Curve-order processing pays off once the coordinates no longer fit in L2 (n >= 2^24, i.e.
 // 128 MB of coordinates); option 1 forces it, 0 disables it.
@@ -295,7 +328,7 @@ sfc_status do_count(sfc_index* idx, const int32_t* d_q, const int32_t* d_delta, 
         idx->qws.pending = {true, d_q, d_delta, 0, d_out_offsets, false, idx->drop, idx->norm};
         return SFC_OK;
     }
-    SFC_TRY(ensure_query_ws(idx, m, idx->n, st));
+    SFC_TRY(ensure_query_ws(idx, m, st));
     QueryWs& w = idx->qws;
     QueryArgs a = base_args(idx, d_q, d_delta, m);
     set_workspace(idx, a);
@@ -553,7 +586,7 @@ sfc_status sfc_reserve(sfc_index* idx, uint64_t n_max, uint64_t m_max, void* str
     SFC_TRY(reserve_sort(idx->sort_ws, n1, st));
     SFC_TRY(idx->box.ensure(box_bytes(idx->dim, n1), st));
     SFC_TRY(idx->dir.ensure(dir_bytes(n1), st));
-    SFC_TRY(ensure_query_ws(idx, m_max, n1, st));
+    SFC_TRY(ensure_query_ws(idx, m_max, st));
     SFC_TRY(reserve_scan(idx->scan_ws, std::max<uint64_t>(m_max, n1) + 1, st));
     if (idx->opt.bounds == SFC_BOUNDS_LEARNED) SFC_TRY(reserve_model(idx, n1, st));
     return SFC_OK;
@@ -932,7 +965,7 @@ sfc_status sfc_reserve_queries(sfc_index* idx, uint64_t m, void* stream)
     if (!idx) return SFC_ERR_INVALID;
     AllocScope alloc_scope(idx->allocator());
     SFC_TRY(ensure_status_buf(idx, as_stream(stream)));
-    return ensure_query_ws(idx, m, idx->n, as_stream(stream));
+    return ensure_query_ws(idx, m, as_stream(stream));
 }
 
 sfc_status sfc_set_bounds_mode(sfc_index* idx, sfc_bounds mode)

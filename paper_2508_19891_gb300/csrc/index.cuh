@@ -24,6 +24,7 @@ struct QueryWs {
     DevBuf recs;                     // the records of the items with hits
     DevBuf flags;                    // look-back words of a batch's scans
     DevBuf qkeys, qkeys_sorted, perm, pstart, dbase;         // curve-order processing
+    uint64_t sized_m = 0;            // queries that the workspace has been sized for
     bool write_ctr_zero = false;     // the write pass's work counter has not been used since the count
     PendingCount pending{false, nullptr, nullptr, 0, nullptr, false, 0, 0};
 };
@@ -116,6 +117,9 @@ sfc_status refit_model(sfc_index* idx, int steps, cudaStream_t st);
 sfc_status apply_update(sfc_index* idx, const int32_t* d_inserts, uint64_t k_ins, const uint32_t* d_del,
                         uint64_t k_del, uint32_t* h_first, cudaStream_t st);
 const RootParams* model_root_device(sfc_index* idx);
+// after the arrays may have grown: the buffers of hits grow with them, so that the batches that the
+// workspace was sized for still allocate nothing (api.cu)
+void follow_arrays(sfc_index* idx, cudaStream_t st);
 // early-termination bitmap of the sorted keys (no-op when opt.occupancy_depth == 0)
 sfc_status build_occupancy(sfc_index* idx, cudaStream_t st);
 uint64_t occupancy_words(int depth);

@@ -415,6 +415,7 @@ sfc_status apply_update(sfc_index* idx, const int32_t* d_inserts, uint64_t k_ins
     idx->qws.pending.valid = false;
     SFC_TRY(build_occupancy(idx, st));
     SFC_TRY(build_boxes(idx, st));
+    follow_arrays(idx, st);
     if (idx->model.trained) {
         const int steps = std::max(20, idx->opt.train_steps / 5);
         SFC_TRY(refit_model(idx, steps, st));

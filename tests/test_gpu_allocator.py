@@ -151,3 +151,55 @@ def test_capture_after_a_batch_over_more_points_allocates_nothing(cuda):
     assert (A.allocs, A.frees) == (allocs, frees) and sfc.sfc_device_status(idx) == (0, 0)
     g.close()
     idx.close()
+
+
+def test_reserved_batches_allocate_nothing_after_the_points_grow(cuda):
+    """sfc_reserve_queries(m) holds after updates that grow the arrays and after a rebuild within
+    them: batches of m queries run no allocator callback, eagerly and under a capture of the
+    caller's own, and a capture made before such a rebuild stays valid."""
+    rng = np.random.default_rng(6)
+    pts = rng.integers(0, 1 << 16, size=(30_000, 2)).astype(np.int32)
+    m = 500
+    q, d = pts[:m].copy(), np.full(m, 900, np.int32)
+    dq, dd = to_dev(q, cuda), to_dev(d, cuda)
+    A = sfc.TorchAllocator(cuda)
+    idx = sfc.sfc_build(to_dev(pts, cuda), "z", allocator=A)
+    sfc.sfc_reserve_queries(idx, m)
+    off = torch.zeros(m + 1, dtype=torch.int64, device=cuda)
+    ids = torch.zeros(4_000_000, dtype=torch.int32, device=cuda)
+
+    def check(points):
+        roff, rids = oracle.query(oracle.build(points), q, d)
+        assert np.array_equal(u64(off), roff) and np.array_equal(u32(ids[: len(rids)]), rids)
+
+    for grown in (30_000, 200_000):
+        ins = rng.integers(0, 1 << 16, size=(grown, 2)).astype(np.int32)
+        sfc.sfc_update(idx, to_dev(ins, cuda), None)
+        pts = np.concatenate([pts, ins])
+        before = (A.allocs, A.frees)
+        sfc.sfc_query_batch(idx, dq, dd, off, ids)
+        check(pts)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            sfc.sfc_query_batch(idx, dq, dd, off, ids)
+        assert (A.allocs, A.frees) == before
+        off.zero_()
+        ids.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        check(pts)
+    sfc.sfc_rebuild(idx, to_dev(pts, cuda))              # the sort's own buffers
+    before = (A.allocs, A.frees)
+    sfc.sfc_rebuild(idx, to_dev(pts[:1000], cuda))
+    sfc.sfc_query_batch(idx, dq, dd, off, ids)
+    check(pts[:1000])
+    sfc.sfc_rebuild(idx, to_dev(pts, cuda))
+    sfc.sfc_query_batch(idx, dq, dd, off, ids)
+    assert (A.allocs, A.frees) == before
+    off.zero_()
+    ids.zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    check(pts)
+    assert sfc.sfc_device_status(idx) == (0, 0)
+    idx.close()
