@@ -99,8 +99,9 @@ typedef struct {
     float learning_rate;    /* learned model: Adam step size (default 0.02) */
     int chunk;              /* scan chunk in points (0 = autotuned/default 1024) */
     int mask_budget_mb;     /* cap on the buffer that carries the hits from the count pass to the
-                               write pass, sized 1 KB per query and 4 bytes per point; queries
-                               whose hits do not fit are filtered again (default cap 4096 MB) */
+                               write pass, sized 1 KB per query and 4 bytes per point (1 KB per
+                               query where the allocator has no room for that); queries whose
+                               hits do not fit are filtered again (default cap 4096 MB) */
     int reorder_queries;    /* order in which queries are processed (outputs are unaffected):
                                0 input order, 1 curve order of the centres (queries that scan
                                overlapping ranges run together and share L2), 2 curve order once

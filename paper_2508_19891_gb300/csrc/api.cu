@@ -11,6 +11,7 @@
 #include "sfc_internal.cuh"
 #include "query.cuh"
 #include "index.cuh"
+#include "sizes.cuh"
 
 namespace sfc {
 
@@ -196,11 +197,9 @@ QueryArgs base_args(sfc_index* idx, const int32_t* q, const int32_t* delta, uint
     return a;
 }
 
-// Bytes for the hits of a batch of m queries over n points: 1 KB per query (about 100 records and
-// 9 batches of 32 items), and 4 bytes per point so that a few queries over large parts of the
-// array fit too; capped by mask_budget_mb.  A quarter goes to the batches, the rest to the
-// records.  Items past either are filtered again by the write pass.
-constexpr uint64_t kBatchBytes = sizeof(uint4) + sizeof(uint32_t) + sizeof(uint64_t);
+static_assert(kHitBatchBytes == sizeof(uint4) + sizeof(uint32_t) + sizeof(uint64_t) && kHitRecordBytes == sizeof(uint2), "");
+
+uint64_t resident_warps() { return (uint64_t)num_sms() * 64; }
 
 // Batches that every per-batch buffer has room for.
 uint64_t batch_capacity(const QueryWs& w)
@@ -219,22 +218,31 @@ bool capturing(cudaStream_t st)
 
 // Sizes the buffers of hits for batches of m queries over as many points as the index's arrays
 // hold (not as it has: a batch over more points within the same arrays, or a replayed graph of one,
-// finds the buffers that it found before).  A capture that was sized for its m uses what is there
-// (any size is right, what does not fit is filtered again) and allocates nothing.
+// finds the buffers that it found before): 1 KB per query (about 100 records and 9 batches of 32
+// items), and 4 bytes per point so that a few queries over large parts of the array fit too, capped by
+// mask_budget_mb.  Any size is right, as what does not fit is filtered again by the write pass: a
+// capture that was sized for its m uses what is there and allocates nothing, and an allocator that has
+// no room for the 4 bytes per point is asked for the 1 KB per query alone.
 sfc_status ensure_hits(sfc_index* idx, uint64_t m, cudaStream_t st)
 {
     QueryWs& w = idx->qws;
     const uint64_t n = idx->keys.bytes / sizeof(uint64_t), kint = (uint64_t)query_intervals(idx->dim, idx->drop);
-    const uint64_t budget = (uint64_t)idx->opt.mask_budget_mb << 20;
-    const uint64_t bytes = std::min<uint64_t>(budget, m * 1024ull + (1ull << 20) + 4 * n);
-    const uint64_t batches = std::min<uint64_t>(bytes / 4 / kBatchBytes, max_batches(idx->dim, m, n, kint));
-    const uint64_t recs = std::min<uint64_t>(bytes / 4 * 3 / sizeof(uint2), 64 * item_groups(idx->dim) * max_batches(idx->dim, m, n, kint) + (1ull << 23));
-    if (batch_capacity(w) >= batches && w.recs.bytes >= recs * sizeof(uint2)) return SFC_OK;
-    if (m <= w.sized_m && w.recs.bytes && capturing(st)) return SFC_OK;
-    SFC_TRY(w.heads.ensure(batches * sizeof(uint4), st));
-    SFC_TRY(w.bhits.ensure(batches * sizeof(uint32_t), st));
-    SFC_TRY(w.bbase.ensure((batches + 1) * sizeof(uint64_t), st));
-    return w.recs.ensure(recs * sizeof(uint2), st);
+    const uint64_t budget = (uint64_t)idx->opt.mask_budget_mb << 20, least = m * 1024ull + (1ull << 20);
+    const uint64_t most = max_batches(idx->dim, m, n, kint), per_batch = 32 * item_groups(idx->dim);
+    for (uint64_t bytes : {least + 4 * n, least}) {
+        const HitSizes h = hit_sizes(std::min(budget, bytes), most, per_batch, resident_warps());
+        const uint64_t total = h.batches * kHitBatchBytes + h.records * kHitRecordBytes;
+        if (batch_capacity(w) >= h.batches && w.recs.bytes >= h.records * kHitRecordBytes) return SFC_OK;
+        if (w.recs.bytes && ((m <= w.sized_m && capturing(st)) || (bytes > least && total >= w.refused))) continue;
+        sfc_status s = w.heads.ensure(h.batches * sizeof(uint4), st);
+        if (s == SFC_OK) s = w.bhits.ensure(h.batches * sizeof(uint32_t), st);
+        if (s == SFC_OK) s = w.bbase.ensure((h.batches + 1) * sizeof(uint64_t), st);
+        if (s == SFC_OK) s = w.recs.ensure(h.records * sizeof(uint2), st);
+        if (s != SFC_ERR_OOM) return s;
+        w.refused = total;   // not asked for again until the caller reserves
+        for (DevBuf* d : {&w.heads, &w.bhits, &w.bbase, &w.recs}) d->release(st);
+    }
+    return w.recs.bytes ? SFC_OK : SFC_ERR_OOM;
 }
 
 sfc_status ensure_query_ws(sfc_index* idx, uint64_t m, cudaStream_t st)
@@ -308,10 +316,7 @@ void set_workspace(sfc_index* idx, QueryArgs& a)
     a.cap_batches = batch_capacity(w);
     a.recs = w.recs.as<uint2>();
     a.cap_recs = std::min<uint64_t>(w.recs.bytes / sizeof(uint2), 0xffffffffull);
-    // records a warp reserves at a time (a batch has up to 32 item_groups): large while an eighth
-    // of the buffer covers every warp's
-    const uint64_t warps = (uint64_t)num_sms() * 64;
-    a.slab = a.cap_recs >= warps * 512 * 8 ? 512 : (uint32_t)(32 * item_groups(idx->dim));
+    a.slab = slab_records(a.cap_recs, max_batches(idx->dim, a.m, a.n, a.kint), 32 * item_groups(idx->dim), resident_warps());
     a.cgrab = idx->batch * std::max(1u, idx->chunk / 1024);
     a.wgrab = idx->qbatch;
     a.work_ctr = w.ctr.as<unsigned long long>();
@@ -586,6 +591,7 @@ sfc_status sfc_reserve(sfc_index* idx, uint64_t n_max, uint64_t m_max, void* str
     SFC_TRY(reserve_sort(idx->sort_ws, n1, st));
     SFC_TRY(idx->box.ensure(box_bytes(idx->dim, n1), st));
     SFC_TRY(idx->dir.ensure(dir_bytes(n1), st));
+    idx->qws.refused = ~0ull;
     SFC_TRY(ensure_query_ws(idx, m_max, st));
     SFC_TRY(reserve_scan(idx->scan_ws, std::max<uint64_t>(m_max, n1) + 1, st));
     if (idx->opt.bounds == SFC_BOUNDS_LEARNED) SFC_TRY(reserve_model(idx, n1, st));
@@ -965,6 +971,7 @@ sfc_status sfc_reserve_queries(sfc_index* idx, uint64_t m, void* stream)
     if (!idx) return SFC_ERR_INVALID;
     AllocScope alloc_scope(idx->allocator());
     SFC_TRY(ensure_status_buf(idx, as_stream(stream)));
+    idx->qws.refused = ~0ull;
     return ensure_query_ws(idx, m, as_stream(stream));
 }
 

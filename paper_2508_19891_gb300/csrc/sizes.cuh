@@ -29,4 +29,36 @@ SFC_HD uint64_t sample_position(uint32_t i, uint64_t n)
     return (((z ^ (z >> 31)) >> 32) * n) >> 32;
 }
 
+// Buffers of the hits of a query batch: per-batch heads and hit counts, and records.
+struct HitSizes {
+    uint64_t batches, records;
+};
+constexpr uint64_t kHitBatchBytes = 28, kHitRecordBytes = 8;
+constexpr uint32_t kSlab = 512;   // records that a warp reserves at a time from a large buffer
+
+// Records from which on an eighth of the buffer covers every warp's slab.
+SFC_HD uint64_t large_records(uint64_t warps) { return warps * kSlab * 8; }
+
+// Records that a warp reserves at a time: one batch's most (per_batch) where the buffer is small or has
+// that many for every batch there can be, so that none goes without; else kSlab.
+SFC_HD uint32_t slab_records(uint64_t records, uint64_t most_batches, uint64_t per_batch, uint64_t warps)
+{
+    return records < large_records(warps) || records / per_batch >= most_batches ? (uint32_t)per_batch : kSlab;
+}
+
+// Sizes within `bytes`, a quarter of them for the batches: at most what most_batches (the most that the
+// batch can have) can use.  (One lookup over 10^8 points: 26 MB; 2^23 records on top of what it can
+// use made that 117 MB.)
+SFC_HD HitSizes hit_sizes(uint64_t bytes, uint64_t most_batches, uint64_t per_batch, uint64_t warps)
+{
+    HitSizes s;
+    s.batches = bytes / 4 / kHitBatchBytes;
+    if (s.batches > most_batches) s.batches = most_batches;
+    uint64_t most = most_batches * per_batch;   // one batch a slab
+    if (most >= large_records(warps)) most = 2 * most + warps * kSlab;   // slabs with unused ends
+    s.records = bytes / 4 * 3 / kHitRecordBytes;
+    if (s.records > most) s.records = most;
+    return s;
+}
+
 }  // namespace sfc

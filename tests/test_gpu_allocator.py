@@ -203,3 +203,39 @@ def test_reserved_batches_allocate_nothing_after_the_points_grow(cuda):
     check(pts)
     assert sfc.sfc_device_status(idx) == (0, 0)
     idx.close()
+
+
+@pytest.mark.parametrize("dim", [2, 3])
+def test_queries_fit_where_the_allocator_has_little_room(cuda, dim):
+    """An allocator that has no room for a buffer of hits that grows with the points still serves a
+    batch of wide windows (what finds no room is filtered again), and is not asked over and over."""
+    rng = np.random.default_rng(dim)
+    n, m, side = 1_000_000, 64, 1 << (30 if dim == 2 else 21)
+    pts = rng.integers(0, side, size=(n, dim)).astype(np.int32)
+    q = rng.integers(0, side, size=(m, dim)).astype(np.int32)
+    d = rng.integers(0, side // 3, m).astype(np.int32)
+    roff, rids = oracle.query(oracle.build(pts), q, d, threads=8) if dim == 2 else oracle.query3(oracle.build3(pts), q, d)
+    A = sfc.TorchAllocator(cuda)
+    roomy, state, refused = A._alloc, {"tight": False}, []
+
+    def alloc(nbytes, stream, ctx):
+        if state["tight"] and nbytes > 2 << 20:
+            refused.append(int(nbytes))
+            return None
+        return roomy(nbytes, stream, ctx)
+
+    A._alloc = sfc.SFC_ALLOC_FN(alloc)
+    A.struct = sfc.sfc_allocator(A._alloc, A._free, None)
+    idx = (sfc.sfc_build if dim == 2 else sfc.sfc_build3)(to_dev(pts, cuda), allocator=A)
+    state["tight"] = True
+    for _ in range(3):
+        off, ids = sfc.query(idx, to_dev(q, cuda), to_dev(d, cuda))
+        assert np.array_equal(u64(off), roff) and np.array_equal(u32(ids), rids)
+    assert len(refused) == 1 and sfc.sfc_device_status(idx) == (0, 0)
+    state["tight"] = False
+    sfc.sfc_reserve_queries(idx, m)                      # asks again
+    off, ids = sfc.query(idx, to_dev(q, cuda), to_dev(d, cuda))
+    assert np.array_equal(u64(off), roff) and np.array_equal(u32(ids), rids)
+    idx.close()
+    torch.cuda.synchronize()
+    assert not A.live

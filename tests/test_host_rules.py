@@ -15,6 +15,13 @@ SOURCE = """
 using namespace sfc;
 extern "C" {
 uint32_t c_tiles_of(uint64_t n, uint32_t per) { return tiles_of(n, per); }
+void c_hit_sizes(uint64_t bytes, uint64_t most, uint64_t per, uint64_t warps, uint64_t* out)
+{
+    const HitSizes h = hit_sizes(bytes, most, per, warps);
+    out[0] = h.batches;
+    out[1] = h.records;
+    out[2] = slab_records(h.records, most, per, warps);
+}
 void c_sample_positions(uint32_t samples, uint64_t n, uint64_t* out)
 {
     for (uint32_t i = 0; i < samples; ++i) out[i] = sample_position(i, n);
@@ -95,3 +102,25 @@ def test_sample_sees_the_runs_whatever_the_order(rules, order, n, samples):
 def test_sample_positions_stay_inside(rules):
     for n in (1, 2, 8192, 10 ** 8, (1 << 32) - 2):
         assert int(_sample(rules, 16384, n).max()) < n
+
+
+@pytest.mark.parametrize("dim,groups,intervals", [(2, 4, 4), (2, 4, 25), (3, 2, 27)])
+@pytest.mark.parametrize("n", [1, 10 ** 6, 10 ** 8])
+def test_sizes_of_the_hit_buffers(rules, dim, groups, intervals, n):
+    """Within the bytes given; when those suffice, a record for every group that a batch can report
+    however the slabs are left; a few lookups over 10^8 points within 32 MB."""
+    warps, per = 152 * 64, 32 * groups
+    for m in (1, 3, 10, 100, 10 ** 4, 10 ** 7):
+        most = m * (n // 32 // groups + 2 * intervals + 1) // 32 + 1
+        for bytes_ in (1 << 20, (1 << 20) + 1024 * m, min(4096 << 20, (1 << 20) + 1024 * m + 4 * n)):
+            out = np.empty(3, np.uint64)
+            rules.c_hit_sizes(*(ctypes.c_uint64(v) for v in (bytes_, most, per, warps)), out.ctypes.data_as(ctypes.c_void_p))
+            batches, records, slab = (int(v) for v in out)
+            assert 28 * batches <= bytes_ // 4 and 8 * records <= bytes_ // 4 * 3
+            assert batches >= 1 and slab in (per, 512)
+            if 28 * most <= bytes_ // 4:
+                assert batches == most
+            if slab == per and 8 * most * per <= bytes_ // 4 * 3:
+                assert records >= most * slab            # a slab for every batch
+            if m == 1:
+                assert 28 * batches + 8 * records <= 32 << 20
