@@ -348,7 +348,6 @@ sfc_status do_count(sfc_index* idx, const int32_t* d_q, const int32_t* d_delta, 
     // per-batch statistics (learned-bounds counters, the scanned total, cells and chunks) start at
     // zero with the rest
     SFC_TRY(launch_reset(model_stats(idx), 7, a.work_ctr, flags_items, 2 * scan_flag_words(m) + scan_flag_words(nb), st));
-    w.write_ctr_zero = true;
     LearnedModelView lv;
     const bool ordered = use_curve_order(idx, m);
     if (ordered) {
@@ -411,10 +410,6 @@ sfc_status do_write_range(sfc_index* idx, const int32_t* d_q, const int32_t* d_d
     a.ids_capacity = d_out_ids ? cap : 0;
     a.q_begin = q_begin;
     a.q_end = q_end;
-    // the write pass's own work counter starts at zero: the count's reset serves the first write
-    // after it, a repeated one or the next slice clears it
-    if (!w.write_ctr_zero) SFC_CUDA_TRY(cudaMemsetAsync(a.work_ctr + kCtrWrite, 0, sizeof(unsigned long long), st));
-    w.write_ctr_zero = false;
     ProfScope ps(idx, "write", st);
     return launch_write(a, st);
 }
@@ -601,7 +596,6 @@ sfc_status sfc_reserve(sfc_index* idx, uint64_t n_max, uint64_t m_max, void* str
 }  // extern "C"
 
 struct sfc_graph {
-    sfc_index* idx = nullptr;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
 };
@@ -634,7 +628,6 @@ sfc_status sfc_graph_capture(sfc_index* idx, unsigned flags, const int32_t* d_po
     if (s == SFC_OK && ce != cudaSuccess) s = SFC_ERR_CUDA;
     if (s == SFC_OK && cudaGraphInstantiate(&g->exec, graph, 0) != cudaSuccess) s = SFC_ERR_CUDA;
     g->graph = graph;
-    g->idx = idx;
     cudaStreamDestroy(cs);
     idx->last_stream = st;
     if (s != SFC_OK) {
@@ -649,7 +642,6 @@ sfc_status sfc_graph_capture(sfc_index* idx, unsigned flags, const int32_t* d_po
 sfc_status sfc_graph_launch(sfc_graph* g, void* stream)
 {
     if (!g || !g->exec) return SFC_ERR_INVALID;
-    g->idx->qws.write_ctr_zero = false;   // a replayed batch uses the write pass's counter
     SFC_CUDA_TRY(cudaGraphLaunch(g->exec, as_stream(stream)));
     count_launch();
     return SFC_OK;

@@ -26,7 +26,6 @@ struct QueryWs {
     DevBuf qkeys, qkeys_sorted, perm, pstart, dbase;         // curve-order processing
     uint64_t sized_m = 0;            // queries that the workspace has been sized for
     uint64_t refused = ~0ull;        // bytes of hits that the allocator had no room for
-    bool write_ctr_zero = false;     // the write pass's work counter has not been used since the count
     PendingCount pending{false, nullptr, nullptr, 0, nullptr, false, 0, 0};
 };
 

@@ -1183,6 +1183,11 @@ __global__ void __launch_bounds__(kThreads, SFC_WRITE_BLOCKS) write_kernel(Query
             head = nhead;
         }
     }
+    // The last block to finish leaves the queue at its start for the next write: of another slice, of
+    // the same batch again, or of a replayed capture that holds no count.
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicInc(reinterpret_cast<unsigned*>(a.work_ctr + kCtrDone), gridDim.x - 1) == gridDim.x - 1)
+        atomicExch(a.work_ctr + kCtrWrite, 0ull);
 }
 
 // Queries of processing ranks [q_begin, q_end) whose items did not all get records (their

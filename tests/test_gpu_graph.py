@@ -84,3 +84,24 @@ def test_rebuild_in_place(cuda):
     off, out = sfc.query(idx, to_dev(b.queries, cuda), to_dev(b.delta, cuda))
     roff, rids = oracle.query(ref, b.queries, b.delta)
     assert np.array_equal(u64(off), roff) and np.array_equal(u32(out), rids)
+
+
+@pytest.mark.parametrize("reorder", [0, 1])
+def test_captured_write_alone(cuda, reorder):
+    """A write captured on its own (the count ran eagerly before it) writes every id on each replay."""
+    wl = W.mixed_1e7(scale=0.01)
+    idx = sfc.sfc_build(to_dev(wl.points, cuda), "z", reorder_queries=reorder)
+    roff, rids = oracle.query(oracle.build(wl.points), wl.queries, wl.delta)
+    q, d = to_dev(wl.queries, cuda), to_dev(wl.delta, cuda)
+    off = sfc.sfc_query_count(idx, q, d)
+    ids = torch.zeros(int(roff[-1]), dtype=torch.int32, device=cuda)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        sfc.sfc_query_write(idx, q, d, off, ids)
+    for _ in range(3):
+        ids.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert np.array_equal(u64(off), roff) and np.array_equal(u32(ids), rids)
+    assert sfc.sfc_device_status(idx) == (0, 0)
