@@ -131,6 +131,20 @@ struct DevBuf {
         bytes = nb;
         return SFC_OK;
     }
+    // the same, keeping the contents; a failure leaves the buffer as it is
+    sfc_status grow(size_t need, cudaStream_t st)
+    {
+        if (need <= bytes) return SFC_OK;
+        DevBuf nb;
+        SFC_TRY(nb.ensure(need, st));
+        if (ptr && cudaMemcpyAsync(nb.ptr, ptr, bytes, cudaMemcpyDeviceToDevice, st) != cudaSuccess) {
+            nb.release(st);
+            return SFC_ERR_CUDA;
+        }
+        release(st);
+        *this = nb;
+        return SFC_OK;
+    }
     void release(cudaStream_t st)
     {
         if (ptr) dev_free(ptr, bytes, st, owner);

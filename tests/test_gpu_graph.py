@@ -105,3 +105,18 @@ def test_captured_write_alone(cuda, reorder):
         torch.cuda.synchronize()
         assert np.array_equal(u64(off), roff) and np.array_equal(u32(ids), rids)
     assert sfc.sfc_device_status(idx) == (0, 0)
+
+
+@pytest.mark.parametrize("dim", [2, 3])
+@pytest.mark.parametrize("n,n_max", [(2000, 2100), (100_000, 110_000), (2000, 1000)])
+def test_reserve_keeps_a_built_index(cuda, dim, n, n_max):
+    """sfc_reserve for a few more points than the index has, within the room that its arrays have
+    left: the index still answers (its directory, which doubles there, is kept)."""
+    rng = np.random.default_rng(n)
+    pts = rng.integers(0, 1 << 16, size=(n, dim)).astype(np.int32)
+    d = rng.integers(0, 5000, 200).astype(np.int32)
+    idx = (sfc.sfc_build if dim == 2 else sfc.sfc_build3)(to_dev(pts, cuda))
+    sfc.sfc_reserve(idx, n_max, 200)
+    off, ids = sfc.query(idx, to_dev(pts[:200], cuda), to_dev(d, cuda))
+    roff, rids = _ref(pts, pts[:200], d, "z") if dim == 2 else oracle.query3(oracle.build3(pts), pts[:200], d)
+    assert np.array_equal(u64(off), roff) and np.array_equal(u32(ids), rids)
