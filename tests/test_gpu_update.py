@@ -137,3 +137,45 @@ def test_sorted_views_outlive_the_callers_index(cuda):
     del keys
     gc.collect()
     assert ref() is None
+
+
+@pytest.mark.parametrize("options", [{}, {"bounds": "learned", "occupancy_depth": 6}])
+def test_update_without_memory_changes_nothing(cuda, options):
+    """An update that finds no memory, at whichever of its requests, returns SFC_ERR_OOM and leaves the
+    index as it was; the same batch then succeeds once there is memory."""
+    rng = np.random.default_rng(12)
+    pts = rng.integers(0, 1 << 14, size=(3000, 2)).astype(np.int32)
+    ins = rng.integers(0, 1 << 14, size=(20_000, 2)).astype(np.int32)
+    dels = rng.permutation(3000)[:700].astype(np.uint32)
+    q, d = pts[:100], np.full(100, 700, np.int32)
+    A = sfc.TorchAllocator(cuda)
+    roomy, left = A._alloc, [1 << 30]
+
+    def alloc(nbytes, stream, ctx):
+        left[0] -= 1
+        return None if left[0] < 0 else roomy(nbytes, stream, ctx)
+
+    A._alloc = sfc.SFC_ALLOC_FN(alloc)
+    A.struct = sfc.sfc_allocator(A._alloc, A._free, None)
+    idx = sfc.sfc_build(to_dev(pts, cuda), "z", allocator=A, **options)
+    dyn = DynamicOracle(pts)
+
+    check_same(idx, dyn, q, d, cuda)
+    failed = 0
+    while True:
+        left[0] = min(failed, 1)                         # one more request succeeds each time
+        try:
+            first = sfc.sfc_update(idx, to_dev(ins, cuda), to_dev(dels.view(np.int32), cuda))
+            break
+        except sfc.SfcError as e:
+            assert e.status == sfc.SFC_ERR_OOM
+            failed += 1
+        finally:
+            left[0] = 1 << 30
+        check_same(idx, dyn, q, d, cuda)
+    assert failed > 5 and first == dyn.apply(ins, dels)
+    check_same(idx, dyn, q, d, cuda)
+    assert sfc.sfc_device_status(idx) == (0, 0)
+    idx.close()
+    torch.cuda.synchronize()
+    assert not A.live
