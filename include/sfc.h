@@ -176,7 +176,8 @@ void sfc_destroy(sfc_index* idx);
 /* Rebuilds the index in place over n new points (device), with the index's curve and
  * options: keys, sort, coordinates, the id table (ids restart at 0..n-1) and, if the index
  * uses learned bounds, a fresh model fit.  Reuses the index's buffers (they only grow), so
- * after sfc_reserve it allocates nothing.  Errors as sfc_build. */
+ * after sfc_reserve it allocates nothing.  Errors as sfc_build; after an error the index is
+ * empty until a rebuild succeeds. */
 sfc_status sfc_rebuild(sfc_index* idx, const int32_t* d_points, uint64_t n, void* stream);
 
 /* As sfc_rebuild with the points in host memory (int32[n][2], or [n][3] for a 3-D index):

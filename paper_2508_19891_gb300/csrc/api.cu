@@ -532,14 +532,8 @@ void sfc_destroy(sfc_index* idx)
     delete idx;
 }
 
-sfc_status sfc_rebuild(sfc_index* idx, const int32_t* d_points, uint64_t n, void* stream)
+static sfc_status rebuild_from_device(sfc_index* idx, const int32_t* d_points, cudaStream_t st)
 {
-    if (!idx || n >= 0xffffffffull || (n && !d_points)) return SFC_ERR_INVALID;
-    AllocScope alloc_scope(idx->allocator());
-    cudaStream_t st = as_stream(stream);
-    idx->last_stream = st;
-    idx->n = n;
-    idx->qws.pending.valid = false;
     SFC_TRY(ensure_status_buf(idx, st));
     // every issued id is live again
     if (idx->dim == 3) return build3_from_device(idx, d_points, st);
@@ -550,6 +544,23 @@ sfc_status sfc_rebuild(sfc_index* idx, const int32_t* d_points, uint64_t n, void
         SFC_TRY(train_model(idx, st));
     }
     return SFC_OK;
+}
+
+sfc_status sfc_rebuild(sfc_index* idx, const int32_t* d_points, uint64_t n, void* stream)
+{
+    if (!idx || n >= 0xffffffffull || (n && !d_points)) return SFC_ERR_INVALID;
+    AllocScope alloc_scope(idx->allocator());
+    cudaStream_t st = as_stream(stream);
+    idx->last_stream = st;
+    idx->n = n;
+    idx->qws.pending.valid = false;
+    const sfc_status s = rebuild_from_device(idx, d_points, st);
+    if (s != SFC_OK) {   // some arrays may be gone: an empty index until a rebuild succeeds
+        idx->n = 0;
+        idx->next_id = 0;
+        idx->model.trained = false;
+    }
+    return s;
 }
 
 sfc_status sfc_rebuild_host(sfc_index* idx, const int32_t* h_points, uint64_t n, void* stream)

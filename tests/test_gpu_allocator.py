@@ -239,3 +239,44 @@ def test_queries_fit_where_the_allocator_has_little_room(cuda, dim):
     idx.close()
     torch.cuda.synchronize()
     assert not A.live
+
+
+@pytest.mark.parametrize("dim,options", [(2, {}), (2, {"bounds": "learned", "occupancy_depth": 5}), (3, {})])
+def test_rebuild_without_memory_leaves_an_empty_index(cuda, dim, options):
+    """A rebuild that finds no memory, at whichever of its requests, returns SFC_ERR_OOM and leaves an
+    empty index that answers queries and takes the next rebuild."""
+    rng = np.random.default_rng(13)
+    pts = rng.integers(0, 1 << 14, size=(40_000, dim)).astype(np.int32)
+    q, d = to_dev(pts[:100], cuda), torch.full((100,), 300, dtype=torch.int32, device=cuda)
+    A = sfc.TorchAllocator(cuda)
+    roomy, left = A._alloc, [1 << 30]
+
+    def alloc(nbytes, stream, ctx):
+        left[0] -= 1
+        return None if left[0] < 0 else roomy(nbytes, stream, ctx)
+
+    A._alloc = sfc.SFC_ALLOC_FN(alloc)
+    A.struct = sfc.sfc_allocator(A._alloc, A._free, None)
+    idx = (sfc.sfc_build if dim == 2 else sfc.sfc_build3)(to_dev(pts[:2000], cuda), allocator=A, **options)
+    failed = 0
+    while True:
+        left[0] = min(failed, 1)                         # one more request succeeds each time
+        try:
+            sfc.sfc_rebuild(idx, to_dev(pts, cuda))
+            break
+        except sfc.SfcError as e:
+            assert e.status == sfc.SFC_ERR_OOM
+            failed += 1
+        finally:
+            left[0] = 1 << 30
+        off, ids = sfc.query(idx, q, d)
+        assert not off.any().item() and ids.numel() == 0 and sfc.sfc_get_sorted(idx)[0].numel() == 0
+    assert failed > 3
+    off, ids = sfc.query(idx, q, d)
+    ref = oracle.build(pts) if dim == 2 else oracle.build3(pts)
+    roff, rids = (oracle.query if dim == 2 else oracle.query3)(ref, pts[:100], np.full(100, 300, np.int32))
+    assert np.array_equal(u64(off), roff) and np.array_equal(u32(ids), rids)
+    assert sfc.sfc_device_status(idx) == (0, 0)
+    idx.close()
+    torch.cuda.synchronize()
+    assert not A.live
