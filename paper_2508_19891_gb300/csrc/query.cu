@@ -1149,12 +1149,21 @@ __global__ void __launch_bounds__(kThreads, SFC_WRITE_BLOCKS) write_kernel(Query
     const uint32_t ra = (uint32_t)a.q_begin, rb = (uint32_t)a.q_end;
     const bool all = ra == 0 && rb == (uint32_t)a.m;
     const uint64_t first = a.gbase[ra] >> 5, nb = min((a.gbase[rb] + 31) >> 5, a.cap_batches);
-    const uint32_t grab = grab_size(nb > first ? nb - first : 0, a.wgrab);
+    const uint64_t todo = nb > first ? nb - first : 0;
+    const uint32_t grab = grab_size(todo, a.wgrab);
     while (true) {
         uint64_t b0 = 0;
         if (lane == 0) b0 = atomicAdd(a.work_ctr + kCtrWrite, (unsigned long long)grab);
-        b0 = first + __shfl_sync(0xffffffffu, b0, 0);
-        if (b0 >= nb) break;
+        b0 = __shfl_sync(0xffffffffu, b0, 0);
+        if (b0 >= todo) {
+            // Every warp fails to grab once, at todo rounded up and `grab` further for each that failed
+            // before it.  The last one puts the queue back to its start for the next write: of another
+            // slice, of the same batch again, or of a replayed capture that holds no count.
+            const uint64_t others = (uint64_t)gridDim.x * (kThreads / 32) - 1;
+            if (lane == 0 && b0 >= todo + others * grab) a.work_ctr[kCtrWrite] = 0;
+            break;
+        }
+        b0 += first;
         const uint32_t left = (uint32_t)min(nb - b0, (uint64_t)grab);
         const uint4* heads = a.heads + b0;
         const uint64_t* bbase = a.bbase + b0;
@@ -1183,11 +1192,6 @@ __global__ void __launch_bounds__(kThreads, SFC_WRITE_BLOCKS) write_kernel(Query
             head = nhead;
         }
     }
-    // The last block to finish leaves the queue at its start for the next write: of another slice, of
-    // the same batch again, or of a replayed capture that holds no count.
-    __syncthreads();
-    if (threadIdx.x == 0 && atomicInc(reinterpret_cast<unsigned*>(a.work_ctr + kCtrDone), gridDim.x - 1) == gridDim.x - 1)
-        atomicExch(a.work_ctr + kCtrWrite, 0ull);
 }
 
 // Queries of processing ranks [q_begin, q_end) whose items did not all get records (their

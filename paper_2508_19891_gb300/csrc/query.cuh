@@ -84,10 +84,9 @@ sfc_status launch_count(const QueryArgs& a, cudaStream_t st);
 // queries that scan at most this many points have no chunks in the statistics
 constexpr uint32_t kSmallScan = 64;
 // work counters of a query batch: the count pass's and the write pass's queues of item batches,
-// the records handed out, whether some item found no room for its record, and the blocks of the write
-// pass that are done (the last one puts that pass's queue and this count back to zero)
-constexpr int kCtrCount = 0, kCtrWrite = 1, kCtrRecs = 2, kCtrOverflow = 3, kCtrDone = 4;
-constexpr int kCtrWords = 5;
+// the records handed out, and whether some item found no room for its record
+constexpr int kCtrCount = 0, kCtrWrite = 1, kCtrRecs = 2, kCtrOverflow = 3;
+constexpr int kCtrWords = 4;
 // most items, and batches of 32 of them, that m queries over n points can have: a range touches at
 // most two items more than its length fills
 inline uint64_t max_batches(int dim, uint64_t m, uint64_t n, uint64_t kint)
