@@ -24,34 +24,43 @@ namespace {
 constexpr int kT = 256;
 constexpr int kU = 4;   // groups per warp and iteration
 
-// Entries [0, 2^bits] of the directory, by the blocks [0, blocks) of a launch.
-__device__ __forceinline__ void fill_directory(const uint64_t* __restrict__ keys, uint32_t n, int bits, uint32_t blocks,
-                                               uint32_t* dir)
+// One step of the directory's search: the answer in [lo, lo + len] given the keys at lo + len / 4,
+// lo + len / 2 and the place between that and the end.  The three are counted, not tested one after
+// another, so that their loads are in flight together.
+__device__ __forceinline__ void narrow(uint32_t& lo, uint32_t& len, uint64_t ka, uint64_t kb, uint64_t kc, uint64_t t)
 {
-    const uint64_t kmin = __ldg(keys), kmax = __ldg(keys + n - 1);
+    const uint32_t q = len >> 2, h = len >> 1, c = (uint32_t)(ka < t) + (kb < t) + (kc < t);
+    const uint32_t from = c == 0 ? 0 : (c & 1 ? q : 0) + (c & 2 ? h : 0) + 1;
+    const uint32_t to = c == 3 ? len : (c == 0 ? q : h + (c == 2 ? q : 0));
+    lo += from;
+    len = to - from;
+}
+
+// Entries [0, 2^bits] of the directory, by the blocks [0, blocks) of a launch.
+__device__ __forceinline__ void fill_directory(const uint64_t* keys, uint32_t n, int bits, uint32_t blocks, uint32_t* dir)
+{
+    // the first step's probes are the same for every entry: loaded with the ends of the range
+    const uint64_t kmin = keys[0], kmax = keys[n - 1];
+    const uint64_t k1 = keys[n >> 2], k2 = keys[n >> 1], k3 = keys[(n >> 2) + (n >> 1)];
     const int shift = dir_shift(kmin, kmax, bits);
     for (uint32_t v = blockIdx.x * kT + threadIdx.x; v <= 1u << bits; v += blocks * kT) {
         const uint64_t t = kmin + ((uint64_t)v << shift);   // at most 2 kmax: 64 bits hold it
         // three probes a step: the latency of the steps, not the loads, sets the time of short arrays
         uint32_t lo = 0, len = n;   // the answer lies in [lo, lo + len]
-        while (len > 0) {
-            const uint32_t q = len >> 2, h = len >> 1;
-            const uint64_t ka = __ldg(keys + lo + q), kb = __ldg(keys + lo + h), kc = __ldg(keys + lo + h + q);
-            const uint32_t from = kc < t ? h + q + 1 : (kb < t ? h + 1 : (ka < t ? q + 1 : 0));
-            const uint32_t to = kc < t ? len : (kb < t ? h + q : (ka < t ? h : q));
-            lo += from;
-            len = to - from;
-        }
+        narrow(lo, len, k1, k2, k3, t);
+        while (len > 0)
+            narrow(lo, len, keys[lo + (len >> 2)], keys[lo + (len >> 1)], keys[lo + (len >> 1) + (len >> 2)], t);
         dir[v] = lo;
     }
 }
 
 // Blocks [0, dblocks) fill the directory, the others the boxes.
-__global__ void __launch_bounds__(kT) boxes_kernel(const int2* __restrict__ xy, const uint64_t* __restrict__ keys,
-                                                   uint32_t n, uint32_t groups, int bits, uint32_t dblocks, uint32_t* dir,
-                                                   int4* box)
+__global__ void __launch_bounds__(kT) boxes_kernel(const int2* xy, const uint64_t* keys, uint32_t n, uint32_t groups,
+                                                   int bits, uint32_t dblocks, uint32_t* dir, int4* box)
 {
     chain_start();
+    xy = after_wait(xy);
+    keys = after_wait(keys);
     if (blockIdx.x < dblocks) {
         fill_directory(keys, n, bits, dblocks, dir);
         return;
@@ -62,7 +71,7 @@ __global__ void __launch_bounds__(kT) boxes_kernel(const int2* __restrict__ xy, 
         int2 p[kU];
 #pragma unroll
         for (int u = 0; u < kU; ++u)   // past the end the last point stands in: it changes no box
-            p[u] = __ldg(xy + (uint32_t)min((uint64_t)(g0 + u) * 32 + lane, (uint64_t)n - 1));
+            p[u] = xy[min((uint64_t)(g0 + u) * 32 + lane, (uint64_t)n - 1)];
 #pragma unroll
         for (int u = 0; u < kU; ++u) {
             const int4 b = make_int4(__reduce_min_sync(0xffffffffu, p[u].x), __reduce_min_sync(0xffffffffu, p[u].y),
@@ -74,11 +83,11 @@ __global__ void __launch_bounds__(kT) boxes_kernel(const int2* __restrict__ xy, 
 
 // 3-D: decodes the sorted keys into the 16-byte records and the packed coordinates on the way (a
 // decoding kernel of its own and boxes read back from its records: 78 us more at 10^7 points).
-__global__ void __launch_bounds__(kT) boxes3_kernel(const uint64_t* __restrict__ keys, uint32_t n, uint32_t groups,
-                                                    int bits, uint32_t dblocks, uint32_t* dir, int4* xyz, uint2* packed,
-                                                    int4* box)
+__global__ void __launch_bounds__(kT) boxes3_kernel(const uint64_t* keys, uint32_t n, uint32_t groups, int bits,
+                                                    uint32_t dblocks, uint32_t* dir, int4* xyz, uint2* packed, int4* box)
 {
     chain_start();
+    keys = after_wait(keys);
     if (blockIdx.x < dblocks) {
         fill_directory(keys, n, bits, dblocks, dir);
         return;
@@ -89,7 +98,7 @@ __global__ void __launch_bounds__(kT) boxes3_kernel(const uint64_t* __restrict__
         uint64_t k[kU];
 #pragma unroll
         for (int u = 0; u < kU; ++u)
-            k[u] = __ldg(keys + (uint32_t)min((uint64_t)(g0 + u) * 32 + lane, (uint64_t)n - 1));
+            k[u] = keys[min((uint64_t)(g0 + u) * 32 + lane, (uint64_t)n - 1)];
 #pragma unroll
         for (int u = 0; u < kU; ++u) {
             const uint64_t i = (uint64_t)(g0 + u) * 32 + lane;

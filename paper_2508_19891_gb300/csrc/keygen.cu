@@ -13,11 +13,11 @@ namespace {
 constexpr int kThreads = 256;
 
 template <int CURVE>
-__global__ void __launch_bounds__(kThreads) keys_kernel(const int2* __restrict__ pts, uint64_t n,
-                                                        uint64_t* __restrict__ keys,
-                                                        uint32_t* status, int vec)
+__global__ void __launch_bounds__(kThreads) keys_kernel(const int2* pts, uint64_t n, uint64_t* keys, uint32_t* status,
+                                                        int vec)
 {
     chain_start();
+    pts = after_wait(pts);
     __shared__ HilbertTables tb;
     if (CURVE == SFC_CURVE_HILBERT) hilbert_tables_init(&tb);
     if (!vec) {   // operands not 16-byte aligned: one point per thread
@@ -53,10 +53,10 @@ __global__ void __launch_bounds__(kThreads) keys_kernel(const int2* __restrict__
 }
 
 template <int CURVE>
-__global__ void __launch_bounds__(kThreads) decode_kernel(const uint64_t* __restrict__ keys,
-                                                          uint64_t n, int2* __restrict__ pts)
+__global__ void __launch_bounds__(kThreads) decode_kernel(const uint64_t* keys, uint64_t n, int2* pts)
 {
     chain_start();
+    keys = after_wait(keys);
     __shared__ HilbertTables tb;
     if (CURVE == SFC_CURVE_HILBERT) hilbert_tables_init(&tb);
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
@@ -71,14 +71,14 @@ __global__ void __launch_bounds__(kThreads) decode_kernel(const uint64_t* __rest
 
 // 3-D Z keys: points are 12-byte records, read as three 32-bit words (consecutive threads read
 // consecutive records, so a warp's loads cover 384 contiguous bytes).
-__global__ void __launch_bounds__(kThreads) keys3_kernel(const int32_t* __restrict__ pts, uint64_t n,
-                                                         uint64_t* __restrict__ keys, uint32_t* status)
+__global__ void __launch_bounds__(kThreads) keys3_kernel(const int32_t* pts, uint64_t n, uint64_t* keys, uint32_t* status)
 {
     chain_start();
+    pts = after_wait(pts);
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     bool bad = false;
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        const int32_t x = __ldg(pts + 3 * i), y = __ldg(pts + 3 * i + 1), z = __ldg(pts + 3 * i + 2);
+        const int32_t x = pts[3 * i], y = pts[3 * i + 1], z = pts[3 * i + 2];
         bad |= !point3_in_domain(x, y, z);
         keys[i] = morton3_key((uint32_t)x, (uint32_t)y, (uint32_t)z);
     }

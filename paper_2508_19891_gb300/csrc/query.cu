@@ -619,19 +619,21 @@ plan_kernel(QueryArgs a, Bounds bounds_in, PlanExport ex)
     // processing order is given: neighbouring threads then search neighbouring keys)
     const uint64_t r = (uint64_t)blockIdx.x * kThreads + threadIdx.x;
     const bool active = r < a.m;
-    const uint64_t i = active && a.perm ? (uint64_t)__ldg(a.perm + r) : r;
+    const uint32_t* perm = after_wait(a.perm);
+    const int32_t *qs = after_wait(a.q), *ds = after_wait(a.delta);
+    const uint64_t i = active && perm ? (uint64_t)perm[r] : r;
     int4 q = make_int4(0, 0, -1, 0);   // x, y, delta, z
     if (active) {
         if (DIM == 3) {
-            q.x = __ldg(a.q + 3 * i);
-            q.y = __ldg(a.q + 3 * i + 1);
-            q.w = __ldg(a.q + 3 * i + 2);
+            q.x = qs[3 * i];
+            q.y = qs[3 * i + 1];
+            q.w = qs[3 * i + 2];
         } else {
-            const int2 c = __ldg(reinterpret_cast<const int2*>(a.q) + i);
+            const int2 c = reinterpret_cast<const int2*>(qs)[i];
             q.x = c.x;
             q.y = c.y;
         }
-        q.z = __ldg(a.delta + i);
+        q.z = ds[i];
     }
     const bool ok = active && q.z >= 0 && (DIM == 3 ? point3_in_domain(q.x, q.y, q.w) : point_in_domain(q.x, q.y));
     if (active && !ok) set_status(a.status, SFC_DEV_BAD_QUERY);
@@ -949,15 +951,16 @@ __device__ __forceinline__ void filter_items(const QueryArgs& a, const Window& w
         if ((slots >> (8 * u)) & 0x80u) word[u] &= sm->hits[(slots >> (8 * u)) & 0x7fu];
 }
 
-// Warp-cooperative search: the query owning item g (largest q with base[q] <= g).
-__device__ __forceinline__ uint64_t owner_query(const uint64_t* __restrict__ base, uint64_t m, uint64_t g)
+// Warp-cooperative search: the query owning item g (largest q with base[q] <= g).  Ordinary loads: base
+// is what the kernel before wrote (after_wait).
+__device__ __forceinline__ uint64_t owner_query(const uint64_t* base, uint64_t m, uint64_t g)
 {
     uint64_t lo = 0, hi = m;   // base[lo] <= g < base[hi]
     const unsigned lane = lane_id();
     while (hi - lo > 1) {
         const uint64_t step = (hi - lo + 31) >> 5;
         const uint64_t pos = lo + lane * step;
-        const bool le = pos < hi && __ldg(base + pos) <= g;
+        const bool le = pos < hi && base[pos] <= g;
         const uint32_t bal = __ballot_sync(0xffffffffu, le);
         const int last = 31 - __clz(bal);
         const uint64_t nlo = lo + (uint64_t)last * step;

@@ -69,6 +69,20 @@ inline void launch_chain(void (*kernel)(P...), unsigned grid, unsigned block, si
 
 __device__ __forceinline__ void chain_start() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// A pointer to what the kernel before may have written (or, at the head of a chain, the caller's
+// kernel).  A read-only load (__ldg, a __restrict__ parameter) promises that the data does not change
+// while this kernel runs, so a compiler may move it ahead of the wait; the grid has started by then, and
+// the writes need not be visible yet.  Such data is read with ordinary loads (or __ldcs) through the
+// pointer that this returns.  Loads whose address depends on something read after the wait
+// cannot move and need no more, nor does what earlier kernels of the chain have written: those were
+// complete before the one before started.
+template <class T>
+__device__ __forceinline__ T* after_wait(T* p)
+{
+    asm volatile("" : "+l"(p)::"memory");
+    return p;
+}
+
 int num_sms();   // SM count of the current device (cached per device)
 
 // Points that a coordinate array has room for: whole groups of 32, so that a group can be loaded

@@ -95,9 +95,10 @@ __global__ void del_locate_kernel(const uint64_t* __restrict__ keys, const uint3
 // Rank of each (sorted) insert among the old entries: all old ids are smaller, so it is the
 // number of old keys <= the insert's key.
 __global__ void ins_rank_kernel(const uint64_t* __restrict__ keys, uint32_t n, const uint32_t* __restrict__ dir, int bits,
-                                const uint64_t* __restrict__ ikeys, uint64_t k, uint32_t* rank)
+                                const uint64_t* ikeys, uint64_t k, uint32_t* rank)
 {
     chain_start();
+    ikeys = after_wait(ikeys);
     for (uint64_t j = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; j < k; j += (uint64_t)gridDim.x * blockDim.x) {
         const uint64_t kk = ikeys[j];
         uint32_t lo, hi;
@@ -116,9 +117,10 @@ __global__ void ins_rank_kernel(const uint64_t* __restrict__ keys, uint32_t n, c
 // starts[t] = how many of the ascending pos[0 .. k) lie before tile t, t = 0 .. tiles.  The
 // thread of pos[j] fills the tiles that begin after pos[j - 1] and not after pos[j] (j == k: the
 // rest).  A position may be n (an insert after every entry).
-__global__ void tile_starts_kernel(const uint32_t* __restrict__ pos, uint64_t k, uint32_t tiles, uint32_t* starts)
+__global__ void tile_starts_kernel(const uint32_t* pos, uint64_t k, uint32_t tiles, uint32_t* starts)
 {
     chain_start();
+    pos = after_wait(pos);
     for (uint64_t j = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; j <= k; j += (uint64_t)gridDim.x * blockDim.x) {
         const uint32_t t0 = j ? pos[j - 1] / kMoveTile + 1 : 0;
         const uint32_t t1 = j < k ? min(pos[j] / kMoveTile, tiles) : tiles;
@@ -134,10 +136,11 @@ __global__ void tile_starts_kernel(const uint32_t* __restrict__ pos, uint64_t k,
 __global__ void __launch_bounds__(kT) move_kernel(const uint64_t* __restrict__ keys, const uint32_t* __restrict__ ids,
                                                   const int2* __restrict__ xy, uint32_t n,
                                                   const uint32_t* __restrict__ dbits, const uint64_t* __restrict__ dstart,
-                                                  const uint32_t* __restrict__ rank, const uint32_t* __restrict__ istart,
+                                                  const uint32_t* __restrict__ rank, const uint32_t* istart,
                                                   uint64_t* nkeys, uint32_t* nids, int2* nxy)
 {
     chain_start();
+    istart = after_wait(istart);
     __shared__ uint32_t s_ins[kMoveTile];   // inserts ranked at each entry, then its slot in the tile's output
     __shared__ uint32_t s_warp[kT / 32];
     const int tid = threadIdx.x;

@@ -1,7 +1,9 @@
 """Sizes and positions that the library computes on the host and the device alike (csrc/sizes.cuh):
 the same source built by the host compiler, at the limits of what the calls accept."""
 import ctypes
+import glob
 import os
+import re
 import shutil
 import subprocess
 
@@ -124,3 +126,37 @@ def test_sizes_of_the_hit_buffers(rules, dim, groups, intervals, n):
                 assert records >= most * slab            # a slab for every batch
             if m == 1:
                 assert 28 * batches + 8 * records <= 32 << 20
+
+
+def _kernels(path):
+    """Name and body of every __global__ function of a file."""
+    src = open(path).read()
+    for mt in re.finditer(r"__global__[^;{]*?(\w+_kernel)\s*\(", src):
+        start = src.index("{", mt.end())
+        depth, end = 1, start + 1
+        while depth:
+            depth += {"{": 1, "}": -1}.get(src[end], 0)
+            end += 1
+        yield mt.group(1), src[start + 1:end - 1]
+
+
+def test_kernels_of_a_chain_wait_before_anything_else():
+    """Every kernel that launch_chain starts begins with the wait, and reads what the kernel (or the
+    caller's kernel) before it writes through after_wait, at addresses known before the wait."""
+    bodies, launched = {}, set()
+    for path in sorted(glob.glob(os.path.join(CSRC, "*.cu"))):
+        for name, body in _kernels(path):
+            bodies[os.path.basename(path), name] = body
+        launched |= {(os.path.basename(path), m) for m in
+                     re.findall(r"launch_chain\(\s*(\w+_kernel)", open(path).read())}
+    assert len(launched) > 20
+    for k in launched:
+        assert bodies[k].lstrip().startswith("chain_start();"), k
+    reads = {("boxes.cu", "boxes_kernel"): ["xy", "keys"], ("boxes.cu", "boxes3_kernel"): ["keys"],
+             ("keygen.cu", "keys_kernel"): ["pts"], ("keygen.cu", "decode_kernel"): ["keys"],
+             ("keygen.cu", "keys3_kernel"): ["pts"], ("update.cu", "ins_rank_kernel"): ["ikeys"],
+             ("update.cu", "tile_starts_kernel"): ["pos"], ("update.cu", "move_kernel"): ["istart"],
+             ("query.cu", "plan_kernel"): ["a.perm", "a.q", "a.delta"]}
+    for k, names in reads.items():
+        for p in names:
+            assert f"after_wait({p})" in bodies[k] and f"__ldg({p} " not in bodies[k], (k, p)
