@@ -97,7 +97,8 @@ typedef struct {
     int train_steps;        /* learned model: Adam steps of the root (default 8) */
     int train_samples;      /* learned model: keys sampled for root training (default 16384) */
     float learning_rate;    /* learned model: Adam step size (default 0.02) */
-    int chunk;              /* scan chunk in points (0 = autotuned/default 1024) */
+    int chunk;              /* points per chunk of sfc_query_stats; past 1024 the count pass takes
+                               proportionally more work per grab (0 = autotuned/default 1024) */
     int mask_budget_mb;     /* cap on the buffer that carries the hits from the count pass to the
                                write pass, sized 1 KB per query and 4 bytes per point (1 KB per
                                query where the allocator has no room for that); queries whose
@@ -260,10 +261,10 @@ sfc_status sfc_reserve_queries(sfc_index* idx, uint64_t m, void* stream);
 
 /* Autotuner: when the index was built with cover_refine = -1, first times whole batches
  * (count + write) under the covers 0, 1 and 2; then times the count pass (plan + scan + count)
- * of this query batch for chunks of {256, 512, 1024, 2048, 4096} points, then for {1, 2, 4, 8,
- * 16} work items per work-queue grab, then the write pass for {1, 2, 4, 8, 16} work items per
- * grab, and keeps the fastest in the index (results do not depend on them).  The choice is cached per (device,
- * curve, log2 n, log2 m, bound search, cover option) for later indexes; force != 0
+ * of this query batch for chunks of {1024, 2048, 4096} points, then for {1, 2, 4, 8, 16} batches
+ * of 32 work items per work-queue grab, then the write pass for {1, 2, 4, 8, 16} batches per
+ * grab, and keeps the fastest in the index (results do not depend on them).  The choice is cached
+ * per (device, curve, log2 n, log2 m, bound search, cover option) for later indexes; force != 0
  * re-measures.  Writes the choice to *h_chunk, *h_batch, *h_qbatch (any may be NULL); the
  * cover is read back with sfc_cover_refine.  Synchronises `stream`; allocates temporary
  * output buffers. */
@@ -271,9 +272,10 @@ sfc_status sfc_autotune(sfc_index* idx, const int32_t* d_q, const int32_t* d_del
                         int* h_chunk, int* h_batch, int* h_qbatch, void* stream);
 
 /* Sets the three scan settings that sfc_autotune chooses, without timing anything: the chunk
- * in points (32 ... 4096, a multiple of 32; past 1024 the count pass takes proportionally more
- * per grab), the work items (up to 4,096 neighbouring points each) per work-queue grab of the count
- * pass (batch) and of the write pass (qbatch), each 1 ... 1024; otherwise
+ * in points (32 ... 4096, a multiple of 32; up to 1024 it sets a statistic only, past that the
+ * count pass takes proportionally more per grab), and how many batches of 32 work items (an item is
+ * up to 128 neighbouring points of one query) a warp takes per grab of the count pass (batch)
+ * and of the write pass (qbatch), each 1 ... 1024; otherwise
  * SFC_ERR_INVALID and nothing changes.  Results do not depend on them, and a count already
  * made is not changed.  For replaying a measured choice where timing it
  * again would give another (under a profiler, whose overhead changes the timings). */

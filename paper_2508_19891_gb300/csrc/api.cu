@@ -317,7 +317,7 @@ void set_workspace(sfc_index* idx, QueryArgs& a)
     a.recs = w.recs.as<uint2>();
     a.cap_recs = std::min<uint64_t>(w.recs.bytes / sizeof(uint2), 0xffffffffull);
     a.slab = slab_records(a.cap_recs, max_batches(idx->dim, a.m, a.n, a.kint), 32 * item_groups(idx->dim), resident_warps());
-    a.cgrab = idx->batch * std::max(1u, idx->chunk / 1024);
+    a.cgrab = idx->batch * std::max(1u, idx->chunk / 1024);   // index.cuh
     a.wgrab = idx->qbatch;
     a.work_ctr = w.ctr.as<unsigned long long>();
 }
@@ -803,7 +803,9 @@ sfc_status sfc_autotune(sfc_index* idx, const int32_t* d_q, const int32_t* d_del
         }
         uint32_t bc = idx->chunk, bb = idx->batch, bq = idx->qbatch;
         best = 1e30f;
-        for (uint32_t c : {256u, 512u, 1024u, 2048u, 4096u}) {
+        // (a chunk of up to 1,024 points changes nothing but a statistic: timing smaller ones as well
+        // would let noise choose)
+        for (uint32_t c : {1024u, 2048u, 4096u}) {
             if (s != SFC_OK) break;
             idx->chunk = c;
             idx->batch = 4;

@@ -75,9 +75,9 @@ struct sfc_index {
     uint32_t next_id = 0;               // first id not yet issued
     sfc_options opt{};
     sfc_bounds bounds = SFC_BOUNDS_BINARY;
-    uint32_t chunk = 1024;              // points per scan chunk
-    uint32_t batch = 4;                 // chunks per work-queue grab
-    uint32_t qbatch = 8;                // queries per write-queue grab
+    uint32_t chunk = 1024;              // points per chunk of the statistics
+    uint32_t batch = 4;                 // item batches per grab of the count pass, times chunk / 1024 past that
+    uint32_t qbatch = 8;                // item batches per grab of the write pass
     int drop = 0;                       // cover refinement: levels below cells(Q) (0..2)
     int norm = 0;                       // query window (sfc_norm)
     int dim = 2;                        // 2, or 3 for indexes made by sfc_build3

@@ -402,3 +402,13 @@ def test_big_queries_with_small_mask_budget(cuda):
         idx, st = assert_same(pts, qs, d, "z", cuda, chunk=chunk, mask_budget_mb=1, cover_refine=1,
                               reorder_queries=1)
         assert st == (0, 0)
+
+
+def test_autotune_times_settings_that_differ(cuda):
+    """Chunks of up to 1,024 points leave the passes as they are, so the tuner does not choose
+    between them."""
+    wl = W.mixed_1e7(scale=0.01)
+    q, d = to_dev(wl.queries, cuda), to_dev(wl.delta, cuda)
+    idx = sfc.sfc_build(to_dev(wl.points, cuda), "z")
+    for _ in range(8):
+        assert sfc.sfc_autotune(idx, q, d, force=True)["chunk"] in (1024, 2048, 4096)
