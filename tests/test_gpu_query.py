@@ -412,3 +412,19 @@ def test_autotune_times_settings_that_differ(cuda):
     idx = sfc.sfc_build(to_dev(wl.points, cuda), "z")
     for _ in range(8):
         assert sfc.sfc_autotune(idx, q, d, force=True)["chunk"] in (1024, 2048, 4096)
+
+
+def test_host_batch_keeps_one_order_when_it_cannot_slice(cuda):
+    """A host batch in curve order whose result buffer is smaller than what the write pass slices keeps
+    one order over the batch (one sort pass fewer than an order by slices); results are the same."""
+    wl = W.mixed_1e7(scale=0.01)
+    roff, rids = oracle.query(oracle.build(wl.points), wl.queries, wl.delta)
+    idx = sfc.sfc_build(to_dev(wl.points, cuda), "z", reorder_queries=1)
+    launches = {}
+    for capacity in (len(rids), (8 << 20) - 1, 8 << 20):
+        for _ in range(2):
+            before = sfc.sfc_launch_count()
+            off, ids = sfc.sfc_query_batch_host(idx, wl.queries, wl.delta, capacity)
+            launches[capacity] = sfc.sfc_launch_count() - before
+            assert np.array_equal(off, roff) and np.array_equal(ids, rids)
+    assert launches[len(rids)] == launches[(8 << 20) - 1] == launches[8 << 20] - 1
