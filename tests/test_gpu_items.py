@@ -110,3 +110,26 @@ def test_bounds_behind_the_directory(cuda, n, spread):
                 for r in range(int(c[i])):
                     assert b[K * i + r] == oracle.lower_bound(ref.keys, int(lo[K * i + r]))
                     assert e[K * i + r] == oracle.lower_bound(ref.keys, int(hi[K * i + r]) + 1)
+
+
+@pytest.mark.parametrize("dim", [2, 3])
+def test_queries_without_records_are_filtered_again(cuda, dim):
+    """Windows over most of the points under a 1 MB budget: their items outnumber the batches that
+    there is room for, so some queries are certainly written by the second filter."""
+    rng = np.random.default_rng(dim)
+    n, m, side = (250_000, 260, 1 << 20) if dim == 2 else (200_000, 180, 1 << 18)
+    pts = rng.integers(0, side, size=(n, dim)).astype(np.int32)
+    qs = rng.integers(side // 3, 2 * side // 3, size=(m, dim)).astype(np.int32)
+    d = rng.integers(side // 2, side, m).astype(np.int32)
+    d[::9] = rng.integers(0, 50, len(d[::9]))            # small ones between them
+    if dim == 2:
+        roff, rids = oracle.query(oracle.build(pts), qs, d, threads=8)
+        idx = sfc.sfc_build(to_dev(pts, cuda), "z", mask_budget_mb=1)
+    else:
+        roff, rids = oracle.query3(oracle.build3(pts), qs, d)
+        idx = sfc.sfc_build3(to_dev(pts, cuda), mask_budget_mb=1)
+    _check(idx, qs, d, roff, rids, cuda)
+    # an item covers at most 128 (3-D: 64) scanned points, a batch 32 items, and 1 MB holds a quarter
+    # of its bytes, and an eighth and 64 more, in 28-byte batches
+    most = ((1 << 20) // 4 // 28) * 9 // 8 + 64
+    assert sfc.sfc_query_stats(idx)["scanned"] > (128 if dim == 2 else 64) * 32 * most
