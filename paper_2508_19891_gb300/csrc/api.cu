@@ -1,7 +1,7 @@
 // C ABI of the library (include/sfc.h): argument checks, the index object and its
 // workspaces, and the order of kernel launches for each call.  No computation of the method
-// happens here; every step runs in the kernels of keygen.cu, radix.cu, scan.cu, query.cu,
-// learned.cu and update.cu.
+// happens here; every step runs in the kernels of keygen.cu, radix.cu, boxes.cu, scan.cu,
+// query.cu, occupancy.cu, learned.cu and update.cu.
 #include <algorithm>
 #include <cstring>
 #include <mutex>

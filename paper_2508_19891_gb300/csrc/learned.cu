@@ -575,10 +575,7 @@ __device__ int2 block_minmax_i(int lo, int hi, int* sh)
 //   predict function.  The leaf's keys are read twice; the second read mostly comes from L2.
 // Threads per leaf block: at 10^8 keys (about 24,000 per leaf) 512 threads take the stage from
 // 1.26 ms (256 threads) to 0.99 ms; 1,024 gain another 2%.
-#ifndef SFC_LEAF_THREADS
-#define SFC_LEAF_THREADS 512
-#endif
-constexpr int kLeafThreads = SFC_LEAF_THREADS;
+constexpr int kLeafThreads = 512;
 
 __global__ void __launch_bounds__(kLeafThreads) leaf_stage_kernel(const uint64_t* __restrict__ keys, uint64_t n,
                                                                   const uint32_t* __restrict__ bound, LeafParams* leaf,

@@ -43,35 +43,14 @@ constexpr int kThreads = 256;
 
 // Binary searches in lock step per thread, and the plan kernel's resident blocks per SM (its
 // register budget) for each bound search.
-#ifndef SFC_BINARY_BATCH
-#define SFC_BINARY_BATCH 4
-#endif
-#ifndef SFC_BINARY_BATCH3
-#define SFC_BINARY_BATCH3 8
-#endif
-#ifndef SFC_PLAN_BLOCKS_BINARY
-#define SFC_PLAN_BLOCKS_BINARY 4
-#endif
-#ifndef SFC_PLAN_BLOCKS_LEARNED
-#define SFC_PLAN_BLOCKS_LEARNED 4
-#endif
-#ifndef SFC_LEARNED_BATCH
-#define SFC_LEARNED_BATCH 2
-#endif
+constexpr int kBinaryBatch = 4, kBinaryBatch3 = 8, kLearnedBatch = 2;
+constexpr int kPlanBlocksBinary = 4, kPlanBlocksLearned = 4;
 // Targets a warp searches per round: the flat list of its 32 queries' interval endpoints is
 // searched in rounds of at most this many (one round for nearly every warp: cover 1 averages
 // about 6.5 endpoints per query).  A multiple of 32.
-#ifndef SFC_PLAN_CAP
-#define SFC_PLAN_CAP 256
-#endif
-constexpr uint32_t kPlanCap = SFC_PLAN_CAP;
+constexpr uint32_t kPlanCap = 256;
 // Resident blocks per SM (the register budgets) of the count and the write pass.
-#ifndef SFC_COUNT_BLOCKS
-#define SFC_COUNT_BLOCKS 6
-#endif
-#ifndef SFC_WRITE_BLOCKS
-#define SFC_WRITE_BLOCKS 7
-#endif
+constexpr int kCountBlocks = 6, kWriteBlocks = 7;
 // Records whose ids a warp of the write pass has in flight.  Measured with the blocks that the
 // registers leave, 10^6 queries over 10^7 mixed points (10^7 over 10^8): two on 8 blocks 597 us (5.77 ms),
 // four on 8 588 (5.81), six on 7 553 (5.62), eight on 7 576 (5.77), on 6 632 (5.97).
@@ -148,8 +127,8 @@ template <int DIM>
 struct BinaryBounds {
     static constexpr bool kStats = false;
     // (3-D: the columns of cell keys leave few warps, which need more loads in flight)
-    static constexpr int kBatch = DIM == 3 ? SFC_BINARY_BATCH3 : SFC_BINARY_BATCH;
-    static constexpr int kMinBlocks = SFC_PLAN_BLOCKS_BINARY;
+    static constexpr int kBatch = DIM == 3 ? kBinaryBatch3 : kBinaryBatch;
+    static constexpr int kMinBlocks = kPlanBlocksBinary;
     const uint32_t* dir;
     int bits;
     uint64_t kmin, kmax;
@@ -193,8 +172,8 @@ struct BinaryBounds {
 
 struct LearnedBounds {
     static constexpr bool kStats = true;
-    static constexpr int kBatch = SFC_LEARNED_BATCH;
-    static constexpr int kMinBlocks = SFC_PLAN_BLOCKS_LEARNED;
+    static constexpr int kBatch = kLearnedBatch;
+    static constexpr int kMinBlocks = kPlanBlocksLearned;
     const RootParams* root;      // device; after prepare() the block's shared-memory copy
     const LeafParams* leaf;
     const uint64_t* fence;       // [leaves][kFence] coarse fence keys
@@ -997,7 +976,7 @@ __device__ __forceinline__ uint32_t lanemask_le() { return lanemask_lt() | (1u <
 // owner of the first and one load of the next 32 queries' first items (past the last query the
 // end of the list stands in, whose items belong to the query rank m: none).
 template <int GEOM>
-__global__ void __launch_bounds__(kThreads, SFC_COUNT_BLOCKS) count_kernel(QueryArgs a)
+__global__ void __launch_bounds__(kThreads, kCountBlocks) count_kernel(QueryArgs a)
 {
     chain_start();
     constexpr int kGroups = Geom<GEOM>::kGroups;
@@ -1141,7 +1120,7 @@ __device__ __forceinline__ void copy_records(const QueryArgs& a, bool fits, uint
 // writes, 1.0 warp instructions per id (11.4 ms and 2.2 with one warp per query,
 // whose dependent loads and per-hit shared-memory store set the time); 129 windows of 2*10^5 ids
 // 48.8 ms -> 0.07 ms, as no warp owns a query.
-__global__ void __launch_bounds__(kThreads, SFC_WRITE_BLOCKS) write_kernel(QueryArgs a)
+__global__ void __launch_bounds__(kThreads, kWriteBlocks) write_kernel(QueryArgs a)
 {
     chain_start();
     __shared__ CopySmem s_copy[kThreads / 32];

@@ -8,13 +8,7 @@ namespace sfc {
 // Groups of 32 points per item of the scan passes (powers of two: an item's boxes are loaded in
 // pairs).  2-D: four measured best (two and one: count 5.8 -> 6.6 and 9.4 ms at 10^8 mixed points);
 // 3-D: two (four the same, one 1.70 -> 2.32 ms at 10^7 points and 10^6 balls).
-#ifndef SFC_ITEM_GROUPS2
-#define SFC_ITEM_GROUPS2 4
-#endif
-#ifndef SFC_ITEM_GROUPS3
-#define SFC_ITEM_GROUPS3 2
-#endif
-constexpr int kItemGroups2 = SFC_ITEM_GROUPS2, kItemGroups3 = SFC_ITEM_GROUPS3;
+constexpr int kItemGroups2 = 4, kItemGroups3 = 2;
 inline uint64_t item_groups(int dim) { return dim == 3 ? kItemGroups3 : kItemGroups2; }
 
 struct QueryArgs {

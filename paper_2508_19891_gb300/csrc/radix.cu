@@ -48,19 +48,11 @@ constexpr int kRadix = 1 << kBits;
 constexpr int kPasses = 8;
 // threads of a pass's block, keys per thread of a tile, and resident blocks per SM (the register
 // budget)
-#ifndef SFC_SORT_THREADS
-#define SFC_SORT_THREADS 256
-#endif
-#ifndef SFC_SORT_ITEMS
-#define SFC_SORT_ITEMS 16
-#endif
-constexpr int kLookBack = 4;   // earlier tiles' words that a thread has in flight
-#ifndef SFC_SORT_BLOCKS
-#define SFC_SORT_BLOCKS 3
-#endif
-constexpr int kThreads = SFC_SORT_THREADS;
+constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
-constexpr int kItems = SFC_SORT_ITEMS;          // keys per thread: tiles of 4096 ...
+constexpr int kSortBlocks = 3;
+constexpr int kLookBack = 4;                    // earlier tiles' words that a thread has in flight
+constexpr int kItems = 16;                      // keys per thread: tiles of 4096 ...
 constexpr int kItemsSmall = 4;                  // ... and of 1024 while those do not fill the GPU
 static_assert(kThreads >= kRadix && kItems % 2 == 0, "thread d owns digit d; two ranks per word");
 constexpr int kHistThreads = 1024;
@@ -70,9 +62,7 @@ constexpr int kHistThreads = 1024;
 constexpr int kSampleLarge = 16384, kSampleSmall = 2048;
 constexpr uint64_t kSampleLargeFrom = 1ull << 22;
 constexpr uint64_t kSampleMin = 8192;           // shorter arrays are sorted by all digits
-#ifndef SFC_SORT_MEAN_RUN
-#define SFC_SORT_MEAN_RUN 16
-#endif
+constexpr uint64_t kMeanRun = 16;
 // Longest run that fix_kernel orders.
 constexpr uint32_t kMaxRun = 512;   // a power of two
 
@@ -150,12 +140,12 @@ __global__ void __launch_bounds__(1024) sample_kernel(SortSource src, uint64_t n
     const int all = (src.bits + kBits - 1) / kBits;
     const int top = live ? 63 - __clzll((long long)live) : 0;
     // pairs of short runs (all pairs there are: SAMPLE^2 / 2 < 2^27)
-    const uint32_t most = (uint32_t)min((uint64_t)SFC_SORT_MEAN_RUN * SAMPLE * SAMPLE / (2 * n), (uint64_t)SAMPLE * SAMPLE);
+    const uint32_t most = (uint32_t)min(kMeanRun * SAMPLE * SAMPLE / (2 * n), (uint64_t)SAMPLE * SAMPLE);
     int passes = 2;
     for (; passes < all; ++passes) {
         const int low = low_bits(src.bits, passes);
         // 2^(top + 1 - low) values of the sorted bits cannot keep n keys apart
-        if (top + 1 <= low || (top + 1 - low < 32 && ((uint64_t)SFC_SORT_MEAN_RUN << (top + 1 - low)) < n)) continue;
+        if (top + 1 <= low || (top + 1 - low < 32 && (kMeanRun << (top + 1 - low)) < n)) continue;
         for (uint32_t i = threadIdx.x; i < kSlots + kSlots / 2; i += 1024) s_slots[i] = 0;
         if (threadIdx.x == 0) s_pairs = 0;
         __syncthreads();
@@ -390,7 +380,7 @@ __device__ __forceinline__ void rank_keys(const uint64_t (&key)[ITEMS], int shif
 // blocks per SM), 256 of 24 6.0; the next tile's keys loaded during the look-back 5.5 instead of
 // 5.9; the values loaded before the warps are combined 5.9.
 template <int CURVE, int ITEMS>
-__global__ void __launch_bounds__(kThreads, SFC_SORT_BLOCKS) onesweep_kernel(PassArgs a)
+__global__ void __launch_bounds__(kThreads, kSortBlocks) onesweep_kernel(PassArgs a)
 {
     chain_start();
     const PassPlan pl = a.sm->plan[a.pass];
@@ -552,10 +542,7 @@ __device__ __forceinline__ void store_final(const SortDest& dst, const HilbertTa
     }
 }
 
-#ifndef SFC_FIX_BLOCKS
-#define SFC_FIX_BLOCKS 4
-#endif
-constexpr int kFixThreads = 256;
+constexpr int kFixThreads = 256, kFixBlocks = 4;   // four blocks per SM
 constexpr int kFixItems = 8;
 constexpr int kFixTile = kFixThreads * kFixItems;
 constexpr int kFixHalo = 64;                         // neighbours kept on each side of the tile
@@ -570,7 +557,7 @@ static_assert(kFixSpan <= 1 << kFixAt && kFixHalo * 2 <= kFixThreads, "");
 // comparison decides ties too).  Bound by HBM (12 bytes read, 20 written per key) and the counting:
 // 10^8 mixed points in runs of 16 on average 0.89 ms.
 template <int CURVE>
-__global__ void __launch_bounds__(kFixThreads, SFC_FIX_BLOCKS) fix_kernel(PassArgs a)
+__global__ void __launch_bounds__(kFixThreads, kFixBlocks) fix_kernel(PassArgs a)
 {
     chain_start();
     const uint32_t low = a.sm->low;
@@ -796,14 +783,14 @@ void launch_pass(const PassArgs& a, cudaStream_t st)
     static bool ok[64] = {false};
     allow_smem((const void*)onesweep_kernel<CURVE, ITEMS>, sizeof(PassSmem<ITEMS>), ok);
     const uint32_t tiles = tiles_of(a.n, kThreads * ITEMS);
-    const unsigned grid = (unsigned)std::min<uint64_t>(tiles, (uint64_t)num_sms() * SFC_SORT_BLOCKS);
+    const unsigned grid = (unsigned)std::min<uint64_t>(tiles, (uint64_t)num_sms() * kSortBlocks);
     launch_chain(onesweep_kernel<CURVE, ITEMS>, grid, kThreads, sizeof(PassSmem<ITEMS>), st, a);
     count_launch();
 }
 
 // Tiles of 1024 keys while they are all resident at once: a pass is then one short chain per
 // block.
-bool small_tiles(uint64_t n) { return n <= (uint64_t)kThreads * kItemsSmall * num_sms() * SFC_SORT_BLOCKS; }
+bool small_tiles(uint64_t n) { return n <= (uint64_t)kThreads * kItemsSmall * num_sms() * kSortBlocks; }
 
 template <int CURVE>
 sfc_status run_sort(const PassArgs& args, uint32_t* epoch, cudaStream_t st)
@@ -863,7 +850,7 @@ sfc_status reserve_sort(SortWorkspace& ws, uint64_t n, cudaStream_t st)
 {
     // the look-back words of the small tiles' longest array cover shorter ones with larger tiles
     const uint64_t per = kThreads * (small_tiles(n) ? kItemsSmall : kItems);
-    const uint64_t most = (uint64_t)num_sms() * SFC_SORT_BLOCKS;   // small tiles at their limit
+    const uint64_t most = (uint64_t)num_sms() * kSortBlocks;   // small tiles at their limit
     const uint64_t tiles = std::max((n + per - 1) / per, std::min((n + kThreads * kItemsSmall - 1) / (kThreads * kItemsSmall), most));
     for (int i = 0; i < 2; ++i) {
         SFC_TRY(ws.tmp_keys[i].ensure(n * sizeof(uint64_t), st));

@@ -47,7 +47,7 @@ inline sfc_status launch_status()
 // chain_start(), which waits until the one before has completed with its writes visible, so
 // nothing it touches is still in use.  After any other stream operation the launch is an ordinary
 // one.  Takes part of the gaps between launches, which set the time of small calls (one lookup 68 ->
-// 54 us, 3*10^5 points built and queried 185 -> 129 us, an update of 5*10^7 points 810 -> 725 us).
+// 62 us, 3*10^5 points built and queried 185 -> 129 us, an update of 5*10^7 points 810 -> 725 us).
 // No kernel lets the next one go before its own blocks end: waiting blocks would take room beside
 // working ones (let go at its start by every kernel, 10^7 3-D points with 10^6 balls took 5.35 ms
 // instead of 3.96, by grids of up to 456 blocks 10^8 points with 10^7 queries 20.7 instead of 19.6).
