@@ -211,9 +211,10 @@ class ClockSampler:
 # roofline of the two query kernels
 # --------------------------------------------------------------------------------------
 
-# Warp instructions that the method itself needs per 32 scanned points in the count pass:
-# one 8-byte load per lane, dx and dy, the two squares as 32x32 -> 64-bit multiply(-add)s,
-# the 64-bit compare against delta^2 (two instructions) and the ballot.
+# Warp instructions that testing every scanned point takes per 32 of them in the count pass: one
+# 8-byte load per lane, dx and dy, the two squares as 32x32 -> 64-bit multiply(-add)s, the 64-bit
+# compare against delta^2 (two instructions) and the ballot.  A common scale for the scans, not
+# what the pass needs: most groups are settled by their bounding box, without reading their points.
 COUNT_MIN_WARP_INST_PER_32 = 8
 
 
@@ -238,6 +239,15 @@ def committed_traffic(kernel: str, workload: str):
         return None
 
 
+def split_phases(phase):
+    """(build, fit, query) ms of a step from its phases: keys, sort and decode with the group boxes
+    and the key directory (a 3-D sort phase contains them); the model fit; every phase of the
+    query batch.  The early-termination bitmap's phase is in none of them."""
+    build = phase.get("sort", float("nan")) + phase.get("boxes", 0.0)
+    query = sum(v for k, v in phase.items() if k not in ("sort", "boxes", "train", "occupancy"))
+    return build, phase.get("train", 0.0), query
+
+
 def query_rooflines(agg, scanned: int, hits: int, dim: int, hbm_peak: float, peak_kind: str,
                     workload: str = WORKLOAD, sm_count: int = 152, sm_mhz: float = 2070.0):
     """Roofline objects of the two query passes, the one with the longer time first.  The count
@@ -247,9 +257,11 @@ def query_rooflines(agg, scanned: int, hits: int, dim: int, hbm_peak: float, pea
 
     write_kernel, bound by HBM: the method must read every reported id and write it, 8 B per
     hit (the hit mask is the two-pass implementation's own traffic and is not counted).
-    count_kernel, bound by instruction issue (the coordinates mostly come from L2, so the HBM
-    roof does not bind): the method needs COUNT_MIN_WARP_INST_PER_32 warp instructions per 32
-    scanned points, against an issue peak of 4 warp instructions per SM and cycle.  Both carry
+    count_kernel, bound by instruction issue (boxes and coordinates mostly come from L2, so the
+    HBM roof does not bind), against an issue peak of 4 warp instructions per SM and cycle:
+    executed_frac is the instructions of the committed capture over the time; achieved and frac
+    are the instructions of testing every scanned point (COUNT_MIN_WARP_INST_PER_32 per 32), an
+    equivalent rate, of which settling groups by their box saves a part.  Both carry
     the DRAM traffic of a committed ncu capture of the same kernel source and workload, as a
     fraction of the measured copy peak (dram_frac) and of the nominal 8 TB/s.
     agg maps a phase name to (launches, total ms) from the CUDA events of the timed steps."""
@@ -276,15 +288,17 @@ def query_rooflines(agg, scanned: int, hits: int, dim: int, hbm_peak: float, pea
                       "algorithmic_bytes": alg, "algorithmic": "8 B per reported id (read + write)"})
         else:
             inst = COUNT_MIN_WARP_INST_PER_32 * scanned / 32.0
+            executed = rec.get("inst_per_scanned_point")
             ach = inst / (avg / 1e3) / 1e9
             peak = sm_count * WARP_SCHEDULERS_PER_SM * sm_mhz * 1e6 / 1e9
             o.update({"bound": "alu", "achieved": ach, "peak": peak, "unit": "G warp-inst/s", "frac": ach / peak,
                       "peak_kind": f"issue rate: {sm_count} SMs x {WARP_SCHEDULERS_PER_SM} warp instructions per "
                                    f"cycle at {sm_mhz:.0f} MHz",
                       "algorithmic_inst": inst,
-                      "algorithmic": f"{COUNT_MIN_WARP_INST_PER_32} warp instructions per 32 scanned points",
-                      "executed_inst_per_32_points": (32 * rec["inst_per_scanned_point"]
-                                                      if rec.get("inst_per_scanned_point") else None),
+                      "algorithmic": f"{COUNT_MIN_WARP_INST_PER_32} warp instructions per 32 scanned points, as if "
+                                     "each were tested",
+                      "executed_inst_per_32_points": 32 * executed if executed else None,
+                      "executed_frac": executed * scanned / (avg / 1e3) / 1e9 / peak if executed else None,
                       "effective_gbs": 4 * dim * scanned / (avg / 1e3) / 1e9})
         out.append(o)
     out.sort(key=lambda k: -k["avg_launch_ms"])
@@ -457,9 +471,7 @@ class StaticBench:
         dominant, others = query_rooflines({k: (v[0], v[1]) for k, v in per.items()}, S, H, self.dim,
                                            hbm_peak, peak_kind, args.workload, sm_count, sm_mhz)
         phase = {k: v[1] for k, v in per.items()}
-        build_ms = phase.get("sort", float("nan"))
-        fit_ms = phase.get("train", 0.0)
-        query_ms = sum(v for k, v in phase.items() if k not in ("sort", "train", "occupancy"))
+        build_ms, fit_ms, query_ms = split_phases(phase)
         config = {"workload": args.workload, "n": wl.n, "m": wl.m, "dim": self.dim, "curve": self.curve,
                   "bounds": self.bounds, "window": self.norm,
                   **({"rel_side": args.rel_side} if args.workload.startswith("paper-") or

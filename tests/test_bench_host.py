@@ -122,3 +122,19 @@ def test_tuning_flag():
                  ["--tuning", "4096,16,2", "--cover", "1", "--workload", "dynamic-5e7"]):
         with pytest.raises(SystemExit):
             bench.parse(argv)
+
+
+def test_phases_of_a_step():
+    """The group boxes belong to the build, not to the query phase; 3-D steps time them in the sort."""
+    phase = {"sort": 4.0, "boxes": 0.25, "train": 0.8, "occupancy": 0.1, "order": 0.5, "plan": 2.0, "scan": 0.2,
+             "count": 5.0, "write": 5.5}
+    assert bench.split_phases(phase) == pytest.approx((4.25, 0.8, 13.2))
+    assert bench.split_phases({"sort": 0.5, "plan": 0.75, "count": 1.5}) == pytest.approx((0.5, 0.0, 2.25))
+
+
+def test_executed_share_of_the_issue_peak(tmp_path, monkeypatch):
+    _write_record(tmp_path, "// kernel source\n", {"count_kernel": {"w1": {"inst_per_scanned_point": 0.5, "command": "ncu y"}}})
+    monkeypatch.setattr(bench, "ROOT", str(tmp_path))
+    dom, _ = bench.query_rooflines({"count": (1, 2.0), "write": (1, 1.0)}, 10 ** 9, 10, 2, 4000.0, "measured", "w1", 100, 2000.0)
+    assert dom["kernel"] == "count_kernel"
+    assert dom["executed_frac"] == pytest.approx(0.5 * 10 ** 9 / 2e-3 / (100 * 4 * 2000e6))
