@@ -596,8 +596,8 @@ sfc_status sfc_reserve(sfc_index* idx, uint64_t n_max, uint64_t m_max, void* str
         SFC_TRY(idx->occ.ensure(occupancy_words(idx->opt.occupancy_depth) * sizeof(uint32_t), st));
     SFC_TRY(reserve_sort(idx->sort_ws, n1, st));
     // (a directory doubles at powers of two, where the arrays above may have room left and stay)
-    SFC_TRY(idx->box.grow(box_bytes(idx->dim, n1), st));
-    SFC_TRY(idx->dir.grow(dir_bytes(n1), st));
+    SFC_TRY(idx->box.grow(box_bytes(idx->dim, n1), box_bytes(idx->dim, idx->n), st));
+    SFC_TRY(idx->dir.grow(dir_bytes(n1), dir_bytes(idx->n), st));
     idx->qws.refused = ~0ull;
     SFC_TRY(ensure_query_ws(idx, m_max, st));
     SFC_TRY(reserve_scan(idx->scan_ws, std::max<uint64_t>(m_max, n1) + 1, st));

@@ -856,7 +856,7 @@ __device__ __forceinline__ void filter_init(FilterSmem<GEOM>* sm)
 // Groups that need their points looked at are gathered in shared memory and taken four at a
 // time, so that four coalesced loads are in flight.  The points' array is padded to whole
 // groups.  Every lane of the warp calls.
-// Bound by instruction issue: a group's side, mask and shared-memory slot are made in one step (all
+// Much of the pass is instruction issue: a group's side, mask and shared-memory slot are made in one step (all
 // classes first, then masks, then slots: count pass of 10^6 queries over 10^7 mixed points 586 us
 // against 564, square windows over Normal points 120 against 110), with masks of two clamped shifts.
 template <int GEOM>
@@ -963,10 +963,11 @@ __device__ __forceinline__ uint32_t lanemask_le() { return lanemask_lt() | (1u <
 // ------------------------------------------------------------------------------------
 // count_kernel
 // ------------------------------------------------------------------------------------
-// Bound by instruction issue (about 60% of it; the points and boxes come from L2), so the design
-// spends as few instructions per scanned point as it can: a lane settles 32 points with one box
-// (about 12 instructions), a warp tests 32 points with about 10, and only where a box is cut by the
-// window's edge.  Measured, count pass only, before (every scanned point tested, a warp per chunk
+// Bound by instruction issue and by the latency of the boxes and points, which come from L2: it issues in
+// 60% of its cycles at 10^6 queries over 10^7 points and 68% at 10^7 over 10^8, and its warps wait on
+// loads for most of the rest (43 of 64 resident).  So the design spends as few instructions per
+// scanned point as it can: a lane settles 32 points with one box (about 12 instructions), a warp
+// tests 32 points with about 10, and only where a box is cut by the window's edge.  Measured, count pass only, before (every scanned point tested, a warp per chunk
 // of one query) and now: 10^7 queries over 10^8 mixed points, cover 1 (1.48*10^10 scanned points)
 // 12.8 -> 5.4 ms; 10^6 over 10^7 1.20 -> 0.56 ms; 10^6 3-D balls over 10^7 3.87 -> 1.66 ms.  Blocks per
 // SM, 10^6 over 10^7 mixed points / Normal points and square windows / 3-D: five 592 / 114 / 1637 us,
@@ -1115,8 +1116,9 @@ __device__ __forceinline__ void copy_records(const QueryArgs& a, bool fits, uint
 }
 
 // The records of the items of the queries of processing ranks [q_begin, q_end).  Bound by the
-// latency of record, id and store and by the L2 (most ids are read from it, all are written once to HBM,
-// 3.6 TB/s): 4.25*10^9 ids of 10^7 queries over 10^8 mixed points in 5.6 ms, 6.1 TB/s of id reads and
+// latency of record, id and store (most ids are read from the L2, all are written once to HBM, 3.6
+// TB/s) about as much as by issue (66% of its cycles at 10^6 queries over 10^7 points, with 62 of 64
+// warps resident; the L1 at 73% of its rate): 4.25*10^9 ids of 10^7 queries over 10^8 mixed points in 5.6 ms, 6.1 TB/s of id reads and
 // writes, 1.0 warp instructions per id (11.4 ms and 2.2 with one warp per query,
 // whose dependent loads and per-hit shared-memory store set the time); 129 windows of 2*10^5 ids
 // 48.8 ms -> 0.07 ms, as no warp owns a query.

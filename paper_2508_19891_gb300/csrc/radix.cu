@@ -374,8 +374,9 @@ __device__ __forceinline__ void rank_keys(const uint64_t (&key)[ITEMS], int shif
     }
 }
 
-// Bound by latency and shared-memory traffic, not yet by HBM (24 bytes per key and pass: 10^8 keys
-// 0.70 ms, 3.4 TB/s; 0.83 ms with one block per tile, ballots and one look-back word at a time).
+// Bound by shared memory (its pipe at 74% of its rate, more than half of its wavefronts bank conflicts)
+// and by the latency of the key loads with 24 warps per SM, not yet by HBM (24 bytes per key and pass:
+// 10^8 keys 0.70 ms, 3.4 TB/s; 0.83 ms with one block per tile, ballots and one look-back word at a time).
 // Measured at 10^8 mixed points (build): 256 threads of 16 keys 5.5 ms, 512 of 8 6.1, of 16 8.2 (two
 // blocks per SM), 256 of 24 6.0; the next tile's keys loaded during the look-back 5.5 instead of
 // 5.9; the values loaded before the warps are combined 5.9.
@@ -554,8 +555,9 @@ static_assert(kFixSpan <= 1 << kFixAt && kFixHalo * 2 <= kFixThreads, "");
 // Orders the runs of keys that agree in the sorted bits.  A bit per key marks where a run begins;
 // a key of a run of one keeps its place, any other counts the keys of its run that come before it
 // (all lanes of a run read the same shared-memory word: the low bits, then the place, so that one
-// comparison decides ties too).  Bound by HBM (12 bytes read, 20 written per key) and the counting:
-// 10^8 mixed points in runs of 16 on average 0.89 ms.
+// comparison decides ties too).  Bound by the issue of the counting (72%
+// of its cycles, the integer pipe at 70%) before HBM (12 bytes read, 20 written per key, 3.7 TB/s):
+// 10^8 mixed points in runs of up to 16 on average 0.89 ms.
 template <int CURVE>
 __global__ void __launch_bounds__(kFixThreads, kFixBlocks) fix_kernel(PassArgs a)
 {

@@ -145,13 +145,14 @@ struct DevBuf {
         bytes = nb;
         return SFC_OK;
     }
-    // the same, keeping the contents; a failure leaves the buffer as it is
-    sfc_status grow(size_t need, cudaStream_t st)
+    // the same, keeping the first `keep` bytes; a failure leaves the buffer as it is
+    sfc_status grow(size_t need, size_t keep, cudaStream_t st)
     {
         if (need <= bytes) return SFC_OK;
         DevBuf nb;
         SFC_TRY(nb.ensure(need, st));
-        if (ptr && cudaMemcpyAsync(nb.ptr, ptr, bytes, cudaMemcpyDeviceToDevice, st) != cudaSuccess) {
+        keep = keep < bytes ? keep : bytes;
+        if (keep && cudaMemcpyAsync(nb.ptr, ptr, keep, cudaMemcpyDeviceToDevice, st) != cudaSuccess) {
             nb.release(st);
             return SFC_ERR_CUDA;
         }

@@ -333,33 +333,21 @@ sfc_status apply_update(sfc_index* idx, const int32_t* d_inserts, uint64_t k_ins
         SFC_CUDA_TRY(cudaStreamSynchronize(st));
         if (hbad) return SFC_ERR_NOT_FOUND;   // nothing has been changed yet
     }
-    // ---- every buffer that the batch needs, before anything of the index changes: a batch that
-    // finds no memory leaves the index as it was (those that hold its contents grow with them) ----
+    // ---- inserts: keys, sort, decoded coordinates ----
     const uint64_t new_n = (uint64_t)n - k_del + k_ins;
     const uint64_t ids_after = (uint64_t)next_id + k_ins;
-    SFC_TRY(U.keys.ensure(std::max<uint64_t>(new_n, 1) * 8, st));
-    SFC_TRY(U.ids.ensure(std::max<uint64_t>(new_n, 1) * 4, st));
-    SFC_TRY(U.xy.ensure(pad_groups(std::max<uint64_t>(new_n, 1)) * 8, st));
-    SFC_TRY(U.istart.ensure(((size_t)tiles + 1) * sizeof(uint32_t), st));
-    SFC_TRY(idx->box.grow(box_bytes(2, new_n), st));
-    SFC_TRY(idx->dir.grow(dir_bytes(new_n), st));
-    if (idx->model.trained) SFC_TRY(reserve_model(idx, new_n, st));
+    uint64_t* ikeys = nullptr;
+    uint32_t* iids = nullptr;
+    int2* ixy = nullptr;
+    uint32_t* irank = nullptr;
     if (k_ins) {
         SFC_TRY(U.e.ensure(k_ins * 8, st));
         SFC_TRY(U.f.ensure(k_ins * 4, st));
         SFC_TRY(U.g.ensure(k_ins * 8, st));
         SFC_TRY(U.h.ensure(k_ins * 4, st));
         if (ids_after * sizeof(uint64_t) > idx->key_by_id.bytes)
-            SFC_TRY(idx->key_by_id.grow(ids_after * sizeof(uint64_t) + ids_after * sizeof(uint64_t) / 2, st));
-        SFC_TRY(ensure_alive_bits(idx, ids_after, st));
-        SFC_TRY(reserve_sort(idx->sort_ws, k_ins, st));
-    }
-    // ---- inserts: keys, sort, decoded coordinates ----
-    uint64_t* ikeys = nullptr;
-    uint32_t* iids = nullptr;
-    int2* ixy = nullptr;
-    uint32_t* irank = nullptr;
-    if (k_ins) {
+            SFC_TRY(idx->key_by_id.grow(ids_after * sizeof(uint64_t) + ids_after * sizeof(uint64_t) / 2,
+                                        (size_t)next_id * sizeof(uint64_t), st));
         ikeys = U.e.as<uint64_t>();
         iids = U.f.as<uint32_t>();
         ixy = U.g.as<int2>();
@@ -379,6 +367,16 @@ sfc_status apply_update(sfc_index* idx, const int32_t* d_inserts, uint64_t k_ins
         dst.curve = curve;
         SFC_TRY(radix_sort(src, k_ins, dst, idx->sort_ws, status, st));
     }
+    // ---- every other buffer that the batch needs (while the sort runs), before anything of the index
+    // changes: a batch that finds no memory leaves it as it was; those that hold contents keep them ----
+    SFC_TRY(U.keys.ensure(std::max<uint64_t>(new_n, 1) * 8, st));
+    SFC_TRY(U.ids.ensure(std::max<uint64_t>(new_n, 1) * 4, st));
+    SFC_TRY(U.xy.ensure(pad_groups(std::max<uint64_t>(new_n, 1)) * 8, st));
+    SFC_TRY(U.istart.ensure(((size_t)tiles + 1) * sizeof(uint32_t), st));
+    SFC_TRY(idx->box.grow(box_bytes(2, new_n), box_bytes(2, n), st));
+    SFC_TRY(idx->dir.grow(dir_bytes(new_n), dir_bytes(n), st));
+    if (k_ins) SFC_TRY(ensure_alive_bits(idx, ids_after, st));
+    if (idx->model.trained) SFC_TRY(reserve_model(idx, new_n, st));
     // ---- shift counts and the new arrays ----
     uint32_t* istart = U.istart.as<uint32_t>();
     const uint64_t* keys = idx->keys.as<uint64_t>();
