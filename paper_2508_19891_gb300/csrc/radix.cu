@@ -181,7 +181,7 @@ constexpr int kHistRow = 16;
 constexpr uint64_t kHistMost = 65000ull * 32;
 
 // Histograms of the sorted digits, one read of the input; the keys of a sort of points are written
-// out for the first pass.  Bound by HBM: 10^8 points, four digits 0.59 -> 0.47 ms (one shared counter
+// out for the first pass.  16 bytes per key: 10^8 points, four digits 0.59 -> 0.47 ms, 3.4 TB/s (one shared counter
 // per digit, keys computed again by the first pass).
 template <int CURVE>
 __global__ void __launch_bounds__(kHistThreads) hist_kernel(SortSource src, uint64_t n, uint64_t* keys_out, Small* sm,
