@@ -599,7 +599,8 @@ sfc_status sfc_reserve(sfc_index* idx, uint64_t n_max, uint64_t m_max, void* str
     SFC_TRY(idx->box.grow(box_bytes(idx->dim, n1), box_bytes(idx->dim, idx->n), st));
     SFC_TRY(idx->dir.grow(dir_bytes(n1), dir_bytes(idx->n), st));
     idx->qws.refused = ~0ull;
-    SFC_TRY(ensure_query_ws(idx, m_max, st));
+    // (not fewer queries than before: what an earlier reserve or batch sized stays sized)
+    SFC_TRY(ensure_query_ws(idx, std::max(m_max, idx->qws.sized_m), st));
     SFC_TRY(reserve_scan(idx->scan_ws, std::max<uint64_t>(m_max, n1) + 1, st));
     if (idx->opt.bounds == SFC_BOUNDS_LEARNED) SFC_TRY(reserve_model(idx, n1, st));
     return SFC_OK;

@@ -280,3 +280,23 @@ def test_rebuild_without_memory_leaves_an_empty_index(cuda, dim, options):
     idx.close()
     torch.cuda.synchronize()
     assert not A.live
+
+
+def test_reserve_for_fewer_queries_keeps_what_was_reserved(cuda):
+    """sfc_reserve for many points and few queries, after batches of many queries: rebuilds within it
+    and batches of either size allocate nothing."""
+    rng = np.random.default_rng(8)
+    pts = rng.integers(0, 1 << 16, size=(300_000, 2)).astype(np.int32)
+    q, d = to_dev(pts[:5000], cuda), torch.full((5000,), 300, dtype=torch.int32, device=cuda)
+    A = sfc.TorchAllocator(cuda)
+    idx = sfc.sfc_build(to_dev(pts[:20_000], cuda), "z", allocator=A)
+    sfc.query(idx, q, d)
+    sfc.sfc_reserve(idx, len(pts), 10)
+    before = (A.allocs, A.frees)
+    sfc.sfc_rebuild(idx, to_dev(pts, cuda))
+    for m in (10, 5000):
+        off, ids = sfc.query(idx, q[:m].contiguous(), d[:m].contiguous())
+        roff, rids = oracle.query(oracle.build(pts), pts[:m], np.full(m, 300, np.int32))
+        assert np.array_equal(u64(off), roff) and np.array_equal(u32(ids), rids)
+    assert (A.allocs, A.frees) == before and sfc.sfc_device_status(idx) == (0, 0)
+    idx.close()
