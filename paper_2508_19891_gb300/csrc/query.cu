@@ -285,7 +285,9 @@ struct LearnedBounds {
                 N = max(N, len[x]);
             }
             // pad every range to the longest: [lo, lo + N) still holds the answer, moved left
-            // where it would run past the end of the array
+            // where it would run past the end of the array (a model kept over a rebuild that did not
+            // fit it again may bracket more keys than there are)
+            N = min(N, n);
             uint32_t lo0[E];
 #pragma unroll
             for (int x = 0; x < E; ++x) {

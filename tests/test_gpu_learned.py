@@ -273,3 +273,22 @@ def test_leaf_stage_matches_oracle(cuda, curve, root, kind):
         checked += c
     assert checked == n   # every key of every leaf was checked
     idx.close()
+
+
+@pytest.mark.parametrize("left", [0, 1, 2, 33, 400])
+def test_model_kept_over_a_rebuild_with_few_points(cuda, left):
+    """A model trained by hand on an index built with binary bounds stays when the index is rebuilt over
+    far fewer points than its leaves bracket: the learned search stays inside the array and right."""
+    rng = np.random.default_rng(left)
+    pts = (rng.normal(1 << 29, 1 << 20, size=(200_000, 2))).astype(np.int32)
+    few = rng.integers(0, 1 << 30, size=(left, 2)).astype(np.int32)
+    q = np.concatenate([few, pts[:50]])
+    d = np.full(len(q), 1 << 24, np.int32)
+    idx = sfc.sfc_build(to_dev(pts, cuda), "z", leaves=16)
+    sfc.sfc_train_model(idx)
+    sfc.sfc_set_bounds_mode(idx, "learned")
+    sfc.sfc_rebuild(idx, to_dev(few, cuda))
+    off, ids = sfc.query(idx, to_dev(q, cuda), to_dev(d, cuda))
+    roff, rids = oracle.query(oracle.build(few), q, d)
+    assert np.array_equal(u64(off), roff) and np.array_equal(u32(ids), rids)
+    assert sfc.sfc_device_status(idx) == (0, 0)
