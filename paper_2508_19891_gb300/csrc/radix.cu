@@ -56,13 +56,17 @@ constexpr int kItems = 16;                      // keys per thread: tiles of 409
 constexpr int kItemsSmall = 4;                  // ... and of 1024 while those do not fill the GPU
 static_assert(kThreads >= kRadix && kItems % 2 == 0, "thread d owns digit d; two ranks per word");
 constexpr int kHistThreads = 1024;
-// Sample: keys looked at (large arrays; smaller ones), and the mean run length up to which fewer
-// passes pay (a run of L keys costs each of them L comparisons in shared memory, a pass 24 bytes
-// of traffic and the ranking).
+// Sample: keys looked at (large arrays; smaller ones), and the mean number of others in a key's run
+// up to which fewer passes are made (a run of L keys costs each of them L comparisons in shared
+// memory, a pass 24 bytes of traffic and the ranking).
 constexpr int kSampleLarge = 16384, kSampleSmall = 2048;
 constexpr uint64_t kSampleLargeFrom = 1ull << 22;
 constexpr uint64_t kSampleMin = 8192;           // shorter arrays are sorted by all digits
-constexpr uint64_t kMeanRun = 16;
+// Fewer passes were faster at every mean measured: builds of 10^6 uniform points in runs of 16 78.9 us,
+// 88.2 with a pass more, of 1.6*10^6 in runs of 24 96.4 and 105.6; sorts of 1.7*10^7 keys in runs of 16 599 and
+// 666 us, of 3.4*10^7 in runs of 32 1195 and 1250.  The line is lower, as the estimate scatters by 8 to
+// 20% and the runs of uneven points are partly much longer than the mean.
+constexpr uint64_t kMeanRun = 20;
 // Longest run that fix_kernel orders.
 constexpr uint32_t kMaxRun = 512;   // a power of two
 
@@ -109,7 +113,8 @@ __device__ __forceinline__ uint64_t source_key(const SortSource& s, const Hilber
 }
 
 // Chooses the number of passes (one block).  Of S sampled keys, C pairs agree in their top bits: the
-// run of a key is about n * 2 C / S^2 keys long, itself counted (a position may be drawn twice).
+// run of a key is about n * 2 C / S^2 keys long, itself counted (a position may be drawn twice): at most
+// kMeanRun others and itself.
 template <int CURVE, int SAMPLE>
 __global__ void __launch_bounds__(1024) sample_kernel(SortSource src, uint64_t n, Small* sm)
 {
@@ -123,7 +128,7 @@ __global__ void __launch_bounds__(1024) sample_kernel(SortSource src, uint64_t n
     constexpr int K = SAMPLE / 1024;
     uint64_t key[K], live = 0;
 #pragma unroll
-    for (int i = 0; i < K; ++i) key[i] = source_key<CURVE>(src, &tb, sample_position(i * 1024 + threadIdx.x, n));
+    for (int i = 0; i < K; ++i) key[i] = source_key<CURVE>(src, &tb, sample_position(i * 1024 + threadIdx.x, SAMPLE, n));
     // bits in which the sampled keys differ: passes above them leave one run
     const uint64_t first = source_key<CURVE>(src, &tb, 0);
 #pragma unroll
@@ -140,7 +145,7 @@ __global__ void __launch_bounds__(1024) sample_kernel(SortSource src, uint64_t n
     const int all = (src.bits + kBits - 1) / kBits;
     const int top = live ? 63 - __clzll((long long)live) : 0;
     // pairs of short runs (all pairs there are: SAMPLE^2 / 2 < 2^27)
-    const uint32_t most = (uint32_t)min(kMeanRun * SAMPLE * SAMPLE / (2 * n), (uint64_t)SAMPLE * SAMPLE);
+    const uint32_t most = (uint32_t)min((kMeanRun + 1) * SAMPLE * SAMPLE / (2 * n), (uint64_t)SAMPLE * SAMPLE);
     int passes = 2;
     for (; passes < all; ++passes) {
         const int low = low_bits(src.bits, passes);

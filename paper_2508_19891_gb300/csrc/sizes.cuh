@@ -16,19 +16,22 @@ namespace sfc {
 // arrays that a sort takes (n < 2^32 - 1).
 SFC_HD uint32_t tiles_of(uint64_t n, uint32_t per) { return (uint32_t)((n + per - 1) / per); }
 
-// Position of sample number i among n elements (n < 2^32): a fixed hash of i (the finaliser of
-// SplitMix64, Steele, Lea & Flood 2014), scaled to n.  Every sample falls anywhere, independently of
-// the others, so pairs of samples meet in a run as often as pairs of keys do whatever the order of
-// the input.  (At positions n i / S two samples of sorted input share a run only if it is n / S long,
-// and input that interleaves kinds of points with a period of n / S shows one kind alone: 10^7 mixed
-// points given in curve order were built in 827 us, 518 now as when shuffled; 2^24 keys of which every
-// second lies in one dense part were sorted in 8.7 ms, 1.0 now.)
-SFC_HD uint64_t sample_position(uint32_t i, uint64_t n)
+// Position of sample number i of `samples` among n elements (n < 2^32; a multiple of 32 samples): each 32
+// consecutive samples fall into one of samples / 32 equal parts of the array, anywhere in it, by a fixed
+// hash of i (the finaliser of SplitMix64, Steele, Lea & Flood 2014).  Two samples of a part meet in a
+// run as often as two of its keys do, whatever the order of the input.  (At positions n i / S two
+// samples of sorted input share a run only if it is n / S long, and input that interleaves kinds of
+// points with a period of n / S shows one kind alone: 10^7 mixed points given in curve order were built
+// in 827 us, 518 now as when shuffled; 2^24 keys of which every second lies in one dense part were
+// sorted in 8.7 ms, 1.0 now.)  A part is what a warp loads at once: 16,384 samples of 6.4*10^6 points
+// scattered over the whole array took 5 us longer, for their address translations.
+SFC_HD uint64_t sample_position(uint32_t i, uint32_t samples, uint64_t n)
 {
     uint64_t z = (i + 1ull) * 0x9e3779b97f4a7c15ull;
     z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ull;
     z = (z ^ (z >> 27)) * 0x94d049bb133111ebull;
-    return (((z ^ (z >> 31)) >> 32) * n) >> 32;
+    const uint64_t parts = samples / 32, part = i / 32, first = n * part / parts;
+    return first + ((((z ^ (z >> 31)) >> 32) * (n * (part + 1) / parts - first)) >> 32);
 }
 
 // Buffers of the hits of a query batch: per-batch heads and hit counts, and records.
